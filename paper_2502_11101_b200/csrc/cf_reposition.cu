@@ -11,6 +11,16 @@ namespace cf {
 
 constexpr int kRepoThreads = 256;
 constexpr int kRepoUnroll = 4;
+constexpr int kRepoPass = kRepoThreads * kRepoUnroll;       // work items a block of the re-positioning kernel takes at a time
+
+// Blocks a key tile is cut into.  One block per tile streams a large store at the copy rate, but a few surviving
+// documents of many heads are a few dozen blocks of a megabyte each, most SMs idle and every block a chain of
+// round trips to memory (ten documents of 160 rows, 32 heads: 61 us, cut into pieces 7.8 us).  Tiles are cut until the grid has about four times the
+// blocks the device holds (eight of 256 threads per SM); a block keeps at least one pass of work.
+static int pieces_per_tile(long long tiles, int passes) {
+    const long long want = 32LL * sm_count();
+    return (int)std::max<long long>(1, std::min<long long>(passes, (want + tiles - 1) / std::max<long long>(1, tiles)));
+}
 
 template <typename T> struct Vec16;
 template <> struct Vec16<__nv_bfloat16> { static constexpr int kElems = 8; };
@@ -58,7 +68,7 @@ __device__ __forceinline__ uint4 pack<float>(const float (&f)[4]) {
 template <typename T, int D, int LAYOUT>
 __global__ void __launch_bounds__(kRepoThreads)
 reposition_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_stride,
-                  const T* k_in, T* k_out) {
+                  const T* k_in, T* k_out, int pieces) {
     constexpr int E = Vec16<T>::kElems;
     constexpr int kVecPerHead = D / E;                                    // 16-byte vectors per (row, head)
     constexpr int kItemsPerHead = LAYOUT == CF_ROPE_HALF ? kVecPerHead / 2 : kVecPerHead;
@@ -72,13 +82,14 @@ reposition_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_str
     T* dst = k_out + (long long)layer * layer_stride;
     const int items_per_row = n_kv_heads * kItemsPerHead;
 
-    for (int ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
+    const int piece = blockIdx.x % pieces, tile_step = gridDim.x / pieces;   // the grid is a multiple of `pieces`
+    for (int ti = blockIdx.x / pieces; ti < n_tiles; ti += tile_step) {
         const int doc = pv.tile_doc[base + ti];
         const long long row0 = pv.tile_row0[base + ti];
         const int len = pv.tile_len[base + ti];
         const float2* trig = pv.trig + (size_t)doc * (D / 2);
         const int n_items = len * items_per_row;
-        for (int it0 = threadIdx.x; it0 < n_items; it0 += kRepoThreads * kRepoUnroll) {
+        for (int it0 = piece * kRepoPass + threadIdx.x; it0 < n_items; it0 += pieces * kRepoPass) {
             uint4 va[kRepoUnroll], vb[kRepoUnroll];
             long long off[kRepoUnroll];
             int slice0[kRepoUnroll];
@@ -136,7 +147,7 @@ __global__ void __launch_bounds__(kRepoThreads)
 assemble_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_stride, long long self_stride,
                 int out_rows, const T* __restrict__ k_in, const T* __restrict__ v_in,
                 const T* __restrict__ k_self, const T* __restrict__ v_self, T* __restrict__ k_out,
-                T* __restrict__ v_out, int* __restrict__ final_rows) {
+                T* __restrict__ v_out, int* __restrict__ final_rows, int pieces) {
     constexpr int E = Vec16<T>::kElems;
     constexpr int kVecPerHead = D / E;
     __shared__ int s_red[kRepoThreads / 32];
@@ -149,7 +160,8 @@ assemble_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_strid
     constexpr int kPartner = LAYOUT == CF_ROPE_HALF ? (D / 2) : 0;
     const int items_per_row = n_kv_heads * kItemsPerHead;
     // blocks stride over the tiles, so a grid smaller than the tile count still covers every tile
-    for (int ti = blockIdx.x; ti <= n_tiles; ti += gridDim.x) {
+    const int piece = blockIdx.x % pieces, tile_step = gridDim.x / pieces;   // the grid is a multiple of `pieces`
+    for (int ti = blockIdx.x / pieces; ti <= n_tiles; ti += tile_step) {
         // rows of the tiles before this one (ti == n_tiles: of all tiles)
         int before = 0;
         for (int t = threadIdx.x; t < ti; t += kRepoThreads) before += pv.tile_len[base + t];
@@ -165,12 +177,12 @@ assemble_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_strid
         if (ti == n_tiles) {                                        // the query tokens' own keys and values
             const int lq = bv.q_len;
             if (before + lq > out_rows) {
-                if (threadIdx.x == 0) atomicCAS(pv.status, 0, CF_ERR_WORKSPACE);
+                if (piece == 0 && threadIdx.x == 0) atomicCAS(pv.status, 0, CF_ERR_WORKSPACE);
                 continue;
             }
-            if (layer == 0 && threadIdx.x == 0) final_rows[b] = before + lq;
+            if (layer == 0 && piece == 0 && threadIdx.x == 0) final_rows[b] = before + lq;
             const long long src0 = (long long)layer * self_stride + (long long)b * lq * n_kv_heads * D;
-            for (int idx = threadIdx.x; idx < lq * row_vecs; idx += kRepoThreads) {
+            for (int idx = piece * kRepoThreads + threadIdx.x; idx < lq * row_vecs; idx += pieces * kRepoThreads) {
                 const long long off = (long long)idx * E;
                 const long long dst = out_base + (long long)before * n_kv_heads * D + off;
                 *reinterpret_cast<uint4*>(k_out + dst) = *reinterpret_cast<const uint4*>(k_self + src0 + off);
@@ -184,7 +196,7 @@ assemble_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_strid
         const float2* trig = pv.trig + (size_t)pv.tile_doc[base + ti] * (D / 2);
         const T* ksrc = k_in + (long long)layer * layer_stride;
         const T* vsrc = v_in + (long long)layer * layer_stride;
-        for (int it = threadIdx.x; it < len * items_per_row; it += kRepoThreads) {
+        for (int it = piece * kRepoThreads + threadIdx.x; it < len * items_per_row; it += pieces * kRepoThreads) {
             const int row = it / items_per_row;
             const int rem = it - row * items_per_row;
             const int head = rem / kItemsPerHead;
@@ -223,15 +235,17 @@ static int launch_assemble_typed(const cf_geom* g, const cf_batch* b, const Plan
                                  long long layer_stride, long long self_stride, int out_rows, const void* k_in,
                                  const void* v_in, const void* k_self, const void* v_self, void* k_out, void* v_out,
                                  int* final_rows, cudaStream_t stream) {
-    const int tiles = std::min(tiles_per_request_bound(b), 1 << 16);
+    const int tiles = std::min(tiles_per_request_bound(b), 1 << 16) + 1;
     if (n_layers > 65535 || b->n_requests > 65535) return CF_ERR_INVALID_ARG;
-    dim3 grid((unsigned)tiles + 1, (unsigned)n_layers, (unsigned)b->n_requests);
+    const int items_per_row = g->n_kv_heads * D / Vec16<T>::kElems / (g->rope_layout == CF_ROPE_HALF ? 2 : 1);
+    const int pieces = pieces_per_tile((long long)tiles * n_layers * b->n_requests, (kTile * items_per_row + kRepoThreads - 1) / kRepoThreads);
+    dim3 grid((unsigned)(tiles * pieces), (unsigned)n_layers, (unsigned)b->n_requests);
     BatchView bv = make_batch_view(b);
     auto args = [&](auto kernel) {
         kernel<<<grid, kRepoThreads, 0, stream>>>(bv, pv, g->n_kv_heads, layer_stride, self_stride, out_rows,
                                                   static_cast<const T*>(k_in), static_cast<const T*>(v_in),
                                                   static_cast<const T*>(k_self), static_cast<const T*>(v_self),
-                                                  static_cast<T*>(k_out), static_cast<T*>(v_out), final_rows);
+                                                  static_cast<T*>(k_out), static_cast<T*>(v_out), final_rows, pieces);
     };
     if (g->rope_layout == CF_ROPE_HALF) args(assemble_kernel<T, D, CF_ROPE_HALF>);
     else args(assemble_kernel<T, D, CF_ROPE_INTERLEAVED>);
@@ -254,16 +268,18 @@ int launch_assemble(const cf_geom* g, const cf_batch* b, const PlanView& pv, int
 template <typename T, int D>
 static int launch_typed(const cf_geom* g, const cf_batch* b, const PlanView& pv, int n_layers,
                         long long layer_stride, const void* k_in, void* k_out, cudaStream_t stream) {
-    const int tiles = tiles_per_request_bound(b);
-    dim3 grid((unsigned)std::min(tiles, 1 << 16), (unsigned)n_layers, (unsigned)b->n_requests);
+    const int tiles = std::min(tiles_per_request_bound(b), 1 << 16);
+    const int items_per_row = g->n_kv_heads * D / Vec16<T>::kElems / (g->rope_layout == CF_ROPE_HALF ? 2 : 1);
+    const int pieces = pieces_per_tile((long long)tiles * n_layers * b->n_requests, (kTile * items_per_row + kRepoPass - 1) / kRepoPass);
+    dim3 grid((unsigned)(tiles * pieces), (unsigned)n_layers, (unsigned)b->n_requests);
     if (n_layers > 65535 || b->n_requests > 65535) return CF_ERR_INVALID_ARG;
     BatchView bv = make_batch_view(b);
     if (g->rope_layout == CF_ROPE_HALF)
         reposition_kernel<T, D, CF_ROPE_HALF><<<grid, kRepoThreads, 0, stream>>>(
-            bv, pv, g->n_kv_heads, layer_stride, static_cast<const T*>(k_in), static_cast<T*>(k_out));
+            bv, pv, g->n_kv_heads, layer_stride, static_cast<const T*>(k_in), static_cast<T*>(k_out), pieces);
     else
         reposition_kernel<T, D, CF_ROPE_INTERLEAVED><<<grid, kRepoThreads, 0, stream>>>(
-            bv, pv, g->n_kv_heads, layer_stride, static_cast<const T*>(k_in), static_cast<T*>(k_out));
+            bv, pv, g->n_kv_heads, layer_stride, static_cast<const T*>(k_in), static_cast<T*>(k_out), pieces);
     return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
 }
 
