@@ -212,7 +212,6 @@ size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, 
         ws->self_l = with_self ? reinterpret_cast<float*>(base + sl) : nullptr;
         ws->part_ld = with_self ? reinterpret_cast<float*>(base + ld) : nullptr;
         ws->self_mode = 0;
-        ws->keys_in_place = 0;
     }
     return off;
 }
@@ -249,7 +248,7 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
                     const void* v_self, long long self_stride, float softmax_scale,
                     void* out, float* lse, float* doc_scores, float* score_accum, void* workspace,
                     size_t workspace_bytes, cudaStream_t s, const void* k_prefix, const void* v_prefix,
-                    long long prefix_stride, int prefix_len, int slot, int n_slots, bool keys_in_place) {
+                    long long prefix_stride, int prefix_len, int slot, int n_slots, int decode_cache_rows) {
     int rc = check_plan(geom, batch, plan);
     if (rc != CF_OK) return rc;
     const bool slotted = slot >= 0;                   // one layer into slot `slot` of n_slots, scored later
@@ -300,6 +299,11 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
     }
     const float scale = softmax_scale == 0.0f ? 1.0f / std::sqrt((float)geom->head_dim) : softmax_scale;
     PlanView pv = make_plan_view(geom, batch, const_cast<void*>(plan));
+    if (decode_cache_rows > 0 && g_attn_path.load() == 0 && decode_attn_supported(geom)) {
+        if (workspace_bytes < decode_attn_workspace_bytes(geom)) return CF_ERR_WORKSPACE;
+        return launch_decode_attn(geom, batch->n_requests, decode_cache_rows, span.n_layers, batch->doc_offsets, span, q, k_cache,
+                                  v_cache, scale * kLog2e, out, lse, workspace, s);
+    }
     const bool tensor_core = g_attn_path.load() == 0 && attn_tc_supported(geom, batch);
     if (with_self && batch->q_len > CF_TILE_TOKENS) return CF_ERR_UNSUPPORTED;
     if (!tensor_core) ws.part_ld = nullptr;           // only the tensor-core kernel reports per-part document sums
@@ -312,7 +316,6 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
     cudaEvent_t ev_start, ev_stop;
     const bool timed = prof_claim(&ev_start, &ev_stop) >= 0;
     if (timed) cudaEventRecord(ev_start, s);
-    ws.keys_in_place = keys_in_place ? 1 : 0;
     if (tensor_core) {
         ws.part_bf16 = 1;
         ws.self_mode = (with_self || with_prefix) ? 2 : 0;   // the blocks ride along as further key tiles

@@ -77,6 +77,24 @@ int configure_smem_once(PerDeviceOnce& once, K kernel, int bytes) {
     if (dev >= 0) once.done[dev] = true;
     return CF_OK;
 }
+// Launches a kernel that may be scheduled while its predecessor in the stream still runs (programmatic stream
+// serialisation): it must execute chain_wait() before it touches memory the predecessor wrote or reads, and
+// every kernel launched this way does so before it ends, so that a chain stays ordered.  Takes the launch latency
+// (1 to 1.5 us) out of chains of kernels that run for a few microseconds each.
+template <typename... P, typename... A>
+int launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+}
 int choose_splits(const cf_geom* g, const cf_batch* b, int n_layers);
 int choose_row_group(const cf_geom* g, const cf_batch* b);
 int tiles_per_request_bound(const cf_batch* b);
@@ -105,7 +123,6 @@ struct AttnWorkspace {
     float* self_l;     // [L*B][Hq*Lq]
     float* part_ld;    // [L*B][n_splits][Hq*Lq]    like part_l, the documents' keys only (self_mode 2)
     int self_mode;
-    int keys_in_place; // every document's destination equals its source (decoding over final caches): no rotation
 };
 // part_layers > 0: the partial results (and the further key blocks' buffers) are sized for that many layers only, the
 // per-tile and per-row log-sum-exps for n_layers (calls that fill one layer slot at a time and score the slots later).
@@ -139,6 +156,12 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
                    long long self_stride, const void* k_prefix, const void* v_prefix, long long prefix_stride,
                    int prefix_len, float scale_log2, const AttnWorkspace& ws, cudaStream_t stream);
 bool attn_tc_supported(const cf_geom* g, const cf_batch* b);
+// One query row per head over the final caches of a decoding step (doc_offsets: of the decode plan).
+bool decode_attn_supported(const cf_geom* g);
+size_t decode_attn_workspace_bytes(const cf_geom* g);
+int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_layers, const int* doc_offsets, const LayerSpan& span,
+                       const void* q, const void* k, const void* v, float scale_log2, void* out, float* lse,
+                       void* workspace, cudaStream_t stream);
 int launch_combine(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span,
                    const AttnWorkspace& ws, void* out, float* lse, float* doc_scores,
                    float* score_accum, cudaStream_t stream);
@@ -153,7 +176,7 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
                     void* out, float* lse, float* doc_scores, float* score_accum, void* workspace,
                     size_t workspace_bytes, cudaStream_t stream, const void* k_prefix = nullptr,
                     const void* v_prefix = nullptr, long long prefix_stride = 0, int prefix_len = 0, int slot = -1,
-                    int n_slots = 0, bool keys_in_place = false);
+                    int n_slots = 0, int decode_cache_rows = 0);
 // Document scores of the layers held in a workspace: doc_scores[l] = s^l (optional), S += s^l in layer order.
 int launch_scores(const cf_geom* g, const cf_batch* b, const PlanView& pv, const AttnWorkspace& ws, float* doc_scores,
                   float* score_accum, cudaStream_t stream);
@@ -173,6 +196,10 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
 int attn_path();
 
 // ---- device helpers -----------------------------------------------------------------------
+// The predecessor in the stream is complete and its writes are visible (returns at once for an ordinary launch).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The successor in the stream may be scheduled on what this grid leaves free.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ float to_float(float x) { return x; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
 template <typename T> __device__ __forceinline__ T from_float(float x);

@@ -1,9 +1,9 @@
 // Decoding over the final caches (Algorithm 2, Phase 3: Y <- LLM(C_final); the "Decoding" loop of
 // Algorithm 1): every generated token appends its key/value rows to each request's packed final cache
 // and attends all rows of it.  The caches come out of cf_assemble_final_cache already re-positioned, so
-// nothing is rotated here: each request's used rows are declared as one document whose destination
-// equals its source (delta 0) and the attention kernels of the query-time path do the rest -- with one
-// query row per head the pass is a stream over the cache, bound by HBM bandwidth.
+// nothing is rotated here.  bf16 / head_dim 128 has a kernel of its own (cf_decode_attn.cu); for other geometries each
+// request's used rows are declared as one document whose destination equals its source (delta 0) and the CUDA-core
+// attention kernel of the query-time path does the rest.
 #include <climits>
 
 #include "cf_common.cuh"
@@ -65,29 +65,56 @@ int check_decode(const cf_geom* geom, int n_requests, int cache_rows) {
     return CF_OK;
 }
 
-__global__ void decode_setup_kernel(DecodeArrays a, int n_requests, int cache_rows, int pos_range,
-                                    const int* __restrict__ rows, int extra_rows, int* status) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b > n_requests) return;
-    if (b == n_requests) {
+// The whole description of a decoding step in one launch, one block per request: the integer arrays and, for the
+// kernels of the query-time path, the plan they would get from cf_plan_init (one kept document in tiles of kTile rows,
+// destination equal to source, identity rotation).
+__global__ void __launch_bounds__(128)
+decode_plan_kernel(DecodeArrays a, PlanView pv, int n_requests, int cache_rows, int pos_range, int half,
+                   const int* __restrict__ rows, int extra_rows) {
+    chain_next();
+    chain_wait();
+    const int b = blockIdx.x, tid = threadIdx.x;
+    if (b == 0) {                                       // the status word: one block looks at every request
+        bool bad = false;
+        for (int r = tid; r < n_requests; r += blockDim.x) {
+            const long long used = (long long)rows[r] + extra_rows;
+            bad |= used < 1 || used > cache_rows;       // the slot cannot hold (or has) that many rows
+        }
+        const int any_bad = __syncthreads_or(bad);
+        if (tid < 4) pv.status[tid] = tid == 0 && any_bad ? CF_ERR_RANGE : 0;
+    }
+    const int used = (int)max(1LL, min((long long)cache_rows, (long long)rows[b] + extra_rows));
+    const int tiles = (used + kTile - 1) / kTile, row0 = b * cache_rows, base = tile_base(2 * b, row0);
+    const int start = pos_range - 1 - used;             // the window ends at the query (pos_range - tail_reserve)
+    if (tid == 0) {
         a.req_doc_begin[b] = 2 * b;
-        a.doc_offsets[2 * b] = b * cache_rows;
-        return;
+        a.doc_offsets[2 * b] = row0;
+        a.doc_offsets[2 * b + 1] = row0 + used;
+        if (b == n_requests - 1) {
+            a.req_doc_begin[b + 1] = 2 * (b + 1);
+            a.doc_offsets[2 * b + 2] = row0 + cache_rows;
+        }
+        a.doc_src_start[2 * b] = start;
+        a.doc_src_start[2 * b + 1] = 0;
+        a.kept_count[b] = pv.kept_count[b] = 1;
+        pv.n_reuse[b] = 1;
+        pv.query_start[b] = pos_range - 1;
+        pv.n_tiles[b] = tiles;
+        pv.tile_begin[b] = base;
     }
-    long long used = (long long)rows[b] + extra_rows;
-    if (used < 1 || used > cache_rows) {                // the slot cannot hold (or has) that many rows
-        atomicCAS(status, 0, CF_ERR_RANGE);
-        used = used < 1 ? 1 : cache_rows;
+    if (tid < 2) {                                      // the rows in use, and the unused tail that is not kept
+        a.order[2 * b + tid] = pv.kept[2 * b + tid] = tid;
+        pv.dst_start[2 * b + tid] = tid == 0 ? start : -1;
+        pv.group[2 * b + tid] = tid == 0 ? 0 : -1;
+        pv.doc_tile_begin[2 * b + tid] = tid == 0 ? base : 0;
+        pv.doc_tile_count[2 * b + tid] = tid == 0 ? tiles : 0;
     }
-    a.req_doc_begin[b] = 2 * b;
-    a.doc_offsets[2 * b] = b * cache_rows;
-    a.doc_offsets[2 * b + 1] = b * cache_rows + (int)used;
-    // cached where the allocation will put it: the window ends at the query (pos_range - tail_reserve)
-    a.doc_src_start[2 * b] = pos_range - 1 - (int)used;
-    a.doc_src_start[2 * b + 1] = 0;
-    a.order[2 * b] = 0;
-    a.order[2 * b + 1] = 1;
-    a.kept_count[b] = 1;
+    for (int t = tid; t < tiles; t += blockDim.x) {
+        pv.tile_doc[base + t] = 2 * b;
+        pv.tile_row0[base + t] = row0 + t * kTile;
+        pv.tile_len[base + t] = min(kTile, used - t * kTile);
+    }
+    if (tid < half) pv.trig[(size_t)2 * b * half + tid] = make_float2(1.f, 0.f);
 }
 
 // One block per (request, layer): the new token's key and value rows go behind the rows in use.
@@ -96,6 +123,8 @@ __global__ void decode_append_kernel(int cache_rows, int row_elems, long long la
                                      const int* __restrict__ rows, int step, const T* __restrict__ k_new,
                                      const T* __restrict__ v_new, T* __restrict__ k_final, T* __restrict__ v_final,
                                      int* status) {
+    chain_next();
+    chain_wait();
     const int b = blockIdx.x, layer = blockIdx.y;
     const long long row = (long long)rows[b] + step;
     if (row < 0 || row >= cache_rows) {
@@ -147,13 +176,8 @@ int cf_decode_plan(const cf_geom* geom, int32_t n_requests, int32_t cache_rows, 
     void* plan = static_cast<char*>(decode_plan) + a.bytes;
     const PlanView pv = make_plan_view(&g, &b, plan);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    rc = launch_clear_status(pv, s);
-    if (rc != CF_OK) return rc;
-    decode_setup_kernel<<<(n_requests + 1 + 255) / 256, 256, 0, s>>>(a, n_requests, cache_rows, g.pos_range, rows,
-                                                                   extra_rows, pv.status);
-    if (cudaGetLastError() != cudaSuccess) return CF_ERR_CUDA;
-    return launch_plan(make_geom_view(&g), make_batch_view(&b), pv, 0, a.order, a.kept_count, -1, nullptr, 0, nullptr,
-                       CF_ALLOC_ALIGN, s);
+    return launch_chained(decode_plan_kernel, dim3((unsigned)n_requests), 128, 0, s, a, pv, n_requests, cache_rows, g.pos_range,
+                          geom->head_dim / 2, rows, extra_rows);
 }
 
 int cf_decode_status(const cf_geom* geom, int32_t n_requests, int32_t cache_rows, const void* decode_plan, void* stream) {
@@ -174,7 +198,8 @@ size_t cf_decode_workspace_bytes(const cf_geom* geom, int32_t n_requests, int32_
     cf_batch b;
     decode_views(geom, n_requests, cache_rows, a, &g, &b);
     b.req_doc_begin = b.doc_offsets = b.doc_src_start = reinterpret_cast<const int32_t*>(geom);
-    return cf_attn_workspace_bytes_layers(&g, &b, n_layers);
+    const size_t general = cf_attn_workspace_bytes_layers(&g, &b, n_layers);
+    return general == 0 || !decode_attn_supported(geom) ? general : general + decode_attn_workspace_bytes(geom);
 }
 
 int cf_decode_attn(const cf_geom* geom, int32_t n_requests, int32_t cache_rows, const void* decode_plan,
@@ -192,8 +217,7 @@ int cf_decode_attn(const cf_geom* geom, int32_t n_requests, int32_t cache_rows, 
     const LayerSpan span = {n_layers, q_layer_stride, kv_layer_stride, out_layer_stride};
     return run_attn_layers(&g, &b, static_cast<const char*>(decode_plan) + a.bytes, span, q, k_final, v_final, nullptr,
                            nullptr, 0, softmax_scale, out, lse, nullptr, nullptr, workspace, workspace_bytes,
-                           static_cast<cudaStream_t>(stream), nullptr, nullptr, 0, 0, -1, 0,
-                           /*keys_in_place=*/true);           // the final caches are used where they lie
+                           static_cast<cudaStream_t>(stream), nullptr, nullptr, 0, 0, -1, 0, cache_rows);
 }
 
 int cf_decode_append(const cf_geom* geom, int32_t n_requests, int32_t cache_rows, int32_t n_layers,
@@ -215,15 +239,12 @@ int cf_decode_append(const cf_geom* geom, int32_t n_requests, int32_t cache_rows
     const dim3 grid((unsigned)n_requests, (unsigned)n_layers);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (geom->dtype == CF_BF16)
-        decode_append_kernel<__nv_bfloat16><<<grid, 128, 0, s>>>(
-            cache_rows, row_elems, kv_layer_stride, new_layer_stride, rows, step, static_cast<const __nv_bfloat16*>(k_new),
-            static_cast<const __nv_bfloat16*>(v_new), static_cast<__nv_bfloat16*>(k_final),
-            static_cast<__nv_bfloat16*>(v_final), status);
-    else
-        decode_append_kernel<float><<<grid, 128, 0, s>>>(cache_rows, row_elems, kv_layer_stride, new_layer_stride, rows, step,
-                                                         static_cast<const float*>(k_new), static_cast<const float*>(v_new),
-                                                         static_cast<float*>(k_final), static_cast<float*>(v_final), status);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+        return launch_chained(decode_append_kernel<__nv_bfloat16>, grid, 128, 0, s, cache_rows, row_elems, kv_layer_stride, new_layer_stride,
+                              rows, step, static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new),
+                              static_cast<__nv_bfloat16*>(k_final), static_cast<__nv_bfloat16*>(v_final), status);
+    return launch_chained(decode_append_kernel<float>, grid, 128, 0, s, cache_rows, row_elems, kv_layer_stride, new_layer_stride, rows, step,
+                          static_cast<const float*>(k_new), static_cast<const float*>(v_new), static_cast<float*>(k_final),
+                          static_cast<float*>(v_final), status);
 }
 
 }  // extern "C"

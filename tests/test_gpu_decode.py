@@ -154,3 +154,42 @@ def test_bench_sized_caches_one_step(layers_per_call):
             got = out[l, b].float().cpu().numpy()
             assert np.all(np.abs(got - o_ref[0]) <= 1e-2 + 2e-2 * np.abs(o_ref[0])), (l, b)
             assert np.all(np.abs(lse[l, b].cpu().numpy() - lse_ref[0]) <= 1e-2), (l, b)
+
+
+@pytest.mark.parametrize("hq,hkv,cache_rows,used", [
+    (12, 2, 90, [1, 15, 16, 17, 63, 64, 65, 90]),        # one cluster per kv head: step and warp edges
+    (5, 5, 40, [40]),                                     # a single head per kv head
+    (16, 2, 600, [600, 3]), (27, 3, 600, [599, 33]),      # eight and nine heads per kv head
+    (40, 1, 200, [200, 1, 129]),                          # forty: tiles of sixteen heads, the last one half empty
+    (8, 1, 6000, [6000, 1, 257]), (20, 2, 9000, [9000, 5]),   # equal shares of all rows, units cut several times
+    (64, 64, 3000, [3000, 2999, 7]),                      # several whole units per share
+])
+def test_decode_kernel_at_the_edges_of_its_splits(hq, hkv, cache_rows, used):
+    L, B, d = 2, len(used), 128
+    geom = cf.make_geom(hq, hkv, d, cf.CF_BF16, 32768, 1e6)
+    gen = torch.Generator().manual_seed(hq + cache_rows)
+    k = torch.randn((L, B, cache_rows, hkv, d), generator=gen).bfloat16()
+    v = torch.randn((L, B, cache_rows, hkv, d), generator=gen).bfloat16()
+    q = (2 * torch.randn((L, B, hq, d), generator=gen)).bfloat16()
+    rows = torch.tensor(used, dtype=torch.int32, device="cuda")
+    plan = torch.full((cf.cf_decode_plan_bytes(geom, B, cache_rows),), 255, dtype=torch.uint8, device="cuda")
+    cf.cf_decode_plan(geom, B, cache_rows, rows, 0, plan)
+    kg, vg, qg = k.cuda(), v.cuda(), q.cuda()
+    for per_call in (1, L):
+        work = torch.full((cf.cf_decode_workspace_bytes(geom, B, cache_rows, per_call),), 255, dtype=torch.uint8, device="cuda")
+        out = torch.full((L, B, hq, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((L, B, hq), float("nan"), device="cuda")
+        for l in range(0, L, per_call):
+            cf.cf_decode_attn(geom, B, cache_rows, plan, qg[l:l + per_call], kg[l:l + per_call], vg[l:l + per_call],
+                              out[l:l + per_call], work, lse[l:l + per_call])
+        assert cf.cf_decode_status(geom, B, cache_rows, plan) == 0
+        for l in range(L):
+            for b, n in enumerate(used):
+                heads = np.arange(hq) // (hq // hkv)
+                logits = np.einsum("hd,nhd->hn", q[l, b].double().numpy(), k[l, b, :n].double().numpy()[:, heads]) / np.sqrt(d)
+                top = logits.max(axis=1, keepdims=True)
+                w = np.exp(logits - top)
+                ref = np.einsum("hn,nhd->hd", w / w.sum(axis=1, keepdims=True), v[l, b, :n].double().numpy()[:, heads])
+                got = out[l, b].double().cpu().numpy()
+                assert np.all(np.abs(got - ref) <= 1e-2 + 2e-2 * np.abs(ref)), (l, b, per_call)
+                assert np.all(np.abs(lse[l, b].cpu().numpy() - (top[:, 0] + np.log(w.sum(axis=1)))) <= 1e-2), (l, b, per_call)
