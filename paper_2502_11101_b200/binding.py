@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libcachefocus.so: same names as the C ABI, argument marshalling only.
+"""Thin binding of libcachefocus.so: same names as the C ABI, argument marshalling only.  The calls a serving loop issues
+per layer or per token are marshalled natively (csrc/binding.cpp), the others through ctypes.
 
 Tensors are torch tensors used purely as device (or host) buffers; every step of the path runs
 in the library's kernels."""
@@ -87,6 +88,7 @@ class CacheFocusError(RuntimeError):
 
 
 _LIB = None
+_NATIVE = None
 
 
 def load_library() -> ctypes.CDLL:
@@ -160,6 +162,16 @@ def load_library() -> ctypes.CDLL:
             getattr(lib, name).restype = ctypes.c_int
     _LIB = lib
     return lib
+
+
+def _native():
+    """The native marshalling module (built next to the library; there is no fallback)."""
+    global _NATIVE
+    if _NATIVE is None:
+        load_library()
+        from . import _native as module
+        _NATIVE = module
+    return _NATIVE
 
 
 def _check(code: int, where: str) -> None:
@@ -243,9 +255,7 @@ def cf_plan_layout_of(geom: cf_geom, batch: cf_batch) -> cf_plan_layout:
 
 def cf_plan_init(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, order: Optional[torch.Tensor] = None,
                  kept_count: Optional[torch.Tensor] = None, query_start: int = -1, stream=None) -> None:
-    rc = load_library().cf_plan_init(ctypes.byref(geom), ctypes.byref(batch), _ptr(order), _ptr(kept_count),
-                                     query_start, plan.data_ptr(), plan.numel() * plan.element_size(), _stream(stream))
-    _check(rc, "cf_plan_init")
+    _check(_native().plan_init(geom, batch, plan, order, kept_count, query_start, stream), "cf_plan_init")
 
 
 def cf_plan_status(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, stream=None) -> int:
@@ -254,9 +264,7 @@ def cf_plan_status(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, stream=No
 
 def cf_reposition_keys(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, k_in: torch.Tensor, k_out: torch.Tensor,
                        n_layers: int = 1, layer_stride: int = 0, stream=None) -> None:
-    rc = load_library().cf_reposition_keys(ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(), n_layers,
-                                           layer_stride, k_in.data_ptr(), k_out.data_ptr(), _stream(stream))
-    _check(rc, "cf_reposition_keys")
+    _check(_native().reposition_keys(geom, batch, plan, k_in, k_out, n_layers, layer_stride, stream), "cf_reposition_keys")
 
 
 def cf_attn_workspace_bytes(geom: cf_geom, batch: cf_batch) -> int:
@@ -267,11 +275,8 @@ def cf_query_prefill_attn(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, q:
                           v_cache: torch.Tensor, out: torch.Tensor, workspace: torch.Tensor,
                           lse: Optional[torch.Tensor] = None, doc_scores: Optional[torch.Tensor] = None,
                           score_accum: Optional[torch.Tensor] = None, softmax_scale: float = 0.0, stream=None) -> None:
-    rc = load_library().cf_query_prefill_attn(ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(), q.data_ptr(),
-                                              k_cache.data_ptr(), v_cache.data_ptr(), softmax_scale, out.data_ptr(),
-                                              _ptr(lse), _ptr(doc_scores), _ptr(score_accum), workspace.data_ptr(),
-                                              workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(rc, "cf_query_prefill_attn")
+    _check(_native().query_prefill_attn(geom, batch, plan, q, k_cache, v_cache, out, workspace, lse, doc_scores, score_accum,
+                                        softmax_scale, stream), "cf_query_prefill_attn")
 
 
 def cf_attn_workspace_bytes_layers(geom: cf_geom, batch: cf_batch, n_layers: int) -> int:
@@ -308,11 +313,8 @@ def cf_query_prefill_attn_slot(geom: cf_geom, batch: cf_batch, plan: torch.Tenso
                                workspace: torch.Tensor, lse: Optional[torch.Tensor] = None, softmax_scale: float = 0.0,
                                stream=None) -> None:
     """One layer (tensors as in cf_query_prefill_attn) whose document scores are left for cf_accumulate_scores."""
-    rc = load_library().cf_query_prefill_attn_slot(
-        ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(), slot, n_slots, q.data_ptr(), k_cache.data_ptr(),
-        v_cache.data_ptr(), softmax_scale, out.data_ptr(), _ptr(lse), workspace.data_ptr(),
-        workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(rc, "cf_query_prefill_attn_slot")
+    _check(_native().query_prefill_attn_slot(geom, batch, plan, slot, n_slots, q, k_cache, v_cache, out, workspace, lse,
+                                             softmax_scale, stream), "cf_query_prefill_attn_slot")
 
 
 def cf_attn_workspace_bytes_slots_full(geom: cf_geom, batch: cf_batch, n_slots: int) -> int:
@@ -340,10 +342,8 @@ def cf_accumulate_scores(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, n_f
                          score_accum: Optional[torch.Tensor] = None, stream=None) -> None:
     """`doc_scores` [n_filled, n_docs_total] (contiguous) and / or `score_accum` [n_docs_total]."""
     assert doc_scores is None or (doc_scores.shape[0] == n_filled and doc_scores.is_contiguous())
-    rc = load_library().cf_accumulate_scores(
-        ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(), n_filled, n_slots, _ptr(doc_scores), _ptr(score_accum),
-        workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(rc, "cf_accumulate_scores")
+    _check(_native().accumulate_scores(geom, batch, plan, n_filled, n_slots, workspace, doc_scores, score_accum, stream),
+           "cf_accumulate_scores")
 
 
 def cf_assemble_final_cache(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, k_cache: torch.Tensor,
@@ -351,13 +351,8 @@ def cf_assemble_final_cache(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, 
                             v_out: torch.Tensor, final_rows: torch.Tensor, stream=None) -> None:
     """k_cache, v_cache [L, T, Hkv, D]; k_self, v_self [L, B, Lq, Hkv, D]; k_out, v_out [L, B, out_rows, Hkv, D]
     (contiguous); final_rows int32 [B]."""
-    assert k_out.is_contiguous() and v_out.is_contiguous() and k_out.shape == v_out.shape
-    assert final_rows.dtype == torch.int32 and k_cache.stride(0) == v_cache.stride(0)
-    rc = load_library().cf_assemble_final_cache(
-        ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(), k_cache.shape[0], k_cache.stride(0),
-        k_cache.data_ptr(), v_cache.data_ptr(), k_self.stride(0), k_self.data_ptr(), v_self.data_ptr(),
-        k_out.shape[2], k_out.data_ptr(), v_out.data_ptr(), final_rows.data_ptr(), _stream(stream))
-    _check(rc, "cf_assemble_final_cache")
+    _check(_native().assemble_final_cache(geom, batch, plan, k_cache, v_cache, k_self, v_self, k_out, v_out, final_rows, stream),
+           "cf_assemble_final_cache")
 
 
 def cf_merge_attn(geom: cf_geom, out_a: torch.Tensor, lse_a: torch.Tensor, out_b: torch.Tensor, lse_b: torch.Tensor,
@@ -439,9 +434,7 @@ def cf_query_prefill_attn_static(geom: cf_geom, batch: cf_batch, plan: torch.Ten
 
 def cf_prune_topk(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, score_accum: torch.Tensor, keep: int,
                   strategy: int, keep_per_request: Optional[torch.Tensor] = None, stream=None) -> None:
-    rc = load_library().cf_prune_topk(ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(), score_accum.data_ptr(),
-                                      keep, _ptr(keep_per_request), strategy, _stream(stream))
-    _check(rc, "cf_prune_topk")
+    _check(_native().prune_topk(geom, batch, plan, score_accum, keep, keep_per_request, strategy, stream), "cf_prune_topk")
 
 
 def cf_prune_topk_host(score_accum: Sequence[float], order: Sequence[int], keep: int, strategy: int) -> List[int]:
@@ -513,21 +506,8 @@ def cf_document_prefill_attn(geom: cf_geom, doc_offsets: torch.Tensor, max_doc_l
     """Attention of the offline cache construction.  q, out [L, T, Hq, D]; k, v [L, T, Hkv, D] (rows may be
     padded to `token_stride`); k_prefix, v_prefix [L, P, Hkv, D] dense; lse [L, Hq, T]; doc_offsets int32
     device [n_docs + 1].  Dimension 0 may be strided."""
-    n_layers, total = q.shape[0], q.shape[1]
-    assert doc_offsets.dtype == torch.int32 and doc_offsets.is_contiguous()
-    assert k.shape[0] == n_layers and v.shape[0] == n_layers and out.shape[0] == n_layers
-    assert k.stride(0) == v.stride(0) and (lse is None or lse.is_contiguous())
-    prefix_len = 0 if k_prefix is None else k_prefix.shape[1]
-    if prefix_len:
-        assert k_prefix.stride(0) == v_prefix.stride(0)
-    stride = k.shape[2] * k.shape[3] if token_stride is None else token_stride
-    docs = cf_doc_batch(doc_offsets.numel() - 1, max_doc_len, prefix_len, 0, total, stride, doc_offsets.data_ptr())
-    rc = load_library().cf_document_prefill_attn(
-        ctypes.byref(geom), ctypes.byref(docs), n_layers, q.data_ptr(), q.stride(0), k.data_ptr(), v.data_ptr(),
-        k.stride(0), _ptr(k_prefix) if prefix_len else None, _ptr(v_prefix) if prefix_len else None,
-        k_prefix.stride(0) if prefix_len else 0, softmax_scale, out.data_ptr(), out.stride(0), _ptr(lse),
-        _ptr(status), _stream(stream))
-    _check(rc, "cf_document_prefill_attn")
+    _check(_native().document_prefill_attn(geom, doc_offsets, max_doc_len, q, k, v, out, k_prefix, v_prefix, lse, softmax_scale,
+                                           token_stride, status, stream), "cf_document_prefill_attn")
 
 
 def cf_debug_wait_timeout(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, limit_cycles: int, stream=None) -> None:
@@ -562,10 +542,7 @@ def cf_decode_workspace_bytes(geom: cf_geom, n_requests: int, cache_rows: int, n
 def cf_decode_plan(geom: cf_geom, n_requests: int, cache_rows: int, rows: torch.Tensor, extra_rows: int,
                    decode_plan: torch.Tensor, stream=None) -> None:
     """One decoding step's description: request b attends rows 0 .. rows[b] + extra_rows - 1 of its slot."""
-    rc = load_library().cf_decode_plan(ctypes.byref(geom), n_requests, cache_rows, rows.data_ptr(), extra_rows,
-                                       decode_plan.data_ptr(), decode_plan.numel() * decode_plan.element_size(),
-                                       _stream(stream))
-    _check(rc, "cf_decode_plan")
+    _check(_native().decode_plan(geom, n_requests, cache_rows, rows, extra_rows, decode_plan, stream), "cf_decode_plan")
 
 
 def cf_decode_status(geom: cf_geom, n_requests: int, cache_rows: int, decode_plan: torch.Tensor, stream=None) -> int:
@@ -577,29 +554,16 @@ def cf_decode_attn(geom: cf_geom, n_requests: int, cache_rows: int, decode_plan:
                    k_final: torch.Tensor, v_final: torch.Tensor, out: torch.Tensor, workspace: torch.Tensor,
                    lse: Optional[torch.Tensor] = None, softmax_scale: float = 0.0, stream=None) -> None:
     """q, out [n_layers, B, Hq, D]; k_final, v_final [n_layers, B, cache_rows, Hkv, D]; lse [n_layers, B, Hq]."""
-    n_layers = q.shape[0]
-    assert k_final.shape[0] == n_layers and v_final.shape[0] == n_layers and out.shape[0] == n_layers
-    assert k_final.stride(0) == v_final.stride(0) and (lse is None or lse.is_contiguous())
-    rc = load_library().cf_decode_attn(ctypes.byref(geom), n_requests, cache_rows, decode_plan.data_ptr(), n_layers,
-                                       q.data_ptr(), q.stride(0), k_final.data_ptr(), v_final.data_ptr(),
-                                       k_final.stride(0), softmax_scale, out.data_ptr(), out.stride(0), _ptr(lse),
-                                       workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-                                       _stream(stream))
-    _check(rc, "cf_decode_attn")
+    _check(_native().decode_attn(geom, n_requests, cache_rows, decode_plan, q, k_final, v_final, out, workspace, lse,
+                                 softmax_scale, stream), "cf_decode_attn")
 
 
 def cf_decode_append(geom: cf_geom, n_requests: int, cache_rows: int, k_final: torch.Tensor, v_final: torch.Tensor,
                      rows: torch.Tensor, step: int, k_new: torch.Tensor, v_new: torch.Tensor,
                      status: Optional[torch.Tensor] = None, stream=None) -> None:
     """k_new, v_new [n_layers, B, Hkv, D] become row rows[b] + step of request b's slot in every layer."""
-    n_layers = k_final.shape[0]
-    assert v_final.shape[0] == n_layers and k_new.shape[0] == n_layers and v_new.shape[0] == n_layers
-    assert k_final.stride(0) == v_final.stride(0) and k_new.stride(0) == v_new.stride(0)
-    rc = load_library().cf_decode_append(ctypes.byref(geom), n_requests, cache_rows, n_layers, k_final.data_ptr(),
-                                         v_final.data_ptr(), k_final.stride(0), rows.data_ptr(), step,
-                                         k_new.data_ptr(), v_new.data_ptr(), k_new.stride(0), _ptr(status),
-                                         _stream(stream))
-    _check(rc, "cf_decode_append")
+    _check(_native().decode_append(geom, n_requests, cache_rows, k_final, v_final, rows, step, k_new, v_new, status, stream),
+           "cf_decode_append")
 
 
 def plan_field(plan: torch.Tensor, layout: cf_plan_layout, name: str, count: int, dtype=torch.int32) -> torch.Tensor:

@@ -37,6 +37,14 @@ class Session:
         self.batch = B.make_batch(self.n_requests, q_len, self.total_tokens, stride, self._req_doc_begin,
                                   self._doc_offsets, self._doc_src_start, prefix_len, tail_reserve, n_reuse, 0)
         self.layout = B.cf_plan_layout_of(self.geom, self.batch)
+        # key tiles of the k longest documents of a request, the most over the requests: [k]
+        self._live_tiles = np.zeros(self.n_docs_total + 1, dtype=np.int64)
+        for b in range(self.n_requests):
+            lens = self.doc_len[self.req_doc_begin_h[b]:self.req_doc_begin_h[b + 1]]
+            tiles = np.cumsum(np.sort((lens + B.CF_TILE_TOKENS - 1) // B.CF_TILE_TOKENS)[::-1])
+            if len(tiles):
+                self._live_tiles[1:len(tiles) + 1] = np.maximum(self._live_tiles[1:len(tiles) + 1], tiles)
+                self._live_tiles[len(tiles) + 1:] = np.maximum(self._live_tiles[len(tiles) + 1:], tiles[-1])
         self.plan = torch.zeros(self.layout.total_bytes, dtype=torch.uint8, device=self.device)
         self.set_live_docs(int(np.diff(self.req_doc_begin_h).max()) if self.n_requests else 0)
         self.workspace = torch.empty(256, dtype=torch.uint8, device=self.device)
@@ -47,12 +55,8 @@ class Session:
     def set_live_docs(self, kept_per_request: int) -> None:
         """Tell the library how many documents a request can still hold (sizes kernel grids only):
         the hint is the tile count of the `kept_per_request` longest documents of any request."""
-        worst = 1
-        for b in range(self.n_requests):
-            lens = self.doc_len[self.req_doc_begin_h[b]:self.req_doc_begin_h[b + 1]]
-            tiles = np.sort((lens + B.CF_TILE_TOKENS - 1) // B.CF_TILE_TOKENS)[::-1]
-            worst = max(worst, int(tiles[:kept_per_request].sum()))
-        self.batch.tiles_hint = worst
+        k = max(0, min(kept_per_request, self.n_docs_total))
+        self.batch.tiles_hint = max(1, int(self._live_tiles[k]))
 
     def reserve_workspace(self, n_layers: int, with_self: bool = False) -> None:
         """Grow the attention workspace to what a call over `n_layers` layers needs with the current
@@ -133,15 +137,15 @@ class Session:
         `driver="library"`: one cf_run_stack call sequences the stack inside the library;
         `driver="calls"`: the same sequence issued from here, one library call per step."""
         if driver == "library":
-            st, keepalive = B.make_stack(q, k, v, out, self.score_accum, schedule, strategy, batch_layers, lse,
-                                         layer_scores, k_final, k_self, v_self, softmax_scale, self.doc_len,
-                                         self.req_doc_begin_h, k_prefix, v_prefix)
             self.batch.tiles_hint = 0
-            need = B.cf_run_stack_workspace_bytes(self.geom, self.batch, st)
-            if need > self.workspace.numel():
+            while True:
+                code, need = B._native().run_stack(self.geom, self.batch, self.plan, self.workspace, q, k, v, out, self.score_accum,
+                                                   schedule, strategy, batch_layers, lse, layer_scores, k_final, k_self, v_self,
+                                                   softmax_scale, self.doc_len, self.req_doc_begin_h, k_prefix, v_prefix, None)
+                if not need:
+                    break
                 self.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
-            B.cf_run_stack(self.geom, self.batch, st, self.plan, self.workspace)
-            del keepalive
+            B._check(code, "cf_run_stack")
             return
         assert driver == "calls" and k_prefix is None, "a prefix cache goes through the library's stack driver"
         sched = dict(schedule)
