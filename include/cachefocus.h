@@ -161,6 +161,12 @@ int cf_plan_init(const cf_geom* geom, const cf_batch* batch, const int32_t* orde
                  const int32_t* kept_count, int32_t query_start, void* plan, size_t plan_bytes,
                  void* stream);
 
+/* cf_plan_init that also sets S = 0 (Algorithm 2, "Init": ids, S) in the same launch: score_accum is device
+ * [n_docs_total], or NULL to leave it alone. */
+int cf_plan_init_scores(const cf_geom* geom, const cf_batch* batch, const int32_t* order,
+                        const int32_t* kept_count, int32_t query_start, float* score_accum, void* plan,
+                        size_t plan_bytes, void* stream);
+
 /* Copies the plan's status word back (synchronises `stream`); returns it as the error code. */
 int cf_plan_status(const cf_geom* geom, const cf_batch* batch, const void* plan, void* stream);
 

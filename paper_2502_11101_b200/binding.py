@@ -24,7 +24,7 @@ TC_KERNEL_BUILT = True      # bf16 / head_dim 128 batches take the tcgen05 atten
 LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libcachefocus.so")
 
 EXPORTS = ["cf_error_string", "cf_allocate_positions", "cf_schedule_linear", "cf_plan_layout_of",
-           "cf_plan_init", "cf_plan_status", "cf_reposition_keys", "cf_attn_workspace_bytes",
+           "cf_plan_init", "cf_plan_init_scores", "cf_plan_status", "cf_reposition_keys", "cf_attn_workspace_bytes",
            "cf_attn_workspace_bytes_layers", "cf_query_prefill_attn", "cf_query_prefill_attn_layers",
            "cf_attn_workspace_bytes_slots", "cf_query_prefill_attn_slot", "cf_accumulate_scores",
            "cf_attn_workspace_bytes_slots_full", "cf_query_prefill_attn_slot_full",
@@ -108,6 +108,7 @@ def load_library() -> ctypes.CDLL:
     lib.cf_schedule_linear.argtypes = [i32, i32, i32, i32, i32, vp, vp, vp]
     lib.cf_plan_layout_of.argtypes = [gp, bp, ctypes.POINTER(cf_plan_layout)]
     lib.cf_plan_init.argtypes = [gp, bp, vp, vp, i32, vp, ctypes.c_size_t, vp]
+    lib.cf_plan_init_scores.argtypes = [gp, bp, vp, vp, i32, vp, vp, ctypes.c_size_t, vp]
     lib.cf_plan_status.argtypes = [gp, bp, vp, vp]
     lib.cf_reposition_keys.argtypes = [gp, bp, vp, i32, i64, vp, vp, vp]
     lib.cf_attn_workspace_bytes.restype = ctypes.c_size_t
@@ -255,7 +256,14 @@ def cf_plan_layout_of(geom: cf_geom, batch: cf_batch) -> cf_plan_layout:
 
 def cf_plan_init(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, order: Optional[torch.Tensor] = None,
                  kept_count: Optional[torch.Tensor] = None, query_start: int = -1, stream=None) -> None:
-    _check(_native().plan_init(geom, batch, plan, order, kept_count, query_start, stream), "cf_plan_init")
+    _check(_native().plan_init(geom, batch, plan, order, kept_count, query_start, None, stream), "cf_plan_init")
+
+
+def cf_plan_init_scores(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, score_accum: torch.Tensor,
+                        order: Optional[torch.Tensor] = None, kept_count: Optional[torch.Tensor] = None,
+                        query_start: int = -1, stream=None) -> None:
+    """cf_plan_init that also clears the accumulated scores, in the same launch."""
+    _check(_native().plan_init(geom, batch, plan, order, kept_count, query_start, score_accum, stream), "cf_plan_init_scores")
 
 
 def cf_plan_status(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, stream=None) -> int:

@@ -139,7 +139,7 @@ PyObject* call(F&& f) {                            // f() returns a CF_* code an
 
 #define NATIVE(name) PyObject* name(PyObject*, PyObject* const* argv, Py_ssize_t argc)
 
-NATIVE(plan_init) {                                // geom, batch, plan, order, kept_count, query_start, stream
+NATIVE(plan_init) {                                // geom, batch, plan, order, kept_count, query_start, score_accum (S = 0) or None, stream
     return guarded([&] {
         Args in(argv, argc);
         Bytes bg, bb;
@@ -149,10 +149,11 @@ NATIVE(plan_init) {                                // geom, batch, plan, order, 
         const int32_t* order = static_cast<const int32_t*>(in.maybe_ptr());
         const int32_t* kept = static_cast<const int32_t*>(in.maybe_ptr());
         const int32_t start = in.i32();
+        float* scores = (float*)in.maybe_ptr();
         void* s = in.stream();
         void* p = plan.data_ptr();
         const size_t n = bytes_of(plan);
-        return call([&] { return cf_plan_init(g, b, order, kept, start, p, n, s); });
+        return call([&] { return cf_plan_init_scores(g, b, order, kept, start, scores, p, n, s); });
     });
 }
 

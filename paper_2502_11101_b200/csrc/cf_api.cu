@@ -424,6 +424,12 @@ int cf_plan_layout_of(const cf_geom* geom, const cf_batch* batch, cf_plan_layout
 int cf_plan_init(const cf_geom* geom, const cf_batch* batch, const int32_t* order,
                  const int32_t* kept_count, int32_t query_start, void* plan, size_t plan_bytes,
                  void* stream) {
+    return cf_plan_init_scores(geom, batch, order, kept_count, query_start, nullptr, plan, plan_bytes, stream);
+}
+
+int cf_plan_init_scores(const cf_geom* geom, const cf_batch* batch, const int32_t* order,
+                        const int32_t* kept_count, int32_t query_start, float* score_accum, void* plan,
+                        size_t plan_bytes, void* stream) {
     int rc = check_plan(geom, batch, plan);
     if (rc != CF_OK) return rc;
     cf_plan_layout L;
@@ -433,10 +439,8 @@ int cf_plan_init(const cf_geom* geom, const cf_batch* batch, const int32_t* orde
         return CF_ERR_RANGE;
     PlanView pv = make_plan_view(geom, batch, plan);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    rc = launch_clear_status(pv, s);
-    if (rc != CF_OK) return rc;
     return launch_plan(make_geom_view(geom), make_batch_view(batch), pv, 0, order, kept_count,
-                       query_start, nullptr, 0, nullptr, CF_ALLOC_ALIGN, s);
+                       query_start, nullptr, 0, nullptr, CF_ALLOC_ALIGN, score_accum, s);
 }
 
 int cf_plan_status(const cf_geom* geom, const cf_batch* batch, const void* plan, void* stream) {
@@ -664,7 +668,7 @@ int cf_prune_topk(const cf_geom* geom, const cf_batch* batch, void* plan,
         return CF_ERR_INVALID_ARG;
     PlanView pv = make_plan_view(geom, batch, plan);
     return launch_plan(make_geom_view(geom), make_batch_view(batch), pv, 1, nullptr, nullptr, -1,
-                       score_accum, keep, keep_per_request, strategy,
+                       score_accum, keep, keep_per_request, strategy, nullptr,
                        static_cast<cudaStream_t>(stream));
 }
 

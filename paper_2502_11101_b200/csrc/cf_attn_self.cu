@@ -39,6 +39,8 @@ __global__ void __launch_bounds__(kSelfThreads)
 self_block_kernel(AttnWorkspace ws, LayerSpan span, ExtraKeys ek, int n_requests, int n_q_heads, int n_kv_heads, int lq,
                   float scale_log2, const T* __restrict__ q) {
     extern __shared__ __align__(16) unsigned char self_smem[];
+    chain_next();
+    chain_wait();
     constexpr int kPitch = D + 2;                                   // odd number of 32-bit words per key row: no bank conflicts
     T* Ks = reinterpret_cast<T*>(self_smem);                        // [kSelfMaxLq][kPitch]
     T* Vs = reinterpret_cast<T*>(self_smem + self_keys_bytes<T, D>(kSelfMaxLq));   // [kSelfMaxLq][D], 16-byte aligned
@@ -173,9 +175,8 @@ int launch_self_typed(const cf_geom* g, const cf_batch* b, const LayerSpan& span
     if (configure_smem_once(configured, self_block_kernel<T, D>, (int)smem) != CF_OK) return CF_ERR_CUDA;
     dim3 grid((unsigned)((rows + kSelfRows - 1) / kSelfRows), (unsigned)g->n_kv_heads,
               (unsigned)(b->n_requests * span.n_layers));
-    self_block_kernel<T, D><<<grid, kSelfThreads, smem, stream>>>(ws, span, ek, b->n_requests, g->n_q_heads, g->n_kv_heads,
-                                                                 b->q_len, scale_log2, static_cast<const T*>(q));
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    return launch_chained(self_block_kernel<T, D>, grid, kSelfThreads, smem, stream, ws, span, ek, b->n_requests, g->n_q_heads,
+                          g->n_kv_heads, b->q_len, scale_log2, static_cast<const T*>(q));
 }
 
 }  // namespace

@@ -25,6 +25,8 @@ attn_simt_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, LayerSpan span, in
                  float scale_log2, const T* __restrict__ q, const T* __restrict__ k_cache,
                  const T* __restrict__ v_cache) {
     extern __shared__ float smem[];
+    chain_next();
+    chain_wait();
     float (*Qs)[D + 1] = reinterpret_cast<float (*)[D + 1]>(smem);
     float (*Ks)[D + 1] = reinterpret_cast<float (*)[D + 1]>(smem + kSimtRows * (D + 1));
     float (*Vs)[D] = reinterpret_cast<float (*)[D]>(smem + (kSimtRows + kSimtSub) * (D + 1));
@@ -201,6 +203,8 @@ template <typename T, int D, typename P>
 __global__ void __launch_bounds__(32 * kCombineRows)
 combine_kernel(AttnWorkspace ws, int n_requests, long long n_rows_all, long long out_layer_stride, int n_q_heads,
                int lq, T* __restrict__ out, float* __restrict__ lse) {
+    chain_next();
+    chain_wait();
     constexpr int V = D / 32;
     static_assert(CF_MAX_SPLITS <= 64, "two parts per lane");
     const int lane = threadIdx.x & 31;
@@ -299,6 +303,8 @@ score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, float*
              float* __restrict__ score_accum) {
     __shared__ float s_red[kScoreThreads / 32];
     __shared__ float s_layer[CF_MAX_LAYERS_PER_CALL];
+    chain_next();
+    chain_wait();
     const int doc = blockIdx.x;
     const int n_layers = ws.n_layers;
     const int count = pv.doc_tile_count[doc];
@@ -357,6 +363,8 @@ template <typename T, int D>
 __global__ void __launch_bounds__(256)
 merge_attn_kernel(long long n_rows, int n_q_heads, int lq, const T* out_a, const float* lse_a,
                   const T* out_b, const float* lse_b, T* out, float* lse) {   // out may alias out_a or out_b, lse likewise
+    chain_next();
+    chain_wait();
     constexpr int V = D / 32;
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);     // index into out: (block, token, head)
@@ -383,17 +391,15 @@ int launch_merge_attn(const cf_geom* g, long long n_rows, int q_len, const void*
     if (blocks <= 0 || blocks > 0x7fffffffLL) return CF_ERR_INVALID_ARG;
     auto run = [&](auto kernel, auto* typed) {
         using T = std::remove_pointer_t<decltype(typed)>;
-        kernel<<<(unsigned)blocks, 256, 0, stream>>>(n_rows, g->n_q_heads, q_len, static_cast<const T*>(out_a), lse_a,
-                                                    static_cast<const T*>(out_b), lse_b, static_cast<T*>(out), lse);
+        return launch_chained(kernel, dim3((unsigned)blocks), 256, 0, stream, n_rows, g->n_q_heads, q_len,
+                              static_cast<const T*>(out_a), lse_a, static_cast<const T*>(out_b), lse_b, static_cast<T*>(out), lse);
     };
     if (g->dtype == CF_BF16) {
-        if (g->head_dim == 128) run(merge_attn_kernel<__nv_bfloat16, 128>, (__nv_bfloat16*)nullptr);
-        else run(merge_attn_kernel<__nv_bfloat16, 64>, (__nv_bfloat16*)nullptr);
-    } else {
-        if (g->head_dim == 128) run(merge_attn_kernel<float, 128>, (float*)nullptr);
-        else run(merge_attn_kernel<float, 64>, (float*)nullptr);
+        if (g->head_dim == 128) return run(merge_attn_kernel<__nv_bfloat16, 128>, (__nv_bfloat16*)nullptr);
+        return run(merge_attn_kernel<__nv_bfloat16, 64>, (__nv_bfloat16*)nullptr);
     }
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    if (g->head_dim == 128) return run(merge_attn_kernel<float, 128>, (float*)nullptr);
+    return run(merge_attn_kernel<float, 64>, (float*)nullptr);
 }
 
 template <typename T, int D>
@@ -410,10 +416,8 @@ static int launch_simt_typed(const cf_geom* g, const cf_batch* b, const PlanView
     static PerDeviceOnce configured[2];              // per (T, D) instantiation and slice layout
     auto run = [&](auto kernel, int which) {
         if (configure_smem_once(configured[which], kernel, (int)smem) != CF_OK) return CF_ERR_CUDA;
-        kernel<<<grid, kSimtThreads, smem, stream>>>(bv, pv, ws, span, g->n_q_heads, g->n_kv_heads, scale_log2,
-                                                     static_cast<const T*>(q), static_cast<const T*>(k),
-                                                     static_cast<const T*>(v));
-        return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+        return launch_chained(kernel, grid, kSimtThreads, smem, stream, bv, pv, ws, span, g->n_q_heads, g->n_kv_heads, scale_log2,
+                              static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v));
     };
     if (g->rope_layout == CF_ROPE_HALF) return run(attn_simt_kernel<T, D, CF_ROPE_HALF>, 0);
     return run(attn_simt_kernel<T, D, CF_ROPE_INTERLEAVED>, 1);
@@ -436,13 +440,9 @@ static int launch_combine_typed(const cf_geom* g, const cf_batch* b, const Layer
     const long long rows_all = (long long)span.n_layers * b->n_requests * g->n_q_heads * b->q_len;
     const long long blocks = (rows_all + kCombineRows - 1) / kCombineRows;
     if (blocks > 0x7fffffffLL || ws.n_splits > CF_MAX_SPLITS) return CF_ERR_INVALID_ARG;
-    if (ws.part_bf16)
-        combine_kernel<T, D, __nv_bfloat16><<<(unsigned)blocks, 32 * kCombineRows, 0, stream>>>(
-            ws, b->n_requests, rows_all, span.out_stride, g->n_q_heads, b->q_len, static_cast<T*>(out), lse);
-    else
-        combine_kernel<T, D, float><<<(unsigned)blocks, 32 * kCombineRows, 0, stream>>>(
-            ws, b->n_requests, rows_all, span.out_stride, g->n_q_heads, b->q_len, static_cast<T*>(out), lse);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    return launch_chained(ws.part_bf16 ? combine_kernel<T, D, __nv_bfloat16> : combine_kernel<T, D, float>, dim3((unsigned)blocks),
+                          32 * kCombineRows, 0, stream, ws, b->n_requests, rows_all, span.out_stride, g->n_q_heads, b->q_len,
+                          static_cast<T*>(out), lse);
 }
 
 int launch_combine(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span,
@@ -461,13 +461,9 @@ int launch_combine(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
 
 int launch_scores(const cf_geom* g, const cf_batch* b, const PlanView& pv, const AttnWorkspace& ws, float* doc_scores,
                   float* score_accum, cudaStream_t stream) {
-    if (b->n_docs_total > 0 && (doc_scores || score_accum)) {
-        score_kernel<<<(unsigned)b->n_docs_total, kScoreThreads, 0, stream>>>(make_batch_view(b), pv, ws,
-                                                                   g->n_q_heads * b->q_len, doc_scores,
-                                                                   score_accum);
-        if (cudaGetLastError() != cudaSuccess) return CF_ERR_CUDA;
-    }
-    return CF_OK;
+    if (b->n_docs_total <= 0 || (!doc_scores && !score_accum)) return CF_OK;
+    return launch_chained(score_kernel, dim3((unsigned)b->n_docs_total), kScoreThreads, 0, stream, make_batch_view(b), pv, ws,
+                          g->n_q_heads * b->q_len, doc_scores, score_accum);
 }
 
 }  // namespace cf

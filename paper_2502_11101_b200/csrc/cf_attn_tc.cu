@@ -122,6 +122,8 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps,
                BatchView bv, PlanView pv, AttnWorkspace ws, long long q_layer_stride, int n_q_heads, int n_kv_heads,
                float scale_log2, const __nv_bfloat16* __restrict__ q, int with_self, int prefix_len) {
     extern __shared__ unsigned char smem_raw[];
+    chain_next();
+    chain_wait();
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t smem_base = smem_u32(smem);
 
@@ -688,10 +690,8 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
     static PerDeviceOnce configured[2];
     auto run = [&](auto kernel, int which) {
         if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return CF_ERR_CUDA;
-        kernel<<<grid, kThreads, kSmemBytes, stream>>>(maps, bv, pv, ws, span.q_stride, g->n_q_heads,
-                                                       g->n_kv_heads, scale_log2, static_cast<const __nv_bfloat16*>(q),
-                                                       k_self ? 1 : 0, prefix_len);
-        return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+        return launch_chained(kernel, grid, kThreads, kSmemBytes, stream, maps, bv, pv, ws, span.q_stride, g->n_q_heads, g->n_kv_heads,
+                              scale_log2, static_cast<const __nv_bfloat16*>(q), k_self ? 1 : 0, prefix_len);
     };
     if (g->rope_layout == CF_ROPE_HALF) return run(attn_tc_kernel<CF_ROPE_HALF>, 0);
     return run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, 1);

@@ -29,6 +29,8 @@ docattn_simt_kernel(DocAttnArgs a, const T* __restrict__ q, const T* __restrict_
                     const T* __restrict__ k_prefix, const T* __restrict__ v_prefix, T* __restrict__ out,
                     float* __restrict__ lse) {
     extern __shared__ float smem[];
+    chain_next();
+    chain_wait();
     float (*Qs)[D + 1] = reinterpret_cast<float (*)[D + 1]>(smem);
     float (*Ks)[D + 1] = reinterpret_cast<float (*)[D + 1]>(smem + kDocRows * (D + 1));
     float (*Vs)[D] = reinterpret_cast<float (*)[D]>(smem + (kDocRows + kDocSub) * (D + 1));
@@ -152,10 +154,9 @@ int launch_docattn_simt_typed(const DocAttnArgs& a, const void* q, const void* k
     static PerDeviceOnce configured;
     if (configure_smem_once(configured, docattn_simt_kernel<T, D>, (int)doc_smem_bytes<D>()) != CF_OK) return CF_ERR_CUDA;
     dim3 grid((unsigned)chunks, (unsigned)a.n_kv_heads, (unsigned)(a.n_docs * a.n_layers));
-    docattn_simt_kernel<T, D><<<grid, kDocThreads, doc_smem_bytes<D>(), stream>>>(
-        a, static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), static_cast<const T*>(kp),
-        static_cast<const T*>(vp), static_cast<T*>(out), lse);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    return launch_chained(docattn_simt_kernel<T, D>, grid, kDocThreads, doc_smem_bytes<D>(), stream, a, static_cast<const T*>(q),
+                          static_cast<const T*>(k), static_cast<const T*>(v), static_cast<const T*>(kp), static_cast<const T*>(vp),
+                          static_cast<T*>(out), lse);
 }
 
 }  // namespace

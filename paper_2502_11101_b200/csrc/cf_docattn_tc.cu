@@ -123,6 +123,8 @@ __global__ void __launch_bounds__(kDocTcThreads, 2)
 docattn_tc_kernel(const __grid_constant__ DocMaps maps, DocAttnArgs a, DocGrid dg,
                   __nv_bfloat16* __restrict__ out_all, float* __restrict__ lse, int* status) {
     extern __shared__ unsigned char smem_raw[];
+    chain_next();
+    chain_wait();
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t q_base = smem_u32(smem), k_base = q_base + kTileBytes, v_base = k_base + kTileBytes;
     DocBars* bars = reinterpret_cast<DocBars*>(smem + 3 * kTileBytes);
@@ -479,8 +481,8 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
     const unsigned grid = (unsigned)std::min<long long>(total, ctas);
     const DocGrid dg = {(int)row_tiles, (int)total, group, (a.prefix_len + kTile - 1) / kTile, rows_per_tile,
                         a.prefix_len % kBoxRows == 0 ? 1 : 0, a.prefix_len};
-    docattn_tc_kernel<<<grid, kDocTcThreads, kDocTcSmem, stream>>>(maps, a, dg, static_cast<__nv_bfloat16*>(out), lse, status);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    return launch_chained(docattn_tc_kernel, dim3(grid), kDocTcThreads, kDocTcSmem, stream, maps, a, dg, static_cast<__nv_bfloat16*>(out),
+                          lse, status);
 }
 
 }  // namespace cf

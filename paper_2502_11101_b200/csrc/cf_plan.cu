@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, const int* __restrict__ order,
             const int* __restrict__ kept_count_in, int query_start_arg,
             const float* __restrict__ score_accum, int keep, const int* __restrict__ keep_per_request,
-            int strategy) {
+            int strategy, float* clear_scores) {
     __shared__ int s_ids[kMaxDocs];       // kept local ids by rank
     __shared__ int s_tmp[kMaxDocs];       // new order; running lengths of the windows; first tile of every rank
     __shared__ int s_row[kMaxDocs + 1];   // first store row of every document (by local id), and the end
@@ -135,8 +135,16 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
     __shared__ int s_longest, s_min_cursor;
     __shared__ int s_warp_sum[kPlanThreads / 32 + 1];
 
+    chain_next();
+    chain_wait();
     const int b = blockIdx.x;
     const int tid = threadIdx.x;
+    // a batch of one request starts with clear status words and, if asked for, S = 0 (larger ones: clear_kernel)
+    if (mode == 0 && gridDim.x == 1) {
+        if (tid == 0) pv.status[0] = pv.status[1] = pv.status[2] = pv.status[3] = 0;
+        if (clear_scores)
+            for (int i = tid; i < bv.n_docs_total; i += blockDim.x) clear_scores[i] = 0.f;
+    }
     const int nthreads = (int)blockDim.x;               // at least the documents of any request, a multiple of 32
     const int doc0 = bv.req_doc_begin[b];
     const int n_docs = bv.req_doc_begin[b + 1] - doc0;
@@ -375,20 +383,19 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
     }
 }
 
-// Clears the status words of a plan (a one-thread kernel: a kernel node after a kernel node costs
-// less than a memset node between two kernels).
-__global__ void clear_status_kernel(int* status) {
-    status[0] = status[1] = status[2] = status[3] = 0;
-}
-
-int launch_clear_status(const PlanView& pv, cudaStream_t stream) {
-    clear_status_kernel<<<1, 1, 0, stream>>>(pv.status);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+// Clears the status words of a plan and the accumulated scores (one kernel: a kernel node after a kernel node costs less
+// than a memset node between two kernels).
+__global__ void __launch_bounds__(256) clear_kernel(int* status, float* scores, int n) {
+    chain_next();
+    chain_wait();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < 4) status[i] = 0;
+    if (scores && i < n) scores[i] = 0.f;
 }
 
 int launch_plan(const GeomView& gv, const BatchView& bv, const PlanView& pv, int mode,
                 const int* order, const int* kept_count, int query_start, const float* score_accum,
-                int keep, const int* keep_per_request, int strategy, cudaStream_t stream) {
+                int keep, const int* keep_per_request, int strategy, float* clear_scores, cudaStream_t stream) {
     if (gv.head_dim > 128) return CF_ERR_UNSUPPORTED;
     InvFreq inv_freq;
     for (int p = 0; p < gv.head_dim / 2; ++p) {
@@ -399,10 +406,13 @@ int launch_plan(const GeomView& gv, const BatchView& bv, const PlanView& pv, int
     // one thread per document of a request; barriers and scans cost less in a small block, the rotation tables (64 slices
     // per kept document) want many threads: 256 is the measured optimum for batches of up to 256 documents
     const int threads = std::min(kPlanThreads, std::max(256, (std::min(bv.n_docs_total, kMaxDocs) + 31) / 32 * 32));
-    plan_kernel<<<bv.n_requests, threads, 0, stream>>>(gv, bv, pv, inv_freq, mode, order, kept_count,
-                                                           query_start, score_accum, keep,
-                                                           keep_per_request, strategy);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    if (mode == 0 && bv.n_requests > 1) {
+        const int rc = launch_chained(clear_kernel, dim3((unsigned)(clear_scores ? (bv.n_docs_total + 255) / 256 + 1 : 1)), 256, 0, stream,
+                                      pv.status, clear_scores, bv.n_docs_total);
+        if (rc != CF_OK) return rc;
+    }
+    return launch_chained(plan_kernel, dim3((unsigned)bv.n_requests), threads, 0, stream, gv, bv, pv, inv_freq, mode, order, kept_count,
+                          query_start, score_accum, keep, keep_per_request, strategy, clear_scores);
 }
 
 }  // namespace cf

@@ -69,6 +69,8 @@ template <typename T, int D, int LAYOUT>
 __global__ void __launch_bounds__(kRepoThreads)
 reposition_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_stride,
                   const T* k_in, T* k_out, int pieces) {
+    chain_next();
+    chain_wait();
     constexpr int E = Vec16<T>::kElems;
     constexpr int kVecPerHead = D / E;                                    // 16-byte vectors per (row, head)
     constexpr int kItemsPerHead = LAYOUT == CF_ROPE_HALF ? kVecPerHead / 2 : kVecPerHead;
@@ -148,6 +150,8 @@ assemble_kernel(BatchView bv, PlanView pv, int n_kv_heads, long long layer_strid
                 int out_rows, const T* __restrict__ k_in, const T* __restrict__ v_in,
                 const T* __restrict__ k_self, const T* __restrict__ v_self, T* __restrict__ k_out,
                 T* __restrict__ v_out, int* __restrict__ final_rows, int pieces) {
+    chain_next();
+    chain_wait();
     constexpr int E = Vec16<T>::kElems;
     constexpr int kVecPerHead = D / E;
     __shared__ int s_red[kRepoThreads / 32];
@@ -241,15 +245,10 @@ static int launch_assemble_typed(const cf_geom* g, const cf_batch* b, const Plan
     const int pieces = pieces_per_tile((long long)tiles * n_layers * b->n_requests, (kTile * items_per_row + kRepoThreads - 1) / kRepoThreads);
     dim3 grid((unsigned)(tiles * pieces), (unsigned)n_layers, (unsigned)b->n_requests);
     BatchView bv = make_batch_view(b);
-    auto args = [&](auto kernel) {
-        kernel<<<grid, kRepoThreads, 0, stream>>>(bv, pv, g->n_kv_heads, layer_stride, self_stride, out_rows,
-                                                  static_cast<const T*>(k_in), static_cast<const T*>(v_in),
-                                                  static_cast<const T*>(k_self), static_cast<const T*>(v_self),
-                                                  static_cast<T*>(k_out), static_cast<T*>(v_out), final_rows, pieces);
-    };
-    if (g->rope_layout == CF_ROPE_HALF) args(assemble_kernel<T, D, CF_ROPE_HALF>);
-    else args(assemble_kernel<T, D, CF_ROPE_INTERLEAVED>);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    return launch_chained(g->rope_layout == CF_ROPE_HALF ? assemble_kernel<T, D, CF_ROPE_HALF> : assemble_kernel<T, D, CF_ROPE_INTERLEAVED>,
+                          grid, kRepoThreads, 0, stream, bv, pv, g->n_kv_heads, layer_stride, self_stride, out_rows,
+                          static_cast<const T*>(k_in), static_cast<const T*>(v_in), static_cast<const T*>(k_self),
+                          static_cast<const T*>(v_self), static_cast<T*>(k_out), static_cast<T*>(v_out), final_rows, pieces);
 }
 
 int launch_assemble(const cf_geom* g, const cf_batch* b, const PlanView& pv, int n_layers, long long layer_stride,
@@ -274,13 +273,9 @@ static int launch_typed(const cf_geom* g, const cf_batch* b, const PlanView& pv,
     dim3 grid((unsigned)(tiles * pieces), (unsigned)n_layers, (unsigned)b->n_requests);
     if (n_layers > 65535 || b->n_requests > 65535) return CF_ERR_INVALID_ARG;
     BatchView bv = make_batch_view(b);
-    if (g->rope_layout == CF_ROPE_HALF)
-        reposition_kernel<T, D, CF_ROPE_HALF><<<grid, kRepoThreads, 0, stream>>>(
-            bv, pv, g->n_kv_heads, layer_stride, static_cast<const T*>(k_in), static_cast<T*>(k_out), pieces);
-    else
-        reposition_kernel<T, D, CF_ROPE_INTERLEAVED><<<grid, kRepoThreads, 0, stream>>>(
-            bv, pv, g->n_kv_heads, layer_stride, static_cast<const T*>(k_in), static_cast<T*>(k_out), pieces);
-    return cudaGetLastError() == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+    return launch_chained(g->rope_layout == CF_ROPE_HALF ? reposition_kernel<T, D, CF_ROPE_HALF> : reposition_kernel<T, D, CF_ROPE_INTERLEAVED>,
+                          grid, kRepoThreads, 0, stream, bv, pv, g->n_kv_heads, layer_stride, static_cast<const T*>(k_in),
+                          static_cast<T*>(k_out), pieces);
 }
 
 int launch_reposition(const cf_geom* g, const cf_batch* b, const PlanView& pv, int n_layers,

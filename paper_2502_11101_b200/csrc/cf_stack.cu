@@ -136,17 +136,15 @@ int cf_run_stack(const cf_geom* geom, const cf_batch* batch, const cf_stack* sta
                                 (stack->k_self && stack->self_layer_stride <= 0) ||
                                 (stack->prefix_len > 0 && stack->prefix_layer_stride <= 0)))
         return CF_ERR_INVALID_ARG;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t esize = geom->dtype == CF_BF16 ? 2 : 4;
     const size_t nd = (size_t)batch->n_docs_total;
     const size_t lse_layer = (size_t)batch->n_requests * geom->n_q_heads * batch->q_len;
 
     // Init: S = 0, every document kept in retrieval order, first allocation
-    if (nd > 0 && cudaMemsetAsync(stack->score_accum, 0, nd * sizeof(float), s) != cudaSuccess) return CF_ERR_CUDA;
     cf_batch local = *batch;
     int keep = max_docs_per_request(batch, stack);
     local.tiles_hint = live_tiles_hint(batch, stack, keep);
-    rc = cf_plan_init(geom, &local, nullptr, nullptr, -1, plan, plan_bytes, stream);
+    rc = cf_plan_init_scores(geom, &local, nullptr, nullptr, -1, stack->score_accum, plan, plan_bytes, stream);
     if (rc != CF_OK) return rc;
 
     // Phase 1: layer_l (attention over the kept caches, S += s^l), pruning and re-allocation at the scheduled layers

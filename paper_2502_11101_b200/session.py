@@ -68,8 +68,7 @@ class Session:
 
     def init(self, order: Optional[torch.Tensor] = None, kept_count: Optional[torch.Tensor] = None,
              query_start: int = -1) -> None:
-        self.score_accum.zero_()
-        B.cf_plan_init(self.geom, self.batch, self.plan, order, kept_count, query_start)
+        B.cf_plan_init_scores(self.geom, self.batch, self.plan, self.score_accum, order, kept_count, query_start)
 
     def attend(self, q: torch.Tensor, k_layer: torch.Tensor, v_layer: torch.Tensor, out: torch.Tensor,
                lse: Optional[torch.Tensor] = None, softmax_scale: float = 0.0) -> None:
