@@ -55,7 +55,7 @@ extern "C" {
 #define CF_ALLOC_ALIGN 1        /* Dynamic Positional Allocation ("align", Sec. 2.5)            */
 #define CF_ALLOC_SORT  2        /* Attention-Guided Allocation ("sort", Sec. 2.5)               */
 
-#define CF_TILE_TOKENS 128      /* key tiles never straddle two documents                       */
+#define CF_TILE_TOKENS 96       /* key tiles never straddle two documents                       */
 #define CF_MAX_DOCS_PER_REQUEST 1024
 #define CF_MAX_SPLITS 64
 #define CF_MAX_LAYERS_PER_CALL 64 /* layers one cf_query_prefill_attn_layers call may batch       */

@@ -16,7 +16,7 @@ CF_OK, CF_ERR_INVALID_ARG, CF_ERR_RANGE, CF_ERR_UNSUPPORTED, CF_ERR_WORKSPACE, C
 CF_BF16, CF_F32 = 0, 1
 CF_ROPE_HALF, CF_ROPE_INTERLEAVED = 0, 1
 CF_ALLOC_NONE, CF_ALLOC_ALIGN, CF_ALLOC_SORT = 0, 1, 2
-CF_TILE_TOKENS = 128
+CF_TILE_TOKENS = 96
 CF_MAX_LAYERS_PER_CALL = 64
 CF_MAX_SPLITS = 64
 TC_KERNEL_BUILT = True      # bf16 / head_dim 128 batches take the tcgen05 attention kernel

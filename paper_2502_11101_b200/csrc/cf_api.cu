@@ -138,37 +138,14 @@ int tiles_per_request_bound(const cf_batch* b) {
     return (int)std::min<long long>(t, 1 << 20);
 }
 
-// Query rows one CTA of the tensor-core kernel owns.  A CTA holds two 128-row tiles; when the rows
-// that share a kv head fill an odd number of such tiles (and more than one), CTAs of one tile each
-// -- whose two warpgroups then take alternate key tiles -- split the work evenly, where pairs would
-// leave a half-empty CTA on the critical path.
-int choose_row_group(const cf_geom* g, const cf_batch* b) {
-    const int rows = (g->n_q_heads / g->n_kv_heads) * b->q_len;
-    const int row_tiles = (rows + 127) / 128;
-    return (row_tiles > 1 && (row_tiles & 1)) ? 128 : 256;
-}
-
-// Parts the key-tile list of a request is cut into.  The tensor-core kernel runs one CTA per
-// (layer, request, kv head, group of query rows, pair of parts): as many CTAs as fit one wave over
-// the SMs, never more CTAs than tiles.  The count is always even.
+// Parts the key-tile list of a request is cut into by the CUDA-core kernel, which runs one CTA per (layer, request, kv
+// head, 64 query rows, part): about two CTAs per SM, never more than tiles.
 int choose_splits(const cf_geom* g, const cf_batch* b, int n_layers) {
     const int rows = (g->n_q_heads / g->n_kv_heads) * b->q_len;
-    const int rg_rows = choose_row_group(g, b);
-    const int row_groups = (rows + rg_rows - 1) / rg_rows;
-    const long long units = (long long)n_layers * b->n_requests * g->n_kv_heads * row_groups;
-    const long long sms = sm_count();
-    long long s = sms / units;                        // whole CTAs per SM: one wave, no ragged second wave
-    if (s == 0) {                                     // more units than SMs: balance the waves instead
-        double best = 0.0;
-        for (long long c = 1; c <= 4; ++c) {
-            const long long ctas = units * c, waves = (ctas + sms - 1) / sms;
-            const double eff = (double)ctas / (double)(waves * sms);
-            if (eff > best + 0.03) { best = eff; s = c; }
-        }
-    }
+    const long long units = (long long)n_layers * b->n_requests * g->n_kv_heads * ((rows + 63) / 64);
+    long long s = (2LL * sm_count() + units - 1) / units;
     s = std::min<long long>(s, tiles_per_request_bound(b));
-    s = std::min<long long>(s, CF_MAX_SPLITS / 2);
-    return 2 * (int)std::max<long long>(s, 1);
+    return (int)std::max<long long>(1, std::min<long long>(s, CF_MAX_SPLITS));
 }
 
 size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, int n_layers, bool with_self,
@@ -184,9 +161,13 @@ size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, 
         off = align_up(off + count * 4, 256);
         return at;
     };
-    size_t o = take(nlb * n_splits * rows * g->head_dim);
-    size_t m = take(nlb * n_splits * rows);
-    size_t l = take(nlb * n_splits * rows);
+    // room for the parts of either kernel family
+    const size_t tc_rows = attn_tc_supported(g, b) ? attn_tc_part_rows() : 0;
+    const size_t parts = std::max(nlb * n_splits * rows, tc_rows);
+    size_t o = take(std::max(nlb * n_splits * rows * g->head_dim, tc_rows * g->head_dim / 2));
+    size_t m = take(parts);
+    size_t l = take(parts);
+    size_t mk = take(tc_rows);
     size_t t = take((size_t)n_layers * max_tiles * rows);
     size_t r = take(nlb_lse * rows);
     size_t so = 0, sm = 0, sl = 0, ld = 0;
@@ -194,19 +175,19 @@ size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, 
         so = take(nlb * rows * g->head_dim);
         sm = take(nlb * rows);
         sl = take(nlb * rows);
-        ld = take(nlb * n_splits * rows);
+        ld = take(parts);
     }
     if (ws) {
         ws->part_o = reinterpret_cast<float*>(base + o);
         ws->part_m = reinterpret_cast<float*>(base + m);
         ws->part_l = reinterpret_cast<float*>(base + l);
+        ws->marks = reinterpret_cast<int*>(base + mk);
         ws->tile_lse2 = reinterpret_cast<float*>(base + t);
         ws->row_lse2 = reinterpret_cast<float*>(base + r);
         ws->n_splits = n_splits;
-        ws->part_bf16 = 0;
         ws->n_layers = n_layers;
         ws->max_tiles = (int)max_tiles;
-        ws->rg_rows = choose_row_group(g, b);
+        ws->rg_rows = attn_tc_supported(g, b) ? attn_tc_row_tile(g, b) : 0;
         ws->self_o = with_self ? reinterpret_cast<float*>(base + so) : nullptr;
         ws->self_m = with_self ? reinterpret_cast<float*>(base + sm) : nullptr;
         ws->self_l = with_self ? reinterpret_cast<float*>(base + sl) : nullptr;
@@ -305,7 +286,7 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
                                   v_cache, scale * kLog2e, out, lse, workspace, s);
     }
     const bool tensor_core = g_attn_path.load() == 0 && attn_tc_supported(geom, batch);
-    if (with_self && batch->q_len > CF_TILE_TOKENS) return CF_ERR_UNSUPPORTED;
+    if (with_self && batch->q_len > 128) return CF_ERR_UNSUPPORTED;
     if (!tensor_core) ws.part_ld = nullptr;           // only the tensor-core kernel reports per-part document sums
     if ((with_self || with_prefix) && !tensor_core) { // the CUDA-core path computes these blocks as a part of their own
         ws.self_mode = 1;
@@ -316,16 +297,15 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
     cudaEvent_t ev_start, ev_stop;
     const bool timed = prof_claim(&ev_start, &ev_stop) >= 0;
     if (timed) cudaEventRecord(ev_start, s);
-    if (tensor_core) {
-        ws.part_bf16 = 1;
-        ws.self_mode = (with_self || with_prefix) ? 2 : 0;   // the blocks ride along as further key tiles
+    if (tensor_core)
         rc = launch_attn_tc(geom, batch, pv, span, q, k_cache, v_cache, k_self, v_self, self_stride, k_prefix, v_prefix,
-                            prefix_stride, prefix_len, scale * kLog2e, ws, s);
-    } else
+                            prefix_stride, prefix_len, scale * kLog2e, ws, out, lse, s);
+    else
         rc = launch_attn_simt(geom, batch, pv, span, q, k_cache, v_cache, scale * kLog2e, ws, s);
     if (timed) cudaEventRecord(ev_stop, s);
+    if (rc == CF_OK && !tensor_core) rc = launch_combine(geom, batch, pv, span, ws, out, lse, s);
     if (rc != CF_OK) return rc;
-    return launch_combine(geom, batch, pv, span, ws, out, lse, doc_scores, score_accum, s);
+    return launch_scores(geom, batch, pv, ws, doc_scores, score_accum, s);
 }
 
 }  // namespace cf

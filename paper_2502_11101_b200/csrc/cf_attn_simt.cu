@@ -158,7 +158,7 @@ attn_simt_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, LayerSpan span, in
     }
 }
 
-// D/32 consecutive elements of a partial O row (fp32 or bf16) as floats.
+// D/32 consecutive elements of a partial O row.
 template <int V>
 __device__ __forceinline__ void load_part(const float* p, float (&x)[V]) {
     if (V == 4) {
@@ -167,17 +167,6 @@ __device__ __forceinline__ void load_part(const float* p, float (&x)[V]) {
     } else {
         const float2 t = *reinterpret_cast<const float2*>(p);
         x[0] = t.x; x[1] = t.y;
-    }
-}
-template <int V>
-__device__ __forceinline__ void load_part(const __nv_bfloat16* p, float (&x)[V]) {
-    if (V == 4) {
-        const uint2 t = *reinterpret_cast<const uint2*>(p);
-        x[0] = __uint_as_float(t.x << 16); x[1] = __uint_as_float(t.x & 0xffff0000u);
-        x[V - 2] = __uint_as_float(t.y << 16); x[V - 1] = __uint_as_float(t.y & 0xffff0000u);
-    } else {
-        const uint32_t t = *reinterpret_cast<const uint32_t*>(p);
-        x[0] = __uint_as_float(t << 16); x[1] = __uint_as_float(t & 0xffff0000u);
     }
 }
 template <int V>
@@ -199,7 +188,7 @@ constexpr int kCombineDepth = 8;      // parts whose loads are in flight togethe
 // out = sum_p w_p O_p / sum_p w_p l_p with w_p = 2^(m_p - max m), and the row's log-sum-exp.
 // Parts are visited in index order and the warp reductions have a fixed shape, so the result does
 // not depend on scheduling.
-template <typename T, int D, typename P>
+template <typename T, int D>
 __global__ void __launch_bounds__(32 * kCombineRows)
 combine_kernel(AttnWorkspace ws, int n_requests, long long n_rows_all, long long out_layer_stride, int n_q_heads,
                int lq, T* __restrict__ out, float* __restrict__ lse) {
@@ -237,7 +226,7 @@ combine_kernel(AttnWorkspace ws, int n_requests, long long n_rows_all, long long
     float acc[V];
 #pragma unroll
     for (int i = 0; i < V; ++i) acc[i] = 0.f;
-    const P* po = reinterpret_cast<const P*>(ws.part_o) + slot0 * D + lane * V;
+    const float* po = ws.part_o + slot0 * D + lane * V;
     const size_t stride = (size_t)rows_total * D;
     for (int p0 = 0; p0 < n_parts; p0 += kCombineDepth) {             // independent loads in flight
         float wp[kCombineDepth], x[kCombineDepth][V];
@@ -256,20 +245,7 @@ combine_kernel(AttnWorkspace ws, int n_requests, long long n_rows_all, long long
             }
     }
     // the documents' share of the row: what the document scores are measured against
-    float docs_l = l_sum;
-    if (ws.self_mode == 2) {
-        // further key blocks were tiles of some parts: every part reports its sum over the documents alone
-        float ld[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int p = lane + 32 * k;
-            ld[k] = (p < n_parts && m[k] > -INFINITY) ? ws.part_ld[slot0 + (size_t)p * rows_total] : 0.f;
-        }
-        docs_l = fmaf(ld[1], w[1], ld[0] * w[0]);                       // same tree as l_sum, no subtraction
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) docs_l += __shfl_xor_sync(0xffffffffu, docs_l, o);
-    }
-    const float docs_lse2 = docs_l > 0.f ? m_max + log2f(docs_l) : -INFINITY;
+    const float docs_lse2 = l_sum > 0.f ? m_max + log2f(l_sum) : -INFINITY;
     float m_all = m_max, l_all = l_sum;
     if (ws.self_mode == 1) {                                           // the query-self block joins as one more part
         const size_t srow = (size_t)lb * rows_total + rg;
@@ -440,23 +416,18 @@ static int launch_combine_typed(const cf_geom* g, const cf_batch* b, const Layer
     const long long rows_all = (long long)span.n_layers * b->n_requests * g->n_q_heads * b->q_len;
     const long long blocks = (rows_all + kCombineRows - 1) / kCombineRows;
     if (blocks > 0x7fffffffLL || ws.n_splits > CF_MAX_SPLITS) return CF_ERR_INVALID_ARG;
-    return launch_chained(ws.part_bf16 ? combine_kernel<T, D, __nv_bfloat16> : combine_kernel<T, D, float>, dim3((unsigned)blocks),
+    return launch_chained(combine_kernel<T, D>, dim3((unsigned)blocks),
                           32 * kCombineRows, 0, stream, ws, b->n_requests, rows_all, span.out_stride, g->n_q_heads, b->q_len,
                           static_cast<T*>(out), lse);
 }
 
 int launch_combine(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span,
-                   const AttnWorkspace& ws, void* out, float* lse, float* doc_scores, float* score_accum,
-                   cudaStream_t stream) {
-    int rc;
+                   const AttnWorkspace& ws, void* out, float* lse, cudaStream_t stream) {
     if (g->dtype == CF_BF16)
-        rc = g->head_dim == 128 ? launch_combine_typed<__nv_bfloat16, 128>(g, b, span, ws, out, lse, stream)
-                                : launch_combine_typed<__nv_bfloat16, 64>(g, b, span, ws, out, lse, stream);
-    else
-        rc = g->head_dim == 128 ? launch_combine_typed<float, 128>(g, b, span, ws, out, lse, stream)
-                                : launch_combine_typed<float, 64>(g, b, span, ws, out, lse, stream);
-    if (rc != CF_OK) return rc;
-    return launch_scores(g, b, pv, ws, doc_scores, score_accum, stream);
+        return g->head_dim == 128 ? launch_combine_typed<__nv_bfloat16, 128>(g, b, span, ws, out, lse, stream)
+                                  : launch_combine_typed<__nv_bfloat16, 64>(g, b, span, ws, out, lse, stream);
+    return g->head_dim == 128 ? launch_combine_typed<float, 128>(g, b, span, ws, out, lse, stream)
+                              : launch_combine_typed<float, 64>(g, b, span, ws, out, lse, stream);
 }
 
 int launch_scores(const cf_geom* g, const cf_batch* b, const PlanView& pv, const AttnWorkspace& ws, float* doc_scores,

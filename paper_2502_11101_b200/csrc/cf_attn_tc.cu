@@ -1,31 +1,33 @@
 // Fused re-position + query-prefill attention on the Blackwell tensor cores (bf16, head_dim 128).
 //
-// Eq. 5 fused into Eq. 1: key tiles are streamed from the un-repositioned store by TMA into
-// 128B-swizzled shared memory, every key is rotated by its document's delta in registers and
-// written back in place, QK^T and PV run as tcgen05.mma with fp32 accumulators in tensor memory,
-// the softmax runs one query row per thread out of tensor memory and hands P back through tensor
-// memory (bf16, aliased onto the upper half of S).  The cache is read once.
+// Eq. 5 fused into Eq. 1: key tiles are streamed from the un-repositioned store by TMA into 128B-swizzled shared memory,
+// rotated there in place by their document's delta (fp32, one rounding: bit for bit what cf_reposition_keys writes) and
+// handed to the tensor cores.
 //
-// One CTA owns a (layer, request, kv head, group of <=256 query rows, range of key tiles).  Two softmax
-// warpgroups work side by side, each with its own S and O accumulators in tensor memory:
-//   - with more than 128 query rows in the group, warpgroup w owns row tile w and both see every
-//     key tile of the CTA's range;
-//   - with at most 128 rows, both own the same rows and take alternate key tiles, i.e. the CTA
-//     produces two independent parts of the split-KV decomposition.
-// Partial results (reference maximum, sum, unnormalised O) go to the workspace and are merged by
-// the combine kernel.  Warp roles (512 threads):
-//   warps 0-3    softmax warpgroup 0 (thread = query row = TMEM lane)
-//   warps 4-7    softmax warpgroup 1
-//   warps 8-11, 14, 15  key rotation in shared memory
-//   warp 12      TMA producer (one lane)     warp 13  TMEM allocation and MMA issue (one lane)
-// The MMA warp interleaves the two warpgroups (PV of one, then the next QK^T of the same one), so
-// one warpgroup's exponentials overlap the other's tensor-core work.
-// The softmax is single-pass: the reference maximum of a row only moves when a 32-key chunk exceeds
-// it by more than 2^8, in which case O, the sums and the P columns already written are rescaled
-// (rare after the first chunk); any reference within the exponent range is exact enough because
-// P (bf16) and the sums (fp32) keep their relative precision.
-// Every wait on an mbarrier is bounded; when a wait expires the CTA raises CF_ERR_TIMEOUT in the
-// plan's status word, all roles leave their loops, and the CTA frees its tensor memory and exits.
+// Work: the key tiles (runs of at most kTile rows of one document, from the plan) of every (layer, request, kv head, tile of
+// at most 128 query rows) laid on one line and cut into equal shares, one per SM: a CTA walks its share, which may end in the
+// middle of a unit and hold several whole ones.  A unit inside one share is finished there; parts of others meet in the merge
+// kernel.  With one CTA per (unit, range) as before, 256 units on 148 SMs left a quarter of the last wave idle and every
+// wave paid set-up and epilogue again.
+//   warps 0-7            two softmax warpgroups, alternate key tiles of the same rows (thread = query row = TMEM lane)
+//   warps 8, 10, 11, 13-15   key rotation in shared memory
+//   warp 9               key, value and rotation-table loads     warp 12  MMA issue
+// The two single-warp roles issue a few dozen dependent instructions per tile and are what the CTA waits for when they have
+// to share their scheduler (warp index mod 4) with too much arithmetic: each has one rotation warp beside it, the other two
+// schedulers have two (all six on three schedulers: 8 x 15 documents, 32 heads 101 us, this way 90).  Tile descriptions are fetched a tile ahead, and what the other roles need to know about a tile they find in shared memory.
+// Tensor memory: O (128 columns), the query tile (64: as the A operand of QK^T it costs no shared-memory reads, which this
+// kernel has none to spare of), three S buffers of 96 columns; P (bf16) overwrites the S columns already consumed.  S(n + 3) is issued behind PV(n), so a softmax warpgroup that has finished a
+// tile finds its next S waiting.
+// Softmax: both warpgroups accumulate into one O under one reference per row, fixed by the first 16 keys of the segment:
+// their maximum plus 40.  P and the sums keep their relative precision for logits up to 80 (log2 units) above that first
+// maximum and as far below as matters, so that no tile has to look at its maximum before its exponentials.  A row that
+// does leave this range is marked (NaN sum) and recomputed from scratch by the merge kernel.
+// What bounds it (per 96-key tile and 128 rows, in SM cycles): tensor cores 768 (8 x 48 + 6 x 64), exponentials 768 on
+// the shared MUFU, shared memory 1150 (copies 384, rotation 384, QK^T 192, PV 192), so these overlap only if nobody
+// waits for a chain.
+// Every wait on an mbarrier is bounded; when a wait expires the CTA raises CF_ERR_TIMEOUT in the plan's status word, all
+// roles leave their loops, and the CTA frees its tensor memory and exits.  Each barrier has one kind of waiter, which waits
+// for every phase in order.
 #include <algorithm>
 
 #include "cf_tc_util.cuh"
@@ -37,558 +39,912 @@ namespace {
 using namespace tc;
 
 constexpr int kThreads = 512;
+constexpr int kRotateWarps = 6;
+constexpr int kRowTile = 128;
+constexpr int kKvHalf = kTile * 128;               // one 64-column half of a key or value tile
+constexpr int kKvBytes = 2 * kKvHalf;
+constexpr int kBoxes = kTile / 16;                 // copy boxes are 16, 32, .. kTile rows high
+constexpr int kKStages = 6, kVStages = 3;          // with the three S buffers of two warpgroups: everything repeats after six tiles
+constexpr int kSBuffers = 3;
+constexpr int kMetaRing = 16, kSegRing = 16;
+constexpr int kPrefSlots = 48;
+constexpr int kLoadWarp = 9, kMmaWarp = 12;
+constexpr int kTrigBytes = kD / 2 * 8;
+constexpr uint32_t kColO = 0, kColQ = 128, kColS = 192;
+constexpr float kRefShift = 40.0f;                 // the reference of a row lies this far (log2 units) above its first maximum
+constexpr float kSumLimit = 1099511627776.0f;      // 2^40: a larger tile sum leaves the range the reference was chosen for
+static_assert(kColS + kSBuffers * kTile <= 512, "tensor memory columns");
+static_assert(kTile % 16 == 0 && kTile <= 96, "three S buffers");
+static_assert(kKStages == 6 && kVStages == 3 && kSBuffers == 3, "rings of one period");
 
-// Tensor maps of the key store and of the value store, one per box height: a tile is fetched by
-// two bulk copies (one per 64-column half) whatever its length.
 struct StoreMaps {
-    CUtensorMap k[4], v[4];
-    CUtensorMap ks[4], vs[4];      // keys and values of the query tokens themselves (calls with a query-self block)
-    CUtensorMap kp[4], vp[4];      // keys and values of a shared prefix cache (calls that attend one)
+    CUtensorMap k[kBoxes], v[kBoxes];              // the stores, one map per box height
+    CUtensorMap ks, vs;                            // keys and values of the query tokens themselves (whole tiles)
+    CUtensorMap kp, vp;                            // keys and values of a shared prefix cache (whole tiles)
 };
-constexpr int kSmemTiles = 7;                      // 2 Q + 5 ring, or 1 Q + 6 ring
-constexpr int kMetaTiles = 128;                    // key tiles of a CTA whose description is staged in shared memory
-constexpr int kSmemBytes = kSmemTiles * kTileBytes + 1024 + 512 + kMetaTiles * 8;   // tiles, alignment slack, barriers, tile list
-constexpr int kMaxStages = 6;
-constexpr int kRotateThreads = 192;
-constexpr float kRescaleThreshold = 8.0f;          // log2 units: the reference maximum moves only
-                                                   // when a tile exceeds it by more than 2^8
 
 struct Barriers {
-    // A parity wait is only meaningful for a waiter that has seen every earlier phase of the barrier.
-    // Key loads and value loads of a ring stage therefore complete on separate barriers: the rotation
-    // warps wait for every key load, the MMA warp for every value load.
-    unsigned long long kv_full[kMaxStages][2];   // [stage][0 = keys, 1 = values]
-    unsigned long long kv_empty[kMaxStages];
-    unsigned long long k_ready[kMaxStages];
-    unsigned long long s_full[2];
-    unsigned long long p_ready[2];
-    unsigned long long o_done[2];
+    unsigned long long k_full[kKStages], k_ready[kKStages], k_empty[kKStages], v_empty[kVStages];
+    unsigned long long s_full[6], pv_ready[6];                          // [tile mod 6]; pv_ready: P is stored and V has landed
+    unsigned long long segment[kSegRing];                               // the description of the segment is there
+    unsigned long long q_ready, q_free, o_done, o_free;                 // one phase per segment
+    unsigned long long ref_full[2], sum_full[2];                        // [segment parity]
     unsigned int tmem_base;
     volatile int abort_flag;
+    volatile int marked;                           // a row of a unit finished here has to be computed from scratch
 };
 
-static_assert(sizeof(Barriers) <= 512, "barrier block must fit its reserved shared memory");
-static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
+// Tile descriptions: flags beside the length, and which keys they are.
+constexpr int kFirstOfSegment = 1 << 8, kLastOfSegment = 1 << 9;
+constexpr int kKindPrefix = -1, kKindSelf = -2;    // tile index of a prefix tile; kKindSelf - n: n-th tile of the query tokens
 
-// A key tile of the CTA's range: first store row, length, document.  The first kMetaTiles come
-// from shared memory (copied there once), later ones from the plan.
-struct TileInfo {
-    int row0, len, doc;
-};
-// Key blocks besides the kept documents, which the CTA of the last pair of parts takes after its documents'
-// tiles: first the tiles of a shared prefix cache (document -2: rows of the prefix tensors, every row of
-// the query sees them), then the query-self block as one tile (document -1: rows of the query's own
-// key/value tensors under the causal mask).  Neither is rotated, neither is a document that is scored.
-struct ExtraTiles {
-    int first;               // index of the first such tile in the CTA's list = number of its document tiles
-    int n_prefix, prefix_len;
-    int self_it, self_row0, self_len;
-};
-__device__ __forceinline__ TileInfo tile_info(const int2* s_meta, const PlanView& pv, int ti0, int it, const ExtraTiles& ex) {
-    TileInfo t;
-    if (it >= ex.first) {
-        if (it == ex.self_it) {
-            t.row0 = ex.self_row0;
-            t.len = ex.self_len;
-            t.doc = -1;
-        } else {
-            t.row0 = (it - ex.first) * kTile;
-            t.len = min(kTile, ex.prefix_len - t.row0);
-            t.doc = -2;
-        }
-    } else if (it < kMetaTiles) {
-        const int2 m = s_meta[it];
-        t.row0 = m.x;
-        t.len = m.y & 0xff;
-        t.doc = m.y >> 8;
-    } else {
-        t.row0 = pv.tile_row0[ti0 + it];
-        t.len = pv.tile_len[ti0 + it];
-        t.doc = pv.tile_doc[ti0 + it];
+// a / b for a >= 0, b > 0 from the reciprocal, exact after its correction: the few divisions on the way to a CTA's first
+// copy are a serial chain, and the integer division of the language is three times as long.
+__device__ __forceinline__ int quick_div(int a, int b) {
+    int q = (int)__fdividef((float)a, (float)b);
+    int r = a - q * b;
+    while (r < 0) {
+        --q;
+        r += b;
     }
-    return t;
+    while (r >= b) {
+        ++q;
+        r -= b;
+    }
+    return q;
 }
 
-// The ring has six stages (one query tile in shared memory) or five (two query tiles); dividing by
-// a literal keeps the index arithmetic of the hot loops to a few instructions.
-__device__ __forceinline__ int ring_mod(int x, bool six) { return six ? x % 6 : x % 5; }
-__device__ __forceinline__ int ring_div(int x, bool six) { return six ? x / 6 : x / 5; }
-// Loads of one kind (keys or values) a stage has received before the one of tile `it`.
-__device__ __forceinline__ int ring_uses(int it, bool six) { return six ? it / 3 : it / 5; }
+// The line of all key tiles (order: layer, request, kv head and tile of query rows, key tile).  A request's tiles are its
+// documents' (plan), then those of the prefix cache, then those of the query tokens.
+struct Line {
+    const int *pref, *begin;
+    int stride, n_requests, row_tiles, tiles;      // tiles = kv heads * tiles of query rows
+    int n_prefix, n_self, per_layer, n_shares, each, rest;
+    __device__ __forceinline__ int cut(int c) const { return c * each + min(c, rest); }
+    __device__ __forceinline__ int share_of(int x) const {
+        const int y = x - rest * (each + 1);
+        return y < 0 ? quick_div(x, each + 1) : rest + quick_div(y, each);
+    }
+};
+
+struct Segment {
+    int lb, layer, b, kvh, row0, rows_here;        // unit: query rows row0 .. of the kv head
+    int t_begin, t_end, n_unit, n_doc, tile0;      // tiles of the unit this segment covers; documents' tiles; first in the plan
+};
+
+constexpr int kMinShare = 2;
+
+// What the line is made from: prefix sums of the requests' tiles (one entry per `stride` requests), and with one entry per
+// request also the requests' first tiles in the plan.  Filled by the first warp.
+struct Requests {
+    int pref[kPrefSlots + 1], begin[kPrefSlots];
+};
+
+__device__ __forceinline__ void scan_requests(const BatchView& bv, const PlanView& pv, int extra, Requests& rq) {
+    const int lane = threadIdx.x & 31, stride = (bv.n_requests + kPrefSlots - 1) / kPrefSlots;
+    int carry = 0;
+    for (int b0 = 0; b0 < bv.n_requests; b0 += 32) {
+        const int b = b0 + lane;
+        int n = 0, begin = 0;
+        if (b < bv.n_requests) {
+            n = pv.n_tiles[b] + extra;
+            if (stride == 1) begin = pv.tile_begin[b];
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, n, o);
+            if (lane >= o) n += up;
+        }
+        if (b < bv.n_requests) {
+            if (stride == 1) rq.begin[b] = begin;
+            if ((b + 1) % stride == 0 || b == bv.n_requests - 1) rq.pref[(b + stride) / stride] = carry + n;
+        }
+        carry += __shfl_sync(0xffffffffu, n, 31);
+    }
+    if (lane == 0) rq.pref[0] = 0;
+}
+
+__device__ __forceinline__ Line make_line(const BatchView& bv, const AttnWorkspace& ws, const Requests& rq, int n_kv_heads, int row_tiles,
+                                          int n_prefix, int n_self, int max_shares) {
+    Line line;
+    line.pref = rq.pref;
+    line.begin = rq.begin;
+    line.n_requests = bv.n_requests;
+    line.stride = (bv.n_requests + kPrefSlots - 1) / kPrefSlots;
+    line.n_prefix = n_prefix;
+    line.n_self = n_self;
+    line.row_tiles = row_tiles;
+    line.tiles = n_kv_heads * line.row_tiles;
+    line.per_layer = rq.pref[(bv.n_requests + line.stride - 1) / line.stride] * line.tiles;
+    const int total = line.per_layer * ws.n_layers;
+    line.n_shares = max(1, min(max_shares, total / kMinShare));
+    line.each = quick_div(total, line.n_shares);
+    line.rest = total - line.each * line.n_shares;
+    return line;
+}
+
+__device__ __forceinline__ Segment segment_at(const BatchView& bv, const PlanView& pv, const AttnWorkspace& ws, const Line& line, int group,
+                                              int x, int end) {
+    Segment sg;
+    sg.layer = quick_div(x, line.per_layer);
+    int r = x - sg.layer * line.per_layer;
+    int lo = 0, hi = (line.n_requests + line.stride - 1) / line.stride;     // the last slot that starts at or before r
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (line.pref[mid] * line.tiles <= r) lo = mid; else hi = mid;
+    }
+    const int extra = line.n_prefix + line.n_self;
+    int b = lo, start = line.pref[lo], n;
+    if (line.stride == 1) {
+        n = line.pref[b + 1] - start;
+        sg.tile0 = line.begin[b];
+    } else {
+        b = lo * line.stride;
+        n = pv.n_tiles[b] + extra;
+        while ((start + n) * line.tiles <= r) {
+            start += n;
+            n = pv.n_tiles[++b] + extra;
+        }
+        sg.tile0 = pv.tile_begin[b];
+    }
+    r -= start * line.tiles;
+    const int unit = quick_div(r, n);
+    sg.n_unit = n;
+    sg.n_doc = n - extra;
+    sg.t_begin = r - unit * n;
+    sg.t_end = min(n, sg.t_begin + (end - x));
+    sg.b = b;
+    sg.lb = sg.layer * line.n_requests + b;
+    sg.kvh = quick_div(unit, line.row_tiles);
+    sg.row0 = (unit - sg.kvh * line.row_tiles) * ws.rg_rows;
+    sg.rows_here = min(ws.rg_rows, group * bv.q_len - sg.row0);
+    return sg;
+}
+
+// What a CTA leaves for the merge kernel: the unit that begins in its share and goes on behind it (n_parts = 0: none), and
+// whether a unit finished in the share has rows to be computed from scratch.
+struct ShareHead {
+    int n_parts, marked, lb, layer, b, row_first, rows_here, n_doc;      // row_first: of the unit among the rows of a request
+};
+static_assert(sizeof(ShareHead) == 32, "two 16-byte loads");
+
+struct Shared {
+    Barriers bars;
+    int4 meta[kMetaRing];                          // tiles in flight: length and flags, tile index or kind, first row, kv head and layer
+    Segment segments[kSegRing];                    // of the share
+    ShareHead head;
+    Line line;
+    float ref[2][kRowTile];                        // [segment parity][row]
+    alignas(16) float2 trig[kKStages][kD / 2];     // cosines and sines of the documents of the key stages
+    float sum[2][2][kRowTile], docs[2][2][kRowTile];   // [segment parity][warpgroup][row]
+    Requests requests;
+};
+constexpr int kSmemBytes = (kKStages + kVStages) * kKvBytes + (int)sizeof(Shared) + 1024;
+static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
+
+// Keys and values of a call outside the tensor maps, for rows that are computed from scratch.
+struct RowSources {
+    const __nv_bfloat16 *q, *k, *v, *ks, *vs, *kp, *vp;
+    long long self_stride, prefix_stride;
+    float scale_log2;
+    int with_self, prefix_len;
+};
+
+// Everything a kernel of this file is told: one constant, so that the rarely taken paths can be handed its address.
+struct Params {
+    BatchView bv;
+    PlanView pv;
+    AttnWorkspace ws;
+    LayerSpan span;
+    RowSources src;
+    int n_q_heads, n_kv_heads, row_tiles, n_prefix, n_self, max_shares;   // n_prefix, n_self: key tiles
+    __nv_bfloat16* out;
+    float* lse;
+};
+#define CF_PARAMS                                                                                                  \
+    const BatchView& bv = p.bv;                                                                                    \
+    const PlanView& pv = p.pv;                                                                                     \
+    const AttnWorkspace& ws = p.ws;                                                                                \
+    const LayerSpan& span = p.span;                                                                                \
+    const RowSources& src = p.src;                                                                                 \
+    const int n_q_heads = p.n_q_heads, n_kv_heads = p.n_kv_heads;                                                  \
+    __nv_bfloat16* const out_all = p.out;                                                                          \
+    float* const lse = p.lse
+
+// One query row by one warp, keys one after the other under a running maximum: its output, its log-sum-exps and those of
+// its document tiles.  Only rows whose logits left the range of the shared reference come here.
+template <int LAYOUT>
+__device__ __noinline__ void row_from_scratch(const Params& p, int lb, int rg, int n_doc) {
+    CF_PARAMS;
+    const int n_prefix = (src.prefix_len + kTile - 1) / kTile, n_self = src.with_self ? (bv.q_len + kTile - 1) / kTile : 0;
+    const int lane = threadIdx.x & 31, lq = bv.q_len, group = n_q_heads / n_kv_heads;
+    const int layer = lb / bv.n_requests, b = lb - layer * bv.n_requests, h = rg / lq, j = rg - h * lq, kvh = h / group;
+    const int d0 = LAYOUT == CF_ROPE_HALF ? 2 * lane : 4 * lane, d1 = LAYOUT == CF_ROPE_HALF ? 64 + 2 * lane : 4 * lane + 2;
+    auto load = [&](const __nv_bfloat16* e, float (&x)[4]) {
+        const uint32_t u = *reinterpret_cast<const uint32_t*>(e + d0), t = *reinterpret_cast<const uint32_t*>(e + d1);
+        x[0] = __uint_as_float(u << 16);
+        x[1] = __uint_as_float(u & 0xffff0000u);
+        x[2] = __uint_as_float(t << 16);
+        x[3] = __uint_as_float(t & 0xffff0000u);
+    };
+    float q[4], acc[4] = {0.f, 0.f, 0.f, 0.f}, m = -INFINITY, l = 0.f, docs_lse2 = -INFINITY;
+    load(src.q + (size_t)layer * span.q_stride + (((size_t)b * lq + j) * n_q_heads + h) * kD, q);
+    for (int t = 0; t < n_doc + n_prefix + n_self; ++t) {
+        const __nv_bfloat16 *kr, *vr;
+        size_t pitch = (size_t)n_kv_heads * kD;
+        int len, index = -1;
+        float2 cs0 = make_float2(1.f, 0.f), cs1 = cs0;
+        if (t < n_doc) {
+            index = pv.tile_begin[b] + t;
+            pitch = bv.token_stride;
+            const size_t at = (size_t)layer * span.kv_stride + (size_t)pv.tile_row0[index] * pitch + kvh * kD;
+            kr = src.k + at;
+            vr = src.v + at;
+            len = pv.tile_len[index];
+            const float2* trig = pv.trig + (size_t)pv.tile_doc[index] * (kD / 2) + 2 * lane;
+            cs0 = trig[0];
+            cs1 = trig[1];
+        } else if (t < n_doc + n_prefix) {
+            const int row0 = (t - n_doc) * kTile;
+            const size_t at = (size_t)layer * src.prefix_stride + (size_t)row0 * pitch + kvh * kD;
+            kr = src.kp + at;
+            vr = src.vp + at;
+            len = min(kTile, src.prefix_len - row0);
+        } else {
+            const int row0 = (t - n_doc - n_prefix) * kTile;
+            const size_t at = (size_t)layer * src.self_stride + ((size_t)b * lq + row0) * pitch + kvh * kD;
+            kr = src.ks + at;
+            vr = src.vs + at;
+            len = min(min(kTile, lq - row0), j + 1 - row0);
+        }
+        if (t == n_doc) docs_lse2 = l > 0.f ? m + log2f(l) : -INFINITY;
+        float tm = -INFINITY, tl = 0.f;
+        for (int i = 0; i < len; ++i) {
+            float k[4], v[4], y[4];
+            load(kr + i * pitch, k);
+            load(vr + i * pitch, v);
+            if (LAYOUT == CF_ROPE_HALF) {
+                rotate_pair(k[0], k[2], cs0.x, cs0.y, y[0], y[2]);
+                rotate_pair(k[1], k[3], cs1.x, cs1.y, y[1], y[3]);
+            } else {
+                rotate_pair(k[0], k[1], cs0.x, cs0.y, y[0], y[1]);
+                rotate_pair(k[2], k[3], cs1.x, cs1.y, y[2], y[3]);
+            }
+            float dot = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dot = fmaf(q[e], __bfloat162float(__float2bfloat16_rn(y[e])), dot);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+            const float s = dot * src.scale_log2;
+            const float m_new = fmaxf(m, s), alpha = exp2f(m - m_new), w = exp2f(s - m_new);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[e] = fmaf(acc[e], alpha, w * v[e]);
+            l = fmaf(l, alpha, w);
+            m = m_new;
+            const float tm_new = fmaxf(tm, s);
+            tl = fmaf(tl, exp2f(tm - tm_new), exp2f(s - tm_new));
+            tm = tm_new;
+        }
+        if (index >= 0 && lane == 0) ws.tile_lse2[((size_t)layer * ws.max_tiles + index) * n_q_heads * lq + rg] = tm + log2f(tl);
+    }
+    const float lse2 = l > 0.f ? m + log2f(l) : -INFINITY, inv = l > 0.f ? 1.f / l : 0.f;
+    __nv_bfloat16* dst = out_all + (size_t)layer * span.out_stride + (((size_t)b * lq + j) * n_q_heads + h) * kD;
+    *reinterpret_cast<uint32_t*>(dst + d0) = pack_bf16(acc[0] * inv, acc[1] * inv);
+    *reinterpret_cast<uint32_t*>(dst + d1) = pack_bf16(acc[2] * inv, acc[3] * inv);
+    if (lane == 0) {
+        ws.row_lse2[(size_t)lb * n_q_heads * lq + rg] = n_prefix + n_self > 0 ? docs_lse2 : lse2;
+        if (lse) lse[(size_t)lb * n_q_heads * lq + rg] = lse2 * kLn2;
+    }
+}
 
 template <int LAYOUT>
 __global__ void __launch_bounds__(kThreads, 1)
-attn_tc_kernel(const __grid_constant__ StoreMaps maps,
-               BatchView bv, PlanView pv, AttnWorkspace ws, long long q_layer_stride, int n_q_heads, int n_kv_heads,
-               float scale_log2, const __nv_bfloat16* __restrict__ q, int with_self, int prefix_len) {
+attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ Params p) {
+    CF_PARAMS;
     extern __shared__ unsigned char smem_raw[];
-    chain_next();
-    chain_wait();
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const uint32_t smem_base = smem_u32(smem);
+    const uint32_t k_base = smem_u32(smem), v_base = k_base + kKStages * kKvBytes;
+    Shared& sh = *reinterpret_cast<Shared*>(smem + (kKStages + kVStages) * kKvBytes);
+    Barriers& bars = sh.bars;
+    volatile int* abort_flag = &bars.abort_flag;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int group = n_q_heads / n_kv_heads, lq = bv.q_len, rows = group * lq, rows_total = n_q_heads * lq;
 
-    const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
-    const int group = n_q_heads / n_kv_heads;
-    const int lq = bv.q_len;
-    const int rows = group * lq;
-    const int rg_rows = ws.rg_rows;                                 // 256, or 128 (one row tile per CTA)
-    const int row_groups = (rows + rg_rows - 1) / rg_rows;
-    const int lb = blockIdx.z;                                      // layer * B + request
-    const int layer = lb / bv.n_requests;
-    const int b = lb - layer * bv.n_requests;
-    q += (size_t)layer * q_layer_stride;
-    const int kvh = blockIdx.y / row_groups;
-    const int rg = blockIdx.y - kvh * row_groups;
-    const int rows_here = min(rg_rows, rows - rg * rg_rows);
-    const bool alternate = rows_here <= 128;                        // both warpgroups on the same rows
-    const int n_qt = alternate ? 1 : 2;                             // query tiles in shared memory
-    const int n_stages = kSmemTiles - n_qt;                         // 6 or 5
-    const int n_parts = ws.n_splits;                                // parts per request, even
-    const int pair = blockIdx.x;                                    // this CTA fills parts 2*pair, 2*pair+1
-    const int rows_total = n_q_heads * lq;
-
-    // shared memory map: [Q tiles][ring][barriers]
-    const uint32_t q_base = smem_base;
-    const uint32_t ring_base = q_base + n_qt * kTileBytes;
-    Barriers* bars = reinterpret_cast<Barriers*>(smem + kSmemTiles * kTileBytes);
-    int2* s_meta = reinterpret_cast<int2*>(smem + kSmemTiles * kTileBytes + 512);
-    volatile int* abort_flag = &bars->abort_flag;
-
-    const int tbase = pv.tile_begin[b];
-    const int n_tiles = pv.n_tiles[b];
-    const int n_pairs = n_parts >> 1;
-    const int t_begin = (int)((long long)n_tiles * pair / n_pairs);
-    const int t_end = (int)((long long)n_tiles * (pair + 1) / n_pairs);
-    // the CTA of the last pair of parts also takes the prefix cache and the query-self block, as more tiles after its
-    // documents'
-    const bool last_pair = pair == n_pairs - 1;
-    const bool has_self = with_self && last_pair;
-    const int n_doc_it = t_end - t_begin;
-    const int n_prefix_it = last_pair ? (prefix_len + kTile - 1) / kTile : 0;
-    const int n_it = n_doc_it + n_prefix_it + (has_self ? 1 : 0);   // key tiles of this CTA
-    const ExtraTiles ex = {n_doc_it, n_prefix_it, prefix_len, has_self ? n_it - 1 : -1, b * lq, lq};
-    // first workspace row of this CTA in part 2*pair
-    const size_t slot0 = ((size_t)lb * n_parts + 2 * pair) * rows_total + (size_t)kvh * rows + rg * rg_rows;
-
-    // rows that will carry no data in one of the two parts: mark them neutral (m = -inf)
-    for (int r = tid; r < rows_here; r += kThreads) {
-        if (n_it <= 0) ws.part_m[slot0 + r] = -INFINITY;
-        if (n_it <= 0 || !alternate || n_it < 2) ws.part_m[slot0 + rows_total + r] = -INFINITY;
-    }
-    if (n_it <= 0) return;
-    const int ti0 = tbase + t_begin;                                // first tile of this CTA in the plan's list
-    if (tid < min(n_doc_it, kMetaTiles)) {
-        const int len = pv.tile_len[ti0 + tid], doc = pv.tile_doc[ti0 + tid];
-        s_meta[tid] = make_int2(pv.tile_row0[ti0 + tid], (len & 0xff) | (doc << 8));   // len 1..128 -> 0x80 at most
-    }
-    // query rows of this CTA: the loads are issued now so that their latency overlaps the set-up below
-    uint4 qval[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int idx = tid + i * kThreads;
-        const int chunk = idx & 15, r = idx >> 4;                   // r: row within the CTA's row group
-        qval[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (i < 4 * n_qt && r < rows_here) {
-            const int row = rg * rg_rows + r;
-            const int g = row / lq, j = row - g * lq;
-            const int h = kvh * group + g;
-            qval[i] = __ldg(reinterpret_cast<const uint4*>(q + (((size_t)b * lq + j) * n_q_heads + h) * kD + chunk * 8));
+    if (warp == kMmaWarp) {
+        if (lane == 0) {
+            auto init = [](unsigned long long* bar, int n, int count) {
+                for (int i = 0; i < n; ++i) mbar_init(smem_u32(bar + i), count);
+            };
+            init(bars.k_full, kKStages, 1);
+            init(bars.k_ready, kKStages, kRotateWarps);
+            init(bars.k_empty, kKStages, 1);
+            init(bars.v_empty, kVStages, 1);
+            init(bars.s_full, 6, 1);
+            init(bars.pv_ready, 6, 5);                              // one arrival per warp, one with the copy of V
+            init(bars.segment, kSegRing, 1);
+            init(&bars.q_ready, 1, 8);
+            init(&bars.q_free, 1, 1);
+            init(&bars.o_done, 1, 1);
+            init(&bars.o_free, 1, 8);
+            init(bars.ref_full, 2, 4);
+            init(bars.sum_full, 2, 8);
+            bars.abort_flag = 0;
+            bars.marked = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
-    }
-
-    if (tid == 0) {
-        const int rows_t0 = min(rows_here, 128), rows_t1 = alternate ? rows_t0 : rows_here - 128;
-        for (int s = 0; s < kMaxStages; ++s) {
-            mbar_init(smem_u32(&bars->kv_full[s][0]), 1);
-            mbar_init(smem_u32(&bars->kv_full[s][1]), 1);
-            mbar_init(smem_u32(&bars->kv_empty[s]), 1);
-            mbar_init(smem_u32(&bars->k_ready[s]), kRotateThreads);
-        }
-        for (int w = 0; w < 2; ++w) {
-            const int active = 32 * (((w ? rows_t1 : rows_t0) + 31) / 32);   // threads of warps that own rows
-            mbar_init(smem_u32(&bars->s_full[w]), 1);
-            mbar_init(smem_u32(&bars->p_ready[w]), active);
-            mbar_init(smem_u32(&bars->o_done[w]), 1);
-        }
-        bars->abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 13) {                                               // all 512 TMEM columns
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&bars->tmem_base)) : "memory");
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&bars.tmem_base)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    __syncthreads();                                                // barriers are initialised
-
-    // the producer starts streaming before the query tile is staged
-    int produced = 0;
-    auto produce = [&](int u) {                                     // u-th ring use: K(u/2) if even, V(u/2) if odd
-        const int st = ring_mod(u, alternate);
-        const TileInfo tile = tile_info(s_meta, pv, ti0, u >> 1, ex);
-        const int row0 = tile.row0;
-        const int boxes = (tile.len + kBoxRows - 1) / kBoxRows;
-        const CUtensorMap* map = tile.doc == -1 ? ((u & 1) ? &maps.vs[boxes - 1] : &maps.ks[boxes - 1])
-                                 : tile.doc == -2 ? ((u & 1) ? &maps.vp[boxes - 1] : &maps.kp[boxes - 1])
-                                                  : ((u & 1) ? &maps.v[boxes - 1] : &maps.k[boxes - 1]);
-        const uint32_t bar = smem_u32(&bars->kv_full[st][u & 1]);
-        const uint32_t dst = ring_base + st * kTileBytes;
-        mbar_expect_tx(bar, boxes * 2 * kBoxBytes);
-        tma_load_4d(dst, map, 0, kvh, row0, layer, bar);
-        tma_load_4d(dst + kHalfBytes, map, 64, kvh, row0, layer, bar);
-    };
-    if (warp == 12 && lane == 0) {
-        for (int i = 0; i < 4; ++i) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.k[i]) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.v[i]) : "memory");
-        }
-        for (; produced < 2; ++produced) produce(produced);        // first key and value tile; the rest follow below
-    }
-
-    // query rows into swizzled shared memory (zero rows beyond the valid ones)
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int idx = tid + i * kThreads;
-        const int chunk = idx & 15, r = idx >> 4;
-        if (i < 4 * n_qt) {
-            const int mt = r >> 7, rr = r & 127;
-            *reinterpret_cast<uint4*>(smem + (size_t)mt * kTileBytes + (chunk >> 3) * kHalfBytes + swz(rr, chunk & 7)) = qval[i];
+    if (warp == kLoadWarp && lane < 2 * kBoxes)
+        asm volatile("prefetch.tensormap [%0];" ::"l"(lane < kBoxes ? &maps.k[lane] : &maps.v[lane - kBoxes]) : "memory");
+    chain_next();
+    chain_wait();
+    if (warp == 0) {
+        scan_requests(bv, pv, p.n_prefix + p.n_self, sh.requests);
+        __syncwarp();
+        if (lane == 0) {
+            const Line l = make_line(bv, ws, sh.requests, n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, (int)gridDim.x);
+            sh.line = l;
+            const int begin = (int)blockIdx.x < l.n_shares ? l.cut(blockIdx.x) : 0, end = (int)blockIdx.x < l.n_shares ? l.cut(blockIdx.x + 1) : 0;
+            if (begin < end) sh.segments[0] = segment_at(bv, pv, ws, l, group, begin, end);
         }
     }
-    fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = bars->tmem_base;
+    const Line& line = sh.line;
+    const uint32_t tmem = bars.tmem_base;
+    const int x_begin = (int)blockIdx.x < line.n_shares ? line.cut(blockIdx.x) : 0, x_end = (int)blockIdx.x < line.n_shares ? line.cut(blockIdx.x + 1) : 0;
+    const int n_items = x_end - x_begin;                            // 0: this CTA has no share, its roles find nothing to do
 
-    // Work of warpgroup w: item j uses key tile kt(w, j) and query tile qt(w).
-    //   side by side (two row tiles): kt = j,          n_items = n_it
-    //   alternating  (one row tile):  kt = 2 j + w,    n_items = ceil((n_it - w) / 2)
-    if (warp == 12 || warp == 13) {
-        if (warp == 12 && lane == 0) {
-            // -------------------------------------------------------------- TMA producer
-            for (int u = produced; u < 2 * n_it; ++u) {
-                const int st = ring_mod(u, alternate);
-                if (u >= n_stages && !mbar_wait(smem_u32(&bars->kv_empty[st]), (ring_div(u, alternate) - 1) & 1, abort_flag)) break;
-                produce(u);
+    if (n_items == 0) {
+    } else if (warp == kLoadWarp) {
+        // ------------------------------------------------------------------ key and value loads, tile descriptions
+        if (lane == 0) {
+            constexpr int kAhead = 3;                               // keys run ahead of values: S(n + 3) is issued beside PV(n)
+            Segment sg = sh.segments[0];
+            int t = sg.t_begin, x = x_begin, row0, len, index, doc = 0, segments = 1;
+            auto fetch = [&]() {                                    // tile t of the segment
+                if (t < sg.n_doc) {
+                    index = sg.tile0 + t;
+                    row0 = __ldg(pv.tile_row0 + index);
+                    len = __ldg(pv.tile_len + index);
+                    doc = __ldg(pv.tile_doc + index);
+                } else if (t < sg.n_doc + line.n_prefix) {
+                    index = kKindPrefix;
+                    row0 = (t - sg.n_doc) * kTile;
+                    len = min(kTile, src.prefix_len - row0);
+                } else {
+                    const int n = t - sg.n_doc - line.n_prefix;
+                    index = kKindSelf - n;
+                    row0 = sg.b * lq + n * kTile;
+                    len = min(kTile, lq - n * kTile);
+                }
+            };
+            fetch();
+            ShareHead head = {};
+            int ks = 0, kp = 1, vs = 0, vp = 1, ps = 0;             // the first lap's waits pass: the phase before a fresh barrier's first
+            for (int n = 0; n < n_items + kAhead; ++n) {
+                if (n < n_items) {
+                    const int4 m = make_int4(len | (t == sg.t_begin ? kFirstOfSegment : 0) | (t == sg.t_end - 1 ? kLastOfSegment : 0), index, row0,
+                                             sg.kvh | (sg.layer << 20));
+                    const float2* trig = pv.trig + (size_t)doc * (kD / 2);
+                    ++x;
+                    if (++t == sg.t_end && x < x_end) {
+                        sg = segment_at(bv, pv, ws, line, group, x, x_end);
+                        t = sg.t_begin;
+                        sh.segments[segments & (kSegRing - 1)] = sg;
+                        mbar_arrive(smem_u32(&bars.segment[segments & (kSegRing - 1)]));
+                        ++segments;
+                    }
+                    if (x < x_end) fetch();                         // the next tile's description travels under this one's wait
+                    if (!mbar_wait(smem_u32(&bars.k_empty[ks]), kp, abort_flag)) break;
+                    sh.meta[n & (kMetaRing - 1)] = m;
+                    const uint32_t bar = smem_u32(&bars.k_full[ks]), dst = k_base + ks * kKvBytes;
+                    const int boxes = m.y >= 0 ? ((m.x & 0xff) + 15) >> 4 : kBoxes;
+                    const CUtensorMap* map = m.y >= 0 ? &maps.k[boxes - 1] : m.y == kKindPrefix ? &maps.kp : &maps.ks;
+                    mbar_expect_tx(bar, (boxes << 12) + (m.y >= 0 ? kTrigBytes : 0));
+                    if (m.y >= 0) bulk_load(smem_u32(sh.trig[ks]), trig, kTrigBytes, bar);
+                    tma_load_4d(dst, map, 0, m.w & 0xfffff, m.z, m.w >> 20, bar);
+                    tma_load_4d(dst + kKvHalf, map, 64, m.w & 0xfffff, m.z, m.w >> 20, bar);
+                    if (++ks == kKStages) {
+                        ks = 0;
+                        kp ^= 1;
+                    }
+                }
+                if (n >= kAhead) {
+                    if (!mbar_wait(smem_u32(&bars.v_empty[vs]), vp, abort_flag)) break;
+                    const int4 m = sh.meta[(n - kAhead) & (kMetaRing - 1)];
+                    const uint32_t bar = smem_u32(&bars.pv_ready[ps]), dst = v_base + vs * kKvBytes;
+                    const int boxes = m.y >= 0 ? ((m.x & 0xff) + 15) >> 4 : kBoxes;
+                    const CUtensorMap* map = m.y >= 0 ? &maps.v[boxes - 1] : m.y == kKindPrefix ? &maps.vp : &maps.vs;
+                    mbar_expect_tx(bar, boxes << 12);
+                    tma_load_4d(dst, map, 0, m.w & 0xfffff, m.z, m.w >> 20, bar);
+                    tma_load_4d(dst + kKvHalf, map, 64, m.w & 0xfffff, m.z, m.w >> 20, bar);
+                    if (++ps == 6) ps = 0;
+                    if (++vs == kVStages) {
+                        vs = 0;
+                        vp ^= 1;
+                    }
+                }
             }
-        } else if (warp == 13 && lane == 0) {
-            // -------------------------------------------------------------- MMA issue
-            // Sequence entry n: warpgroup w = n & 1, its item j = n >> 1, key tile = n (alternating)
-            // or j (side by side).  Issue order: S(0) S(1), then PV(n) followed by S(n + 2): the
-            // next QK^T of a warpgroup follows its own PV in the pipe, so S may overwrite the P it aliases.
-            // This one thread is the pacemaker of the CTA: whatever it executes between two bursts of
-            // tcgen05.mma is time in which the tensor cores idle.  Its ring positions and barrier parities are
-            // therefore running counters, and every descriptor is a precomputed base plus a stage offset.
-            const uint32_t idesc_o = instr_desc(kD, true);
-            const uint32_t idesc_s0 = instr_desc(0, false);
-            const int n_seq = alternate ? n_it : 2 * n_it;
-            const int period = alternate ? 3 : 5;                   // tiles after which a stage's parity flips
-            const uint64_t a_desc0 = smem_desc(q_base, 16, 1024);
-            const uint64_t a_desc1 = alternate ? a_desc0 : smem_desc(q_base + kTileBytes, 16, 1024);
-            const uint64_t bk_desc = smem_desc(ring_base, 16, 1024);
-            const uint64_t bv_desc = smem_desc(ring_base, kHalfBytes, 1024);
-            const uint32_t bar_k_ready = smem_u32(&bars->k_ready[0]), bar_kv_full = smem_u32(&bars->kv_full[0][0]);
-            const uint32_t bar_kv_empty = smem_u32(&bars->kv_empty[0]);
-            const uint32_t bar_s_full = smem_u32(&bars->s_full[0]), bar_p_ready = smem_u32(&bars->p_ready[0]);
-            const uint32_t bar_o_done = smem_u32(&bars->o_done[0]);
-            // position of the next tile of one kind (keys: stages 0, 2, 4, ...; values: 1, 3, 5, ...) in the ring
-            struct Cursor {
-                int stage, parity, count, tile;
-            };
-            auto advance = [&](Cursor& c) {
-                c.stage += 2;
-                if (c.stage >= n_stages) c.stage -= n_stages;
-                if (++c.count == period) {
-                    c.count = 0;
-                    c.parity ^= 1;
-                }
-                ++c.tile;
-            };
-            auto keys_of = [&](int it) -> int {                     // MMA extent of a tile: its rows rounded up to 16
-                return (tile_info(s_meta, pv, ti0, it, ex).len + 15) & ~15;
-            };
-            Cursor ck = {0, 0, 0, 0}, cv = {1, 0, 0, 0};            // keys for the next QK^T, values for the next PV
-            auto issue_s = [&](int n) -> bool {
-                const int w = n & 1;
-                const int n_keys = keys_of(ck.tile);
-                if (!mbar_wait(bar_k_ready + ck.stage * 8, ck.parity, abort_flag)) return false;
-                tc_fence_after();
-                const uint64_t a0 = w ? a_desc1 : a_desc0;
-                const uint64_t b0 = bk_desc + (uint64_t)(ck.stage * (kTileBytes >> 4));
-                const uint32_t idesc_s = idesc_s0 | ((uint32_t)(n_keys >> 3) << 17);
-                const uint32_t s_tmem = tmem + w * 128;
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {                    // 16 dims per instruction
-                    const uint64_t off = (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
-                    umma(s_tmem, a0 + off, b0 + off, idesc_s, kk > 0);
-                }
-                umma_commit(bar_s_full + w * 8);
-                if (alternate || w == 1) {                          // last reader of the keys
-                    umma_commit(bar_kv_empty + ck.stage * 8);
-                    advance(ck);
-                }
-                return true;
-            };
-            auto issue_pv = [&](int n) -> bool {
-                const int w = n & 1, j = n >> 1;
-                const int n_steps = keys_of(cv.tile) >> 4;          // 16 keys = 8 packed columns per instruction
-                if (!mbar_wait(bar_kv_full + cv.stage * 16 + 8, cv.parity, abort_flag)) return false;
-                if (!mbar_wait(bar_p_ready + w * 8, j & 1, abort_flag)) return false;
-                tc_fence_after();
-                const uint64_t b0 = bv_desc + (uint64_t)(cv.stage * (kTileBytes >> 4));
-                const uint32_t o_tmem = tmem + 256 + w * 128, p_tmem = tmem + w * 128;
-                umma_ts(o_tmem, p_tmem, b0, idesc_o, j > 0);
-#pragma unroll
-                for (int kk = 1; kk < kTile / 16; ++kk)
-                    if (kk < n_steps) umma_ts(o_tmem, p_tmem + kk * 8, b0 + (uint64_t)(kk * 128), idesc_o, 1u);
-                umma_commit(bar_o_done + w * 8);
-                if (alternate || w == 1) {                          // last reader of the values
-                    umma_commit(bar_kv_empty + cv.stage * 8);
-                    advance(cv);
-                }
-                return true;
-            };
-            bool ok = issue_s(0);
-            if (ok && n_seq > 1) ok = issue_s(1);
-            for (int n = 0; n < n_seq && ok; ++n) {
-                ok = issue_pv(n);
-                if (ok && n + 2 < n_seq) ok = issue_s(n + 2);
+            // sg is the share's last segment
+            if (sg.t_begin == 0 && sg.t_end < sg.n_unit) {
+                head.n_parts = line.share_of(x_end - sg.t_end + sg.n_unit - 1) - (int)blockIdx.x + 1;
+                head.lb = sg.lb;
+                head.layer = sg.layer;
+                head.b = sg.b;
+                head.row_first = sg.kvh * rows + sg.row0;
+                head.rows_here = sg.rows_here;
+                head.n_doc = sg.n_doc;
             }
+            sh.head = head;
+        }
+    } else if (warp == kMmaWarp) {
+        // ------------------------------------------------------------------ MMA issue: the warp walks, one lane issues
+        const bool lead = elect_one();
+        const uint32_t idesc_o = instr_desc(kD, true), idesc_s0 = instr_desc(0, false);
+        const uint64_t bk_desc = smem_desc(k_base, 16, 1024), bv_desc = smem_desc(v_base, kKvHalf, 1024);
+        const uint32_t bar_k_ready = smem_u32(bars.k_ready), bar_k_empty = smem_u32(bars.k_empty), bar_v_empty = smem_u32(bars.v_empty);
+        const uint32_t bar_s_full = smem_u32(bars.s_full), bar_pv_ready = smem_u32(bars.pv_ready);
+        // One rolled loop (unrolled by the rings' period of six it was some instructions per tile shorter, and every lap's first
+        // pass through it cost 2 to 3 thousand cycles per tile of instruction fetches).
+        struct Ring {
+            int it, j, parity;                                      // tile, tile mod 6, parity of its lap
+        } s = {0, 0, 0}, v = {0, 0, 0};
+        auto next = [](Ring& r) {
+            ++r.it;
+            if (++r.j == 6) {
+                r.j = 0;
+                r.parity ^= 1;
+            }
+        };
+        int segments_s = 0, segments = 0;                           // segments begun by QK^T, finished by PV
+        bool ok = true;
+        while (v.it < n_items && ok) {
+            // QK^T runs up to three tiles ahead; into the next segment only once its query tile is there
+            bool do_s = s.it < n_items && s.it < v.it + kSBuffers;
+            int m = 0;
+            if (do_s) {
+                ok = warp_wait(bar_k_ready + s.j * 8, s.parity, abort_flag);
+                if (!ok) break;
+                m = sh.meta[s.it & (kMetaRing - 1)].x;
+                if (m & kFirstOfSegment) {
+                    const uint32_t bar = smem_u32(&bars.q_ready);
+                    if (s.it == v.it) ok = warp_wait(bar, segments_s & 1, abort_flag);
+                    else do_s = __all_sync(0xffffffffu, mbar_try_wait(bar, segments_s & 1));
+                    if (!ok) break;
+                    if (do_s) ++segments_s;
+                }
+            }
+            if (do_s) {
+                tc_fence_after();
+                const uint32_t idesc = idesc_s0 | ((uint32_t)(((m & 0xff) + 15) >> 4) << 18);
+                const uint64_t b0 = bk_desc + (uint64_t)(s.j * (kKvBytes >> 4));
+                const uint32_t s_tmem = tmem + kColS + (s.j >= 3 ? s.j - 3 : s.j) * kTile, q_tmem = tmem + kColQ;
+                if (lead) {
+                    umma_ts_lit<false>(s_tmem, q_tmem, b0, idesc);
+#pragma unroll
+                    for (int kk = 1; kk < 8; ++kk)                  // 16 dims per instruction
+                        umma_ts_lit<true>(s_tmem, q_tmem + kk * 8, b0 + (uint64_t)(((kk >> 2) * kKvHalf + (kk & 3) * 32) >> 4), idesc);
+                    umma_commit(bar_s_full + s.j * 8);
+                    umma_commit(bar_k_empty + s.j * 8);
+                    if (m & kLastOfSegment) umma_commit(smem_u32(&bars.q_free));
+                }
+                __syncwarp();
+                next(s);
+                if (s.it < v.it + kSBuffers && s.it < n_items) continue;
+            }
+            m = sh.meta[v.it & (kMetaRing - 1)].x;
+            ok = warp_wait(bar_pv_ready + v.j * 8, v.parity, abort_flag);
+            if (ok && (m & kFirstOfSegment) && segments > 0) ok = warp_wait(smem_u32(&bars.o_free), (segments - 1) & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            const int steps = ((m & 0xff) + 15) >> 4;               // 16 keys = 8 packed columns per instruction
+            const int buffer = v.j >= 3 ? v.j - 3 : v.j;            // both of the S buffers and of the value stages
+            const uint64_t b0 = bv_desc + (uint64_t)(buffer * (kKvBytes >> 4));
+            const uint32_t p_tmem = tmem + kColS + buffer * kTile, o_tmem = tmem + kColO;
+            if (lead) {
+                umma_ts(o_tmem, p_tmem, b0, idesc_o, (m & kFirstOfSegment) ? 0u : 1u);
+                for (int kk = 1; kk < steps; ++kk) umma_ts_lit<true>(o_tmem, p_tmem + kk * 8, b0 + (uint64_t)(kk * 128), idesc_o);
+                umma_commit(bar_v_empty + buffer * 8);
+                if (m & kLastOfSegment) umma_commit(smem_u32(&bars.o_done));
+            }
+            __syncwarp();
+            if (m & kLastOfSegment) ++segments;
+            next(v);
         }
     } else if (warp >= 8) {
         // ------------------------------------------------------------------ key rotation (Eq. 5)
-        const int t = warp < 12 ? tid - 256 : tid - 320;            // 0..191 (warps 8-11, 14, 15)
-        const int chunk = t & 7, rsub = t >> 3;
-        for (int it = 0; it < n_it; ++it) {
-            const TileInfo tile = tile_info(s_meta, pv, ti0, it, ex);
-            const int len = tile.len;
-            const float2* trig = pv.trig + (size_t)max(tile.doc, 0) * (kD / 2);
-            const int st = ring_mod(2 * it, alternate);
-            float2 cs[8];
-            if (tile.doc < 0) {                                     // the query's own keys are already in place
+        const int rw = warp == 8 ? 0 : warp < kMmaWarp ? warp - 9 : warp - 10, rt = rw * 32 + lane;   // 0 .. 191
+        const int chunk = rt & 7, rsub = rt >> 3;                   // 16-byte chunk of each half row; first row
+        int stage = 0, phase = 0;
+        for (int it = 0; it < n_items; ++it) {
+            if (!warp_wait(smem_u32(&bars.k_full[stage]), phase, abort_flag)) break;
+            const int2 meta = *reinterpret_cast<const int2*>(&sh.meta[it & (kMetaRing - 1)]);
+            if (meta.y >= 0) {                                      // a document's tile: its table came with the keys
+                const int len = meta.x & 0xff;
+                uint64_t c2[4], s2[4], n2[4];                       // cosines, sines and their negatives as pairs for the packed arithmetic
+                const float4* trig = reinterpret_cast<const float4*>(sh.trig[stage]);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) cs[e] = make_float2(1.f, 0.f);
-            } else if (LAYOUT == CF_ROPE_HALF) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) cs[e] = __ldg(trig + chunk * 8 + e);
-            } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    cs[e] = __ldg(trig + chunk * 4 + e);            // first half: dims chunk*8 .. +7
-                    cs[4 + e] = __ldg(trig + 32 + chunk * 4 + e);   // second half: dims 64 + chunk*8 ..
+                for (int e = 0; e < 4; ++e) {                       // half layout: slices chunk*8 .. +7; interleaved: chunk*4 .. +3 of either half
+                    const float4 cs = trig[LAYOUT == CF_ROPE_HALF ? chunk * 4 + e : (e >> 1) * 16 + chunk * 2 + (e & 1)];
+                    c2[e] = pack_f2(cs.x, cs.z);
+                    s2[e] = pack_f2(cs.y, cs.w);
+                    n2[e] = pack_f2(-cs.y, -cs.w);
                 }
-            }
-            const int kuse = ring_uses(it, alternate);                        // key loads this stage has seen
-            if (!mbar_wait(smem_u32(&bars->kv_full[st][0]), kuse & 1, abort_flag)) break;
-            unsigned char* buf = smem + (ring_base - smem_base) + (size_t)st * kTileBytes;
+                // rows 24 apart keep their swizzle phase: one pointer walks
+                unsigned char* at = smem + (size_t)stage * kKvBytes + swz(rsub, chunk);
 #pragma unroll 2
-            for (int r = rsub; r < len; r += kRotateThreads / 8) {
-                uint4* pa = reinterpret_cast<uint4*>(buf + swz(r, chunk));
-                uint4* pb = reinterpret_cast<uint4*>(buf + kHalfBytes + swz(r, chunk));
-                uint4 va = *pa, vb = *pb;
-                uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
-                if (LAYOUT == CF_ROPE_HALF) {
+                for (int r = rsub; r < len; r += kRotateWarps * 4, at += kRotateWarps * 4 * 128) {
+                    uint4* pa = reinterpret_cast<uint4*>(at);
+                    uint4* pb = reinterpret_cast<uint4*>(at + kKvHalf);
+                    const uint4 va = *pa, vb = *pb;
+                    uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
+                    if (LAYOUT == CF_ROPE_HALF) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float a0 = __uint_as_float(wa[i] << 16), a1 = __uint_as_float(wa[i] & 0xffff0000u);
-                        float b0 = __uint_as_float(wb[i] << 16), b1 = __uint_as_float(wb[i] & 0xffff0000u);
-                        float ya0, yb0, ya1, yb1;
-                        rotate_pair(a0, b0, cs[2 * i].x, cs[2 * i].y, ya0, yb0);
-                        rotate_pair(a1, b1, cs[2 * i + 1].x, cs[2 * i + 1].y, ya1, yb1);
-                        wa[i] = pack_bf16(ya0, ya1);
-                        wb[i] = pack_bf16(yb0, yb1);
-                    }
-                } else {
+                        for (int e = 0; e < 4; ++e) {
+                            const uint64_t fa = pack_f2(__uint_as_float(wa[e] << 16), __uint_as_float(wa[e] & 0xffff0000u));
+                            const uint64_t fb = pack_f2(__uint_as_float(wb[e] << 16), __uint_as_float(wb[e] & 0xffff0000u));
+                            float y0, y1;
+                            unpack_f2(fma_f2(fa, c2[e], mul_f2(fb, n2[e])), y0, y1);
+                            wa[e] = pack_bf16(y0, y1);
+                            unpack_f2(fma_f2(fa, s2[e], mul_f2(fb, c2[e])), y0, y1);
+                            wb[e] = pack_bf16(y0, y1);
+                        }
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float a0 = __uint_as_float(wa[i] << 16), a1 = __uint_as_float(wa[i] & 0xffff0000u);
-                        float b0 = __uint_as_float(wb[i] << 16), b1 = __uint_as_float(wb[i] & 0xffff0000u);
-                        float ya0, ya1, yb0, yb1;
-                        rotate_pair(a0, a1, cs[i].x, cs[i].y, ya0, ya1);
-                        rotate_pair(b0, b1, cs[4 + i].x, cs[4 + i].y, yb0, yb1);
-                        wa[i] = pack_bf16(ya0, ya1);
-                        wb[i] = pack_bf16(yb0, yb1);
+                        for (int e = 0; e < 4; ++e) {               // the two elements of a word are a slice; words in pairs
+                            uint32_t& w0 = e < 2 ? wa[2 * e] : wb[2 * e - 4];
+                            uint32_t& w1 = e < 2 ? wa[2 * e + 1] : wb[2 * e - 3];
+                            const uint64_t fa = pack_f2(__uint_as_float(w0 << 16), __uint_as_float(w1 << 16));
+                            const uint64_t fb = pack_f2(__uint_as_float(w0 & 0xffff0000u), __uint_as_float(w1 & 0xffff0000u));
+                            float a0, a1, b0, b1;
+                            unpack_f2(fma_f2(fa, c2[e], mul_f2(fb, n2[e])), a0, a1);
+                            unpack_f2(fma_f2(fa, s2[e], mul_f2(fb, c2[e])), b0, b1);
+                            w0 = pack_bf16(a0, b0);
+                            w1 = pack_bf16(a1, b1);
+                        }
                     }
+                    *pa = make_uint4(wa[0], wa[1], wa[2], wa[3]);
+                    *pb = make_uint4(wb[0], wb[1], wb[2], wb[3]);
                 }
-                *pa = make_uint4(wa[0], wa[1], wa[2], wa[3]);
-                *pb = make_uint4(wb[0], wb[1], wb[2], wb[3]);
+                fence_proxy_async();
             }
-            fence_proxy_async();
-            mbar_arrive(smem_u32(&bars->k_ready[st]));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bars.k_ready[stage]));
+            if (++stage == kKStages) {
+                stage = 0;
+                phase ^= 1;
+            }
         }
     } else {
         // ------------------------------------------------------------------ softmax, one row per thread
-        const int w = warp >> 2;                                    // warpgroup
-        const int r = tid & 127;                                    // row within the tile = TMEM lane
-        const int row_in_group = (alternate ? 0 : w * 128) + r;
-        const int n_items = alternate ? (n_it - w + 1) / 2 : n_it;
-        // a warp none of whose rows exist does not take part (the barrier counts exclude it)
-        const bool warp_active = (alternate ? 0 : w * 128) + (warp & 3) * 32 < rows_here;
-        if (warp_active && n_items > 0) {
-            const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-            const uint32_t s_addr = tmem + lane_addr + w * 128;
-            const uint32_t o_addr = tmem + lane_addr + 256 + w * 128;
-            const bool row_valid = row_in_group < rows_here;
-            const size_t tile_row = (size_t)kvh * rows + rg * rg_rows + row_in_group;
-            float* tile_lse2 = ws.tile_lse2 + (size_t)layer * ws.max_tiles * rows_total;
-            float m_ref = -INFINITY, l_run = 0.f, l_docs = 0.f;     // l_docs: the sum over the documents' keys alone
-            bool seen_extra = false;
-            const int q_index = (rg * rg_rows + row_in_group) % lq;     // position of this row's token in the query
-            bool ok = true;
-            for (int j = 0; j < n_items; ++j) {
-                const int it = alternate ? 2 * j + w : j;
-                const int ti = ti0 + it;
-                const int len = tile_info(s_meta, pv, ti0, it, ex).len;
-                // keys this row may see: the whole tile of a document, the query tokens 0..q_index of the
-                // query-self block (causal mask, footnote to Eq. 1)
-                const int vis = it == ex.self_it ? min(len, q_index + 1) : len;
-                if (it >= ex.first && !seen_extra) {                // from here on the keys are not the documents'
+        const int w = warp >> 2, r = tid & 127;                     // warpgroup; row of the tile = TMEM lane
+        const uint32_t lane_tmem = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint64_t scale2 = pack_f2(src.scale_log2, src.scale_log2);
+        const uint32_t bar_s_full = smem_u32(bars.s_full), bar_pv_ready = smem_u32(bars.pv_ready);
+        int k = w, phase = 0;                                       // this warpgroup's next tile, mod 6, and its parity
+        int it0 = 0;                                                // tiles before the current segment
+        float ref = 0.f, l_run = 0.f, l_docs = 0.f;
+        const bool wide_out = ((reinterpret_cast<uintptr_t>(out_all) | (uintptr_t)(span.out_stride * 2)) & 31) == 0;   // rows start at 32-byte addresses
+        bool ok = true;
+        for (int seg = 0; ok; ++seg) {
+            const bool more = it0 < n_items;
+            const int slot = seg & (kSegRing - 1);
+            if (more && seg > 0) {
+                ok = warp_wait(smem_u32(&bars.segment[slot]), (seg / kSegRing) & 1 ^ (slot == 0 ? 1 : 0), abort_flag);
+                if (!ok) break;
+            }
+            const Segment& sg = sh.segments[slot];
+            if (more) {
+                // the query tile of the segment goes into tensor memory, half of every row by each warpgroup (before the
+                // epilogue of the last segment)
+                const bool active = (warp & 3) * 32 < sg.rows_here;
+                const int row = sg.row0 + min(r, sg.rows_here - 1), g = row / lq, j = row - g * lq;
+                const uint4* q = reinterpret_cast<const uint4*>(src.q + (size_t)sg.layer * span.q_stride + (((size_t)sg.b * lq + j) * n_q_heads + sg.kvh * group + g) * kD) + w * 8;
+                uint32_t qw[32];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint4 v = __ldg(q + i);
+                    qw[4 * i] = v.x;
+                    qw[4 * i + 1] = v.y;
+                    qw[4 * i + 2] = v.z;
+                    qw[4 * i + 3] = v.w;
+                }
+                if (seg > 0) ok = warp_wait(smem_u32(&bars.q_free), (seg - 1) & 1, abort_flag);   // read by its last QK^T
+                if (!ok) break;
+                if (active) {
+                    tc_fence_after();
+                    tmem_st16_from<0>(lane_tmem + kColQ + w * 32, qw);
+                    tmem_st16_from<16>(lane_tmem + kColQ + w * 32 + 16, qw);
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    tc_fence_before();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bars.q_ready));
+            }
+            if (seg > 0) {
+                // ---- end of a segment: the two sums meet, each warpgroup takes half of the columns of O
+                const int par = (seg - 1) & 1;
+                sh.sum[par][w][r] = l_run;
+                sh.docs[par][w][r] = l_docs;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bars.sum_full[par]));
+                ok = warp_wait(smem_u32(&bars.sum_full[par]), ((seg - 1) >> 1) & 1, abort_flag) && warp_wait(smem_u32(&bars.o_done), par, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const Segment& done = sh.segments[(seg - 1) & (kSegRing - 1)];
+                const bool whole = done.t_end - done.t_begin == done.n_unit;
+                const int row = done.row0 + r;
+                const float l_all = sh.sum[par][0][r] + sh.sum[par][1][r], d_all = sh.docs[par][0][r] + sh.docs[par][1][r];
+                const bool row_valid = r < done.rows_here, marked = l_all != l_all;
+                const size_t at = (size_t)done.lb * rows_total + (size_t)done.kvh * rows + row;
+                if ((warp & 3) * 32 < done.rows_here) {
+                    const int g = row / lq, j = row - g * lq;
+                    const size_t slot = ((size_t)2 * blockIdx.x + (done.t_begin == 0 ? 1 : 0)) * kRowTile + r;
+                    const float f = whole ? (l_all > 0.f ? 1.f / l_all : 0.f) : 1.f;
+                    __nv_bfloat16* dst = (whole ? out_all + (size_t)done.layer * span.out_stride + (((size_t)done.b * lq + j) * n_q_heads + done.kvh * group + g) * kD
+                                                : reinterpret_cast<__nv_bfloat16*>(ws.part_o) + slot * kD) + w * 64;
+#pragma unroll 1
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t o[32];
+                        tmem_ld32(lane_tmem + kColO + w * 64 + c * 32, o);
+                        if (row_valid) {
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {           // whole 32-byte sectors: rows are 256 bytes apart
+                                uint32_t y[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) y[e] = pack_bf16(__uint_as_float(o[16 * i + 2 * e]) * f, __uint_as_float(o[16 * i + 2 * e + 1]) * f);
+                                if (wide_out) {
+                                    store32(dst + c * 32 + i * 16, y);
+                                } else {
+                                    *reinterpret_cast<uint4*>(dst + c * 32 + i * 16) = make_uint4(y[0], y[1], y[2], y[3]);
+                                    *reinterpret_cast<uint4*>(dst + c * 32 + i * 16 + 8) = make_uint4(y[4], y[5], y[6], y[7]);
+                                }
+                            }
+                        }
+                    }
+                    if (w == 0 && row_valid) {
+                        if (!whole) {
+                            ws.part_m[slot] = l_all == 0.f ? -INFINITY : ref;   // a row may see none of the segment's keys
+                            ws.part_l[slot] = l_all;
+                            if (ws.part_ld) ws.part_ld[slot] = d_all;   // what the document scores are measured against
+                        } else {
+                            ws.row_lse2[at] = marked ? l_all : ref + log2f(d_all);
+                            if (lse) lse[at] = (ref + log2f(l_all)) * kLn2;
+                            if (marked) bars.marked = 1;
+                        }
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bars.o_free));
+            }
+            if (!more) break;
+            // ---- the tiles of the segment
+            const int n = sg.t_end - sg.t_begin, par = seg & 1;
+            const bool active = (warp & 3) * 32 < sg.rows_here, row_valid = r < sg.rows_here;
+            const int q_index = (sg.row0 + r) % lq;                 // position of this row's token in the query
+            float* tile_lse2 = ws.tile_lse2 + (size_t)sg.layer * ws.max_tiles * rows_total + (size_t)sg.kvh * rows + sg.row0 + r;
+            const bool leads = (it0 & 1) == w;                      // this warpgroup has the segment's first tile
+            bool have_ref = false, seen_extra = false;
+            l_run = l_docs = 0.f;
+            for (int i = leads ? 0 : 1; i < n; i += 2) {
+                ok = warp_wait(bar_s_full + k * 8, phase, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const int4 meta = sh.meta[(it0 + i) & (kMetaRing - 1)];
+                const int len = meta.x & 0xff, n_chunks = (len + 15) >> 4;
+                // keys this row may see: a whole tile of a document or of the prefix, the query tokens up to its own (causal
+                // mask, footnote to Eq. 1)
+                const int vis = meta.y <= kKindSelf ? min(len, q_index + 1 - (kKindSelf - meta.y) * kTile) : len;
+                const uint32_t s_addr = lane_tmem + kColS + (k >= 3 ? k - 3 : k) * kTile;
+                uint32_t va[16], vb[16];
+                if (active) {
+                    tmem_ld16_async(s_addr, va);
+                    tmem_ld16_wait(va);
+                }
+                if (i == 0) {                                       // the reference of the segment, from its first 16 keys
+                    float m = -INFINITY;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) m = fmaxf(m, e < vis ? __uint_as_float(va[e]) : -INFINITY);
+                    sh.ref[par][r] = m > -INFINITY ? fmaf(m, src.scale_log2, kRefShift) : 0.f;   // a row that sees none of them sees none of the tile
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.ref_full[par]));
+                }
+                if (!have_ref) {
+                    ok = warp_wait(smem_u32(&bars.ref_full[par]), (seg >> 1) & 1, abort_flag);
+                    if (!ok) break;
+                    ref = sh.ref[par][r];
+                    have_ref = true;
+                }
+                if (meta.y < 0 && !seen_extra) {                    // from here on the keys are not the documents'
                     l_docs = l_run;
                     seen_extra = true;
                 }
-                ok = mbar_wait(smem_u32(&bars->s_full[w]), j & 1, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                if (j > 0) {
-                    // PV(j-1) sits before S(j) in the tensor pipe, so it is complete; waiting here keeps
-                    // this thread's view of the barrier in step (every phase is waited for, in order)
-                    ok = mbar_wait(smem_u32(&bars->o_done[w]), (j - 1) & 1, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                }
-                // Single pass over S in 32-key chunks, loads double-buffered.  The reference maximum only
-                // moves when a chunk exceeds it by more than 2^8; then O, the sums and the P chunks of this
-                // tile that are already written are rescaled (rare after the first chunk of the first tile).
-                const int n_chunks = (len + 31) >> 5;
-                float tile_sum = 0.f;
-                uint32_t va[32], vb[32];
-                // step 1 of a chunk; no tensor-memory load may be in flight across these branches
-                auto prepare = [&](const uint32_t (&v)[32], int valid, int c) {
-                    const float cmax = (valid >= 32 ? chunk_max<false>(v, 32) : chunk_max<true>(v, valid)) * scale_log2;
-                    const bool move = cmax > m_ref + kRescaleThreshold;       // very first chunk: m_ref = -inf
-                    if (__any_sync(0xffffffffu, move)) {
-                        float alpha = 1.f;
-                        if (move) {
-                            alpha = fast_exp2(m_ref - cmax);                  // 0 when nothing is accumulated yet
-                            m_ref = cmax;
-                        }
-                        if (j > 0) {
-                            for (int cc = 0; cc < 8; ++cc) {
-                                uint32_t o[16];
-                                tmem_ld16(o_addr + cc * 16, o);
+                if (active) {
+                    // single pass in chunks of 16 keys: P chunk c goes over the S columns 8c .. 8c + 7, which are in registers by then
+                    const uint64_t neg_ref2 = pack_f2(-ref, -ref);
+                    uint64_t sum2 = 0;
+                    auto finish = [&](uint32_t (&v)[16], int c) {
+                        if (vis - c * 16 < 16) {                    // the ragged end of a tile, the causal mask
 #pragma unroll
-                                for (int k = 0; k < 16; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * alpha);
-                                tmem_st16(o_addr + cc * 16, o);
-                            }
+                            for (int e = 0; e < 16; ++e) v[e] = e < vis - c * 16 ? v[e] : 0xff800000u;
                         }
-                        if (c > 0) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");   // P stores in flight
-                        for (int cc = 0; cc < c; ++cc) {
-                            uint32_t pk[16];
-                            tmem_ld16(s_addr + cc * 16, pk);
-#pragma unroll
-                            for (int k = 0; k < 16; ++k)
-                                pk[k] = pack_bf16(__uint_as_float(pk[k] << 16) * alpha, __uint_as_float(pk[k] & 0xffff0000u) * alpha);
-                            tmem_st16(s_addr + cc * 16, pk);
-                        }
-                        l_run *= alpha;
-                        l_docs *= alpha;
-                        tile_sum *= alpha;
+                        chunk16_exp(v, scale2, neg_ref2, sum2);
+                        tmem_st8_async(s_addr + c * 8, v);
+                    };
+#pragma unroll 1
+                    for (int c = 0;;) {
+                        if (c + 1 < n_chunks) tmem_ld16_async(s_addr + (c + 1) * 16, vb);
+                        finish(va, c);
+                        if (++c == n_chunks) break;
+                        tmem_ld16_wait(vb);
+                        if (c + 1 < n_chunks) tmem_ld16_async(s_addr + (c + 1) * 16, va);
+                        finish(vb, c);
+                        if (++c == n_chunks) break;
+                        tmem_ld16_wait(va);
                     }
-                };
-                // step 2 (straight-line): exponentials, packing; P chunk c lands in S columns 16c..16c+15,
-                // which belong to S chunks already held in registers
-                auto finish = [&](uint32_t (&v)[32], int valid, int c) {
-                    tile_sum += valid >= 32 ? chunk_exp<false>(v, 32, scale_log2, -m_ref) : chunk_exp<true>(v, valid, scale_log2, -m_ref);
-                    tmem_st16_async(s_addr + c * 16, v);
-                };
-                tmem_ld32_async(s_addr, va);
-                tmem_ld_wait(va);
-                for (int c = 0; c < n_chunks; c += 2) {
-                    prepare(va, vis - c * 32, c);
-                    if (c + 1 < n_chunks) tmem_ld32_async(s_addr + (c + 1) * 32, vb);
-                    finish(va, vis - c * 32, c);
-                    if (c + 1 < n_chunks) {
-                        tmem_ld_wait(vb);
-                        prepare(vb, vis - c * 32 - 32, c + 1);
-                        if (c + 2 < n_chunks) tmem_ld32_async(s_addr + (c + 2) * 32, va);
-                        finish(vb, vis - c * 32 - 32, c + 1);
-                        if (c + 2 < n_chunks) tmem_ld_wait(va);
-                    }
+                    float tile_sum, odd;
+                    unpack_f2(sum2, tile_sum, odd);
+                    tile_sum += odd;
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_pv_ready + k * 8);
+                    if (!(tile_sum < kSumLimit)) tile_sum = __int_as_float(0x7fffffff);     // out of range: the row is marked
+                    l_run += tile_sum;
+                    if (meta.y >= 0 && row_valid) tile_lse2[(size_t)meta.y * rows_total] = ref + __log2f(tile_sum);
+                } else if (lane == 0) {
+                    mbar_arrive(bar_pv_ready + k * 8);
                 }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bars->p_ready[w]));
-                if (it < ex.first && row_valid) tile_lse2[(size_t)ti * rows_total + tile_row] = m_ref + log2f(tile_sum);
-                l_run += tile_sum;
-            }
-            if (ok) ok = mbar_wait(smem_u32(&bars->o_done[w]), (n_items - 1) & 1, abort_flag);
-            if (ok) {
-                tc_fence_after();
-                const size_t slot = slot0 + (alternate ? (size_t)w * rows_total : 0) + row_in_group;
-                // Partial O rows leave as bf16 through shared memory so that global stores are full
-                // 256-byte rows.  Staging space: this warpgroup's own query tile (every QK^T that read
-                // it has completed), or, when both warpgroups share one query tile, the ring stage of
-                // the next unused key or value slot (its last reader completed before this point).
-                unsigned char* stage = alternate ? smem + (ring_base - smem_base) + (size_t)((2 * n_it + w) % n_stages) * kTileBytes
-                                                 : smem + (size_t)w * kTileBytes;
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t o[32];
-                    tmem_ld32(o_addr + c * 32, o);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {                   // 8 dims = one 16-byte chunk
-                        const int chunk = c * 4 + i;
-                        *reinterpret_cast<uint4*>(stage + r * 256 + ((chunk ^ (r & 15)) << 4)) =
-                            make_uint4(pack_bf16(__uint_as_float(o[8 * i]), __uint_as_float(o[8 * i + 1])),
-                                       pack_bf16(__uint_as_float(o[8 * i + 2]), __uint_as_float(o[8 * i + 3])),
-                                       pack_bf16(__uint_as_float(o[8 * i + 4]), __uint_as_float(o[8 * i + 5])),
-                                       pack_bf16(__uint_as_float(o[8 * i + 6]), __uint_as_float(o[8 * i + 7])));
-                    }
-                }
-                __syncwarp();
-                {
-                    const int warp_row0 = r & ~31;                  // this warp's 32 rows
-                    const int rows_left = rows_here - ((alternate ? 0 : w * 128) + warp_row0);
-                    unsigned char* dst = reinterpret_cast<unsigned char*>(ws.part_o) + (slot - lane) * (size_t)(kD * 2);
-#pragma unroll 4
-                    for (int i = 0; i < 16; ++i) {                  // two rows per step, 16 lanes each
-                        const int rr = 2 * i + (lane >> 4), chunk = lane & 15;
-                        if (rr < rows_left) {
-                            const int srow = warp_row0 + rr;
-                            const uint4 val = *reinterpret_cast<const uint4*>(stage + srow * 256 + ((chunk ^ (srow & 15)) << 4));
-                            *reinterpret_cast<uint4*>(dst + (size_t)rr * (kD * 2) + chunk * 16) = val;
-                        }
-                    }
-                }
-                if (row_valid) {
-                    ws.part_m[slot] = m_ref;
-                    ws.part_l[slot] = l_run;
-                    // this part's sum over the documents alone: what the document scores are measured against
-                    if (ws.part_ld) ws.part_ld[slot] = seen_extra ? l_docs : l_run;
+                k += 2;
+                if (k >= 6) {
+                    k -= 6;
+                    phase ^= 1;
                 }
             }
+            if (ok && !have_ref) ok = warp_wait(smem_u32(&bars.ref_full[par]), (seg >> 1) & 1, abort_flag);   // every phase is waited for
+            if (!have_ref && ok) ref = sh.ref[par][r];
+            if (!seen_extra) l_docs = l_run;
+            it0 += n;
         }
     }
 
     // ---------------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
-    if (bars->abort_flag) {
-        // a wait expired: let loads already in flight land before the shared memory is given back
-        if (warp == 12 && lane == 0) {
-            for (int u = 0; u < 2 * n_it; ++u) {
-                const int use = (n_stages & 1) ? (u >> 1) / n_stages : u / n_stages;
-                const uint32_t bar = smem_u32(&bars->kv_full[u % n_stages][u & 1]);
-                const long long t0 = clock64();
-                while (!mbar_try_wait(bar, use & 1) && clock64() - t0 < kWaitLimitCycles / 16) {}
-            }
+    if (tid == 0) {
+        ShareHead head = {};
+        if (n_items > 0) head = sh.head;
+        head.marked = bars.marked;
+        reinterpret_cast<ShareHead*>(ws.marks)[blockIdx.x] = head;
+    }
+    if (bars.abort_flag) {
+        // a wait expired: let the copies in flight land before the shared memory is given back
+        if (tid == 0) {
+            const long long t0 = clock64();
+            while (clock64() - t0 < kWaitLimitCycles / 64) {}
+            atomicCAS(pv.status, 0, CF_ERR_TIMEOUT);
         }
-        if (tid == 0) atomicCAS(pv.status, 0, CF_ERR_TIMEOUT);
         __syncthreads();
     }
-    if (warp == 13) {
+    if (warp == kMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
+}
+
+constexpr int kMergeRows = 32;                     // rows of a unit per block: four per warp, eight lanes each
+
+// Units that lie in several shares, four blocks per share: those of the share a unit begins in merge its parts, in the order
+// of the line.  They also see to rows of the share's whole units that left the range of their reference; the last share's
+// blocks to the (empty) results of requests that have nothing to attend.  A chain of two memory latencies: what a block
+// has to know about the unit was left by the CTA that began it, and all parts of a row are loaded together.
+template <int LAYOUT>
+__global__ void __launch_bounds__(256, 3)
+attn_tc_merge_kernel(const __grid_constant__ Params p) {
+    CF_PARAMS;
+    const int max_shares = p.max_shares;
+    __shared__ Requests s_rq;
+    const int lq = bv.q_len, rows_total = n_q_heads * lq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kBlocks = kRowTile / kMergeRows;
+    const int share = blockIdx.x / kBlocks, block = blockIdx.x - share * kBlocks;
+    chain_next();
+    chain_wait();
+    const int4* words = reinterpret_cast<const int4*>(reinterpret_cast<const ShareHead*>(ws.marks) + share);
+    const int4 w0 = words[0], w1 = words[1];
+    const ShareHead head = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+    if (share == max_shares - 1 && p.n_prefix + p.n_self == 0)
+        for (int b = block; b < bv.n_requests; b += kBlocks)
+            if (pv.n_tiles[b] == 0)
+                for (int layer = 0; layer < ws.n_layers; ++layer) {
+                    uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)layer * span.out_stride + (size_t)b * rows_total * kD);
+                    for (int i = threadIdx.x; i < rows_total * (kD / 8); i += 256) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+                    const size_t at = ((size_t)layer * bv.n_requests + b) * rows_total;
+                    for (int i = threadIdx.x; i < rows_total; i += 256) {
+                        ws.row_lse2[at + i] = -INFINITY;
+                        if (lse) lse[at + i] = -INFINITY;
+                    }
+                }
+    if (head.marked) {
+        if (warp == 0) scan_requests(bv, pv, p.n_prefix + p.n_self, s_rq);
+        __syncthreads();
+        const Line line = make_line(bv, ws, s_rq, n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, max_shares);
+        const int group = n_q_heads / n_kv_heads, end = line.cut(share + 1);
+        for (int y = line.cut(share); y < end;) {
+            const Segment own = segment_at(bv, pv, ws, line, group, y, end);
+            if (own.t_end - own.t_begin == own.n_unit)
+                for (int r = block * kMergeRows + warp; r < min(own.rows_here, (block + 1) * kMergeRows); r += 8) {
+                    const int rg = own.kvh * group * lq + own.row0 + r;
+                    const float v = ws.row_lse2[(size_t)own.lb * rows_total + rg];
+                    if (v != v) row_from_scratch<LAYOUT>(p, own.lb, rg, own.n_doc);
+                }
+            y += own.t_end - own.t_begin;
+        }
+    }
+    const int n_parts = head.n_parts;
+    if (n_parts == 0) return;
+    const int r = block * kMergeRows + warp * 4 + (lane >> 3), e0 = (lane & 7) * 16;         // row of the unit; this lane's dims
+    const bool valid = r < head.rows_here;
+    float acc[16], m = -INFINITY, l = 0.f, ld = 0.f;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) acc[e] = 0.f;
+    // part i: the share's slot for what goes on behind it (i = 0), the others' for what began before them
+    const size_t slot0 = ((size_t)2 * share + 1) * kRowTile + min(r, head.rows_here - 1), slot1 = slot0 + kRowTile;
+    auto slot_of = [&](int i) { return i == 0 ? slot0 : slot1 + (size_t)(i - 1) * 2 * kRowTile; };
+    const __nv_bfloat16* part_o = reinterpret_cast<const __nv_bfloat16*>(ws.part_o) + e0;
+    for (int i0 = 0; i0 < n_parts; i0 += 4) {
+        float mp[4], lp[4], dp[4];
+        uint4 o[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const size_t slot = slot_of(min(i0 + u, n_parts - 1));
+            mp[u] = i0 + u < n_parts ? ws.part_m[slot] : -INFINITY;
+            lp[u] = ws.part_l[slot];
+            dp[u] = ws.part_ld ? ws.part_ld[slot] : lp[u];
+            o[u][0] = *reinterpret_cast<const uint4*>(part_o + slot * kD);
+            o[u][1] = *reinterpret_cast<const uint4*>(part_o + slot * kD + 8);
+        }
+        const float m_new = fmaxf(fmaxf(m, fmaxf(mp[0], mp[1])), fmaxf(mp[2], mp[3]));
+        const float keep = m > -INFINITY ? exp2f(m - m_new) : 0.f;
+        m = m_new;
+        l *= keep;
+        ld *= keep;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] *= keep;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (mp[u] > -INFINITY) {
+                const float w = exp2f(mp[u] - m_new);
+                l = fmaf(lp[u], w, l);
+                ld = fmaf(dp[u], w, ld);
+                const uint32_t words[8] = {o[u][0].x, o[u][0].y, o[u][0].z, o[u][0].w, o[u][1].x, o[u][1].y, o[u][1].z, o[u][1].w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    acc[2 * e] = fmaf(__uint_as_float(words[e] << 16), w, acc[2 * e]);
+                    acc[2 * e + 1] = fmaf(__uint_as_float(words[e] & 0xffff0000u), w, acc[2 * e + 1]);
+                }
+            }
+    }
+    const int rg = head.row_first + r, h = rg / lq, j = rg - h * lq;
+    if (valid && l == l) {
+        const float inv = l > 0.f ? 1.f / l : 0.f;
+        uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)head.layer * span.out_stride + (((size_t)head.b * lq + j) * n_q_heads + h) * kD + e0);
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            dst[e] = make_uint4(pack_bf16(acc[8 * e] * inv, acc[8 * e + 1] * inv), pack_bf16(acc[8 * e + 2] * inv, acc[8 * e + 3] * inv),
+                                pack_bf16(acc[8 * e + 4] * inv, acc[8 * e + 5] * inv), pack_bf16(acc[8 * e + 6] * inv, acc[8 * e + 7] * inv));
+        if ((lane & 7) == 0) {
+            ws.row_lse2[(size_t)head.lb * rows_total + rg] = ld > 0.f ? m + log2f(ld) : -INFINITY;
+            if (lse) lse[(size_t)head.lb * rows_total + rg] = (l > 0.f ? m + log2f(l) : -INFINITY) * kLn2;
+        }
+    }
+    // marked: out of the range of its reference
+    for (unsigned todo = __ballot_sync(0xffffffffu, valid && l != l && (lane & 7) == 0); todo; todo &= todo - 1)
+        row_from_scratch<LAYOUT>(p, head.lb, __shfl_sync(0xffffffffu, rg, __ffs(todo) - 1), head.n_doc);
 }
 
 // Exercises the bounded wait by itself: one CTA initialises an mbarrier that nothing ever arrives on,
@@ -609,35 +965,6 @@ __global__ void __launch_bounds__(128) wait_probe_kernel(int* status, long long 
     if (threadIdx.x == 0 && !ok && abort_word) atomicCAS(status, 0, CF_ERR_TIMEOUT);
 }
 
-// The store as a 4-D tensor (head_dim, kv heads, rows, layers).
-int make_store_map(CUtensorMap* map, const void* base, const cf_geom* g, const cf_batch* b, const LayerSpan& span,
-                   int box_rows) {
-    const unsigned long long layer_bytes = span.n_layers > 1 ? (unsigned long long)span.kv_stride * 2
-                                                             : (unsigned long long)b->total_tokens * b->token_stride * 2;
-    return make_rows_map(map, base, g->n_kv_heads, (unsigned long long)b->total_tokens,
-                         (unsigned long long)b->token_stride * 2, span.n_layers, layer_bytes, box_rows);
-}
-
-// Keys or values of the query tokens, [layers][requests][q_len][kv heads][head_dim], as a 4-D tensor
-// (head_dim, kv heads, requests * q_len rows, layers).
-int make_self_map(CUtensorMap* map, const void* base, const cf_geom* g, const cf_batch* b, const LayerSpan& span,
-                  long long self_stride, int box_rows) {
-    const unsigned long long rows = (unsigned long long)b->n_requests * b->q_len;
-    const unsigned long long row_bytes = (unsigned long long)g->n_kv_heads * kD * 2;
-    const unsigned long long layer_bytes = span.n_layers > 1 ? (unsigned long long)self_stride * 2 : rows * row_bytes;
-    return make_rows_map(map, base, g->n_kv_heads, rows, row_bytes, span.n_layers, layer_bytes, box_rows);
-}
-
-// Keys or values of a shared prefix cache, [layers][prefix_len][kv heads][head_dim] dense, as a 4-D tensor
-// (head_dim, kv heads, prefix rows, layers).
-int make_prefix_map(CUtensorMap* map, const void* base, const cf_geom* g, const LayerSpan& span, int prefix_len,
-                    long long prefix_stride, int box_rows) {
-    const unsigned long long row_bytes = (unsigned long long)g->n_kv_heads * kD * 2;
-    const unsigned long long layer_bytes = span.n_layers > 1 ? (unsigned long long)prefix_stride * 2
-                                                             : (unsigned long long)prefix_len * row_bytes;
-    return make_rows_map(map, base, g->n_kv_heads, (unsigned long long)prefix_len, row_bytes, span.n_layers, layer_bytes, box_rows);
-}
-
 }  // namespace
 
 int launch_wait_probe(const PlanView& pv, long long limit_cycles, cudaStream_t stream) {
@@ -646,55 +973,68 @@ int launch_wait_probe(const PlanView& pv, long long limit_cycles, cudaStream_t s
 }
 
 bool attn_tc_supported(const cf_geom* g, const cf_batch* b) {
-    return g->dtype == CF_BF16 && g->head_dim == 128 && b->total_tokens > 0 && b->n_docs_total < (1 << 23);
+    return g->dtype == CF_BF16 && g->head_dim == 128 && b->total_tokens > 0;
 }
+
+// Query rows of a tile: the rows that share a kv head, spread evenly over as few 128-row tiles as hold them, whole warps.
+int attn_tc_row_tile(const cf_geom* g, const cf_batch* b) {
+    const long long rows = (long long)(g->n_q_heads / g->n_kv_heads) * b->q_len, tiles = (rows + kRowTile - 1) / kRowTile;
+    return (int)std::min<long long>(kRowTile, ((rows + tiles - 1) / tiles + 31) / 32 * 32);
+}
+
+// Two parts per share of the line, one share per SM.
+size_t attn_tc_part_rows() { return (size_t)2 * sm_count() * kRowTile; }
 
 int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span, const void* q,
                    const void* k, const void* v, const void* k_self, const void* v_self, long long self_stride,
                    const void* k_prefix, const void* v_prefix, long long prefix_stride, int prefix_len,
-                   float scale_log2, const AttnWorkspace& ws, cudaStream_t stream) {
-    const int rows = (g->n_q_heads / g->n_kv_heads) * b->q_len;
-    const int row_groups = (rows + ws.rg_rows - 1) / ws.rg_rows;
-    if ((long long)g->n_kv_heads * row_groups > 65535 || (long long)b->n_requests * span.n_layers > 65535 ||
-        (ws.n_splits & 1) || (ws.rg_rows != 128 && ws.rg_rows != 256))
-        return CF_ERR_INVALID_ARG;
+                   float scale_log2, const AttnWorkspace& ws, void* out, float* lse, cudaStream_t stream) {
+    const int group = g->n_q_heads / g->n_kv_heads;
+    const long long row_tiles = ((long long)group * b->q_len + ws.rg_rows - 1) / ws.rg_rows;
+    // the line's positions are 32-bit
+    const long long most = ((long long)pv.max_tiles + (long long)b->n_requests * (prefix_len / kTile + b->q_len / kTile + 2)) *
+                           g->n_kv_heads * row_tiles * span.n_layers;
+    if (most > 0x7fffffffLL || g->n_kv_heads >= (1 << 20)) return CF_ERR_INVALID_ARG;
     StoreMaps maps;
-    for (int i = 0; i < 4; ++i) {
-        int rc = make_store_map(&maps.k[i], k, g, b, span, (i + 1) * kBoxRows);
+    const unsigned long long rows = (unsigned long long)b->total_tokens, row_bytes = (unsigned long long)b->token_stride * 2;
+    const unsigned long long layer_bytes = span.n_layers > 1 ? (unsigned long long)span.kv_stride * 2 : rows * row_bytes;
+    for (int i = 0; i < kBoxes; ++i) {
+        int rc = make_rows_map(&maps.k[i], k, g->n_kv_heads, rows, row_bytes, span.n_layers, layer_bytes, (i + 1) * 16);
+        if (rc == CF_OK) rc = make_rows_map(&maps.v[i], v, g->n_kv_heads, rows, row_bytes, span.n_layers, layer_bytes, (i + 1) * 16);
         if (rc != CF_OK) return rc;
-        rc = make_store_map(&maps.v[i], v, g, b, span, (i + 1) * kBoxRows);
-        if (rc != CF_OK) return rc;
-        if (k_self) {
-            rc = make_self_map(&maps.ks[i], k_self, g, b, span, self_stride, (i + 1) * kBoxRows);
-            if (rc != CF_OK) return rc;
-            rc = make_self_map(&maps.vs[i], v_self, g, b, span, self_stride, (i + 1) * kBoxRows);
-            if (rc != CF_OK) return rc;
-        } else {
-            maps.ks[i] = maps.k[i];
-            maps.vs[i] = maps.v[i];
-        }
-        if (prefix_len > 0) {
-            rc = make_prefix_map(&maps.kp[i], k_prefix, g, span, prefix_len, prefix_stride, (i + 1) * kBoxRows);
-            if (rc != CF_OK) return rc;
-            rc = make_prefix_map(&maps.vp[i], v_prefix, g, span, prefix_len, prefix_stride, (i + 1) * kBoxRows);
-            if (rc != CF_OK) return rc;
-        } else {
-            maps.kp[i] = maps.k[i];
-            maps.vp[i] = maps.v[i];
-        }
     }
-    if (k_self && b->q_len > kTile) return CF_ERR_UNSUPPORTED;   // the query-self block is one key tile
-    dim3 grid((unsigned)(ws.n_splits / 2), (unsigned)(g->n_kv_heads * row_groups),
-              (unsigned)(b->n_requests * span.n_layers));
-    BatchView bv = make_batch_view(b);
-    static PerDeviceOnce configured[2];
-    auto run = [&](auto kernel, int which) {
-        if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return CF_ERR_CUDA;
-        return launch_chained(kernel, grid, kThreads, kSmemBytes, stream, maps, bv, pv, ws, span.q_stride, g->n_q_heads, g->n_kv_heads,
-                              scale_log2, static_cast<const __nv_bfloat16*>(q), k_self ? 1 : 0, prefix_len);
+    // further key blocks: dense rows of the kv heads, layers `stride` elements apart
+    const unsigned long long dense = (unsigned long long)g->n_kv_heads * kD * 2;
+    auto block_maps = [&](CUtensorMap* mk, CUtensorMap* mv, const void* pk, const void* pvv, unsigned long long n, long long stride) {
+        const unsigned long long layer = span.n_layers > 1 ? (unsigned long long)stride * 2 : n * dense;
+        const int rc = make_rows_map(mk, pk, g->n_kv_heads, n, dense, span.n_layers, layer, kTile);
+        return rc != CF_OK ? rc : make_rows_map(mv, pvv, g->n_kv_heads, n, dense, span.n_layers, layer, kTile);
     };
-    if (g->rope_layout == CF_ROPE_HALF) return run(attn_tc_kernel<CF_ROPE_HALF>, 0);
-    return run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, 1);
+    maps.ks = maps.kp = maps.k[0];
+    maps.vs = maps.vp = maps.v[0];
+    if (k_self) {
+        const int rc = block_maps(&maps.ks, &maps.vs, k_self, v_self, (unsigned long long)b->n_requests * b->q_len, self_stride);
+        if (rc != CF_OK) return rc;
+    }
+    if (prefix_len > 0) {
+        const int rc = block_maps(&maps.kp, &maps.vp, k_prefix, v_prefix, (unsigned long long)prefix_len, prefix_stride);
+        if (rc != CF_OK) return rc;
+    }
+    const BatchView bv = make_batch_view(b);
+    const int shares = sm_count();
+    typedef const __nv_bfloat16* In;
+    const RowSources src = {static_cast<In>(q), static_cast<In>(k), static_cast<In>(v), static_cast<In>(k_self), static_cast<In>(v_self),
+                            static_cast<In>(k_prefix), static_cast<In>(v_prefix), self_stride, prefix_stride, scale_log2, k_self ? 1 : 0, prefix_len};
+    const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
+                      k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, static_cast<__nv_bfloat16*>(out), lse};
+    static PerDeviceOnce configured[2];
+    auto run = [&](auto kernel, auto merge, int which) {
+        if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return (int)CF_ERR_CUDA;
+        const int rc = launch_chained(kernel, dim3((unsigned)shares), kThreads, kSmemBytes, stream, maps, p);
+        return rc != CF_OK ? rc : launch_chained(merge, dim3((unsigned)(shares * (kRowTile / kMergeRows))), 256, 0, stream, p);
+    };
+    if (g->rope_layout == CF_ROPE_HALF) return run(attn_tc_kernel<CF_ROPE_HALF>, attn_tc_merge_kernel<CF_ROPE_HALF>, 0);
+    return run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, attn_tc_merge_kernel<CF_ROPE_INTERLEAVED>, 1);
 }
 
 }  // namespace cf

@@ -96,32 +96,30 @@ int launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cu
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? CF_OK : CF_ERR_CUDA;
 }
 int choose_splits(const cf_geom* g, const cf_batch* b, int n_layers);
-int choose_row_group(const cf_geom* g, const cf_batch* b);
 int tiles_per_request_bound(const cf_batch* b);
 
 // Partial results of the attention kernels, one slice per split, merged by the combine kernel.
 // All logits are in base-2 units: t = (q.k) * softmax_scale * log2(e).
 // A call covers n_layers layers; (layer, request) pairs are numbered lb = layer * B + request.
 struct AttnWorkspace {
-    float* part_o;     // [L*B][n_splits][Hq*Lq][D] sum_t 2^(t - m) v_t, not normalised (unset if m = -inf);
-                       //                           fp32, or bf16 in the same index order when part_bf16 is set
+    float* part_o;     // [L*B][n_splits][Hq*Lq][D] sum_t 2^(t - m) v_t, not normalised (unset if m = -inf)
     float* part_m;     // [L*B][n_splits][Hq*Lq]    reference maximum m (-inf if the part is empty)
     float* part_l;     // [L*B][n_splits][Hq*Lq]    sum_t 2^(t - m)
     float* tile_lse2;  // [L][max_tiles][Hq*Lq]     log2 of sum over the tile's tokens of 2^t
     float* row_lse2;   // [L*B][Hq*Lq]              log2 of the full softmax denominator
+    int* marks;        // [shares]                  tensor-core path: a unit of the share has rows to be computed from scratch
     int n_splits;
-    int part_bf16;     // the tensor-core kernel stores its partial O rows as bf16
     int n_layers;
     int max_tiles;     // tile slots per layer in tile_lse2
-    int rg_rows;       // query rows per CTA of the tensor-core kernel: 256 (two row tiles) or 128
+    int rg_rows;       // query rows of a row tile of the tensor-core kernel, whose parts are numbered by share (cf_attn_tc.cu)
     // Key blocks besides the documents (the query-self block, a shared prefix cache) of a call that has some.
-    // self_mode 1 (CUDA-core path): the query-self block is one more part, (self_m, self_l, self_o) like
-    // (part_m, part_l, part_o) in fp32.  self_mode 2 (tensor-core path): the blocks are further key tiles of
-    // the last parts, and part_ld holds every part's sum over the documents' keys alone.  self_mode 0: none.
+    // self_mode 1 (CUDA-core path): the blocks are one more part, (self_m, self_l, self_o) like (part_m, part_l,
+    // part_o).  On the tensor-core path they are further key tiles, and part_ld holds every part's sum over the
+    // documents' keys alone.
     float* self_o;     // [L*B][Hq*Lq][D]
     float* self_m;     // [L*B][Hq*Lq]
     float* self_l;     // [L*B][Hq*Lq]
-    float* part_ld;    // [L*B][n_splits][Hq*Lq]    like part_l, the documents' keys only (self_mode 2)
+    float* part_ld;    // like part_l, the documents' keys only (tensor-core path with further key blocks)
     int self_mode;
 };
 // part_layers > 0: the partial results (and the further key blocks' buffers) are sized for that many layers only, the
@@ -153,7 +151,9 @@ int launch_attn_simt(const cf_geom* g, const cf_batch* b, const PlanView& pv, co
 int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span,
                    const void* q, const void* k, const void* v, const void* k_self, const void* v_self,
                    long long self_stride, const void* k_prefix, const void* v_prefix, long long prefix_stride,
-                   int prefix_len, float scale_log2, const AttnWorkspace& ws, cudaStream_t stream);
+                   int prefix_len, float scale_log2, const AttnWorkspace& ws, void* out, float* lse, cudaStream_t stream);
+int attn_tc_row_tile(const cf_geom* g, const cf_batch* b);
+size_t attn_tc_part_rows();
 bool attn_tc_supported(const cf_geom* g, const cf_batch* b);
 // One query row per head over the final caches of a decoding step (doc_offsets: of the decode plan).
 bool decode_attn_supported(const cf_geom* g);
@@ -162,8 +162,7 @@ int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_l
                        const void* q, const void* k, const void* v, float scale_log2, void* out, float* lse,
                        void* workspace, cudaStream_t stream);
 int launch_combine(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span,
-                   const AttnWorkspace& ws, void* out, float* lse, float* doc_scores,
-                   float* score_accum, cudaStream_t stream);
+                   const AttnWorkspace& ws, void* out, float* lse, cudaStream_t stream);
 int launch_self_block(const cf_geom* g, const cf_batch* b, const LayerSpan& span, long long self_stride,
                       const void* q, const void* k_self, const void* v_self, const void* k_prefix, const void* v_prefix,
                       long long prefix_stride, int prefix_len, float scale_log2, const AttnWorkspace& ws,

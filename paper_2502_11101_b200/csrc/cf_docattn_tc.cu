@@ -57,21 +57,21 @@ struct KeyTile {
 __device__ __forceinline__ KeyTile key_tile(int i, bool joined, int n_prefix_tiles, int prefix_len, int row_first, int n_doc_keys) {
     KeyTile t;
     if (joined) {
-        const int k0 = i * kTile;
+        const int k0 = i * kTile128;
         t.p_row0 = k0;
-        t.p_len = max(0, min(kTile, prefix_len - k0));
+        t.p_len = max(0, min(kTile128, prefix_len - k0));
         t.doc_first = max(0, k0 - prefix_len);
-        t.d_len = max(0, min(kTile - t.p_len, n_doc_keys - t.doc_first));
+        t.d_len = max(0, min(kTile128 - t.p_len, n_doc_keys - t.doc_first));
     } else if (i < n_prefix_tiles) {
-        t.p_row0 = i * kTile;
-        t.p_len = min(kTile, prefix_len - t.p_row0);
+        t.p_row0 = i * kTile128;
+        t.p_len = min(kTile128, prefix_len - t.p_row0);
         t.doc_first = 0;
         t.d_len = 0;
     } else {
         t.p_row0 = 0;
         t.p_len = 0;
-        t.doc_first = (i - n_prefix_tiles) * kTile;
-        t.d_len = min(kTile, n_doc_keys - t.doc_first);
+        t.doc_first = (i - n_prefix_tiles) * kTile128;
+        t.d_len = min(kTile128, n_doc_keys - t.doc_first);
     }
     t.d_row0 = row_first + t.doc_first;
     t.len = t.p_len + t.d_len;
@@ -107,8 +107,8 @@ __device__ __forceinline__ DocItem doc_item(const DocAttnArgs& a, const DocGrid&
     if (it.r0 >= rows) return it;
     it.rows_here = min(dg.rows_per_tile, rows - it.r0);
     it.n_doc_keys = (it.r0 + it.rows_here - 1) / group + 1;       // document tokens 0 .. the last row's token
-    it.n_tiles = dg.joined ? (dg.prefix_len + it.n_doc_keys + kTile - 1) / kTile
-                           : n_prefix_tiles + (it.n_doc_keys + kTile - 1) / kTile;
+    it.n_tiles = dg.joined ? (dg.prefix_len + it.n_doc_keys + kTile128 - 1) / kTile128
+                           : n_prefix_tiles + (it.n_doc_keys + kTile128 - 1) / kTile128;
     it.valid = true;
     return it;
 }
@@ -163,7 +163,7 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, DocAttnArgs a, DocGrid d
         tma_load_4d(q_base + kHalfBytes, &maps.qm, 64, it.kvh * group, it.row_first + it.r0 / group, it.layer, bar);
     };
     // rows of the query tile behind the box are never written: zero them once (their results are not stored)
-    for (int idx = tid; idx < (kTile - dg.rows_per_tile) * 16; idx += kDocTcThreads) {
+    for (int idx = tid; idx < (kTile128 - dg.rows_per_tile) * 16; idx += kDocTcThreads) {
         const int chunk = idx & 15, r = dg.rows_per_tile + (idx >> 4);
         *reinterpret_cast<uint4*>(smem + (chunk >> 3) * kHalfBytes + swz(r, chunk & 7)) = make_uint4(0u, 0u, 0u, 0u);
     }
@@ -417,14 +417,14 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, DocAttnArgs a, DocGrid d
 
 bool docattn_tc_supported(const cf_geom* g, const cf_doc_batch* docs) {
     return g->dtype == CF_BF16 && g->head_dim == 128 && docs->total_tokens > 0 &&
-           g->n_q_heads / g->n_kv_heads <= kTile;                   // an item holds at least one whole token
+           g->n_q_heads / g->n_kv_heads <= kTile128;                   // an item holds at least one whole token
 }
 
 int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, const void* k, const void* v,
                       const void* kp, const void* vp, void* out, float* lse, int* status, cudaStream_t stream) {
     const int group = a.n_q_heads / a.n_kv_heads;
-    if (group > kTile) return CF_ERR_UNSUPPORTED;
-    const int rows_per_tile = (kTile / group) * group;              // whole tokens
+    if (group > kTile128) return CF_ERR_UNSUPPORTED;
+    const int rows_per_tile = (kTile128 / group) * group;              // whole tokens
     const long long row_tiles = ((long long)a.max_doc_len * group + rows_per_tile - 1) / rows_per_tile;
     const long long total = row_tiles * a.n_kv_heads * (long long)a.n_docs * a.n_layers;   // work items, empty ones included
     if (row_tiles <= 0 || total > 0x7fffffffLL - 65536) return CF_ERR_INVALID_ARG;
@@ -462,7 +462,7 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
                                                           : (unsigned long long)a.total_tokens * qrow;
         const cuuint64_t dims[4] = {(cuuint64_t)kD, (cuuint64_t)a.n_q_heads, (cuuint64_t)a.total_tokens, (cuuint64_t)a.n_layers};
         const cuuint64_t strides[3] = {(cuuint64_t)kD * 2, (cuuint64_t)qrow, (cuuint64_t)qlayer};
-        const cuuint32_t box[4] = {64, (cuuint32_t)group, (cuuint32_t)(kTile / group), 1};
+        const cuuint32_t box[4] = {64, (cuuint32_t)group, (cuuint32_t)(kTile128 / group), 1};
         const cuuint32_t elem[4] = {1, 1, 1, 1};
         if (fn(&maps.qm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(q), dims, strides, box, elem,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -479,7 +479,7 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
     if (configure_smem_once(configured, docattn_tc_kernel, kDocTcSmem) != CF_OK) return CF_ERR_CUDA;
     const int ctas = sm_count() > 0 ? 2 * sm_count() : 296;         // persistent: two CTAs per SM
     const unsigned grid = (unsigned)std::min<long long>(total, ctas);
-    const DocGrid dg = {(int)row_tiles, (int)total, group, (a.prefix_len + kTile - 1) / kTile, rows_per_tile,
+    const DocGrid dg = {(int)row_tiles, (int)total, group, (a.prefix_len + kTile128 - 1) / kTile128, rows_per_tile,
                         a.prefix_len % kBoxRows == 0 ? 1 : 0, a.prefix_len};
     return launch_chained(docattn_tc_kernel, dim3(grid), kDocTcThreads, kDocTcSmem, stream, maps, a, dg, static_cast<__nv_bfloat16*>(out),
                           lse, status);

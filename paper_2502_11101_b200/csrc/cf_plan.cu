@@ -353,9 +353,9 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
         const int len = s_row[id + 1] - row0;
         const int count = __float_as_int(s_score[lo]);
         const int t = x - s_tmp[lo];
-        // the document's rows are spread evenly over its tiles, in steps of 32 rows (160 rows make
-        // tiles of 96 and 64, not 128 and 32), so consecutive tiles cost about the same
-        const int step = min(kTile, ((len + count - 1) / count + 31) & ~31);
+        // the document's rows are spread evenly over its tiles, in steps of 16 (160 rows make
+        // tiles of 80 and 80, not 96 and 64), so consecutive tiles cost about the same
+        const int step = min(kTile, ((len + count - 1) / count + 15) & ~15);
         pv.tile_doc[base + x] = doc0 + id;
         pv.tile_row0[base + x] = row0 + t * step;
         pv.tile_len[base + x] = min(step, len - t * step);

@@ -13,7 +13,8 @@ namespace cf {
 namespace tc {
 
 constexpr int kD = 128;                            // head_dim of the tensor-core kernels
-constexpr int kHalfBytes = kTile * 128;            // one 64-column half of a 128-row tile, 128 B per row
+constexpr int kTile128 = 128;                      // rows of the tiles of the cache-construction kernel
+constexpr int kHalfBytes = kTile128 * 128;         // one 64-column half of a 128-row tile, 128 B per row
 constexpr int kTileBytes = 2 * kHalfBytes;         // 32 KiB: a K tile, a V tile, a Q tile or a P tile
 constexpr int kBoxRows = 32;                       // TMA boxes are 32, 64, 96 or 128 rows high
 constexpr int kBoxBytes = kBoxRows * 128;
@@ -67,6 +68,11 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// `bytes` contiguous bytes (a multiple of 16, both addresses 16-byte aligned).
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 // A tile of shared memory to a box of a 4-D tensor; the issuing thread commits and awaits the group itself.
 __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int x, int y, int z, int w) {
     asm volatile(
@@ -155,6 +161,49 @@ __device__ __forceinline__ void tmem_st16_async(uint32_t taddr, const uint32_t (
                  : : "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(taddr)
                  : "memory");
 }
+// One lane of a converged warp.  Descriptors and predicates of a tcgen05.mma live in uniform registers: with the whole warp
+// walking the issuing role and this lane under the branch, 8 QK^T and 6 PV instructions of 96 keys issue at the math rate of
+// the pipe (770 cycles against 768); one thread of a diverged warp needs 983.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
+// A bounded wait of a whole warp: the same answer in every lane.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+// tcgen05.mma with the accumulate predicate a literal, in its two operand forms.
+template <bool ACCUMULATE>
+__device__ __forceinline__ void umma_ts_lit(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "n"(ACCUMULATE ? 1 : 0)
+        : "memory");
+}
+// Two fp32 values in one 64-bit register pair, for the packed arithmetic of sm_100.
+__device__ __forceinline__ uint64_t pack_f2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack_f2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_f2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul_f2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -164,9 +213,61 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&h);
 }
+// Thirty-two bytes to a 32-byte aligned address in one store.
+__device__ __forceinline__ void store32(void* p, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
 // Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a 128B-swizzled half tile.
 __device__ __forceinline__ uint32_t swz(int row, int chunk) {
     return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4));
+}
+
+// Columns of the P operand or of the rotated query tile, from consecutive registers; awaited by the caller.
+template <int FIRST, int N>
+__device__ __forceinline__ void tmem_st16_from(uint32_t taddr, const uint32_t (&v)[N]) {
+    static_assert(FIRST + 16 <= N, "sixteen registers");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};"
+                 : : "r"(v[FIRST]), "r"(v[FIRST + 1]), "r"(v[FIRST + 2]), "r"(v[FIRST + 3]), "r"(v[FIRST + 4]), "r"(v[FIRST + 5]),
+                 "r"(v[FIRST + 6]), "r"(v[FIRST + 7]), "r"(v[FIRST + 8]), "r"(v[FIRST + 9]), "r"(v[FIRST + 10]), "r"(v[FIRST + 11]),
+                 "r"(v[FIRST + 12]), "r"(v[FIRST + 13]), "r"(v[FIRST + 14]), "r"(v[FIRST + 15]), "r"(taddr)
+                 : "memory");
+}
+
+// Sixteen columns, asynchronous: the registers may only be used after tmem_ld16_wait.
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld16_wait(uint32_t (&v)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]),
+                   "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+                 :
+                 : "memory");
+}
+// Eight columns (16 packed bf16) of the P operand.
+__device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
+                 : : "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(taddr)
+                 : "memory");
+}
+// p = 2^(s*scale - ref) of 16 key columns with packed multiply-adds, packed in place to bf16 pairs (v[0..7]); the sums of
+// the even and the odd keys are added to sum2.
+__device__ __forceinline__ void chunk16_exp(uint32_t (&v)[16], uint64_t scale2, uint64_t neg_ref2, uint64_t& sum2) {
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+        float p0, p1;
+        unpack_f2(fma_f2(pack_f2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), scale2, neg_ref2), p0, p1);
+        p0 = fast_exp2(p0);
+        p1 = fast_exp2(p1);
+        sum2 = add_f2(sum2, pack_f2(p0, p1));
+        v[i >> 1] = pack_bf16(p0, p1);
+    }
 }
 
 // Maximum of the first `valid` of 32 logits (MASKED=false: all 32).

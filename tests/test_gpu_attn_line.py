@@ -1,0 +1,91 @@
+"""The tensor-core attention kernel cuts the key tiles of all units into equal shares: parity with the CUDA-core kernel where
+shares end inside units, hold several of them, or find nothing to do, and for rows that leave the range of their reference."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _library():
+    assert torch.cuda.is_available()
+    from paper_2502_11101_b200 import build
+    build.build()
+    import paper_2502_11101_b200 as cf
+    cf.load_library()
+
+
+def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_block=False, kept=None, peak=None):
+    """Outputs, log-sum-exps and scores of both kernel families on the same inputs."""
+    import paper_2502_11101_b200 as cf
+    from paper_2502_11101_b200.session import Session
+    b = len(docs_per_request)
+    begin = np.concatenate([[0], np.cumsum(docs_per_request)]).astype(np.int32)
+    total, (hq, hkv) = int(sum(lens)), heads
+    gen = torch.Generator(device="cuda").manual_seed(total + hq)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rand(layers, b, q_len, hq, 128), rand(layers, total, hkv, 128), rand(layers, total, hkv, 128)
+    if peak is not None:                                     # one key per kv head far above all others for every row
+        q.abs_()
+        k[:, peak] = 12.0
+    ks, vs = rand(layers, b, q_len, hkv, 128), rand(layers, b, q_len, hkv, 128)
+    kp, vp = rand(layers, max(prefix, 1), hkv, 128), rand(layers, max(prefix, 1), hkv, 128)
+    results = []
+    try:
+        for path in (1, 0):
+            cf.cf_set_attn_path(path)
+            sess = Session(hq, hkv, 128, torch.bfloat16, 32768, 1e6, q_len, np.asarray(lens, np.int32), begin,
+                           np.zeros(len(lens), np.int32), tail_reserve=q_len, prefix_len=prefix)
+            counts = None if kept is None else torch.tensor(kept, dtype=torch.int32, device="cuda")
+            sess.init(kept_count=counts)
+            out = torch.full_like(q, float("nan"))
+            lse = torch.full((layers, b, hq, q_len), float("nan"), device="cuda")
+            scores = torch.full((layers, len(lens)), float("nan"), device="cuda")
+            work = torch.full((cf.cf_attn_workspace_bytes_full(sess.geom, sess.batch, layers),), 255, dtype=torch.uint8, device="cuda")
+            if prefix:
+                cf.cf_query_prefill_attn_prefix(sess.geom, sess.batch, sess.plan, q, k, v, kp, vp, out, work,
+                                                ks if self_block else None, vs if self_block else None, lse, scores, sess.score_accum)
+            elif self_block:
+                cf.cf_query_prefill_attn_full(sess.geom, sess.batch, sess.plan, q, k, v, ks, vs, out, work, lse, scores, sess.score_accum)
+            else:
+                cf.cf_query_prefill_attn_layers(sess.geom, sess.batch, sess.plan, q, k, v, out, work, lse, scores, sess.score_accum)
+            torch.cuda.synchronize()
+            assert sess.status() == 0
+            results.append((out.float().cpu(), lse.cpu(), scores.cpu()))
+    finally:
+        cf.cf_set_attn_path(0)
+    (o_a, l_a, s_a), (o_b, l_b, s_b) = results
+    assert torch.all((o_a - o_b).abs() <= 1e-2 + 2e-2 * o_a.abs()), float((o_a - o_b).abs().max())
+    inf = torch.isinf(l_a)
+    assert torch.equal(inf, torch.isinf(l_b))
+    assert torch.all((l_a - l_b)[~inf].abs() <= 1e-3 + 1e-5 * l_a[~inf].abs())
+    assert torch.all((s_a - s_b).abs() <= 1e-3 * s_a.abs() + 1e-5)
+    return results[1]
+
+
+@pytest.mark.parametrize("heads,q_len,lens,docs,layers,prefix,self_block", [
+    ((1, 1), 1, [1], [1], 1, 0, False),                              # one row, one key
+    ((2, 1), 65, [95, 96, 97, 15, 16, 17, 193], [7], 1, 0, False),   # tile edges; two row tiles of 96 and 34 rows
+    ((8, 8), 33, [160] * 12, [5, 4, 3], 2, 0, False),                # several units per share
+    ((6, 2), 128, [96, 31], [2], 1, 97, True),                       # the query's own keys are two tiles, the prefix too
+    ((4, 2), 97, [40], [1], 3, 5, True),                             # rows that see nothing of a share's one tile
+    ((2, 2), 9, [20] * 130, [2, 1] * 43 + [1], 1, 0, False),         # more requests than the line's table has entries
+])
+def test_shares_at_their_edges(heads, q_len, lens, docs, layers, prefix, self_block):
+    _both_paths(heads, q_len, lens, docs, layers, prefix, self_block)
+
+
+@pytest.mark.parametrize("self_block", [False, True])
+def test_requests_that_keep_nothing(self_block):
+    out, lse, _ = _both_paths((4, 2), 12, [50, 130, 64, 33], [1, 2, 1], 2, 0, self_block, kept=[1, 0, 1])
+    if not self_block:
+        assert float(out[:, 1].abs().max()) == 0.0 and bool(torch.all(torch.isinf(lse[:, 1])))
+
+
+@pytest.mark.parametrize("heads,docs", [((4, 2), [9]), ((16, 16), [3, 3, 3])])
+def test_rows_far_outside_the_range_of_their_reference(heads, docs):
+    """A key more than 2^80 heavier than the first sixteen of its segment: the row is computed from scratch, whether its unit
+    was cut between shares or finished by one."""
+    out, lse, _ = _both_paths(heads, 20, [150] * 9, docs, peak=[149 + 150 * 1, 149 + 150 * 4, 149 + 150 * 7])
+    assert float(lse.max()) > 60.0
