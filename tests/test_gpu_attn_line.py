@@ -28,7 +28,7 @@ def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_b
     q, k, v = rand(layers, b, q_len, hq, 128), rand(layers, total, hkv, 128), rand(layers, total, hkv, 128)
     if peak is not None:                                     # one key per kv head far above all others for every row
         q.abs_()
-        k[:, peak] = 12.0
+        k[:, peak] = 40.0
     ks, vs = rand(layers, b, q_len, hkv, 128), rand(layers, b, q_len, hkv, 128)
     kp, vp = rand(layers, max(prefix, 1), hkv, 128), rand(layers, max(prefix, 1), hkv, 128)
     results = []
