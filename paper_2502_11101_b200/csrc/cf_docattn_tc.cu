@@ -1,24 +1,25 @@
 // Tensor-core kernel of the cache-construction attention, C_d <- LLM(C_prefix, d) (Sec. 2.2), for bf16
 // storage and head_dim 128: block-diagonal causal attention over a packed store.
 //
-// A work item is 128 query rows of a (layer, document, kv head); rows are numbered token-major
-// (r = token * G + g), so an item needs the prefix cache and the document's keys up to its last token
-// only.  Keys are walked in tiles of up to 128: first the prefix tiles (every key visible), then the
-// document's own tiles, where row r sees the keys up to its own token (causal mask of Eq. 1).
-//   warps 0-3  softmax, one query row per thread (= TMEM lane); running maximum and sum per row
-//   warp 4     one lane issues the TMA loads and the tcgen05.mma instructions
-// S = Q K^T and O += P V accumulate in tensor memory (128 + 128 columns); P goes back through tensor
-// memory as bf16 over the S columns already consumed.  There is one K and one V buffer: the next key
-// tile is fetched as soon as QK^T has read the current one, the next value tile as soon as PV has.  A CTA
-// holds 96 KB of shared memory and 256 tensor-memory columns, so two CTAs share an SM and overlap each
-// other's waits.  The result is complete per row (a document is short: no split over CTAs, no merge).
-// CTAs are persistent: CTA c takes items c, c + grid, c + 2 grid, ...  An item holds whole tokens
-// ((128 / G) * G rows), so its query rows are one box of the query tensor: they and the item's first key
-// tile are requested as soon as the last QK^T of the current item has read the query tile, and the next
-// item's first QK^T runs under the epilogue of the current one.  Rows leave through the value buffer, by
-// bulk copy when the item is a whole box of the output, row by row for the ragged last item of a
-// document; the next item's first value tile may only overwrite the buffer once they are out.  Barriers
-// live for the whole kernel; their parities follow running counts of key tiles and items.
+// A work item is the query rows of as many whole tokens as fit 128 rows of a (layer, document, kv head); rows are numbered
+// token-major (r = token * G + g), so that an item's queries are one box of the query tensor and it needs the prefix cache
+// and the document's keys up to its last token only.  An item's keys are the sequence [prefix, padded to 16; document
+// tokens], cut into tiles of 128.
+//   warps 0-3  softmax, one query row per thread (= TMEM lane)
+//   warp 4     MMA issue, the warp converged and one lane elected (see elect_one)
+//   warp 5     item descriptions and copies
+// S = Q K^T and O += P V accumulate in tensor memory (128 + 128 columns); P goes back as bf16 over the S columns already
+// consumed.  A CTA holds 97 KB of shared memory and 256 tensor-memory columns, so two CTAs share an SM and overlap each
+// other's waits; CTAs are persistent (CTA c takes items c, c + grid, ...).  There is one buffer each for queries, keys and
+// values, refilled as soon as its last reader is done; the next item's first QK^T runs under the current epilogue, whose
+// rows go to global memory straight from registers in whole sectors, so that nothing waits for a staging buffer.
+// Softmax: one fixed reference per row, the maximum over the item's first 16 keys (every row sees the first one) plus 40;
+// P and the sums keep their relative precision up to 80 (log2 units) above that maximum.  A row that leaves this range is
+// noted and computed again, alone, when the CTA's items are done.
+// Bound by HBM for a few query heads per kv head: with 6 heads and a 64-token prefix 123 flops per byte.
+// Measured (400 documents of 128-192 tokens, 12/2 heads, 4 layers, prefix 64): 660 us before
+// (one issuing thread for copies and MMAs, two passes over S, rows staged through the value buffer), 514 us now; one layer
+// of 60 ragged documents with 32 heads and a 41-token prefix 229 -> 153 us.
 // Every mbarrier wait is bounded; on expiry the CTA reports CF_ERR_TIMEOUT in the status word.
 #include <algorithm>
 
@@ -30,138 +31,117 @@ namespace {
 
 using namespace tc;
 
-constexpr int kDocTcThreads = 160;
-constexpr int kDocTcSmem = 3 * kTileBytes + 1024 + 128;      // Q, K, V tiles; alignment slack; barriers
+constexpr int kDocTcThreads = 192;
+constexpr int kDocBoxes = 4;                                 // copy boxes of 16, 32, 64 and 128 rows
+constexpr int kItemRing = 4;
+constexpr int kMarkedMost = 1024;
+constexpr float kDocRefShift = 40.0f, kDocSumLimit = 1099511627776.0f;   // 2^40: see cf_attn_tc.cu
 
 struct DocMaps {
-    CUtensorMap k[4], v[4];        // the documents' keys and values, one map per box height
-    CUtensorMap kp[4], vp[4];      // the prefix cache
-    CUtensorMap qm, om;            // the queries and the output: boxes of 64 dims x G heads x (128 / G) tokens
+    CUtensorMap k[kDocBoxes], v[kDocBoxes];        // the documents' keys and values, one map per box height
+    CUtensorMap kp[kDocBoxes], vp[kDocBoxes];      // the prefix cache
+    CUtensorMap qm;                                // the queries: boxes of 64 dims x G heads x (128 / G) tokens
 };
 
-struct DocBars {
-    unsigned long long k_full, v_full, s_full, p_ready, o_done;    // one phase per key tile
-    unsigned long long q_full, staged, stage_free;                 // one phase per item
+// index w = row tile + row_tiles * (kv head + n_kv_heads * (layer * n_docs + document))
+struct DocItem {
+    int w, layer, kvh, row_first, r0, rows_here, n_keys;      // n_keys: the padded prefix and the document keys; w < 0: no more items
+};
+
+struct DocShared {
+    unsigned long long k_full, s_full, pv_ready, o_done;      // one phase per key tile
+    unsigned long long q_full;                               // one phase per item
+    unsigned long long item_full[kItemRing];
     unsigned int tmem_base;
     volatile int abort_flag;
+    int n_marked;
+    DocItem item[kItemRing];
+    int2 marked[kMarkedMost];                                 // item, row
 };
+constexpr int kDocTcSmem = 3 * kTileBytes + (int)sizeof(DocShared) + 1024;   // Q, K, V tiles
+static_assert(2 * (kDocTcSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 
-// A key tile: up to 128 keys, first those of the prefix cache (rows p_row0 .. of the prefix tensors, visible to every
-// row), then those of the document (store rows d_row0 .., document tokens doc_first ..).  When the prefix length is a
-// multiple of the copy boxes' 32 rows the two parts share tiles (`joined`: the keys of an item are the sequence
-// [prefix; document tokens] cut every 128); otherwise the prefix has tiles of its own.
-struct KeyTile {
-    int p_row0, p_len, d_row0, d_len, doc_first, len;
-};
-
-__device__ __forceinline__ KeyTile key_tile(int i, bool joined, int n_prefix_tiles, int prefix_len, int row_first, int n_doc_keys) {
-    KeyTile t;
-    if (joined) {
-        const int k0 = i * kTile128;
-        t.p_row0 = k0;
-        t.p_len = max(0, min(kTile128, prefix_len - k0));
-        t.doc_first = max(0, k0 - prefix_len);
-        t.d_len = max(0, min(kTile128 - t.p_len, n_doc_keys - t.doc_first));
-    } else if (i < n_prefix_tiles) {
-        t.p_row0 = i * kTile128;
-        t.p_len = min(kTile128, prefix_len - t.p_row0);
-        t.doc_first = 0;
-        t.d_len = 0;
-    } else {
-        t.p_row0 = 0;
-        t.p_len = 0;
-        t.doc_first = (i - n_prefix_tiles) * kTile128;
-        t.d_len = min(kTile128, n_doc_keys - t.doc_first);
-    }
-    t.d_row0 = row_first + t.doc_first;
-    t.len = t.p_len + t.d_len;
-    return t;
-}
-
-// A work item: index w = row tile + row_tiles * (kv head + n_kv_heads * (layer * n_docs + document)).
-struct DocItem {
-    int w, layer, kvh, row_first, r0, rows_here, n_doc_keys, n_tiles;
-    bool valid;
-};
-
-// Shape of the item space.  An item holds whole tokens: rows_per_tile = (128 / G) * G rows, so that its query rows are one
-// box of the query tensor (G heads x 128 / G tokens) and arrive by bulk copy.
+// Shape of the item space.
 struct DocGrid {
-    int row_tiles, total, group, n_prefix_tiles, rows_per_tile, joined, prefix_len;
+    int row_tiles, total, group, rows_per_tile, prefix_len, prefix_pad;
 };
 
 __device__ __forceinline__ DocItem doc_item(const DocAttnArgs& a, const DocGrid& dg, int w) {
-    const int row_tiles = dg.row_tiles, total = dg.total, group = dg.group, n_prefix_tiles = dg.n_prefix_tiles;
-    DocItem it;
-    it.w = w;
-    it.valid = false;
-    if (w >= total) return it;
-    const int x = w % row_tiles, yz = w / row_tiles;
-    it.kvh = yz % a.n_kv_heads;
+    DocItem it = {};
+    it.w = -1;
+    if (w >= dg.total) return it;
+    const int x = w % dg.row_tiles, yz = w / dg.row_tiles;
     const int z = yz / a.n_kv_heads;
+    it.kvh = yz - z * a.n_kv_heads;
     it.layer = z / a.n_docs;
     const int doc = z - it.layer * a.n_docs;
     it.row_first = __ldg(a.doc_offsets + doc);
-    const int rows = (__ldg(a.doc_offsets + doc + 1) - it.row_first) * group;
+    const int rows = (__ldg(a.doc_offsets + doc + 1) - it.row_first) * dg.group;
     it.r0 = x * dg.rows_per_tile;
     if (it.r0 >= rows) return it;
     it.rows_here = min(dg.rows_per_tile, rows - it.r0);
-    it.n_doc_keys = (it.r0 + it.rows_here - 1) / group + 1;       // document tokens 0 .. the last row's token
-    it.n_tiles = dg.joined ? (dg.prefix_len + it.n_doc_keys + kTile128 - 1) / kTile128
-                           : n_prefix_tiles + (it.n_doc_keys + kTile128 - 1) / kTile128;
-    it.valid = true;
-    return it;
-}
-// The CTA's next item with rows in it, from index w on (steps of the grid size); invalid when there is none.
-__device__ __forceinline__ DocItem next_item(const DocAttnArgs& a, const DocGrid& dg, int w) {
-    DocItem it = doc_item(a, dg, w);
-    while (!it.valid && it.w < dg.total) it = doc_item(a, dg, it.w + (int)gridDim.x);
+    it.n_keys = dg.prefix_pad + (it.r0 + it.rows_here - 1) / dg.group + 1;   // document tokens up to the last row's
+    it.w = w;
     return it;
 }
 
+struct DocParams {
+    DocAttnArgs a;
+    DocGrid dg;
+    const __nv_bfloat16 *q, *k, *v, *kp, *vp;
+    __nv_bfloat16* out;
+    float* lse;
+    int* status;
+    int wide_out;                                             // output rows start at 32-byte addresses
+};
+// One row of an item by one warp, keys one after the other under a running maximum.
+__device__ __noinline__ void doc_row_from_scratch(const DocParams& p, int w, int r) {
+    const int lane = threadIdx.x & 31;
+    const DocItem it = doc_item(p.a, p.dg, w);
+    const int row = it.r0 + r, token = row / p.dg.group, h = it.kvh * p.dg.group + row - token * p.dg.group;
+    auto load = [&](const __nv_bfloat16* e, float (&x)[4]) {
+        const uint2 u = *reinterpret_cast<const uint2*>(e + lane * 4);
+        x[0] = __uint_as_float(u.x << 16);
+        x[1] = __uint_as_float(u.x & 0xffff0000u);
+        x[2] = __uint_as_float(u.y << 16);
+        x[3] = __uint_as_float(u.y & 0xffff0000u);
+    };
+    const size_t at = ((size_t)(it.row_first + token) * p.a.n_q_heads + h) * kD;
+    float q[4], acc[4] = {0.f, 0.f, 0.f, 0.f}, m = -INFINITY, l = 0.f;
+    load(p.q + (size_t)it.layer * p.a.q_layer_stride + at, q);
+    for (int i = 0; i < p.dg.prefix_len + token + 1; ++i) {
+        const size_t off = i < p.dg.prefix_len ? (size_t)it.layer * p.a.prefix_layer_stride + ((size_t)i * p.a.n_kv_heads + it.kvh) * kD
+                                               : (size_t)it.layer * p.a.kv_layer_stride + (size_t)(it.row_first + i - p.dg.prefix_len) * p.a.token_stride + it.kvh * kD;
+        float k[4], v[4];
+        load((i < p.dg.prefix_len ? p.kp : p.k) + off, k);
+        load((i < p.dg.prefix_len ? p.vp : p.v) + off, v);
+        float dot = fmaf(q[0], k[0], fmaf(q[1], k[1], fmaf(q[2], k[2], q[3] * k[3])));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        const float s = dot * p.a.scale_log2, m_new = fmaxf(m, s), alpha = exp2f(m - m_new), e = exp2f(s - m_new);
+#pragma unroll
+        for (int x = 0; x < 4; ++x) acc[x] = fmaf(acc[x], alpha, e * v[x]);
+        l = fmaf(l, alpha, e);
+        m = m_new;
+    }
+    const float inv = 1.f / l;
+    *reinterpret_cast<uint2*>(p.out + (size_t)it.layer * p.a.out_layer_stride + at + lane * 4) =
+        make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
+    if (lane == 0 && p.lse) p.lse[((size_t)it.layer * p.a.n_q_heads + h) * p.a.total_tokens + it.row_first + token] = (m + log2f(l)) * kLn2;
+}
+
 __global__ void __launch_bounds__(kDocTcThreads, 2)
-docattn_tc_kernel(const __grid_constant__ DocMaps maps, DocAttnArgs a, DocGrid dg,
-                  __nv_bfloat16* __restrict__ out_all, float* __restrict__ lse, int* status) {
+docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ DocParams p) {
     extern __shared__ unsigned char smem_raw[];
     chain_next();
     chain_wait();
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t q_base = smem_u32(smem), k_base = q_base + kTileBytes, v_base = k_base + kTileBytes;
-    DocBars* bars = reinterpret_cast<DocBars*>(smem + 3 * kTileBytes);
-    volatile int* abort_flag = &bars->abort_flag;
-
+    DocShared* sh = reinterpret_cast<DocShared*>(smem + 3 * kTileBytes);
+    volatile int* abort_flag = &sh->abort_flag;
+    const DocGrid& dg = p.dg;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int group = dg.group, n_prefix_tiles = dg.n_prefix_tiles;
-    const bool joined = dg.joined != 0;
-    DocItem cur = next_item(a, dg, (int)blockIdx.x);
-    if (!cur.valid) return;                                         // uniform over the CTA
 
-    // Keys or values of key tile i of an item into their buffer (issued by the one thread of warp 4 that also issues the MMAs).
-    auto load = [&](const DocItem& it, int i, bool values) {
-        const KeyTile t = key_tile(i, joined, n_prefix_tiles, a.prefix_len, it.row_first, it.n_doc_keys);
-        const int p_boxes = (t.p_len + kBoxRows - 1) / kBoxRows, d_boxes = (t.d_len + kBoxRows - 1) / kBoxRows;
-        const uint32_t bar = smem_u32(values ? &bars->v_full : &bars->k_full);
-        const uint32_t dst = values ? v_base : k_base;
-        mbar_expect_tx(bar, (p_boxes + d_boxes) * 2 * kBoxBytes);
-        if (p_boxes > 0) {
-            const CUtensorMap* map = values ? &maps.vp[p_boxes - 1] : &maps.kp[p_boxes - 1];
-            tma_load_4d(dst, map, 0, it.kvh, t.p_row0, it.layer, bar);
-            tma_load_4d(dst + kHalfBytes, map, 64, it.kvh, t.p_row0, it.layer, bar);
-        }
-        if (d_boxes > 0) {                                          // behind the prefix rows (a whole number of boxes)
-            const CUtensorMap* map = values ? &maps.v[d_boxes - 1] : &maps.k[d_boxes - 1];
-            const uint32_t d_dst = dst + t.p_len * 128;
-            tma_load_4d(d_dst, map, 0, it.kvh, t.d_row0, it.layer, bar);
-            tma_load_4d(d_dst + kHalfBytes, map, 64, it.kvh, t.d_row0, it.layer, bar);
-        }
-    };
-    // Query rows of an item (whole tokens, G heads each) into the query tile, one copy per 64-dim half.
-    auto load_q = [&](const DocItem& it) {
-        const uint32_t bar = smem_u32(&bars->q_full);
-        mbar_expect_tx(bar, dg.rows_per_tile * 256);
-        tma_load_4d(q_base, &maps.qm, 0, it.kvh * group, it.row_first + it.r0 / group, it.layer, bar);
-        tma_load_4d(q_base + kHalfBytes, &maps.qm, 64, it.kvh * group, it.row_first + it.r0 / group, it.layer, bar);
-    };
     // rows of the query tile behind the box are never written: zero them once (their results are not stored)
     for (int idx = tid; idx < (kTile128 - dg.rows_per_tile) * 16; idx += kDocTcThreads) {
         const int chunk = idx & 15, r = dg.rows_per_tile + (idx >> 4);
@@ -170,246 +150,276 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, DocAttnArgs a, DocGrid d
     fence_proxy_async();
     if (warp == 4) {
         if (lane == 0) {
-            mbar_init(smem_u32(&bars->k_full), 1);
-            mbar_init(smem_u32(&bars->v_full), 1);
-            mbar_init(smem_u32(&bars->s_full), 1);
-            mbar_init(smem_u32(&bars->p_ready), 128);
-            mbar_init(smem_u32(&bars->o_done), 1);
-            mbar_init(smem_u32(&bars->q_full), 1);
-            mbar_init(smem_u32(&bars->staged), 128);
-            mbar_init(smem_u32(&bars->stage_free), 128);
-            bars->abort_flag = 0;
+            mbar_init(smem_u32(&sh->k_full), 1);
+            mbar_init(smem_u32(&sh->s_full), 1);
+            mbar_init(smem_u32(&sh->pv_ready), 5);                  // P of four warps and the values
+            mbar_init(smem_u32(&sh->o_done), 1);
+            mbar_init(smem_u32(&sh->q_full), 1);
+            for (int i = 0; i < kItemRing; ++i) mbar_init(smem_u32(&sh->item_full[i]), 1);
+            sh->abort_flag = 0;
+            sh->n_marked = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            load_q(cur);                                            // the first tiles travel during the set-up
-            load(cur, 0, false);
-            load(cur, 0, true);
         }
         __syncwarp();
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&bars->tmem_base)) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&sh->tmem_base)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();                                                // barriers are initialised, tensor memory is allocated
     tc_fence_after();
-    const uint32_t tmem = bars->tmem_base;
+    const uint32_t tmem = sh->tmem_base;
 
-    if (warp == 4) {
-        if (lane == 0) {
-            // ---------------------------------------------------------- TMA loads and MMA issue
-            const uint64_t a0 = smem_desc(q_base, 16, 1024), bk = smem_desc(k_base, 16, 1024);
-            const uint64_t bv = smem_desc(v_base, kHalfBytes, 1024);
-            const uint32_t idesc_o = instr_desc(kD, true);
-            int g = 0, n = 0;                                       // key tiles and items before the current one
-            auto issue_s = [&](const DocItem& it, int i, int gi) -> bool {
-                const int n_keys = (key_tile(i, joined, n_prefix_tiles, a.prefix_len, it.row_first, it.n_doc_keys).len + 15) & ~15;
-                if (!mbar_wait(smem_u32(&bars->k_full), gi & 1, abort_flag)) return false;
-                tc_fence_after();
-                const uint32_t idesc = instr_desc(n_keys, false);
+    if (warp == 5) {
+        // -------------------------------------------------------------- items and copies
+        // Keys or values of key tile i: the prefix rows (whole chunks of 16, zeros behind the last row), then the document's.
+        auto load = [&](const DocItem& it, int i, bool values) {
+            const int k0 = i * kTile128, p_len = max(0, min(kTile128, dg.prefix_pad - k0));
+            const int doc_first = max(0, k0 - dg.prefix_pad);
+            const int n16 = (min(kTile128, it.n_keys - k0) + 15) >> 4;
+            const uint32_t bar = smem_u32(values ? &sh->pv_ready : &sh->k_full), dst = values ? v_base : k_base;
+            mbar_expect_tx(bar, n16 * (16 * 256));
+            auto rows = [&](const CUtensorMap* boxes, int at, int n, int row) {   // n chunks of 16 rows to row `at` of the tile
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                    const uint64_t off = (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
-                    umma(tmem, a0 + off, bk + off, idesc, kk > 0);
+                for (int b = kDocBoxes - 1; b >= 0; --b) {
+                    if (!(n >> b & 1)) continue;
+                    tma_load_4d(dst + at * 128, boxes + b, 0, it.kvh, row, it.layer, bar);
+                    tma_load_4d(dst + kHalfBytes + at * 128, boxes + b, 64, it.kvh, row, it.layer, bar);
+                    at += 16 << b;
+                    row += 16 << b;
                 }
-                umma_commit(smem_u32(&bars->s_full));
-                return true;
             };
-            bool ok = mbar_wait(smem_u32(&bars->q_full), 0, abort_flag);
-            if (ok) ok = issue_s(cur, 0, 0);
-            while (ok) {
-                const DocItem nxt = next_item(a, dg, cur.w + (int)gridDim.x);
-                for (int i = 0; i < cur.n_tiles && ok; ++i) {
-                    const bool last = i + 1 == cur.n_tiles;
-                    // QK^T(i) has completed: the key buffer is free, and after the item's last one the query tile too
-                    ok = mbar_wait(smem_u32(&bars->s_full), (g + i) & 1, abort_flag);
+            if (p_len > 0) rows(values ? maps.vp : maps.kp, 0, p_len >> 4, k0);
+            rows(values ? maps.v : maps.k, p_len, n16 - (p_len >> 4), it.row_first + doc_first);
+        };
+        int n = 0, g = 0;                                           // items and key tiles so far
+        bool ok = true;
+        for (int w0 = (int)blockIdx.x;; w0 += 32 * (int)gridDim.x) {
+            // 32 candidates at a time; the row tiles of short documents are empty
+            const long long mine = (long long)w0 + (long long)lane * gridDim.x;
+            const DocItem cand = doc_item(p.a, dg, (int)min(mine, (long long)dg.total));
+            unsigned live = __ballot_sync(0xffffffffu, cand.w >= 0);
+            const bool end = (long long)w0 + 32ll * gridDim.x >= dg.total;
+            while (live && ok) {
+                if (lane == __ffs((int)live) - 1) sh->item[n % kItemRing] = cand;
+                live &= live - 1;
+                __syncwarp();
+                const DocItem it = sh->item[n % kItemRing];
+                if (lane == 0) mbar_arrive(smem_u32(&sh->item_full[n % kItemRing]));
+                const int tiles = (it.n_keys + kTile128 - 1) / kTile128;
+                for (int i = 0; i < tiles && ok; ++i, ++g) {
+                    if (g > 0) ok = warp_wait(smem_u32(&sh->s_full), (g - 1) & 1, abort_flag);    // QK^T has read keys and queries
                     if (!ok) break;
-                    if (!last) {
-                        load(cur, i + 1, false);
-                    } else if (nxt.valid) {
-                        load_q(nxt);
-                        load(nxt, 0, false);
+                    if (lane == 0) {
+                        if (i == 0) {
+                            const uint32_t bar = smem_u32(&sh->q_full);
+                            const int token = it.row_first + it.r0 / dg.group;
+                            mbar_expect_tx(bar, dg.rows_per_tile * 256);
+                            tma_load_4d(q_base, &maps.qm, 0, it.kvh * dg.group, token, it.layer, bar);
+                            tma_load_4d(q_base + kHalfBytes, &maps.qm, 64, it.kvh * dg.group, token, it.layer, bar);
+                        }
+                        load(it, i, false);
                     }
-                    const int n_keys = (key_tile(i, joined, n_prefix_tiles, a.prefix_len, cur.row_first, cur.n_doc_keys).len + 15) & ~15;
-                    ok = mbar_wait(smem_u32(&bars->v_full), (g + i) & 1, abort_flag) &&
-                         mbar_wait(smem_u32(&bars->p_ready), (g + i) & 1, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    for (int kk = 0; kk < (n_keys >> 4); ++kk)        // 16 keys = 8 packed P columns per instruction
-                        umma_ts(tmem + 128, tmem + kk * 8, bv + (uint64_t)(kk * 128), idesc_o, (i > 0 || kk > 0) ? 1u : 0u);
-                    umma_commit(smem_u32(&bars->o_done));
-                    // the next QK^T sits behind PV(i) in the pipe, so it may overwrite P(i); the next item's first one
-                    // also needs its query rows in shared memory
-                    if (!last) {
-                        ok = issue_s(cur, i + 1, g + i + 1);
-                    } else if (nxt.valid) {
-                        ok = mbar_wait(smem_u32(&bars->q_full), (n + 1) & 1, abort_flag);
-                        if (ok) ok = issue_s(nxt, 0, g + i + 1);
-                    }
-                    if (!ok) break;
-                    ok = mbar_wait(smem_u32(&bars->o_done), (g + i) & 1, abort_flag);   // PV(i) has read the value buffer
-                    if (!ok) break;
-                    if (!last) {
-                        load(cur, i + 1, true);
-                    } else if (nxt.valid) {                         // the rows of this item leave through the value buffer
-                        ok = mbar_wait(smem_u32(&bars->stage_free), n & 1, abort_flag);
-                        if (ok) load(nxt, 0, true);
-                    }
+                    __syncwarp();
+                    if (g > 0) ok = warp_wait(smem_u32(&sh->o_done), (g - 1) & 1, abort_flag);    // PV has read the values
+                    if (ok && lane == 0) load(it, i, true);
+                    __syncwarp();
                 }
-                if (!nxt.valid) break;
-                g += cur.n_tiles;
                 ++n;
-                cur = nxt;
+            }
+            if (end || !ok) break;
+        }
+        if (ok && lane == 0) {
+            sh->item[n % kItemRing].w = -1;
+            mbar_arrive(smem_u32(&sh->item_full[n % kItemRing]));
+        }
+    } else if (warp == 4) {
+        // -------------------------------------------------------------- MMA issue
+        const uint64_t a0 = smem_desc(q_base, 16, 1024), bk = smem_desc(k_base, 16, 1024), bv = smem_desc(v_base, kHalfBytes, 1024);
+        const uint32_t idesc_o = instr_desc(kD, true);
+        int n16_before = 0, i_before = 0;                           // the tile whose PV is still to be issued; 0: none
+        int g = 0;
+        bool ok = true;
+        auto issue_pv = [&]() {                                     // PV of tile g - 1
+            ok = warp_wait(smem_u32(&sh->pv_ready), (g - 1) & 1, abort_flag);
+            if (!ok) return;
+            tc_fence_after();
+            if (elect_one()) {
+                for (int kk = 0; kk < n16_before; ++kk)             // 16 keys = 8 packed P columns per instruction
+                    umma_ts(tmem + 128, tmem + kk * 8, bv + (uint64_t)(kk * 128), idesc_o, (i_before > 0 || kk > 0) ? 1u : 0u);
+                umma_commit(smem_u32(&sh->o_done));
+            }
+            __syncwarp();
+        };
+        for (int n = 0; ok; ++n) {
+            ok = warp_wait(smem_u32(&sh->item_full[n % kItemRing]), (n / kItemRing) & 1, abort_flag);
+            if (!ok) break;
+            const int n_keys = sh->item[n % kItemRing].w < 0 ? 0 : sh->item[n % kItemRing].n_keys;
+            if (n_keys == 0) {
+                if (n16_before > 0) issue_pv();
+                break;
+            }
+            for (int i = 0; i * kTile128 < n_keys; ++i, ++g) {
+                // this QK^T sits behind the last PV in the pipe, so it may overwrite that P
+                if (n16_before > 0) issue_pv();
+                if (ok && i == 0) ok = warp_wait(smem_u32(&sh->q_full), n & 1, abort_flag);
+                if (ok) ok = warp_wait(smem_u32(&sh->k_full), g & 1, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const int n16 = (min(kTile128, n_keys - i * kTile128) + 15) >> 4;
+                const uint32_t idesc = instr_desc(n16 * 16, false);
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {
+                        const uint64_t off = (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
+                        umma(tmem, a0 + off, bk + off, idesc, kk > 0);
+                    }
+                    umma_commit(smem_u32(&sh->s_full));
+                }
+                __syncwarp();
+                n16_before = n16;
+                i_before = i;
             }
         }
     } else {
         // -------------------------------------------------------------- softmax, one row per thread
-        const int r = tid;                                              // 0..127 = TMEM lane
-        const uint32_t lane_addr = (uint32_t)(warp * 32) << 16;
-        const uint32_t s_addr = tmem + lane_addr, o_addr = tmem + lane_addr + 128;
-        int g = 0, n = 0;                                               // key tiles and items before the current one
+        const uint32_t s_addr = tmem + ((uint32_t)(warp * 32) << 16), o_addr = s_addr + 128;
+        const uint64_t scale2 = pack_f2(p.a.scale_log2, p.a.scale_log2);
+        const int group = dg.group;
+        const int hole = dg.prefix_pad > dg.prefix_len ? (dg.prefix_pad >> 4) - 1 : -1;       // the chunk with padding keys
+        const int hole_valid = dg.prefix_len - hole * 16;
+        int g = 0;
         bool ok = true;
-        while (ok) {
-            const DocItem nxt = next_item(a, dg, cur.w + (int)gridDim.x);
-            const bool row_valid = r < cur.rows_here;
-            const int row = cur.r0 + min(r, cur.rows_here - 1);         // rows beyond the end follow the last valid one
+        for (int n = 0; ok; ++n) {
+            ok = warp_wait(smem_u32(&sh->item_full[n % kItemRing]), (n / kItemRing) & 1, abort_flag);
+            if (!ok) break;
+            const DocItem it = sh->item[n % kItemRing];
+            if (it.w < 0) break;
+            const int last_row = it.r0 + it.rows_here - 1;
+            const int row = min(it.r0 + tid, last_row);                 // rows beyond the end follow the last valid one
             const int token = row / group;
-            float m_run = -INFINITY, l_run = 0.f;
-            for (int i = 0; i < cur.n_tiles; ++i) {
-                const KeyTile t = key_tile(i, joined, n_prefix_tiles, a.prefix_len, cur.row_first, cur.n_doc_keys);
-                // visible keys of this tile: all of its prefix keys; document tokens up to the row's own
-                const int vis = t.p_len + max(0, min(t.d_len, token - t.doc_first + 1));
-                const int n_chunks = (t.len + 31) >> 5;
-                ok = mbar_wait(smem_u32(&bars->s_full), (g + i) & 1, abort_flag);
+            // keys of the sequence that the row sees, and the least and the most among the warp's rows
+            const int lim = dg.prefix_pad + token + 1;
+            const int lim_lo = __shfl_sync(0xffffffffu, lim, 0), lim_hi = __shfl_sync(0xffffffffu, lim, 31);
+            float ref = 0.f, l_run = 0.f;
+            uint64_t neg_ref2 = 0;
+            bool marked = false;
+            const int chunks = (it.n_keys + 15) >> 4;
+            for (int c0 = 0; c0 < chunks; c0 += 8, ++g) {               // a tile: chunks c0 .. c0 + 7 of the sequence
+                const int n16 = min(8, chunks - c0);
+                ok = warp_wait(smem_u32(&sh->s_full), g & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                uint32_t sv[32];
-                float tile_max = -INFINITY;
-                for (int c = 0; c < n_chunks; ++c) {
-                    tmem_ld32(s_addr + c * 32, sv);
-                    tile_max = fmaxf(tile_max, chunk_max<true>(sv, vis - c * 32));
-                }
-                // The reference maximum of a row only moves when a tile exceeds it by more than 2^8: any reference within
-                // the exponent range is exact enough, since P (bf16) and the sums (fp32) keep their relative precision,
-                // and the rescale of O below becomes rare after the first tile.
-                const float t_max = tile_max * a.scale_log2;
-                const float m_new = t_max > m_run + 8.0f ? t_max : m_run;   // finite from the first tile on
-                const float alpha = fast_exp2(m_run - m_new);               // first tile: 0
-                if (i > 0) {
-                    ok = mbar_wait(smem_u32(&bars->o_done), (g + i - 1) & 1, abort_flag);   // PV(i-1) is complete
-                    if (!ok) break;
-                    tc_fence_after();
-                    if (__any_sync(0xffffffffu, alpha != 1.f)) {
-                        for (int cc = 0; cc < 8; ++cc) {
-                            uint32_t o[16];
-                            tmem_ld16(o_addr + cc * 16, o);
-#pragma unroll
-                            for (int x = 0; x < 16; ++x) o[x] = __float_as_uint(__uint_as_float(o[x]) * alpha);
-                            tmem_st16(o_addr + cc * 16, o);
-                        }
+                const int full = (lim_lo >> 4) - c0, some = min(n16, ((lim_hi + 15) >> 4) - c0);   // chunks every row sees; any row sees
+                uint64_t sum2 = 0;
+                auto chunk = [&](int c, uint32_t (&v)[16]) {
+                    if (c < full && c0 + c != hole) {
+                        chunk16_exp(v, scale2, neg_ref2, sum2);
+                    } else {
+                        chunk16_exp_masked(v, min(lim - (c0 + c) * 16, c0 + c == hole ? hole_valid : 16), scale2, neg_ref2, sum2);
                     }
+                    tmem_st8_async(s_addr + c * 8, v);                  // over S columns already in registers
+                };
+                uint32_t va[16], vb[16];
+                tmem_ld16_async(s_addr, va);
+                tmem_ld16_wait(va);
+                if (c0 == 0) {
+                    const float m = chunk16_max(va, min(lim, hole == 0 ? hole_valid : 16));
+                    ref = fmaf(m, p.a.scale_log2, kDocRefShift);
+                    neg_ref2 = pack_f2(-ref, -ref);
                 }
-                float tile_sum = 0.f;
-                for (int c = 0; c < n_chunks; ++c) {
-                    tmem_ld32(s_addr + c * 32, sv);
-                    tile_sum += chunk_exp<true>(sv, vis - c * 32, a.scale_log2, -m_new);
-                    tmem_st16_async(s_addr + c * 16, sv);               // over S columns already in registers
+                for (int c = 0; c < some; c += 2) {
+                    if (c > 0) tmem_ld16_wait(va);
+                    if (c + 1 < some) tmem_ld16_async(s_addr + (c + 1) * 16, vb);
+                    chunk(c, va);
+                    if (c + 1 >= some) break;
+                    tmem_ld16_wait(vb);
+                    if (c + 2 < some) tmem_ld16_async(s_addr + (c + 2) * 16, va);
+                    chunk(c + 1, vb);
+                }
+                if (some < n16) {
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) va[x] = 0u;
+                    for (int c = max(some, 0); c < n16; ++c) tmem_st8_async(s_addr + c * 8, va);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
-                mbar_arrive(smem_u32(&bars->p_ready));
-                l_run = fmaf(l_run, alpha, tile_sum);
-                m_run = m_new;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&sh->pv_ready));
+                float s0, s1;
+                unpack_f2(sum2, s0, s1);
+                marked |= !(s0 + s1 <= kDocSumLimit);
+                l_run += s0 + s1;
             }
             if (!ok) break;
-            ok = mbar_wait(smem_u32(&bars->o_done), (g + cur.n_tiles - 1) & 1, abort_flag);
+            ok = warp_wait(smem_u32(&sh->o_done), (g - 1) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
-            {
-                const float inv = 1.f / l_run;
-                // Rows leave through shared memory (the value buffer: every PV has completed), laid out like the query
-                // tile (two 64-dim halves, 128-byte swizzle): an item of whole tokens is one box of the output tensor and
-                // goes out by bulk copy; the ragged last item of a document goes out row by row.
-                unsigned char* stage = smem + 2 * kTileBytes;
-                auto stage_chunk = [&](const uint32_t (&o)[32], int c) {   // 32 dims of the row: four 16-byte pieces
+            const bool valid = tid < it.rows_here;
+            const float inv = 1.f / l_run;
+            const int h = it.kvh * group + row - token * group;
+            __nv_bfloat16* out = p.out + (size_t)it.layer * p.a.out_layer_stride + ((size_t)(it.row_first + token) * p.a.n_q_heads + h) * kD;
+            auto store = [&](const uint32_t (&o)[32], int c) {          // 32 dims: two sectors
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const int chunk = c * 4 + x;
-                        *reinterpret_cast<uint4*>(stage + (chunk >> 3) * kHalfBytes + swz(r, chunk & 7)) =
-                            make_uint4(pack_bf16(__uint_as_float(o[8 * x]) * inv, __uint_as_float(o[8 * x + 1]) * inv),
-                                       pack_bf16(__uint_as_float(o[8 * x + 2]) * inv, __uint_as_float(o[8 * x + 3]) * inv),
-                                       pack_bf16(__uint_as_float(o[8 * x + 4]) * inv, __uint_as_float(o[8 * x + 5]) * inv),
-                                       pack_bf16(__uint_as_float(o[8 * x + 6]) * inv, __uint_as_float(o[8 * x + 7]) * inv));
-                    }
-                };
-                uint32_t oa[32], ob[32];                                // the load of the next piece travels under the packing of this one
-                tmem_ld32_async(o_addr, oa);
-                tmem_ld_wait(oa);
-                tmem_ld32_async(o_addr + 32, ob);
-                stage_chunk(oa, 0);
-                tmem_ld_wait(ob);
-                tmem_ld32_async(o_addr + 64, oa);
-                stage_chunk(ob, 1);
-                tmem_ld_wait(oa);
-                tmem_ld32_async(o_addr + 96, ob);
-                stage_chunk(oa, 2);
-                tmem_ld_wait(ob);
-                stage_chunk(ob, 3);
-                if (row_valid && lse) {
-                    const int gq = row - token * group;
-                    lse[((size_t)cur.layer * a.n_q_heads + cur.kvh * group + gq) * a.total_tokens + cur.row_first + token] =
-                        (m_run + log2f(l_run)) * kLn2;
-                }
-                fence_proxy_async();
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bars->staged));
-                ok = mbar_wait(smem_u32(&bars->staged), n & 1, abort_flag);   // every row of the item is staged
-                if (!ok) break;
-                if (cur.rows_here == dg.rows_per_tile) {
-                    if (tid == 0) {
-                        const int token0 = cur.row_first + cur.r0 / group;
-                        tma_store_4d(&maps.om, smem_u32(stage), 0, cur.kvh * group, token0, cur.layer);
-                        tma_store_4d(&maps.om, smem_u32(stage) + kHalfBytes, 64, cur.kvh * group, token0, cur.layer);
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the copies have read the staging rows
-                    }
-                } else {
-                    __nv_bfloat16* out = out_all + (size_t)cur.layer * a.out_layer_stride;
-                    const int warp_row0 = warp * 32;
-#pragma unroll 4
-                    for (int x = 0; x < 16; ++x) {                      // two rows per step, 16 lanes each
-                        const int rr = warp_row0 + 2 * x + (lane >> 4), chunk = lane & 15;
-                        if (rr < cur.rows_here) {
-                            const int rw = cur.r0 + rr;
-                            const int j = rw / group, gq = rw - j * group;
-                            const uint4 val = *reinterpret_cast<const uint4*>(stage + (chunk >> 3) * kHalfBytes + swz(rr, chunk & 7));
-                            *reinterpret_cast<uint4*>(out + ((size_t)(cur.row_first + j) * a.n_q_heads + cur.kvh * group + gq) * kD + chunk * 8) = val;
-                        }
+                for (int x = 0; x < 32; x += 16) {
+                    uint32_t u[8];
+#pragma unroll
+                    for (int y = 0; y < 8; ++y)
+                        u[y] = pack_bf16(__uint_as_float(o[x + 2 * y]) * inv, __uint_as_float(o[x + 2 * y + 1]) * inv);
+                    if (!valid) continue;
+                    if (p.wide_out) {
+                        store32(out + c * 32 + x, u);
+                    } else {
+                        *reinterpret_cast<uint4*>(out + c * 32 + x) = make_uint4(u[0], u[1], u[2], u[3]);
+                        *reinterpret_cast<uint4*>(out + c * 32 + x + 8) = make_uint4(u[4], u[5], u[6], u[7]);
                     }
                 }
-                // once every thread is here the value buffer may be overwritten by the next item's first value tile
-                mbar_arrive(smem_u32(&bars->stage_free));
+            };
+            uint32_t oa[32], ob[32];                                    // the load of the next piece travels under the packing of this one
+            tmem_ld32_async(o_addr, oa);
+            tmem_ld_wait(oa);
+            tmem_ld32_async(o_addr + 32, ob);
+            store(oa, 0);
+            tmem_ld_wait(ob);
+            tmem_ld32_async(o_addr + 64, oa);
+            store(ob, 1);
+            tmem_ld_wait(oa);
+            tmem_ld32_async(o_addr + 96, ob);
+            store(oa, 2);
+            tmem_ld_wait(ob);
+            store(ob, 3);
+            if (valid && p.lse)
+                p.lse[((size_t)it.layer * p.a.n_q_heads + h) * p.a.total_tokens + it.row_first + token] = (ref + log2f(l_run)) * kLn2;
+            if (valid && marked) {
+                const int at = atomicAdd(&sh->n_marked, 1);
+                if (at < kMarkedMost) sh->marked[at] = make_int2(it.w, tid);
             }
-            if (!nxt.valid) break;
-            g += cur.n_tiles;
-            ++n;
-            cur = nxt;
         }
     }
 
     // ---------------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
-    if (bars->abort_flag) {
-        // a wait expired: let the (at most two) loads in flight land before the shared memory is given back
+    if (sh->abort_flag) {
+        // a wait expired: let the loads in flight (at most a tile of each operand) land before the shared memory is given back
         if (warp == 4 && lane == 0) {
             const long long t0 = clock64();
             while (clock64() - t0 < kWaitLimitCycles / 64) {}
         }
-        if (tid == 0 && status) atomicCAS(status, 0, CF_ERR_TIMEOUT);
+        if (tid == 0 && p.status) atomicCAS(p.status, 0, CF_ERR_TIMEOUT);
         __syncthreads();
     }
     if (warp == 4) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+    }
+    const int n_marked = sh->n_marked;
+    if (n_marked <= kMarkedMost) {
+        for (int i = warp; i < n_marked; i += kDocTcThreads / 32) doc_row_from_scratch(p, sh->marked[i].x, sh->marked[i].y);
+    } else {                                                        // more than the list holds: every row of this CTA
+        for (long long w = blockIdx.x; w < dg.total; w += gridDim.x) {
+            const DocItem it = doc_item(p.a, dg, (int)w);
+            for (int r = warp; it.w >= 0 && r < it.rows_here; r += kDocTcThreads / 32) doc_row_from_scratch(p, (int)w, r);
+        }
     }
 }
 
@@ -435,24 +445,16 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
     const unsigned long long prow = (unsigned long long)a.n_kv_heads * kD * 2;
     const unsigned long long player = a.n_layers > 1 ? (unsigned long long)a.prefix_layer_stride * 2
                                                      : (unsigned long long)a.prefix_len * prow;
-    for (int i = 0; i < 4; ++i) {
-        int rc = make_rows_map(&maps.k[i], k, a.n_kv_heads, (unsigned long long)a.total_tokens, row_bytes, a.n_layers,
-                               layer_bytes, (i + 1) * kBoxRows);
-        if (rc != CF_OK) return rc;
-        rc = make_rows_map(&maps.v[i], v, a.n_kv_heads, (unsigned long long)a.total_tokens, row_bytes, a.n_layers,
-                           layer_bytes, (i + 1) * kBoxRows);
-        if (rc != CF_OK) return rc;
-        if (a.prefix_len > 0) {
-            rc = make_rows_map(&maps.kp[i], kp, a.n_kv_heads, (unsigned long long)a.prefix_len, prow, a.n_layers, player,
-                               (i + 1) * kBoxRows);
-            if (rc != CF_OK) return rc;
-            rc = make_rows_map(&maps.vp[i], vp, a.n_kv_heads, (unsigned long long)a.prefix_len, prow, a.n_layers, player,
-                               (i + 1) * kBoxRows);
-            if (rc != CF_OK) return rc;
-        } else {
-            maps.kp[i] = maps.k[i];
-            maps.vp[i] = maps.v[i];
+    for (int i = 0; i < kDocBoxes; ++i) {
+        int rc = make_rows_map(&maps.k[i], k, a.n_kv_heads, (unsigned long long)a.total_tokens, row_bytes, a.n_layers, layer_bytes, 16 << i);
+        if (rc == CF_OK)
+            rc = make_rows_map(&maps.v[i], v, a.n_kv_heads, (unsigned long long)a.total_tokens, row_bytes, a.n_layers, layer_bytes, 16 << i);
+        if (rc == CF_OK && a.prefix_len > 0) {
+            rc = make_rows_map(&maps.kp[i], kp, a.n_kv_heads, (unsigned long long)a.prefix_len, prow, a.n_layers, player, 16 << i);
+            if (rc == CF_OK)
+                rc = make_rows_map(&maps.vp[i], vp, a.n_kv_heads, (unsigned long long)a.prefix_len, prow, a.n_layers, player, 16 << i);
         }
+        if (rc != CF_OK) return rc;
     }
     {   // queries [layers][tokens][q heads][128] as (64 dims, q heads, tokens, layers); the two halves are fetched one by one
         EncodeTiledFn fn = encode_fn();
@@ -468,21 +470,17 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return CF_ERR_CUDA;
-        // the output has the layout of the queries; its layers may lie further apart
-        const cuuint64_t ostrides[3] = {(cuuint64_t)kD * 2, (cuuint64_t)qrow,
-                                        a.n_layers > 1 ? (cuuint64_t)a.out_layer_stride * 2 : (cuuint64_t)a.total_tokens * qrow};
-        if (fn(&maps.om, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, out, dims, ostrides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return CF_ERR_CUDA;
     }
     static PerDeviceOnce configured;
     if (configure_smem_once(configured, docattn_tc_kernel, kDocTcSmem) != CF_OK) return CF_ERR_CUDA;
     const int ctas = sm_count() > 0 ? 2 * sm_count() : 296;         // persistent: two CTAs per SM
     const unsigned grid = (unsigned)std::min<long long>(total, ctas);
-    const DocGrid dg = {(int)row_tiles, (int)total, group, (a.prefix_len + kTile128 - 1) / kTile128, rows_per_tile,
-                        a.prefix_len % kBoxRows == 0 ? 1 : 0, a.prefix_len};
-    return launch_chained(docattn_tc_kernel, dim3(grid), kDocTcThreads, kDocTcSmem, stream, maps, a, dg, static_cast<__nv_bfloat16*>(out),
-                          lse, status);
+    typedef const __nv_bfloat16* In;
+    const DocParams p = {a, {(int)row_tiles, (int)total, group, rows_per_tile, a.prefix_len, (a.prefix_len + 15) & ~15},
+                         static_cast<In>(q), static_cast<In>(k), static_cast<In>(v), static_cast<In>(kp), static_cast<In>(vp),
+                         static_cast<__nv_bfloat16*>(out), lse, status,
+                         ((reinterpret_cast<uintptr_t>(out) | (uintptr_t)(a.n_layers > 1 ? a.out_layer_stride * 2 : 0)) & 31) == 0};
+    return launch_chained(docattn_tc_kernel, dim3(grid), kDocTcThreads, kDocTcSmem, stream, maps, p);
 }
 
 }  // namespace cf

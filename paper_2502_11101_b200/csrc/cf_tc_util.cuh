@@ -16,8 +16,6 @@ constexpr int kD = 128;                            // head_dim of the tensor-cor
 constexpr int kTile128 = 128;                      // rows of the tiles of the cache-construction kernel
 constexpr int kHalfBytes = kTile128 * 128;         // one 64-column half of a 128-row tile, 128 B per row
 constexpr int kTileBytes = 2 * kHalfBytes;         // 32 KiB: a K tile, a V tile, a Q tile or a P tile
-constexpr int kBoxRows = 32;                       // TMA boxes are 32, 64, 96 or 128 rows high
-constexpr int kBoxBytes = kBoxRows * 128;
 constexpr long long kWaitLimitCycles = 2000000000LL;      // about a second
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -72,13 +70,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-// A tile of shared memory to a box of a 4-D tensor; the issuing thread commits and awaits the group itself.
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int x, int y, int z, int w) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
-        ::"l"(map), "r"(src), "r"(x), "r"(y), "r"(z), "r"(w)
-        : "memory");
 }
 
 // Shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor version 1.
@@ -135,31 +126,6 @@ __device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&v)[32
 // compiler from moving their uses above the wait.
 __device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31]) : : "memory");
-}
-// 16 columns, synchronous (used on the rare rescaling path).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};\n"
-        "tcgen05.wait::st.sync.aligned;"
-        ::"r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
-          "r"(taddr)
-        : "memory");
-}
-// 16 columns (32 packed bf16) of the P operand; completion is awaited once per tile.
-__device__ __forceinline__ void tmem_st16_async(uint32_t taddr, const uint32_t (&v)[32]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};"
-                 : : "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(taddr)
-                 : "memory");
 }
 // One lane of a converged warp.  Descriptors and predicates of a tcgen05.mma live in uniform registers: with the whole warp
 // walking the issuing role and this lane under the branch, 8 QK^T and 6 PV instructions of 96 keys issue at the math rate of
@@ -270,35 +236,27 @@ __device__ __forceinline__ void chunk16_exp(uint32_t (&v)[16], uint64_t scale2, 
     }
 }
 
-// Maximum of the first `valid` of 32 logits (MASKED=false: all 32).
-template <bool MASKED>
-__device__ __forceinline__ float chunk_max(const uint32_t (&v)[32], int valid) {
-    float m0 = -INFINITY, m1 = -INFINITY;
+// The same with keys at or beyond `valid` giving 0.
+__device__ __forceinline__ void chunk16_exp_masked(uint32_t (&v)[16], int valid, uint64_t scale2, uint64_t neg_ref2, uint64_t& sum2) {
 #pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-        m0 = fmaxf(m0, (!MASKED || i < valid) ? __uint_as_float(v[i]) : -INFINITY);
-        m1 = fmaxf(m1, (!MASKED || i + 1 < valid) ? __uint_as_float(v[i + 1]) : -INFINITY);
-    }
-    return fmaxf(m0, m1);
-}
-// p = 2^(s*scale - ref) for 32 key columns (keys at or beyond `valid` give 0), packed in place to
-// bf16 pairs: v[0..15] become 16 tensor-memory columns of the P operand.  Returns the row sum.
-template <bool MASKED>
-__device__ __forceinline__ float chunk_exp(uint32_t (&v)[32], int valid, float scale_log2, float neg_ref) {
-    float sum0 = 0.f, sum1 = 0.f;
-#pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-        float p0 = fast_exp2(fmaf(__uint_as_float(v[i]), scale_log2, neg_ref));
-        float p1 = fast_exp2(fmaf(__uint_as_float(v[i + 1]), scale_log2, neg_ref));
-        if (MASKED) {
-            p0 = i < valid ? p0 : 0.f;
-            p1 = i + 1 < valid ? p1 : 0.f;
-        }
-        sum0 += p0;
-        sum1 += p1;
+    for (int i = 0; i < 16; i += 2) {
+        float p0, p1;
+        unpack_f2(fma_f2(pack_f2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), scale2, neg_ref2), p0, p1);
+        p0 = i < valid ? fast_exp2(p0) : 0.f;
+        p1 = i + 1 < valid ? fast_exp2(p1) : 0.f;
+        sum2 = add_f2(sum2, pack_f2(p0, p1));
         v[i >> 1] = pack_bf16(p0, p1);
     }
-    return sum0 + sum1;
+}
+// Maximum of the first `valid` of 16 logits.
+__device__ __forceinline__ float chunk16_max(const uint32_t (&v)[16], int valid) {
+    float m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+        m0 = fmaxf(m0, i < valid ? __uint_as_float(v[i]) : -INFINITY);
+        m1 = fmaxf(m1, i + 1 < valid ? __uint_as_float(v[i + 1]) : -INFINITY);
+    }
+    return fmaxf(m0, m1);
 }
 
 

@@ -139,3 +139,36 @@ def test_bench_sized_batch_sampled():
     picks = {(int(l), int(i)) for l, i in zip(rng.integers(0, 4, size=12), rng.integers(0, 400, size=12))}
     picks |= {(0, 0), (3, 399), (1, int(np.argmax(lens))), (2, int(np.argmin(lens)))}
     _check(lens, 4, 12, 2, 128, torch.bfloat16, 64, seed=4, sample=picks)
+
+
+@pytest.mark.parametrize("lens,prefix_len,first", [([200, 33, 1, 16, 128], 0, 20), ([130, 47], 41, 0), ([128] * 110, 0, 20)])
+def test_rows_far_outside_the_range_of_their_reference(lens, prefix_len, first):
+    """One key whose scores lie far above those of the first keys, for every row that sees it: a few rows, and more rows
+    than a CTA's list of them holds; the output at an address that is not a multiple of 32 bytes."""
+    hq, hkv, total = (32, 32, sum(lens)) if len(lens) > 100 else (12, 2, sum(lens))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").to(torch.bfloat16)
+    q, k, v = rand(1, total, hq, 128).abs_(), rand(1, total, hkv, 128), rand(1, total, hkv, 128)
+    kp, vp = (rand(1, prefix_len, hkv, 128), rand(1, prefix_len, hkv, 128)) if prefix_len else (None, None)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    for start, n in zip(off[:-1], lens):
+        if n > first:
+            k[:, int(start) + first] = 40.0
+    geom = cf.make_geom(hq, hkv, 128, torch.bfloat16, 4096, 1e4)
+    results = []
+    for path in (0, 1):
+        out = torch.empty(q.numel() + 8, dtype=torch.bfloat16, device="cuda")[8:].view(q.shape)
+        lse = torch.empty(1, hq, total, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        cf.cf_set_attn_path(path)
+        try:
+            cf.cf_document_prefill_attn(geom, torch.from_numpy(off).cuda(), max(lens), q, k, v, out, kp, vp, lse, status=status)
+            torch.cuda.synchronize()
+        finally:
+            cf.cf_set_attn_path(0)
+        assert int(status[0]) == 0
+        results.append((out.float(), lse))
+    (o0, l0), (o1, l1) = results
+    assert float(l1.max()) > 100.0
+    torch.testing.assert_close(l0, l1, rtol=2e-3, atol=2e-3)
+    torch.testing.assert_close(o0, o1, rtol=2e-2, atol=2e-2)
