@@ -10,7 +10,7 @@
 //   warp 5     item descriptions and copies
 // S = Q K^T and O += P V accumulate in tensor memory (128 + 128 columns); P goes back as bf16 over the S columns already
 // consumed.  A CTA holds 97 KB of shared memory and 256 tensor-memory columns, so two CTAs share an SM and overlap each
-// other's waits; CTAs are persistent (CTA c takes items c, c + grid, ...).  There is one buffer each for queries, keys and
+// other's waits; CTAs are persistent.  There is one buffer each for queries, keys and
 // values, refilled as soon as its last reader is done; the next item's first QK^T runs under the current epilogue, whose
 // rows go to global memory straight from registers in whole sectors, so that nothing waits for a staging buffer.
 // Softmax: one fixed reference per row, the maximum over the item's first 16 keys (every row sees the first one) plus 40;
@@ -48,6 +48,109 @@ struct DocItem {
     int w, layer, kvh, row_first, r0, rows_here, n_keys;      // n_keys: the padded prefix and the document keys; w < 0: no more items
 };
 
+// Shape of the item space.
+struct DocGrid {
+    int row_tiles, group, rows_per_tile, prefix_len, prefix_pad;
+};
+
+__device__ __forceinline__ DocItem doc_item(const DocAttnArgs& a, const DocGrid& dg, int layer, int doc, int kvh, int x) {
+    DocItem it;
+    it.w = x + dg.row_tiles * (kvh + a.n_kv_heads * (layer * a.n_docs + doc));
+    it.layer = layer;
+    it.kvh = kvh;
+    it.row_first = __ldg(a.doc_offsets + doc);
+    const int rows = (__ldg(a.doc_offsets + doc + 1) - it.row_first) * dg.group;
+    it.r0 = x * dg.rows_per_tile;
+    it.rows_here = min(dg.rows_per_tile, rows - it.r0);
+    it.n_keys = dg.prefix_pad + (it.r0 + it.rows_here - 1) / dg.group + 1;   // document tokens up to the last row's
+    return it;
+}
+__device__ __forceinline__ DocItem doc_item(const DocAttnArgs& a, const DocGrid& dg, int w) {
+    const int yz = w / dg.row_tiles, z = yz / a.n_kv_heads, layer = z / a.n_docs;
+    return doc_item(a, dg, layer, z - layer * a.n_docs, yz - z * a.n_kv_heads, w - yz * dg.row_tiles);
+}
+
+// The items of all layers, documents and kv heads lie on a line, each as long as its estimated cost, kItemCost + its keys;
+// a CTA takes those that start in its equal share of the line.  Items dealt out in turn instead leave the slowest of 296 CTAs
+// with 1.75 times the mean (60 ragged documents with 32 heads), since neighbours on a CTA come from row tiles of like number.
+// kItemCost is what an item costs beside its keys, in keys: the first QK^T, the last PV and the epilogue.
+constexpr int kItemCost = 256;
+struct DocWalk {
+    int layer, doc, kvh, x, tiles, len;                       // the current item; row tiles and tokens of its document
+    long long pos, end;                                       // where it starts on the line; where the share ends
+};
+__device__ __forceinline__ int walk_len(const DocAttnArgs& a, int doc) {
+    return doc < a.n_docs ? __ldg(a.doc_offsets + doc + 1) - __ldg(a.doc_offsets + doc) : 0;
+}
+__device__ __forceinline__ int walk_tiles(const DocGrid& dg, int len) {
+    const int tokens = dg.rows_per_tile / dg.group;
+    return max(0, min(dg.row_tiles, (len + tokens - 1) / tokens));
+}
+__device__ __forceinline__ int tile_cost(const DocGrid& dg, int len, int x) {
+    return kItemCost + dg.prefix_pad + min((x + 1) * (dg.rows_per_tile / dg.group), len);
+}
+__device__ __forceinline__ long long doc_cost(const DocGrid& dg, int len) {
+    const long long tokens = dg.rows_per_tile / dg.group, tiles = walk_tiles(dg, len);
+    return tiles == 0 ? 0 : tiles * (kItemCost + dg.prefix_pad) + tokens * (tiles * (tiles - 1) / 2) + min(tiles * tokens, (long long)len);
+}
+__device__ __forceinline__ void walk_next(const DocAttnArgs& a, const DocGrid& dg, DocWalk& w) {
+    w.pos += tile_cost(dg, w.len, w.x);
+    if (++w.x < w.tiles) return;
+    w.x = 0;
+    if (++w.kvh < a.n_kv_heads) return;
+    w.kvh = 0;
+    do {
+        if (w.pos >= w.end) return;                           // the share ends here, perhaps the line with it
+        if (++w.doc == a.n_docs) {
+            w.doc = 0;
+            ++w.layer;
+        }
+        w.len = walk_len(a, w.doc);
+        w.tiles = walk_tiles(dg, w.len);
+    } while (w.tiles == 0);
+}
+// The first item of this CTA's share, by a whole warp; pos >= end: there is none.
+__device__ __forceinline__ DocWalk walk_begin(const DocAttnArgs& a, const DocGrid& dg) {
+    const int lane = threadIdx.x & 31;
+    DocWalk w = {};
+    long long all = 0;
+    for (int d = lane; d < a.n_docs; d += 32) all += doc_cost(dg, walk_len(a, d));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+    if (all == 0) return w;
+    const long long per_layer = all * a.n_kv_heads, line = per_layer * a.n_layers;
+    const long long begin = line / gridDim.x * blockIdx.x + line % gridDim.x * blockIdx.x / gridDim.x;
+    w.end = line / gridDim.x * (blockIdx.x + 1) + line % gridDim.x * (blockIdx.x + 1) / gridDim.x;
+    if (begin == w.end) return w;
+    w.layer = (int)(begin / per_layer);
+    long long rest = begin - w.layer * per_layer;             // within the layer, then within the document, then within the kv head
+    for (int d0 = 0; d0 < a.n_docs; d0 += 32) {
+        const int len = walk_len(a, d0 + lane);
+        const long long mine = doc_cost(dg, len) * a.n_kv_heads;
+        long long upto = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long below = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += below;
+        }
+        const unsigned past = __ballot_sync(0xffffffffu, upto > rest);
+        if (past) {
+            const int at = __ffs((int)past) - 1;
+            rest -= __shfl_sync(0xffffffffu, upto - mine, at);
+            w.doc = d0 + at;
+            w.len = __shfl_sync(0xffffffffu, len, at);
+            break;
+        }
+        rest -= __shfl_sync(0xffffffffu, upto, 31);
+    }
+    w.tiles = walk_tiles(dg, w.len);
+    const long long per_head = doc_cost(dg, w.len);
+    w.kvh = (int)(rest / per_head);
+    w.pos = begin - (rest - w.kvh * per_head);                // start of the kv head's first item
+    while (w.pos < begin) walk_next(a, dg, w);
+    return w;
+}
+
 struct DocShared {
     unsigned long long k_full, s_full, pv_ready, o_done;      // one phase per key tile
     unsigned long long q_full;                               // one phase per item
@@ -56,34 +159,11 @@ struct DocShared {
     volatile int abort_flag;
     int n_marked;
     DocItem item[kItemRing];
+    DocWalk walk;
     int2 marked[kMarkedMost];                                 // item, row
 };
 constexpr int kDocTcSmem = 3 * kTileBytes + (int)sizeof(DocShared) + 1024;   // Q, K, V tiles
 static_assert(2 * (kDocTcSmem + 1024) <= 228 * 1024, "two CTAs per SM");
-
-// Shape of the item space.
-struct DocGrid {
-    int row_tiles, total, group, rows_per_tile, prefix_len, prefix_pad;
-};
-
-__device__ __forceinline__ DocItem doc_item(const DocAttnArgs& a, const DocGrid& dg, int w) {
-    DocItem it = {};
-    it.w = -1;
-    if (w >= dg.total) return it;
-    const int x = w % dg.row_tiles, yz = w / dg.row_tiles;
-    const int z = yz / a.n_kv_heads;
-    it.kvh = yz - z * a.n_kv_heads;
-    it.layer = z / a.n_docs;
-    const int doc = z - it.layer * a.n_docs;
-    it.row_first = __ldg(a.doc_offsets + doc);
-    const int rows = (__ldg(a.doc_offsets + doc + 1) - it.row_first) * dg.group;
-    it.r0 = x * dg.rows_per_tile;
-    if (it.r0 >= rows) return it;
-    it.rows_here = min(dg.rows_per_tile, rows - it.r0);
-    it.n_keys = dg.prefix_pad + (it.r0 + it.rows_here - 1) / dg.group + 1;   // document tokens up to the last row's
-    it.w = w;
-    return it;
-}
 
 struct DocParams {
     DocAttnArgs a;
@@ -193,40 +273,34 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
         };
         int n = 0, g = 0;                                           // items and key tiles so far
         bool ok = true;
-        for (int w0 = (int)blockIdx.x;; w0 += 32 * (int)gridDim.x) {
-            // 32 candidates at a time; the row tiles of short documents are empty
-            const long long mine = (long long)w0 + (long long)lane * gridDim.x;
-            const DocItem cand = doc_item(p.a, dg, (int)min(mine, (long long)dg.total));
-            unsigned live = __ballot_sync(0xffffffffu, cand.w >= 0);
-            const bool end = (long long)w0 + 32ll * gridDim.x >= dg.total;
-            while (live && ok) {
-                if (lane == __ffs((int)live) - 1) sh->item[n % kItemRing] = cand;
-                live &= live - 1;
-                __syncwarp();
-                const DocItem it = sh->item[n % kItemRing];
-                if (lane == 0) mbar_arrive(smem_u32(&sh->item_full[n % kItemRing]));
-                const int tiles = (it.n_keys + kTile128 - 1) / kTile128;
-                for (int i = 0; i < tiles && ok; ++i, ++g) {
-                    if (g > 0) ok = warp_wait(smem_u32(&sh->s_full), (g - 1) & 1, abort_flag);    // QK^T has read keys and queries
-                    if (!ok) break;
-                    if (lane == 0) {
-                        if (i == 0) {
-                            const uint32_t bar = smem_u32(&sh->q_full);
-                            const int token = it.row_first + it.r0 / dg.group;
-                            mbar_expect_tx(bar, dg.rows_per_tile * 256);
-                            tma_load_4d(q_base, &maps.qm, 0, it.kvh * dg.group, token, it.layer, bar);
-                            tma_load_4d(q_base + kHalfBytes, &maps.qm, 64, it.kvh * dg.group, token, it.layer, bar);
-                        }
-                        load(it, i, false);
-                    }
-                    __syncwarp();
-                    if (g > 0) ok = warp_wait(smem_u32(&sh->o_done), (g - 1) & 1, abort_flag);    // PV has read the values
-                    if (ok && lane == 0) load(it, i, true);
-                    __syncwarp();
-                }
-                ++n;
+        DocWalk walk = walk_begin(p.a, dg);
+        if (lane == 0) sh->walk = walk;
+        for (; ok && walk.pos < walk.end; ++n) {
+            const DocItem it = doc_item(p.a, dg, walk.layer, walk.doc, walk.kvh, walk.x);
+            if (lane == 0) {
+                sh->item[n % kItemRing] = it;
+                mbar_arrive(smem_u32(&sh->item_full[n % kItemRing]));
             }
-            if (end || !ok) break;
+            walk_next(p.a, dg, walk);
+            const int tiles = (it.n_keys + kTile128 - 1) / kTile128;
+            for (int i = 0; i < tiles && ok; ++i, ++g) {
+                if (g > 0) ok = warp_wait(smem_u32(&sh->s_full), (g - 1) & 1, abort_flag);    // QK^T has read keys and queries
+                if (!ok) break;
+                if (lane == 0) {
+                    if (i == 0) {
+                        const uint32_t bar = smem_u32(&sh->q_full);
+                        const int token = it.row_first + it.r0 / dg.group;
+                        mbar_expect_tx(bar, dg.rows_per_tile * 256);
+                        tma_load_4d(q_base, &maps.qm, 0, it.kvh * dg.group, token, it.layer, bar);
+                        tma_load_4d(q_base + kHalfBytes, &maps.qm, 64, it.kvh * dg.group, token, it.layer, bar);
+                    }
+                    load(it, i, false);
+                }
+                __syncwarp();
+                if (g > 0) ok = warp_wait(smem_u32(&sh->o_done), (g - 1) & 1, abort_flag);    // PV has read the values
+                if (ok && lane == 0) load(it, i, true);
+                __syncwarp();
+            }
         }
         if (ok && lane == 0) {
             sh->item[n % kItemRing].w = -1;
@@ -416,9 +490,9 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
     if (n_marked <= kMarkedMost) {
         for (int i = warp; i < n_marked; i += kDocTcThreads / 32) doc_row_from_scratch(p, sh->marked[i].x, sh->marked[i].y);
     } else {                                                        // more than the list holds: every row of this CTA
-        for (long long w = blockIdx.x; w < dg.total; w += gridDim.x) {
-            const DocItem it = doc_item(p.a, dg, (int)w);
-            for (int r = warp; it.w >= 0 && r < it.rows_here; r += kDocTcThreads / 32) doc_row_from_scratch(p, (int)w, r);
+        for (DocWalk walk = sh->walk; walk.pos < walk.end; walk_next(p.a, dg, walk)) {
+            const DocItem it = doc_item(p.a, dg, walk.layer, walk.doc, walk.kvh, walk.x);
+            for (int r = warp; r < it.rows_here; r += kDocTcThreads / 32) doc_row_from_scratch(p, it.w, r);
         }
     }
 }
@@ -476,7 +550,7 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
     const int ctas = sm_count() > 0 ? 2 * sm_count() : 296;         // persistent: two CTAs per SM
     const unsigned grid = (unsigned)std::min<long long>(total, ctas);
     typedef const __nv_bfloat16* In;
-    const DocParams p = {a, {(int)row_tiles, (int)total, group, rows_per_tile, a.prefix_len, (a.prefix_len + 15) & ~15},
+    const DocParams p = {a, {(int)row_tiles, group, rows_per_tile, a.prefix_len, (a.prefix_len + 15) & ~15},
                          static_cast<In>(q), static_cast<In>(k), static_cast<In>(v), static_cast<In>(kp), static_cast<In>(vp),
                          static_cast<__nv_bfloat16*>(out), lse, status,
                          ((reinterpret_cast<uintptr_t>(out) | (uintptr_t)(a.n_layers > 1 ? a.out_layer_stride * 2 : 0)) & 31) == 0};
