@@ -6,13 +6,16 @@
 // and the document's keys up to its last token only.  An item's keys are the sequence [prefix, padded to 16; document
 // tokens], cut into tiles of 128.
 //   warps 0-3  softmax, one query row per thread (= TMEM lane)
-//   warp 4     MMA issue, the warp converged and one lane elected (see elect_one)
-//   warp 5     item descriptions and copies
+//   warps 4-7  epilogue: O / sum to global memory while the softmax is at the next item
+//   warp 8     MMA issue, the warp converged and one lane elected (see elect_one)
+//   warp 9     item descriptions and copies
 // S = Q K^T and O += P V accumulate in tensor memory (128 + 128 columns); P goes back as bf16 over the S columns already
-// consumed.  A CTA holds 97 KB of shared memory and 256 tensor-memory columns, so two CTAs share an SM and overlap each
-// other's waits; CTAs are persistent.  There is one buffer each for queries, keys and
-// values, refilled as soon as its last reader is done; the next item's first QK^T runs under the current epilogue, whose
-// rows go to global memory straight from registers in whole sectors, so that nothing waits for a staging buffer.
+// consumed.  A CTA holds 107 KB of shared memory and 256 tensor-memory columns, so two CTAs share an SM and overlap each
+// other's waits; CTAs are persistent.  There is one buffer each for queries, keys and values, refilled as soon as its last
+// reader is done, and the next item's first QK^T runs behind the current one's last PV.  What bounds an item is the chain
+// QK^T, softmax, PV per key tile: no unit is busy for more than a quarter of the time, so the epilogue is taken out of the
+// chain.  Rows pass through 2 KB of staging per warp, so that a store instruction writes 64 bytes to each of 8 rows: one row
+// per thread in 32-byte pieces kept the warps waiting for 2100 cycles per item.
 // Softmax: one fixed reference per row, the maximum over the item's first 16 keys (every row sees the first one) plus 40;
 // P and the sums keep their relative precision up to 80 (log2 units) above that maximum.  A row that leaves this range is
 // noted and computed again, alone, when the CTA's items are done.
@@ -21,6 +24,8 @@
 // (one issuing thread for copies and MMAs, two passes over S, rows staged through the value buffer), 514 us now; one layer
 // of 60 ragged documents with 32 heads and a 41-token prefix 229 -> 153 us.
 // Every mbarrier wait is bounded; on expiry the CTA reports CF_ERR_TIMEOUT in the status word.
+#include <math_constants.h>
+
 #include <algorithm>
 
 #include "cf_tc_util.cuh"
@@ -31,10 +36,10 @@ namespace {
 
 using namespace tc;
 
-constexpr int kDocTcThreads = 192;
+constexpr int kDocMmaWarp = 8, kDocLoadWarp = 9, kDocTcThreads = 320;   // behind four softmax and four epilogue warps
 constexpr int kDocBoxes = 4;                                 // copy boxes of 16, 32, 64 and 128 rows
 constexpr int kItemRing = 4;
-constexpr int kMarkedMost = 1024;
+constexpr int kMarkedMost = 512;
 constexpr float kDocRefShift = 40.0f, kDocSumLimit = 1099511627776.0f;   // 2^40: see cf_attn_tc.cu
 
 struct DocMaps {
@@ -151,13 +156,20 @@ __device__ __forceinline__ DocWalk walk_begin(const DocAttnArgs& a, const DocGri
     return w;
 }
 
+// Byte offset of 16-byte piece x (0..3) of row r in a staging block of 32 rows of 64 bytes: eight lanes of consecutive rows, and
+// of consecutive pieces, fall on all banks.
+__device__ __forceinline__ int stage_at(int r, int x) { return r * 64 + ((x ^ ((r >> 1) & 3)) << 4); }
+
 struct DocShared {
+    unsigned char stage[4][32 * 64];
+
     unsigned long long k_full, s_full, pv_ready, o_done;      // one phase per key tile
-    unsigned long long q_full;                               // one phase per item
+    unsigned long long q_full, sums_full, o_full, o_free;    // one phase per item
     unsigned long long item_full[kItemRing];
     unsigned int tmem_base;
     volatile int abort_flag;
     int n_marked;
+    float row_sum[2][kTile128], row_ref[2][kTile128];         // of even and of odd items; sum NaN: the row left the range of its reference
     DocItem item[kItemRing];
     DocWalk walk;
     int2 marked[kMarkedMost];                                 // item, row
@@ -172,7 +184,6 @@ struct DocParams {
     __nv_bfloat16* out;
     float* lse;
     int* status;
-    int wide_out;                                             // output rows start at 32-byte addresses
 };
 // One row of an item by one warp, keys one after the other under a running maximum.
 __device__ __noinline__ void doc_row_from_scratch(const DocParams& p, int w, int r) {
@@ -228,13 +239,16 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
         *reinterpret_cast<uint4*>(smem + (chunk >> 3) * kHalfBytes + swz(r, chunk & 7)) = make_uint4(0u, 0u, 0u, 0u);
     }
     fence_proxy_async();
-    if (warp == 4) {
+    if (warp == kDocMmaWarp) {
         if (lane == 0) {
             mbar_init(smem_u32(&sh->k_full), 1);
             mbar_init(smem_u32(&sh->s_full), 1);
             mbar_init(smem_u32(&sh->pv_ready), 5);                  // P of four warps and the values
             mbar_init(smem_u32(&sh->o_done), 1);
             mbar_init(smem_u32(&sh->q_full), 1);
+            mbar_init(smem_u32(&sh->sums_full), 4);
+            mbar_init(smem_u32(&sh->o_full), 1);
+            mbar_init(smem_u32(&sh->o_free), 4);
             for (int i = 0; i < kItemRing; ++i) mbar_init(smem_u32(&sh->item_full[i]), 1);
             sh->abort_flag = 0;
             sh->n_marked = 0;
@@ -249,7 +263,7 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
 
-    if (warp == 5) {
+    if (warp == kDocLoadWarp) {
         // -------------------------------------------------------------- items and copies
         // Keys or values of key tile i: the prefix rows (whole chunks of 16, zeros behind the last row), then the document's.
         auto load = [&](const DocItem& it, int i, bool values) {
@@ -306,21 +320,28 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
             sh->item[n % kItemRing].w = -1;
             mbar_arrive(smem_u32(&sh->item_full[n % kItemRing]));
         }
-    } else if (warp == 4) {
+    } else if (warp == kDocMmaWarp) {
         // -------------------------------------------------------------- MMA issue
         const uint64_t a0 = smem_desc(q_base, 16, 1024), bk = smem_desc(k_base, 16, 1024), bv = smem_desc(v_base, kHalfBytes, 1024);
         const uint32_t idesc_o = instr_desc(kD, true);
-        int n16_before = 0, i_before = 0;                           // the tile whose PV is still to be issued; 0: none
+        int n16_before = 0, i_before = 0, n_before = 0;             // the tile whose PV is still to be issued (0: none) and its item
+        bool last_before = false;
         int g = 0;
         bool ok = true;
         auto issue_pv = [&]() {                                     // PV of tile g - 1
             ok = warp_wait(smem_u32(&sh->pv_ready), (g - 1) & 1, abort_flag);
             if (!ok) return;
             tc_fence_after();
+            if (i_before == 0 && n_before > 0) {                    // the epilogue has read the rows of the item before
+                ok = warp_wait(smem_u32(&sh->o_free), (n_before - 1) & 1, abort_flag);
+                if (!ok) return;
+                tc_fence_after();
+            }
             if (elect_one()) {
                 for (int kk = 0; kk < n16_before; ++kk)             // 16 keys = 8 packed P columns per instruction
                     umma_ts(tmem + 128, tmem + kk * 8, bv + (uint64_t)(kk * 128), idesc_o, (i_before > 0 || kk > 0) ? 1u : 0u);
                 umma_commit(smem_u32(&sh->o_done));
+                if (last_before) umma_commit(smem_u32(&sh->o_full));
             }
             __syncwarp();
         };
@@ -352,11 +373,13 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
                 __syncwarp();
                 n16_before = n16;
                 i_before = i;
+                n_before = n;
+                last_before = (i + 1) * kTile128 >= n_keys;
             }
         }
-    } else {
+    } else if (warp < 4) {
         // -------------------------------------------------------------- softmax, one row per thread
-        const uint32_t s_addr = tmem + ((uint32_t)(warp * 32) << 16), o_addr = s_addr + 128;
+        const uint32_t s_addr = tmem + ((uint32_t)(warp * 32) << 16);
         const uint64_t scale2 = pack_f2(p.a.scale_log2, p.a.scale_log2);
         const int group = dg.group;
         const int hole = dg.prefix_pad > dg.prefix_len ? (dg.prefix_pad >> 4) - 1 : -1;       // the chunk with padding keys
@@ -376,7 +399,6 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
             const int lim_lo = __shfl_sync(0xffffffffu, lim, 0), lim_hi = __shfl_sync(0xffffffffu, lim, 31);
             float ref = 0.f, l_run = 0.f;
             uint64_t neg_ref2 = 0;
-            bool marked = false;
             const int chunks = (it.n_keys + 15) >> 4;
             for (int c0 = 0; c0 < chunks; c0 += 8, ++g) {               // a tile: chunks c0 .. c0 + 7 of the sequence
                 const int n16 = min(8, chunks - c0);
@@ -421,51 +443,71 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
                 if (lane == 0) mbar_arrive(smem_u32(&sh->pv_ready));
                 float s0, s1;
                 unpack_f2(sum2, s0, s1);
-                marked |= !(s0 + s1 <= kDocSumLimit);
-                l_run += s0 + s1;
+                l_run += s0 + s1 <= kDocSumLimit ? s0 + s1 : CUDART_NAN_F;
             }
             if (!ok) break;
-            ok = warp_wait(smem_u32(&sh->o_done), (g - 1) & 1, abort_flag);
+            sh->row_sum[n & 1][tid] = l_run;                            // item n - 2 has left: its rows made way for PV of item n - 1
+            sh->row_ref[n & 1][tid] = ref;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sh->sums_full));
+        }
+    } else {
+        // -------------------------------------------------------------- epilogue, one row per thread
+        const int r = tid - 128;
+        const uint32_t o_addr = tmem + 128 + ((uint32_t)((warp & 3) * 32) << 16);
+        unsigned char* stage = sh->stage[warp & 3];
+        const int group = dg.group;
+        bool ok = true;
+        for (int n = 0; ok; ++n) {
+            ok = warp_wait(smem_u32(&sh->item_full[n % kItemRing]), (n / kItemRing) & 1, abort_flag);
+            if (!ok) break;
+            const DocItem it = sh->item[n % kItemRing];
+            if (it.w < 0) break;
+            const int row = it.r0 + min(r, it.rows_here - 1), token = row / group;
+            const int at = token * p.a.n_q_heads + it.kvh * group + row - token * group;   // the row among the document's
+            __nv_bfloat16* out = p.out + (size_t)it.layer * p.a.out_layer_stride + (size_t)it.row_first * p.a.n_q_heads * kD + (lane & 3) * 8;
+            ok = warp_wait(smem_u32(&sh->sums_full), n & 1, abort_flag);
+            if (!ok) break;
+            const float sum = sh->row_sum[n & 1][r], inv = 1.f / sum;
+            if (r < it.rows_here) {
+                if (p.lse)
+                    p.lse[((size_t)it.layer * p.a.n_q_heads + it.kvh * group + row - token * group) * p.a.total_tokens + it.row_first + token] =
+                        (sh->row_ref[n & 1][r] + log2f(sum)) * kLn2;
+                if (sum != sum) {
+                    const int m = atomicAdd(&sh->n_marked, 1);
+                    if (m < kMarkedMost) sh->marked[m] = make_int2(it.w, r);
+                }
+            }
+            ok = warp_wait(smem_u32(&sh->o_full), n & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
-            const bool valid = tid < it.rows_here;
-            const float inv = 1.f / l_run;
-            const int h = it.kvh * group + row - token * group;
-            __nv_bfloat16* out = p.out + (size_t)it.layer * p.a.out_layer_stride + ((size_t)(it.row_first + token) * p.a.n_q_heads + h) * kD;
-            auto store = [&](const uint32_t (&o)[32], int c) {          // 32 dims: two sectors
+            uint32_t o[32];
+            tmem_ld32_async(o_addr, o);
 #pragma unroll
-                for (int x = 0; x < 32; x += 16) {
-                    uint32_t u[8];
+            for (int c = 0; c < 4; ++c) {                               // 32 dims at a time, four 16-byte pieces
+                uint32_t u[16];
+                tmem_ld_wait(o);
 #pragma unroll
-                    for (int y = 0; y < 8; ++y)
-                        u[y] = pack_bf16(__uint_as_float(o[x + 2 * y]) * inv, __uint_as_float(o[x + 2 * y + 1]) * inv);
-                    if (!valid) continue;
-                    if (p.wide_out) {
-                        store32(out + c * 32 + x, u);
-                    } else {
-                        *reinterpret_cast<uint4*>(out + c * 32 + x) = make_uint4(u[0], u[1], u[2], u[3]);
-                        *reinterpret_cast<uint4*>(out + c * 32 + x + 8) = make_uint4(u[4], u[5], u[6], u[7]);
-                    }
+                for (int x = 0; x < 16; ++x) u[x] = pack_bf16(__uint_as_float(o[2 * x]) * inv, __uint_as_float(o[2 * x + 1]) * inv);
+                if (c < 3) {
+                    tmem_ld32_async(o_addr + (c + 1) * 32, o);
+                } else {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&sh->o_free));
                 }
-            };
-            uint32_t oa[32], ob[32];                                    // the load of the next piece travels under the packing of this one
-            tmem_ld32_async(o_addr, oa);
-            tmem_ld_wait(oa);
-            tmem_ld32_async(o_addr + 32, ob);
-            store(oa, 0);
-            tmem_ld_wait(ob);
-            tmem_ld32_async(o_addr + 64, oa);
-            store(ob, 1);
-            tmem_ld_wait(oa);
-            tmem_ld32_async(o_addr + 96, ob);
-            store(oa, 2);
-            tmem_ld_wait(ob);
-            store(ob, 3);
-            if (valid && p.lse)
-                p.lse[((size_t)it.layer * p.a.n_q_heads + h) * p.a.total_tokens + it.row_first + token] = (ref + log2f(l_run)) * kLn2;
-            if (valid && marked) {
-                const int at = atomicAdd(&sh->n_marked, 1);
-                if (at < kMarkedMost) sh->marked[at] = make_int2(it.w, tid);
+                __syncwarp();                                           // the pieces before have been read
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    *reinterpret_cast<uint4*>(stage + stage_at(lane, x)) = make_uint4(u[4 * x], u[4 * x + 1], u[4 * x + 2], u[4 * x + 3]);
+                __syncwarp();
+#pragma unroll
+                for (int x = 0; x < 32; x += 8) {
+                    const int rr = x + (lane >> 2);
+                    const int to = __shfl_sync(0xffffffffu, at, rr);
+                    if ((warp & 3) * 32 + rr < it.rows_here)
+                        *reinterpret_cast<uint4*>(out + (size_t)to * kD + c * 32) = *reinterpret_cast<const uint4*>(stage + stage_at(rr, lane & 3));
+                }
             }
         }
     }
@@ -475,14 +517,14 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
     __syncthreads();
     if (sh->abort_flag) {
         // a wait expired: let the loads in flight (at most a tile of each operand) land before the shared memory is given back
-        if (warp == 4 && lane == 0) {
+        if (warp == kDocMmaWarp && lane == 0) {
             const long long t0 = clock64();
             while (clock64() - t0 < kWaitLimitCycles / 64) {}
         }
         if (tid == 0 && p.status) atomicCAS(p.status, 0, CF_ERR_TIMEOUT);
         __syncthreads();
     }
-    if (warp == 4) {
+    if (warp == kDocMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
     }
@@ -552,8 +594,7 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
     typedef const __nv_bfloat16* In;
     const DocParams p = {a, {(int)row_tiles, group, rows_per_tile, a.prefix_len, (a.prefix_len + 15) & ~15},
                          static_cast<In>(q), static_cast<In>(k), static_cast<In>(v), static_cast<In>(kp), static_cast<In>(vp),
-                         static_cast<__nv_bfloat16*>(out), lse, status,
-                         ((reinterpret_cast<uintptr_t>(out) | (uintptr_t)(a.n_layers > 1 ? a.out_layer_stride * 2 : 0)) & 31) == 0};
+                         static_cast<__nv_bfloat16*>(out), lse, status};
     return launch_chained(docattn_tc_kernel, dim3(grid), kDocTcThreads, kDocTcSmem, stream, maps, p);
 }
 
