@@ -4,18 +4,18 @@
 // A work item is the query rows of as many whole tokens as fit 128 rows of a (layer, document, kv head); rows are numbered
 // token-major (r = token * G + g), so that an item's queries are one box of the query tensor and it needs the prefix cache
 // and the document's keys up to its last token only.  An item's keys are the sequence [prefix, padded to 16; document
-// tokens], cut into tiles of 128.
+// tokens], cut into tiles of 64.
 //   warps 0-3  softmax, one query row per thread (= TMEM lane)
 //   warps 4-7  epilogue: O / sum to global memory while the softmax is at the next item
 //   warp 8     MMA issue, the warp converged and one lane elected (see elect_one)
 //   warp 9     item descriptions and copies
-// S = Q K^T and O += P V accumulate in tensor memory (128 + 128 columns); P goes back as bf16 over the S columns already
-// consumed.  A CTA holds 107 KB of shared memory and 256 tensor-memory columns, so two CTAs share an SM and overlap each
-// other's waits; CTAs are persistent.  There is one buffer each for queries, keys and values, refilled as soon as its last
-// reader is done, and the next item's first QK^T runs behind the current one's last PV.  What bounds an item is the chain
-// QK^T, softmax, PV per key tile: no unit is busy for more than a quarter of the time, so the epilogue is taken out of the
-// chain.  Rows pass through 2 KB of staging per warp, so that a store instruction writes 64 bytes to each of 8 rows: one row
-// per thread in 32-byte pieces kept the warps waiting for 2100 cycles per item.
+// S = Q K^T and O += P V accumulate in tensor memory (two buffers of 64 columns and 128); P goes back as bf16 over the S
+// columns already consumed.  A CTA holds 109 KB of shared memory and 256 tensor-memory columns, so two CTAs share an SM;
+// CTAs are persistent.  What bounds an item is the chain QK^T, softmax, PV per key tile: no unit is busy for more than a
+// quarter of the time.  So QK^T of the next tile, the next item's first one too, runs while the softmax is at the current
+// one (tiles of 128 with one S buffer: the softmax waited 2200 cycles per tile for its S and worked for 2000), and the
+// epilogue is taken out of the chain.  Rows pass through 2 KB of staging per warp, so that a store instruction writes 64
+// bytes to each of 8 rows: one row per thread in 32-byte pieces kept the warps waiting for 2100 cycles per item.
 // Softmax: one fixed reference per row, the maximum over the item's first 16 keys (every row sees the first one) plus 40;
 // P and the sums keep their relative precision up to 80 (log2 units) above that maximum.  A row that leaves this range is
 // noted and computed again, alone, when the CTA's items are done.
@@ -37,9 +37,11 @@ namespace {
 using namespace tc;
 
 constexpr int kDocMmaWarp = 8, kDocLoadWarp = 9, kDocTcThreads = 320;   // behind four softmax and four epilogue warps
-constexpr int kDocBoxes = 4;                                 // copy boxes of 16, 32, 64 and 128 rows
-constexpr int kItemRing = 4;
-constexpr int kMarkedMost = 512;
+constexpr int kKeys = 64, kKeyChunks = kKeys / 16;           // keys of a tile
+constexpr int kKeyHalf = kKeys * 128, kKeyTile = 2 * kKeyHalf;   // bytes: 64 dims of a tile, a tile
+constexpr int kDocBoxes = 3;                                 // copy boxes of 16, 32 and 64 rows
+constexpr int kItemRing = 8, kSumRing = 4;                   // QK^T runs two tiles, perhaps two items, ahead of PV, and the epilogue one behind
+constexpr int kMarkedMost = 256;
 constexpr float kDocRefShift = 40.0f, kDocSumLimit = 1099511627776.0f;   // 2^40: see cf_attn_tc.cu
 
 struct DocMaps {
@@ -163,13 +165,13 @@ __device__ __forceinline__ int stage_at(int r, int x) { return r * 64 + ((x ^ ((
 struct DocShared {
     unsigned char stage[4][32 * 64];
 
-    unsigned long long k_full, s_full, pv_ready, o_done;      // one phase per key tile
-    unsigned long long q_full, sums_full, o_full, o_free;    // one phase per item
-    unsigned long long item_full[kItemRing];
+    unsigned long long k_full[2], s_full[2], pv_ready[2], o_done[2];   // of even and of odd key tiles
+    unsigned long long q_full, o_full, o_free;               // one phase per item
+    unsigned long long item_full[kItemRing], sums_full[kSumRing];
     unsigned int tmem_base;
     volatile int abort_flag;
     int n_marked;
-    float row_sum[2][kTile128], row_ref[2][kTile128];         // of even and of odd items; sum NaN: the row left the range of its reference
+    float row_sum[kSumRing][kTile128], row_ref[kSumRing][kTile128];   // sum NaN: the row left the range of its reference
     DocItem item[kItemRing];
     DocWalk walk;
     int2 marked[kMarkedMost];                                 // item, row
@@ -227,7 +229,7 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
     chain_next();
     chain_wait();
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const uint32_t q_base = smem_u32(smem), k_base = q_base + kTileBytes, v_base = k_base + kTileBytes;
+    const uint32_t q_base = smem_u32(smem), k_base = q_base + kTileBytes, v_base = k_base + 2 * kKeyTile;
     DocShared* sh = reinterpret_cast<DocShared*>(smem + 3 * kTileBytes);
     volatile int* abort_flag = &sh->abort_flag;
     const DocGrid& dg = p.dg;
@@ -241,12 +243,14 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
     fence_proxy_async();
     if (warp == kDocMmaWarp) {
         if (lane == 0) {
-            mbar_init(smem_u32(&sh->k_full), 1);
-            mbar_init(smem_u32(&sh->s_full), 1);
-            mbar_init(smem_u32(&sh->pv_ready), 5);                  // P of four warps and the values
-            mbar_init(smem_u32(&sh->o_done), 1);
+            for (int i = 0; i < 2; ++i) {
+                mbar_init(smem_u32(&sh->k_full[i]), 1);
+                mbar_init(smem_u32(&sh->s_full[i]), 1);
+                mbar_init(smem_u32(&sh->pv_ready[i]), 5);           // P of four warps and the values
+                mbar_init(smem_u32(&sh->o_done[i]), 1);
+            }
             mbar_init(smem_u32(&sh->q_full), 1);
-            mbar_init(smem_u32(&sh->sums_full), 4);
+            for (int i = 0; i < kSumRing; ++i) mbar_init(smem_u32(&sh->sums_full[i]), 4);
             mbar_init(smem_u32(&sh->o_full), 1);
             mbar_init(smem_u32(&sh->o_free), 4);
             for (int i = 0; i < kItemRing; ++i) mbar_init(smem_u32(&sh->item_full[i]), 1);
@@ -265,19 +269,19 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
 
     if (warp == kDocLoadWarp) {
         // -------------------------------------------------------------- items and copies
-        // Keys or values of key tile i: the prefix rows (whole chunks of 16, zeros behind the last row), then the document's.
-        auto load = [&](const DocItem& it, int i, bool values) {
-            const int k0 = i * kTile128, p_len = max(0, min(kTile128, dg.prefix_pad - k0));
+        // Keys or values of key tile i of an item, the g-th of this CTA: the prefix rows (whole chunks of 16, zeros behind the last row), then the document's.
+        auto load = [&](const DocItem& it, int i, int g, bool values) {
+            const int k0 = i * kKeys, p_len = max(0, min(kKeys, dg.prefix_pad - k0));
             const int doc_first = max(0, k0 - dg.prefix_pad);
-            const int n16 = (min(kTile128, it.n_keys - k0) + 15) >> 4;
-            const uint32_t bar = smem_u32(values ? &sh->pv_ready : &sh->k_full), dst = values ? v_base : k_base;
+            const int n16 = (min(kKeys, it.n_keys - k0) + 15) >> 4;
+            const uint32_t bar = smem_u32(values ? &sh->pv_ready[g & 1] : &sh->k_full[g & 1]), dst = (values ? v_base : k_base) + (g & 1) * kKeyTile;
             mbar_expect_tx(bar, n16 * (16 * 256));
             auto rows = [&](const CUtensorMap* boxes, int at, int n, int row) {   // n chunks of 16 rows to row `at` of the tile
 #pragma unroll
                 for (int b = kDocBoxes - 1; b >= 0; --b) {
                     if (!(n >> b & 1)) continue;
                     tma_load_4d(dst + at * 128, boxes + b, 0, it.kvh, row, it.layer, bar);
-                    tma_load_4d(dst + kHalfBytes + at * 128, boxes + b, 64, it.kvh, row, it.layer, bar);
+                    tma_load_4d(dst + kKeyHalf + at * 128, boxes + b, 64, it.kvh, row, it.layer, bar);
                     at += 16 << b;
                     row += 16 << b;
                 }
@@ -287,6 +291,13 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
         };
         int n = 0, g = 0;                                           // items and key tiles so far
         bool ok = true;
+        DocItem before = {};
+        int i_before = 0;
+        auto values_before = [&](int g) {                               // the values of tile g - 1
+            if (g > 2) ok = warp_wait(smem_u32(&sh->o_done[(g - 1) & 1]), (((g - 1) >> 1) - 1) & 1, abort_flag);   // PV has read those of g - 3
+            if (ok && lane == 0) load(before, i_before, g - 1, true);
+            __syncwarp();
+        };
         DocWalk walk = walk_begin(p.a, dg);
         if (lane == 0) sh->walk = walk;
         for (; ok && walk.pos < walk.end; ++n) {
@@ -296,40 +307,43 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
                 mbar_arrive(smem_u32(&sh->item_full[n % kItemRing]));
             }
             walk_next(p.a, dg, walk);
-            const int tiles = (it.n_keys + kTile128 - 1) / kTile128;
-            for (int i = 0; i < tiles && ok; ++i, ++g) {
-                if (g > 0) ok = warp_wait(smem_u32(&sh->s_full), (g - 1) & 1, abort_flag);    // QK^T has read keys and queries
-                if (!ok) break;
-                if (lane == 0) {
-                    if (i == 0) {
+            const int tiles = (it.n_keys + kKeys - 1) / kKeys;
+            for (int i = 0; i < tiles && ok; ++i, ++g) {                // the values travel one tile behind the keys
+                if (g > 1) ok = warp_wait(smem_u32(&sh->s_full[g & 1]), ((g >> 1) - 1) & 1, abort_flag);   // QK^T has read tile g - 2
+                if (ok && lane == 0) load(it, i, g, false);
+                __syncwarp();
+                if (ok && i == 0) {
+                    if (g > 0) ok = warp_wait(smem_u32(&sh->s_full[(g - 1) & 1]), ((g - 1) >> 1) & 1, abort_flag);   // and the last queries
+                    if (ok && lane == 0) {
                         const uint32_t bar = smem_u32(&sh->q_full);
                         const int token = it.row_first + it.r0 / dg.group;
                         mbar_expect_tx(bar, dg.rows_per_tile * 256);
                         tma_load_4d(q_base, &maps.qm, 0, it.kvh * dg.group, token, it.layer, bar);
                         tma_load_4d(q_base + kHalfBytes, &maps.qm, 64, it.kvh * dg.group, token, it.layer, bar);
                     }
-                    load(it, i, false);
+                    __syncwarp();
                 }
-                __syncwarp();
-                if (g > 0) ok = warp_wait(smem_u32(&sh->o_done), (g - 1) & 1, abort_flag);    // PV has read the values
-                if (ok && lane == 0) load(it, i, true);
-                __syncwarp();
+                if (ok && g > 0) values_before(g);
+                before = it;
+                i_before = i;
             }
         }
+        if (ok && g > 0) values_before(g);
         if (ok && lane == 0) {
             sh->item[n % kItemRing].w = -1;
             mbar_arrive(smem_u32(&sh->item_full[n % kItemRing]));
         }
     } else if (warp == kDocMmaWarp) {
         // -------------------------------------------------------------- MMA issue
-        const uint64_t a0 = smem_desc(q_base, 16, 1024), bk = smem_desc(k_base, 16, 1024), bv = smem_desc(v_base, kHalfBytes, 1024);
+        const uint64_t a0 = smem_desc(q_base, 16, 1024), bk = smem_desc(k_base, 16, 1024), bv = smem_desc(v_base, kKeyHalf, 1024);
         const uint32_t idesc_o = instr_desc(kD, true);
         int n16_before = 0, i_before = 0, n_before = 0;             // the tile whose PV is still to be issued (0: none) and its item
         bool last_before = false;
         int g = 0;
         bool ok = true;
         auto issue_pv = [&]() {                                     // PV of tile g - 1
-            ok = warp_wait(smem_u32(&sh->pv_ready), (g - 1) & 1, abort_flag);
+            const int b = (g - 1) & 1;
+            ok = warp_wait(smem_u32(&sh->pv_ready[b]), ((g - 1) >> 1) & 1, abort_flag);
             if (!ok) return;
             tc_fence_after();
             if (i_before == 0 && n_before > 0) {                    // the epilogue has read the rows of the item before
@@ -339,8 +353,8 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
             }
             if (elect_one()) {
                 for (int kk = 0; kk < n16_before; ++kk)             // 16 keys = 8 packed P columns per instruction
-                    umma_ts(tmem + 128, tmem + kk * 8, bv + (uint64_t)(kk * 128), idesc_o, (i_before > 0 || kk > 0) ? 1u : 0u);
-                umma_commit(smem_u32(&sh->o_done));
+                    umma_ts(tmem + 128, tmem + b * kKeys + kk * 8, bv + (uint64_t)(b * (kKeyTile >> 4) + kk * 128), idesc_o, (i_before > 0 || kk > 0) ? 1u : 0u);
+                umma_commit(smem_u32(&sh->o_done[b]));
                 if (last_before) umma_commit(smem_u32(&sh->o_full));
             }
             __syncwarp();
@@ -353,33 +367,34 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
                 if (n16_before > 0) issue_pv();
                 break;
             }
-            for (int i = 0; i * kTile128 < n_keys; ++i, ++g) {
-                // this QK^T sits behind the last PV in the pipe, so it may overwrite that P
-                if (n16_before > 0) issue_pv();
-                if (ok && i == 0) ok = warp_wait(smem_u32(&sh->q_full), n & 1, abort_flag);
-                if (ok) ok = warp_wait(smem_u32(&sh->k_full), g & 1, abort_flag);
+            for (int i = 0; i * kKeys < n_keys; ++i, ++g) {
+                // S of this tile, into the buffer that the PV before the last has read, while the softmax is at the tile before
+                const int b = g & 1;
+                if (i == 0) ok = warp_wait(smem_u32(&sh->q_full), n & 1, abort_flag);
+                if (ok) ok = warp_wait(smem_u32(&sh->k_full[b]), (g >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                const int n16 = (min(kTile128, n_keys - i * kTile128) + 15) >> 4;
+                const int n16 = (min(kKeys, n_keys - i * kKeys) + 15) >> 4;
                 const uint32_t idesc = instr_desc(n16 * 16, false);
                 if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        const uint64_t off = (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
-                        umma(tmem, a0 + off, bk + off, idesc, kk > 0);
-                    }
-                    umma_commit(smem_u32(&sh->s_full));
+                    for (int kk = 0; kk < 8; ++kk)
+                        umma(tmem + b * kKeys, a0 + (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4),
+                             bk + (uint64_t)((b * kKeyTile + (kk >> 2) * kKeyHalf + (kk & 3) * 32) >> 4), idesc, kk > 0);
+                    umma_commit(smem_u32(&sh->s_full[b]));
                 }
                 __syncwarp();
+                if (n16_before > 0) issue_pv();
+                if (!ok) break;
                 n16_before = n16;
                 i_before = i;
                 n_before = n;
-                last_before = (i + 1) * kTile128 >= n_keys;
+                last_before = (i + 1) * kKeys >= n_keys;
             }
         }
     } else if (warp < 4) {
         // -------------------------------------------------------------- softmax, one row per thread
-        const uint32_t s_addr = tmem + ((uint32_t)(warp * 32) << 16);
+        const uint32_t lane_tmem = tmem + ((uint32_t)(warp * 32) << 16);
         const uint64_t scale2 = pack_f2(p.a.scale_log2, p.a.scale_log2);
         const int group = dg.group;
         const int hole = dg.prefix_pad > dg.prefix_len ? (dg.prefix_pad >> 4) - 1 : -1;       // the chunk with padding keys
@@ -400,9 +415,10 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
             float ref = 0.f, l_run = 0.f;
             uint64_t neg_ref2 = 0;
             const int chunks = (it.n_keys + 15) >> 4;
-            for (int c0 = 0; c0 < chunks; c0 += 8, ++g) {               // a tile: chunks c0 .. c0 + 7 of the sequence
-                const int n16 = min(8, chunks - c0);
-                ok = warp_wait(smem_u32(&sh->s_full), g & 1, abort_flag);
+            for (int c0 = 0; c0 < chunks; c0 += kKeyChunks, ++g) {      // a tile: chunks c0 .. c0 + 3 of the sequence
+                const int n16 = min(kKeyChunks, chunks - c0);
+                const uint32_t s_addr = lane_tmem + (g & 1) * kKeys;
+                ok = warp_wait(smem_u32(&sh->s_full[g & 1]), (g >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 const int full = (lim_lo >> 4) - c0, some = min(n16, ((lim_hi + 15) >> 4) - c0);   // chunks every row sees; any row sees
@@ -440,16 +456,16 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sh->pv_ready));
+                if (lane == 0) mbar_arrive(smem_u32(&sh->pv_ready[g & 1]));
                 float s0, s1;
                 unpack_f2(sum2, s0, s1);
                 l_run += s0 + s1 <= kDocSumLimit ? s0 + s1 : CUDART_NAN_F;
             }
             if (!ok) break;
-            sh->row_sum[n & 1][tid] = l_run;                            // item n - 2 has left: its rows made way for PV of item n - 1
-            sh->row_ref[n & 1][tid] = ref;
+            sh->row_sum[n % kSumRing][tid] = l_run;                     // item n - 4 has left: its rows made way for the PV of item n - 2
+            sh->row_ref[n % kSumRing][tid] = ref;
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sh->sums_full));
+            if (lane == 0) mbar_arrive(smem_u32(&sh->sums_full[n % kSumRing]));
         }
     } else {
         // -------------------------------------------------------------- epilogue, one row per thread
@@ -466,13 +482,13 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
             const int row = it.r0 + min(r, it.rows_here - 1), token = row / group;
             const int at = token * p.a.n_q_heads + it.kvh * group + row - token * group;   // the row among the document's
             __nv_bfloat16* out = p.out + (size_t)it.layer * p.a.out_layer_stride + (size_t)it.row_first * p.a.n_q_heads * kD + (lane & 3) * 8;
-            ok = warp_wait(smem_u32(&sh->sums_full), n & 1, abort_flag);
+            ok = warp_wait(smem_u32(&sh->sums_full[n % kSumRing]), (n / kSumRing) & 1, abort_flag);
             if (!ok) break;
-            const float sum = sh->row_sum[n & 1][r], inv = 1.f / sum;
+            const float sum = sh->row_sum[n % kSumRing][r], inv = 1.f / sum;
             if (r < it.rows_here) {
                 if (p.lse)
                     p.lse[((size_t)it.layer * p.a.n_q_heads + it.kvh * group + row - token * group) * p.a.total_tokens + it.row_first + token] =
-                        (sh->row_ref[n & 1][r] + log2f(sum)) * kLn2;
+                        (sh->row_ref[n % kSumRing][r] + log2f(sum)) * kLn2;
                 if (sum != sum) {
                     const int m = atomicAdd(&sh->n_marked, 1);
                     if (m < kMarkedMost) sh->marked[m] = make_int2(it.w, r);
