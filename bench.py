@@ -190,10 +190,11 @@ class GpuWorkload:
 
     def launches_per_step(self):
         cfg = self.cfg
-        # clear status + plan init + per attention call (attention, merge, scores; the query-self block if asked
+        # plan init (behind a clearing kernel for more than one request) + per attention call (attention, merge, scores; the query-self block if asked
         # for) + prune/plan kernels + final re-positioning
         # (on the tensor-core path the block is a key tile of the attention kernel, not a launch)
         per_call = 4 if self.self_kernel else 3
+        first = 1 if cfg.batch == 1 else 2
         prunes = sum(1 for l, _ in cfg.schedule if l <= cfg.n_layers)
         if not self.batch_layers:
             # one call per layer: the stack driver leaves the layers' scores in up to eight workspace
@@ -203,8 +204,8 @@ class GpuWorkload:
                 filled += 1
                 if layer in cuts or filled == slots or layer == cfg.n_layers:
                     groups, filled = groups + 1, 0
-            return 2 + (per_call - 1) * cfg.n_layers + groups + prunes + 1
-        return 2 + per_call * len(self.calls()) + prunes + 1
+            return first + (per_call - 1) * cfg.n_layers + groups + prunes + 1
+        return first + per_call * len(self.calls()) + prunes + 1
 
 
 def time_steps(fn, steps, warmup, world):
