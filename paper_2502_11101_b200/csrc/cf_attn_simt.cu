@@ -268,68 +268,86 @@ combine_kernel(AttnWorkspace ws, int n_requests, long long n_rows_all, long long
     }
 }
 
-constexpr int kScoreThreads = 1024;
+constexpr int kScoreThreads = 256, kScoreCluster = 8;
 
-// Document scores (footnote of Sec. 2.4; Algorithm 2: S <- S + s^l): one block per document sums
-// 2^(tile_lse - row_lse) over the document's tiles and all query rows of every layer of the call,
-// each layer in a fixed order, then adds the layers' scores to S in layer order.  Up to eight
-// layers are reduced side by side by groups of threads.
+// One float to the same place in the shared memory of the cluster's first block.
+__device__ __forceinline__ void store_to_first(float* at, float v) {
+    asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, 0;\nst.shared::cluster.f32 [a], %1;\n}"
+                 ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(at))), "f"(v) : "memory");
+}
+
+// Document scores (footnote of Sec. 2.4; Algorithm 2: S <- S + s^l): 2^(tile_lse - row_lse) summed over a document's tiles
+// and all query rows of a layer in a fixed order, then the layers' scores added to S in layer order.  A cluster per
+// document, a layer per block of it (the n_layers-th one on by the first block again), which hands its sum to the first
+// block through distributed shared memory.  A chain of memory latencies: a thread has a row's denominator and its tiles in
+// flight together, four rows to a load.  Measured against one block of 1024 threads per document: 28
+// calls of one layer each, 50 documents, 12 heads: 660 -> 598 us.
 __global__ void __launch_bounds__(kScoreThreads)
-score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, float* __restrict__ doc_scores,
+score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, int cluster, float* __restrict__ doc_scores,
              float* __restrict__ score_accum) {
     __shared__ float s_red[kScoreThreads / 32];
     __shared__ float s_layer[CF_MAX_LAYERS_PER_CALL];
     chain_next();
+    const int doc = blockIdx.x / cluster, rank = blockIdx.x - doc * cluster;
+    if (cluster > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     chain_wait();
-    const int doc = blockIdx.x;
     const int n_layers = ws.n_layers;
     const int count = pv.doc_tile_count[doc];
-    if (count == 0) {
-        if (doc_scores)
-            for (int l = threadIdx.x; l < n_layers; l += kScoreThreads) doc_scores[(size_t)l * bv.n_docs_total + doc] = 0.f;
-        return;
-    }
+    const size_t tile0 = (size_t)pv.doc_tile_begin[doc];
+    const float before = score_accum && rank == 0 ? score_accum[doc] : 0.f;
     int lo = 0, hi = bv.n_requests;                 // request that owns the document
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (bv.req_doc_begin[mid] <= doc) lo = mid; else hi = mid;
     }
-    int groups = 1;                                 // power of two, at most min(n_layers, 8)
-    while (groups * 2 <= n_layers && groups < 8) groups *= 2;
-    const int gs = kScoreThreads / groups;          // threads per group, a multiple of 128
-    const int g = threadIdx.x / gs, t = threadIdx.x - g * gs;
+    if (cluster > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");    // every block has begun: its memory may be written
+    if (count == 0) {                               // the whole cluster
+        if (doc_scores && rank == 0)
+            for (int l = threadIdx.x; l < n_layers; l += kScoreThreads) doc_scores[(size_t)l * bv.n_docs_total + doc] = 0.f;
+        return;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int warps_per_group = gs >> 5;
-    const int rounds = (n_layers + groups - 1) / groups;
-    const size_t tile0 = (size_t)pv.doc_tile_begin[doc];
-    const int n = count * rows_total;
-    for (int rd = 0; rd < rounds; ++rd) {
-        const int layer = rd * groups + g;
+    for (int layer = rank; layer < n_layers; layer += cluster) {
         float sum = 0.f;
-        if (layer < n_layers) {
-            const float* __restrict__ row_lse2 = ws.row_lse2 + ((size_t)layer * bv.n_requests + lo) * rows_total;
-            const float* __restrict__ tile_lse2 = ws.tile_lse2 + ((size_t)layer * ws.max_tiles + tile0) * rows_total;
+        const float* __restrict__ row_lse2 = ws.row_lse2 + ((size_t)layer * bv.n_requests + lo) * rows_total;
+        const float* __restrict__ tile_lse2 = ws.tile_lse2 + ((size_t)layer * ws.max_tiles + tile0) * rows_total;
+        if ((rows_total & 3) == 0) {                // every tile's rows start at a 16-byte address
+#pragma unroll 2
+            for (int r = threadIdx.x * 4; r < rows_total; r += kScoreThreads * 4) {
+                const float4 row = *reinterpret_cast<const float4*>(row_lse2 + r);
 #pragma unroll 4
-            for (int idx = t; idx < n; idx += gs) sum += exp2f(tile_lse2[idx] - row_lse2[idx % rows_total]);
+                for (int t = 0; t < count; ++t) {
+                    const float4 x = *reinterpret_cast<const float4*>(tile_lse2 + (size_t)t * rows_total + r);
+                    sum += (exp2f(x.x - row.x) + exp2f(x.y - row.y)) + (exp2f(x.z - row.z) + exp2f(x.w - row.w));
+                }
+            }
+        } else {
+#pragma unroll 2
+            for (int r = threadIdx.x; r < rows_total; r += kScoreThreads) {
+                const float row = row_lse2[r];
+#pragma unroll 4
+                for (int t = 0; t < count; ++t) sum += exp2f(tile_lse2[(size_t)t * rows_total + r] - row);
+            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (lane == 0) s_red[warp] = sum;
         __syncthreads();
-        if (t == 0 && layer < n_layers) {
+        if (threadIdx.x == 0) {
             float total = 0.f;
-            for (int k = 0; k < warps_per_group; ++k) total += s_red[g * warps_per_group + k];
-            s_layer[layer] = total / (float)rows_total;
+            for (int k = 0; k < kScoreThreads / 32; ++k) total += s_red[k];
+            total /= (float)rows_total;
+            if (doc_scores) doc_scores[(size_t)layer * bv.n_docs_total + doc] = total;
+            if (rank == 0) s_layer[layer] = total;
+            else store_to_first(&s_layer[layer], total);
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        float acc = score_accum ? score_accum[doc] : 0.f;
-        for (int l = 0; l < n_layers; ++l) {
-            if (doc_scores) doc_scores[(size_t)l * bv.n_docs_total + doc] = s_layer[l];
-            acc += s_layer[l];
-        }
-        if (score_accum) score_accum[doc] = acc;
+    if (cluster > 1) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank == 0 && threadIdx.x == 0 && score_accum) {
+        float acc = before;
+        for (int l = 0; l < n_layers; ++l) acc += s_layer[l];
+        score_accum[doc] = acc;
     }
 }
 
@@ -433,8 +451,11 @@ int launch_combine(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
 int launch_scores(const cf_geom* g, const cf_batch* b, const PlanView& pv, const AttnWorkspace& ws, float* doc_scores,
                   float* score_accum, cudaStream_t stream) {
     if (b->n_docs_total <= 0 || (!doc_scores && !score_accum)) return CF_OK;
-    return launch_chained(score_kernel, dim3((unsigned)b->n_docs_total), kScoreThreads, 0, stream, make_batch_view(b), pv, ws,
-                          g->n_q_heads * b->q_len, doc_scores, score_accum);
+    int cluster = 1;                                // a power of two, at most n_layers and 8, the portable size
+    while (cluster * 2 <= std::min(ws.n_layers, kScoreCluster)) cluster *= 2;
+    const int rows_total = g->n_q_heads * b->q_len;
+    return launch_chained_clusters(score_kernel, dim3((unsigned)(cluster * b->n_docs_total)), kScoreThreads, 0, (unsigned)cluster, stream, make_batch_view(b), pv,
+                          ws, rows_total, cluster, doc_scores, score_accum);
 }
 
 }  // namespace cf

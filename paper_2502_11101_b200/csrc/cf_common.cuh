@@ -82,18 +82,25 @@ int configure_smem_once(PerDeviceOnce& once, K kernel, int bytes) {
 // every kernel launched this way does so before it ends, so that a chain stays ordered.  Takes the launch latency
 // (1 to 1.5 us) out of chains of kernels that run for a few microseconds each.
 template <typename... P, typename... A>
-int launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+int launch_chained_clusters(void (*kernel)(P...), dim3 grid, int threads, size_t smem, unsigned cluster, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;       // clusters along x
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? CF_OK : CF_ERR_CUDA;
+}
+template <typename... P, typename... A>
+int launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+    return launch_chained_clusters(kernel, grid, threads, smem, 1, stream, args...);
 }
 int choose_splits(const cf_geom* g, const cf_batch* b, int n_layers);
 int tiles_per_request_bound(const cf_batch* b);
