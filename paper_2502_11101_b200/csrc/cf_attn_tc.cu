@@ -837,114 +837,152 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
     }
 }
 
-constexpr int kMergeRows = 32;                     // rows of a unit per block: four per warp, eight lanes each
-
-// Units that lie in several shares, four blocks per share: those of the share a unit begins in merge its parts, in the order
-// of the line.  They also see to rows of the share's whole units that left the range of their reference; the last share's
-// blocks to the (empty) results of requests that have nothing to attend.  A chain of two memory latencies: what a block
-// has to know about the unit was left by the CTA that began it, and all parts of a row are loaded together.
-template <int LAYOUT>
-__global__ void __launch_bounds__(256, 3)
+// Units that lie in several shares: the parts of a row are merged in the order of the line by eight lanes, in a block of the
+// share the unit begins in.  The blocks of a share also see to rows of its whole units that left the range of their reference,
+// those of the last share to the (empty) results of requests that have nothing to attend.  A chain of two memory latencies:
+// what a block has to know about the unit was left by the CTA that began it, and four parts of a row are loaded together.
+// ROWS = 32: a block has 32 rows of one share's unit.  ROWS = 8: it has 8 rows of the units of four shares (of which few have
+// one), and the parts of a row are cut into four runs, walked side by side and joined in order through shared memory.
+// Measured (one layer of 25 documents, 12/2 heads, with the attention): 19.5 us with 32 rows, 17.0 us with 8.
+template <int LAYOUT, int ROWS>
+__global__ void __launch_bounds__(256, 2)
 attn_tc_merge_kernel(const __grid_constant__ Params p) {
     CF_PARAMS;
+    constexpr int kRuns = 32 / ROWS, kSlices = kRowTile / ROWS, kRunThreads = 256 / kRuns;
     const int max_shares = p.max_shares;
     __shared__ Requests s_rq;
+    __shared__ float s_run[kRuns > 1 ? kRuns - 1 : 1][19][kRuns > 1 ? kRunThreads : 1];   // m, l, ld and 16 dims per thread
     const int lq = bv.q_len, rows_total = n_q_heads * lq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kBlocks = kRowTile / kMergeRows;
-    const int share = blockIdx.x / kBlocks, block = blockIdx.x - share * kBlocks;
+    const int n_classes = (max_shares + kRuns - 1) / kRuns, share0 = blockIdx.x / kSlices, slice = blockIdx.x - share0 * kSlices;
     chain_next();
     chain_wait();
-    const int4* words = reinterpret_cast<const int4*>(reinterpret_cast<const ShareHead*>(ws.marks) + share);
-    const int4 w0 = words[0], w1 = words[1];
-    const ShareHead head = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-    if (share == max_shares - 1 && p.n_prefix + p.n_self == 0)
-        for (int b = block; b < bv.n_requests; b += kBlocks)
-            if (pv.n_tiles[b] == 0)
-                for (int layer = 0; layer < ws.n_layers; ++layer) {
-                    uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)layer * span.out_stride + (size_t)b * rows_total * kD);
-                    for (int i = threadIdx.x; i < rows_total * (kD / 8); i += 256) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-                    const size_t at = ((size_t)layer * bv.n_requests + b) * rows_total;
-                    for (int i = threadIdx.x; i < rows_total; i += 256) {
-                        ws.row_lse2[at + i] = -INFINITY;
-                        if (lse) lse[at + i] = -INFINITY;
+    // lanes 2 i, 2 i + 1: the head of share share0 + i * n_classes
+    int4 words = make_int4(0, 0, 0, 0);
+    if (lane < 2 * kRuns && share0 + (lane >> 1) * n_classes < max_shares)
+        words = reinterpret_cast<const int4*>(reinterpret_cast<const ShareHead*>(ws.marks) + share0 + (lane >> 1) * n_classes)[lane & 1];
+    auto word = [&](int v, int from) { return __shfl_sync(0xffffffffu, v, from); };
+#pragma unroll 1
+    for (int u = 0; u < kRuns; ++u) {
+        const int share = share0 + u * n_classes;
+        if (share >= max_shares) break;
+        const ShareHead head = {word(words.x, 2 * u), word(words.y, 2 * u), word(words.z, 2 * u), word(words.w, 2 * u),
+                                word(words.x, 2 * u + 1), word(words.y, 2 * u + 1), word(words.z, 2 * u + 1), word(words.w, 2 * u + 1)};
+        if (share == max_shares - 1 && p.n_prefix + p.n_self == 0)
+            for (int b = slice; b < bv.n_requests; b += kSlices)
+                if (pv.n_tiles[b] == 0)
+                    for (int layer = 0; layer < ws.n_layers; ++layer) {
+                        uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)layer * span.out_stride + (size_t)b * rows_total * kD);
+                        for (int i = threadIdx.x; i < rows_total * (kD / 8); i += 256) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+                        const size_t at = ((size_t)layer * bv.n_requests + b) * rows_total;
+                        for (int i = threadIdx.x; i < rows_total; i += 256) {
+                            ws.row_lse2[at + i] = -INFINITY;
+                            if (lse) lse[at + i] = -INFINITY;
+                        }
+                    }
+        if (head.marked) {
+            __syncthreads();
+            if (warp == 0) scan_requests(bv, pv, p.n_prefix + p.n_self, s_rq);
+            __syncthreads();
+            const Line line = make_line(bv, ws, s_rq, n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, max_shares);
+            const int group = n_q_heads / n_kv_heads, end = line.cut(share + 1);
+            for (int y = line.cut(share); y < end;) {
+                const Segment own = segment_at(bv, pv, ws, line, group, y, end);
+                if (own.t_end - own.t_begin == own.n_unit)
+                    for (int r = slice * ROWS + warp; r < min(own.rows_here, (slice + 1) * ROWS); r += 8) {
+                        const int rg = own.kvh * group * lq + own.row0 + r;
+                        const float v = ws.row_lse2[(size_t)own.lb * rows_total + rg];
+                        if (v != v) row_from_scratch<LAYOUT>(p, own.lb, rg, own.n_doc);
+                    }
+                y += own.t_end - own.t_begin;
+            }
+        }
+        const int n_parts = head.n_parts;
+        if (n_parts == 0 || slice * ROWS >= head.rows_here) continue;                       // the whole block
+        const int run = warp / (8 / kRuns), part_end = n_parts * (run + 1) / kRuns;
+        const int r = slice * ROWS + (warp - run * (8 / kRuns)) * 4 + (lane >> 3), e0 = (lane & 7) * 16;   // row of the unit; this lane's dims
+        const bool valid = run == 0 && r < head.rows_here;
+        float acc[16], m = -INFINITY, l = 0.f, ld = 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] = 0.f;
+        // part i: the share's slot for what goes on behind it (i = 0), the others' for what began before them
+        const size_t slot0 = ((size_t)2 * share + 1) * kRowTile + min(r, head.rows_here - 1), slot1 = slot0 + kRowTile;
+        auto slot_of = [&](int i) { return i == 0 ? slot0 : slot1 + (size_t)(i - 1) * 2 * kRowTile; };
+        const __nv_bfloat16* part_o = reinterpret_cast<const __nv_bfloat16*>(ws.part_o) + e0;
+        for (int i0 = n_parts * run / kRuns; i0 < part_end; i0 += 4) {
+            float mp[4], lp[4], dp[4];
+            uint4 o[4][2];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const size_t slot = slot_of(min(i0 + x, part_end - 1));
+                mp[x] = i0 + x < part_end ? ws.part_m[slot] : -INFINITY;
+                lp[x] = ws.part_l[slot];
+                dp[x] = ws.part_ld ? ws.part_ld[slot] : lp[x];
+                o[x][0] = *reinterpret_cast<const uint4*>(part_o + slot * kD);
+                o[x][1] = *reinterpret_cast<const uint4*>(part_o + slot * kD + 8);
+            }
+            const float m_new = fmaxf(fmaxf(m, fmaxf(mp[0], mp[1])), fmaxf(mp[2], mp[3]));
+            const float keep = m > -INFINITY ? exp2f(m - m_new) : 0.f;
+            m = m_new;
+            l *= keep;
+            ld *= keep;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) acc[e] *= keep;
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (mp[x] > -INFINITY) {
+                    const float w = exp2f(mp[x] - m_new);
+                    l = fmaf(lp[x], w, l);
+                    ld = fmaf(dp[x], w, ld);
+                    const uint32_t pairs[8] = {o[x][0].x, o[x][0].y, o[x][0].z, o[x][0].w, o[x][1].x, o[x][1].y, o[x][1].z, o[x][1].w};
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        acc[2 * e] = fmaf(__uint_as_float(pairs[e] << 16), w, acc[2 * e]);
+                        acc[2 * e + 1] = fmaf(__uint_as_float(pairs[e] & 0xffff0000u), w, acc[2 * e + 1]);
                     }
                 }
-    if (head.marked) {
-        if (warp == 0) scan_requests(bv, pv, p.n_prefix + p.n_self, s_rq);
-        __syncthreads();
-        const Line line = make_line(bv, ws, s_rq, n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, max_shares);
-        const int group = n_q_heads / n_kv_heads, end = line.cut(share + 1);
-        for (int y = line.cut(share); y < end;) {
-            const Segment own = segment_at(bv, pv, ws, line, group, y, end);
-            if (own.t_end - own.t_begin == own.n_unit)
-                for (int r = block * kMergeRows + warp; r < min(own.rows_here, (block + 1) * kMergeRows); r += 8) {
-                    const int rg = own.kvh * group * lq + own.row0 + r;
-                    const float v = ws.row_lse2[(size_t)own.lb * rows_total + rg];
-                    if (v != v) row_from_scratch<LAYOUT>(p, own.lb, rg, own.n_doc);
-                }
-            y += own.t_end - own.t_begin;
         }
-    }
-    const int n_parts = head.n_parts;
-    if (n_parts == 0) return;
-    const int r = block * kMergeRows + warp * 4 + (lane >> 3), e0 = (lane & 7) * 16;         // row of the unit; this lane's dims
-    const bool valid = r < head.rows_here;
-    float acc[16], m = -INFINITY, l = 0.f, ld = 0.f;
+        if (kRuns > 1) {
+            __syncthreads();                                        // the unit before has been joined
+            if (run > 0) {
+                float* mine = &s_run[run - 1][0][threadIdx.x % kRunThreads];
+                mine[0] = m;
+                mine[kRunThreads] = l;
+                mine[2 * kRunThreads] = ld;
 #pragma unroll
-    for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-    // part i: the share's slot for what goes on behind it (i = 0), the others' for what began before them
-    const size_t slot0 = ((size_t)2 * share + 1) * kRowTile + min(r, head.rows_here - 1), slot1 = slot0 + kRowTile;
-    auto slot_of = [&](int i) { return i == 0 ? slot0 : slot1 + (size_t)(i - 1) * 2 * kRowTile; };
-    const __nv_bfloat16* part_o = reinterpret_cast<const __nv_bfloat16*>(ws.part_o) + e0;
-    for (int i0 = 0; i0 < n_parts; i0 += 4) {
-        float mp[4], lp[4], dp[4];
-        uint4 o[4][2];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t slot = slot_of(min(i0 + u, n_parts - 1));
-            mp[u] = i0 + u < n_parts ? ws.part_m[slot] : -INFINITY;
-            lp[u] = ws.part_l[slot];
-            dp[u] = ws.part_ld ? ws.part_ld[slot] : lp[u];
-            o[u][0] = *reinterpret_cast<const uint4*>(part_o + slot * kD);
-            o[u][1] = *reinterpret_cast<const uint4*>(part_o + slot * kD + 8);
-        }
-        const float m_new = fmaxf(fmaxf(m, fmaxf(mp[0], mp[1])), fmaxf(mp[2], mp[3]));
-        const float keep = m > -INFINITY ? exp2f(m - m_new) : 0.f;
-        m = m_new;
-        l *= keep;
-        ld *= keep;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) acc[e] *= keep;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (mp[u] > -INFINITY) {
-                const float w = exp2f(mp[u] - m_new);
-                l = fmaf(lp[u], w, l);
-                ld = fmaf(dp[u], w, ld);
-                const uint32_t words[8] = {o[u][0].x, o[u][0].y, o[u][0].z, o[u][0].w, o[u][1].x, o[u][1].y, o[u][1].z, o[u][1].w};
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    acc[2 * e] = fmaf(__uint_as_float(words[e] << 16), w, acc[2 * e]);
-                    acc[2 * e + 1] = fmaf(__uint_as_float(words[e] & 0xffff0000u), w, acc[2 * e + 1]);
-                }
+                for (int e = 0; e < 16; ++e) mine[(3 + e) * kRunThreads] = acc[e];
             }
-    }
-    const int rg = head.row_first + r, h = rg / lq, j = rg - h * lq;
-    if (valid && l == l) {
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-        uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)head.layer * span.out_stride + (((size_t)head.b * lq + j) * n_q_heads + h) * kD + e0);
+            __syncthreads();
+            if (run > 0) continue;
 #pragma unroll
-        for (int e = 0; e < 2; ++e)
-            dst[e] = make_uint4(pack_bf16(acc[8 * e] * inv, acc[8 * e + 1] * inv), pack_bf16(acc[8 * e + 2] * inv, acc[8 * e + 3] * inv),
-                                pack_bf16(acc[8 * e + 4] * inv, acc[8 * e + 5] * inv), pack_bf16(acc[8 * e + 6] * inv, acc[8 * e + 7] * inv));
-        if ((lane & 7) == 0) {
-            ws.row_lse2[(size_t)head.lb * rows_total + rg] = ld > 0.f ? m + log2f(ld) : -INFINITY;
-            if (lse) lse[(size_t)head.lb * rows_total + rg] = (l > 0.f ? m + log2f(l) : -INFINITY) * kLn2;
+            for (int k = 0; k < kRuns - 1; ++k) {
+                const float* other = &s_run[k][0][threadIdx.x];
+                const float mo = other[0];
+                if (mo == -INFINITY) continue;
+                const float m_new = fmaxf(m, mo), keep = m > -INFINITY ? exp2f(m - m_new) : 0.f, w = exp2f(mo - m_new);
+                m = m_new;
+                l = fmaf(other[kRunThreads], w, l * keep);
+                ld = fmaf(other[2 * kRunThreads], w, ld * keep);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) acc[e] = fmaf(other[(3 + e) * kRunThreads], w, acc[e] * keep);
+            }
         }
+        const int rg = head.row_first + r, h = rg / lq, j = rg - h * lq;
+        if (valid && l == l) {
+            const float inv = l > 0.f ? 1.f / l : 0.f;
+            uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)head.layer * span.out_stride + (((size_t)head.b * lq + j) * n_q_heads + h) * kD + e0);
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                dst[e] = make_uint4(pack_bf16(acc[8 * e] * inv, acc[8 * e + 1] * inv), pack_bf16(acc[8 * e + 2] * inv, acc[8 * e + 3] * inv),
+                                    pack_bf16(acc[8 * e + 4] * inv, acc[8 * e + 5] * inv), pack_bf16(acc[8 * e + 6] * inv, acc[8 * e + 7] * inv));
+            if ((lane & 7) == 0) {
+                ws.row_lse2[(size_t)head.lb * rows_total + rg] = ld > 0.f ? m + log2f(ld) : -INFINITY;
+                if (lse) lse[(size_t)head.lb * rows_total + rg] = (l > 0.f ? m + log2f(l) : -INFINITY) * kLn2;
+            }
+        }
+        // marked: out of the range of its reference
+        for (unsigned todo = __ballot_sync(0xffffffffu, valid && l != l && (lane & 7) == 0); todo; todo &= todo - 1)
+            row_from_scratch<LAYOUT>(p, head.lb, __shfl_sync(0xffffffffu, rg, __ffs(todo) - 1), head.n_doc);
     }
-    // marked: out of the range of its reference
-    for (unsigned todo = __ballot_sync(0xffffffffu, valid && l != l && (lane & 7) == 0); todo; todo &= todo - 1)
-        row_from_scratch<LAYOUT>(p, head.lb, __shfl_sync(0xffffffffu, rg, __ffs(todo) - 1), head.n_doc);
 }
 
 // Exercises the bounded wait by itself: one CTA initialises an mbarrier that nothing ever arrives on,
@@ -1028,13 +1066,18 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
     const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
                       k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, static_cast<__nv_bfloat16*>(out), lse};
     static PerDeviceOnce configured[2];
+    // Few units in many shares each.  Measured (attention and merge of a call, us, 32 rows against 8): 6 units of 25 parts 19.5
+    // against 17.0; 24 units of 6 parts 33.0 against 36.2; 32 units of 5 parts 33.1 against 36.6.
+    const bool many_parts = (long long)span.n_layers * b->n_requests * g->n_kv_heads * row_tiles * 8 <= shares;
+    const int merge_rows = many_parts ? 8 : 32;
     auto run = [&](auto kernel, auto merge, int which) {
         if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return (int)CF_ERR_CUDA;
         const int rc = launch_chained(kernel, dim3((unsigned)shares), kThreads, kSmemBytes, stream, maps, p);
-        return rc != CF_OK ? rc : launch_chained(merge, dim3((unsigned)(shares * (kRowTile / kMergeRows))), 256, 0, stream, p);
+        return rc != CF_OK ? rc : launch_chained(merge, dim3((unsigned)((shares + 32 / merge_rows - 1) / (32 / merge_rows) * (kRowTile / merge_rows))), 256, 0, stream, p);
     };
-    if (g->rope_layout == CF_ROPE_HALF) return run(attn_tc_kernel<CF_ROPE_HALF>, attn_tc_merge_kernel<CF_ROPE_HALF>, 0);
-    return run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, attn_tc_merge_kernel<CF_ROPE_INTERLEAVED>, 1);
+    constexpr int H = CF_ROPE_HALF, I = CF_ROPE_INTERLEAVED;
+    if (g->rope_layout == H) return run(attn_tc_kernel<H>, many_parts ? attn_tc_merge_kernel<H, 8> : attn_tc_merge_kernel<H, 32>, 0);
+    return run(attn_tc_kernel<I>, many_parts ? attn_tc_merge_kernel<I, 8> : attn_tc_merge_kernel<I, 32>, 1);
 }
 
 }  // namespace cf

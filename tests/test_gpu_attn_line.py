@@ -89,3 +89,42 @@ def test_rows_far_outside_the_range_of_their_reference(heads, docs):
     was cut between shares or finished by one."""
     out, lse, _ = _both_paths(heads, 20, [150] * 9, docs, peak=[149 + 150 * 1, 149 + 150 * 4, 149 + 150 * 7])
     assert float(lse.max()) > 60.0
+
+
+@pytest.mark.parametrize("docs,q_len", [(37, 3), (14, 128)])
+def test_few_units_in_many_shares(docs, q_len):
+    """Two to six units whose rows have many parts each, merged in runs; the last slice of rows is not whole."""
+    _both_paths((6, 2), q_len, [200 - 3 * i for i in range(docs)], [docs])
+
+
+@pytest.mark.parametrize("heads,q_len", [((3, 1), 1), ((5, 5), 3), ((4, 2), 7), ((12, 2), 48)])
+@pytest.mark.parametrize("layers", [1, 2, 3, 9, 17])
+def test_scores_do_not_depend_on_the_layers_beside_them(heads, q_len, layers):
+    """The same layer several times in one call (clusters of one to eight blocks, layers beyond them, rows that are no multiple
+    of four): every layer's scores are those of a call with one, they sum to 1 per request, and S takes them in order."""
+    import paper_2502_11101_b200 as cf
+    from paper_2502_11101_b200.session import Session
+    hq, hkv = heads
+    lens, begin = [97, 1, 40, 200, 13], np.asarray([0, 3, 5], np.int32)
+    gen = torch.Generator(device="cuda").manual_seed(layers)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rand(1, 2, q_len, hq, 128), rand(1, sum(lens), hkv, 128), rand(1, sum(lens), hkv, 128)
+    got = []
+    for n in (1, layers):
+        sess = Session(hq, hkv, 128, torch.bfloat16, 32768, 1e6, q_len, np.asarray(lens, np.int32), begin,
+                       np.zeros(len(lens), np.int32), tail_reserve=q_len)
+        sess.init(kept_count=torch.tensor([2, 2], dtype=torch.int32, device="cuda"))
+        scores = torch.full((n, len(lens)), float("nan"), device="cuda")
+        qn, kn, vn = (x.expand(n, *x.shape[1:]).contiguous() for x in (q, k, v))
+        sess.attend_layers(qn, kn, vn, torch.empty_like(qn), layer_scores=scores)
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        got.append((scores.cpu(), sess.score_accum.cpu()))
+    (one, _), (scores, accum) = got
+    torch.testing.assert_close(scores, one.expand_as(scores), rtol=1e-3, atol=1e-6)
+    torch.testing.assert_close(scores[:, :3].sum(1), torch.ones(layers), rtol=1e-3, atol=0)
+    torch.testing.assert_close(scores[:, 3:].sum(1), torch.ones(layers), rtol=1e-3, atol=0)
+    total = torch.zeros_like(accum)
+    for s in scores:
+        total += s
+    assert torch.equal(accum[[0, 1, 3, 4]], total[[0, 1, 3, 4]]) and float(scores[:, 2].abs().max()) == 0.0
