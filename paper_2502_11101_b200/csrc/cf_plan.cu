@@ -81,8 +81,9 @@ __device__ __forceinline__ void sincos_turns(int delta, unsigned long long turns
     cs = ((q + 1) & 2) ? -c1 : c1;
 }
 
-// Exclusive prefix sum of one value per thread over the block; *total receives the sum.  Every
-// thread of the block must call it.
+// Exclusive prefix sum of one value per thread over the block; *total receives the sum.  Every thread of the block must call
+// it, with a buffer that nothing else uses until the kernel ends: one barrier instead of three, every warp scans the (at most
+// 32) warp sums by itself.
 __device__ __forceinline__ int block_scan(int value, int* s_warp_sum, int* total) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int incl = value;
@@ -93,22 +94,9 @@ __device__ __forceinline__ int block_scan(int value, int* s_warp_sum, int* total
     }
     if (lane == 31) s_warp_sum[warp] = incl;
     __syncthreads();
-    if (warp == 0) {                                     // scan of the (at most 32) warp sums
-        const int mine = lane < (int)(blockDim.x >> 5) ? s_warp_sum[lane] : 0;
-        int acc = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int up = __shfl_up_sync(0xffffffffu, acc, o);
-            if (lane >= o) acc += up;
-        }
-        s_warp_sum[lane] = acc - mine;                   // sum of the warps before this one
-        if (lane == 31) s_warp_sum[32] = acc;
-    }
-    __syncthreads();
-    const int before = s_warp_sum[warp] + incl - value;
-    *total = s_warp_sum[32];
-    __syncthreads();
-    return before;
+    const int sum = lane < (int)(blockDim.x >> 5) ? s_warp_sum[lane] : 0;
+    *total = __reduce_add_sync(0xffffffffu, sum);
+    return __reduce_add_sync(0xffffffffu, lane < warp ? sum : 0) + incl - value;
 }
 
 // mode 0: initialise from (order, kept_count); mode 1: prune by score, then rebuild.
@@ -129,16 +117,22 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
     __shared__ int s_first[kMaxDocs];      // first tile by local id
     __shared__ int s_cnt[kMaxDocs];       // tile count by local id
     __shared__ int s_src[kMaxDocs];       // positions the documents were cached at, by local id
-    __shared__ float s_score[kMaxDocs];
+    __shared__ int2 s_score[kMaxDocs];    // score (its bits) and local id by rank; later first tile and tiles by rank
     __shared__ float s_all[kMaxDocs];     // accumulated scores of all documents of the request, by local id
-    __shared__ unsigned char s_flag[kMaxDocs];
+    __shared__ unsigned char s_flag[kMaxDocs], s_survives[kMaxDocs];
     __shared__ int s_longest, s_min_cursor;
-    __shared__ int s_warp_sum[kPlanThreads / 32 + 1];
+    __shared__ int s_warp_sum[3][kPlanThreads / 32];
 
     chain_next();
-    chain_wait();
     const int b = blockIdx.x;
     const int tid = threadIdx.x;
+    const int half = gv.head_dim / 2;
+    const int half_log2 = half == 64 ? 6 : 5;
+    // this thread's rotary frequency (a constant-bank load that differs between the lanes is served one lane at a time: here it
+    // passes under the predecessor)
+    const unsigned long long turns = inv_freq.turns[tid & (half - 1)];
+    const double freq = inv_freq.f[tid & (half - 1)];
+    chain_wait();
     // a batch of one request starts with clear status words and, if asked for, S = 0 (larger ones: clear_kernel)
     if (mode == 0 && gridDim.x == 1) {
         if (tid == 0) pv.status[0] = pv.status[1] = pv.status[2] = pv.status[3] = 0;
@@ -148,6 +142,12 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
     const int nthreads = (int)blockDim.x;               // at least the documents of any request, a multiple of 32
     const int doc0 = bv.req_doc_begin[b];
     const int n_docs = bv.req_doc_begin[b + 1] - doc0;
+    const int kept_count_old = mode == 0 ? 0 : pv.kept_count[b];
+    const int kept_in = mode == 0 && kept_count_in ? kept_count_in[b] : n_docs;
+    const int keep_arg = (mode != 0 && keep_per_request) ? keep_per_request[b] : keep;
+    int query_start = mode == 0 ? (query_start_arg < 0 ? gv.pos_range - bv.tail_reserve : query_start_arg)
+                                : pv.query_start[b];
+    int windows = mode == 0 ? max(1, bv.n_reuse) : pv.n_reuse[b];
     if (n_docs > kMaxDocs || n_docs < 0) {
         if (tid == 0) {
             raise_status(pv.status, CF_ERR_INVALID_ARG);
@@ -157,37 +157,38 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
         }
         return;
     }
-    const int half = gv.head_dim / 2;
-    const int half_log2 = half == 64 ? 6 : 5;
 
-    // ---- stage the inputs (everything here depends on doc0 alone: one round trip to global memory) ----
+    // ---- stage the inputs (everything here depends on doc0 alone: one round trip to global memory, every load issued before
+    // the first result is put down) ----
     int n_old = 0, keep_b = 0, n_kept = 0;
-    const int kept_count_old = mode == 0 ? 0 : pv.kept_count[b];
-    const int keep_arg = (mode != 0 && keep_per_request) ? keep_per_request[b] : keep;
-    const int kept_raw = (mode != 0 && tid < n_docs) ? pv.kept[doc0 + tid] : 0;    // rank tid, if there is one
-    if (mode != 0 && tid < n_docs) s_all[tid] = score_accum[doc0 + tid];            // S of every document, by local id
-    for (int i = tid; i <= n_docs; i += nthreads) s_row[i] = bv.doc_offsets[doc0 + i];
-    for (int i = tid; i < n_docs; i += nthreads) {
-        s_src[i] = bv.doc_src_start[doc0 + i];
-        s_dst[i] = mode == 0 ? -1 : pv.dst_start[doc0 + i];
-        s_group[i] = mode == 0 ? -1 : pv.group[doc0 + i];
+    const bool own = tid < n_docs, again = own && mode != 0;                       // a document, a rank of its own
+    const int kept_raw = again ? pv.kept[doc0 + tid] : 0;
+    const float score_raw = again ? score_accum[doc0 + tid] : 0.f;                 // S of every document, by local id
+    const int dst_raw = again ? pv.dst_start[doc0 + tid] : -1, group_raw = again ? pv.group[doc0 + tid] : -1;
+    const int order_raw = own && mode == 0 && order ? order[doc0 + tid] : tid;
+    const int row_raw = tid <= n_docs ? bv.doc_offsets[doc0 + tid] : 0;
+    const int src_raw = own ? bv.doc_src_start[doc0 + tid] : 0;
+    if (tid == 0 && n_docs == nthreads) s_row[n_docs] = bv.doc_offsets[doc0 + n_docs];
+    if (tid <= n_docs) s_row[tid] = row_raw;
+    if (own) {
+        s_all[tid] = score_raw;
+        s_src[tid] = src_raw;
+        s_dst[tid] = dst_raw;
+        s_group[tid] = group_raw;
+        s_flag[tid] = 0;
     }
-    int query_start = mode == 0 ? (query_start_arg < 0 ? gv.pos_range - bv.tail_reserve : query_start_arg)
-                                : pv.query_start[b];
-    int windows = mode == 0 ? max(1, bv.n_reuse) : pv.n_reuse[b];
     if (mode == 0) {
-        n_kept = kept_count_in ? kept_count_in[b] : n_docs;
-        n_kept = max(0, min(n_kept, n_docs));
-        for (int i = tid; i < n_docs; i += nthreads) s_cnt[i] = 0;
+        n_kept = max(0, min(kept_in, n_docs));
+        if (own) s_cnt[tid] = 0;
         __syncthreads();
-        for (int r = tid; r < n_kept; r += nthreads) {
-            int id = order ? order[doc0 + r] : r;
+        if (tid < n_kept) {
+            int id = order_raw;
             if (id < 0 || id >= n_docs) {
                 raise_status(pv.status, CF_ERR_INVALID_ARG);
                 id = 0;
             }
             if (atomicAdd(&s_cnt[id], 1) != 0) raise_status(pv.status, CF_ERR_INVALID_ARG);   // an id listed twice
-            s_ids[r] = id;
+            s_ids[tid] = id;
         }
     } else {
         n_old = max(0, min(kept_count_old, n_docs));
@@ -202,55 +203,59 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
 
     // ---- the kept list, in rank order -------------------------------------------------------
     if (mode != 0) {
-        if (tid < n_old) s_score[tid] = s_all[s_ids[tid]];
+        if (tid < n_old) s_score[tid] = make_int2(__float_as_int(s_all[s_ids[tid]]), s_ids[tid]);
         __syncthreads();
         // rank by counting: how many kept documents beat this one (ties: lower id wins); eight
         // lanes share the count of one document
         for (int r0 = 0; r0 < n_old; r0 += nthreads / 8) {
             const int r = r0 + (tid >> 3);
-            const float sc = r < n_old ? s_score[r] : 0.f;
-            const int id = r < n_old ? s_ids[r] : 0;
+            const int2 me = r < n_old ? s_score[r] : make_int2(0, 0);
+            const float sc = __int_as_float(me.x);
+            const int id = me.y;
             int better = 0;
             if (r < n_old)
+#pragma unroll 8
                 for (int o = tid & 7; o < n_old; o += 8) {
-                    const float so = s_score[o];
-                    better += (so > sc) || (so == sc && s_ids[o] < id);
+                    const int2 other = s_score[o];
+                    const float so = __int_as_float(other.x);
+                    better += (so > sc) || (so == sc && other.y < id);
                 }
             better += __shfl_xor_sync(0xffffffffu, better, 1);
             better += __shfl_xor_sync(0xffffffffu, better, 2);
             better += __shfl_xor_sync(0xffffffffu, better, 4);
             if (r < n_old && (tid & 7) == 0) {
-                s_flag[r] = better < keep_b;
+                s_survives[r] = better < keep_b;
                 if (strategy == CF_ALLOC_SORT && better < keep_b) s_tmp[better] = id;
             }
         }
         __syncthreads();
         if (strategy != CF_ALLOC_SORT) {                  // survivors keep their order: slot = survivors before
-            const int survives = tid < n_old ? (int)s_flag[tid] : 0;
+            const int survives = tid < n_old ? (int)s_survives[tid] : 0;
             int n_survive;
-            const int before = block_scan(survives, s_warp_sum, &n_survive);
+            const int before = block_scan(survives, s_warp_sum[0], &n_survive);
             if (survives) s_tmp[before] = s_ids[tid];
+            __syncthreads();
         }
-        __syncthreads();
         n_kept = keep_b;
         // (the clamp only matters for malformed input -- duplicate ids, NaN scores -- where two
         //  documents can claim one slot and leave another unwritten)
-        for (int r = tid; r < n_kept; r += nthreads) s_ids[r] = max(0, min(s_tmp[r], n_docs - 1));
-        __syncthreads();
+        if (tid < n_kept) {
+            const int id = max(0, min(s_tmp[tid], n_docs - 1));
+            s_ids[tid] = id;
+            s_flag[id] = 1;
+        }
+    } else {
+        if (tid < n_kept) s_flag[s_ids[tid]] = 1;
     }
 
-    // ---- documents that are not kept ----------------------------------------------------------
     const bool reallocate = (mode == 0) || (strategy != CF_ALLOC_NONE);
-    for (int i = tid; i < n_docs; i += nthreads) s_flag[i] = 0;
-    __syncthreads();
-    for (int r = tid; r < n_kept; r += nthreads) s_flag[s_ids[r]] = 1;
     __syncthreads();
 
     // ---- positional allocation ----------------------------------------------------------------
     if (reallocate && n_kept > 0) {
-        int longest = 0;
-        for (int r = tid; r < n_kept; r += nthreads) longest = max(longest, s_row[s_ids[r] + 1] - s_row[s_ids[r]]);
-        atomicMax(&s_longest, longest);
+        int longest = tid < n_kept ? s_row[s_ids[tid] + 1] - s_row[s_ids[tid]] : 0;
+        longest = __reduce_max_sync(0xffffffffu, longest);
+        if ((tid & 31) == 0 && tid < n_kept) atomicMax(&s_longest, longest);
         __syncthreads();
         longest = s_longest;
         const int capacity = gv.pos_range - bv.prefix_len - bv.tail_reserve;
@@ -287,7 +292,7 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
             len = s_row[id + 1] - s_row[id];
         }
         int all_rows;
-        const int before = block_scan(len, s_warp_sum, &all_rows);
+        const int before = block_scan(len, s_warp_sum[1], &all_rows);
         if (rank >= 0) s_tmp[x] = before;
         __syncthreads();
         int lowest = 0x7fffffff;
@@ -298,7 +303,8 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
             s_group[id] = rank % windows;
             lowest = start;
         }
-        atomicMin(&s_min_cursor, lowest);
+        lowest = __reduce_min_sync(0xffffffffu, lowest);
+        if ((tid & 31) == 0 && lowest != 0x7fffffff) atomicMin(&s_min_cursor, lowest);
         __syncthreads();
         if (tid == 0 && (s_min_cursor < bv.prefix_len || query_start + bv.tail_reserve > gv.pos_range))
             raise_status(pv.status, CF_ERR_RANGE);
@@ -307,7 +313,7 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
     // ---- key tiles: runs of at most kTile rows that never straddle two documents -----------------
     const int my_tiles = tid < n_kept ? (s_row[s_ids[tid] + 1] - s_row[s_ids[tid]] + kTile - 1) / kTile : 0;
     int total;
-    const int first_tile = block_scan(my_tiles, s_warp_sum, &total);
+    const int first_tile = block_scan(my_tiles, s_warp_sum[2], &total);
     const int base = tile_base(doc0, s_row[0]);
     const bool fail = base + total > pv.max_tiles;       // cannot happen with a plan sized by cf_plan_layout_of
 
@@ -324,12 +330,8 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
     // every array is written with consecutive threads on consecutive elements: per-document fields
     // by document, the kept list by rank, the tile list by tile
     if (tid < n_kept) {
-        s_tmp[tid] = first_tile;                             // first tile of rank tid (ascending)
-        s_score[tid] = __int_as_float(my_tiles);
-    }
-    __syncthreads();
-    if (tid < n_kept) {                                      // per-document view of the same numbers
-        const int id = s_ids[tid];
+        const int id = s_ids[tid];                           // per-document view of the same numbers
+        s_score[tid] = make_int2(first_tile, my_tiles);      // first tile of rank tid (ascending)
         s_first[id] = first_tile;
         s_cnt[id] = my_tiles;
     }
@@ -346,13 +348,13 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
         int lo = 0, hi = n_kept;                             // last rank whose first tile is <= x
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (s_tmp[mid] <= x) lo = mid; else hi = mid;
+            if (s_score[mid].x <= x) lo = mid; else hi = mid;
         }
         const int id = s_ids[lo];
         const int row0 = s_row[id];
         const int len = s_row[id + 1] - row0;
-        const int count = __float_as_int(s_score[lo]);
-        const int t = x - s_tmp[lo];
+        const int count = s_score[lo].y;
+        const int t = x - s_score[lo].x;
         // the document's rows are spread evenly over its tiles, in steps of 16 (160 rows make
         // tiles of 80 and 80, not 96 and 64), so consecutive tiles cost about the same
         const int step = min(kTile, ((len + count - 1) / count + 15) & ~15);
@@ -362,11 +364,9 @@ plan_kernel(GeomView gv, BatchView bv, PlanView pv, InvFreq inv_freq, int mode, 
     }
 
     // ---- rotation tables: cos, sin of (dst - src) * theta^(-2p/D) -------------------------------
-    // thread = (slice p, every (nthreads / half)-th rank): the frequency is read once per thread
+    // thread = (slice p, every (nthreads / half)-th rank)
     {
         const int p = tid & (half - 1);
-        const unsigned long long turns = inv_freq.turns[p];
-        const double freq = inv_freq.f[p];
         for (int r = tid >> half_log2; r < n_kept; r += nthreads >> half_log2) {
             const int id = s_ids[r];
             const int delta = s_dst[id] - s_src[id];
