@@ -278,10 +278,10 @@ __device__ __forceinline__ void store_to_first(float* at, float v) {
 
 // Document scores (footnote of Sec. 2.4; Algorithm 2: S <- S + s^l): 2^(tile_lse - row_lse) summed over a document's tiles
 // and all query rows of a layer in a fixed order, then the layers' scores added to S in layer order.  A cluster per
-// document, a layer per block of it (the n_layers-th one on by the first block again), which hands its sum to the first
-// block through distributed shared memory.  A chain of memory latencies: a thread has a row's denominator and its tiles in
-// flight together, four rows to a load.  Measured against one block of 1024 threads per document: 28
-// calls of one layer each, 50 documents, 12 heads: 660 -> 598 us.
+// document, a layer per block of it (several from the ninth on), which hands its sum to the first block through distributed
+// shared memory.  A chain of memory latencies: a thread has a row's denominator and its tiles in flight together, four rows
+// to a load.  Measured against one block of 1024 threads per document: 28 calls of one layer each, 50 documents, 12 heads,
+// 660 -> 598 us a pass.
 __global__ void __launch_bounds__(kScoreThreads)
 score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, int cluster, float* __restrict__ doc_scores,
              float* __restrict__ score_accum) {
@@ -295,10 +295,12 @@ score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, int cl
     const int count = pv.doc_tile_count[doc];
     const size_t tile0 = (size_t)pv.doc_tile_begin[doc];
     const float before = score_accum && rank == 0 ? score_accum[doc] : 0.f;
-    int lo = 0, hi = bv.n_requests;                 // request that owns the document
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (bv.req_doc_begin[mid] <= doc) lo = mid; else hi = mid;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int lo = 0;                                     // request that owns the document: those that begin at or before it, less one
+    for (int b0 = 1; b0 < bv.n_requests; b0 += 32) {
+        const int n = __popc(__ballot_sync(0xffffffffu, b0 + lane < bv.n_requests && bv.req_doc_begin[min(b0 + lane, bv.n_requests)] <= doc));
+        lo += n;
+        if (n < 32) break;
     }
     if (cluster > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");    // every block has begun: its memory may be written
     if (count == 0) {                               // the whole cluster
@@ -306,7 +308,6 @@ score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, int cl
             for (int l = threadIdx.x; l < n_layers; l += kScoreThreads) doc_scores[(size_t)l * bv.n_docs_total + doc] = 0.f;
         return;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int layer = rank; layer < n_layers; layer += cluster) {
         float sum = 0.f;
         const float* __restrict__ row_lse2 = ws.row_lse2 + ((size_t)layer * bv.n_requests + lo) * rows_total;
@@ -451,8 +452,8 @@ int launch_combine(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
 int launch_scores(const cf_geom* g, const cf_batch* b, const PlanView& pv, const AttnWorkspace& ws, float* doc_scores,
                   float* score_accum, cudaStream_t stream) {
     if (b->n_docs_total <= 0 || (!doc_scores && !score_accum)) return CF_OK;
-    int cluster = 1;                                // a power of two, at most n_layers and 8, the portable size
-    while (cluster * 2 <= std::min(ws.n_layers, kScoreCluster)) cluster *= 2;
+    const int rounds = (ws.n_layers + kScoreCluster - 1) / kScoreCluster;   // layers per block, evenly; 8 is the portable cluster size
+    const int cluster = (ws.n_layers + rounds - 1) / rounds;
     const int rows_total = g->n_q_heads * b->q_len;
     return launch_chained_clusters(score_kernel, dim3((unsigned)(cluster * b->n_docs_total)), kScoreThreads, 0, (unsigned)cluster, stream, make_batch_view(b), pv,
                           ws, rows_total, cluster, doc_scores, score_accum);

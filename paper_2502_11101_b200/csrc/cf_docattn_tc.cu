@@ -21,8 +21,8 @@
 // noted and computed again, alone, when the CTA's items are done.
 // Bound by HBM for a few query heads per kv head: with 6 heads and a 64-token prefix 123 flops per byte.
 // Measured (400 documents of 128-192 tokens, 12/2 heads, 4 layers, prefix 64): 660 us before
-// (one issuing thread for copies and MMAs, two passes over S, rows staged through the value buffer), 514 us now; one layer
-// of 60 ragged documents with 32 heads and a 41-token prefix 229 -> 153 us.
+// (one issuing thread for copies and MMAs, two passes over S, rows staged through the value buffer), 449 us now; one layer
+// of 60 ragged documents with 32 heads and a 41-token prefix 229 -> 100 us.
 // Every mbarrier wait is bounded; on expiry the CTA reports CF_ERR_TIMEOUT in the status word.
 #include <math_constants.h>
 
