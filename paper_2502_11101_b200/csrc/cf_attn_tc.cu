@@ -112,6 +112,8 @@ struct Segment {
     int t_begin, t_end, n_unit, n_doc, tile0;      // tiles of the unit this segment covers; documents' tiles; first in the plan
 };
 
+// A share has at least two tiles: at one layer per call, 28 calls of a small request take 582 us a pass with 1 or 2, 611 / 635 /
+// 676 / 753 with 3 / 4 / 6 / 8 (a longer share costs more than the parts it saves); larger calls do not notice.
 constexpr int kMinShare = 2;
 
 // What the line is made from: prefix sums of the requests' tiles (one entry per `stride` requests), and with one entry per
