@@ -281,7 +281,7 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
     const float scale = softmax_scale == 0.0f ? 1.0f / std::sqrt((float)geom->head_dim) : softmax_scale;
     PlanView pv = make_plan_view(geom, batch, const_cast<void*>(plan));
     if (decode_cache_rows > 0 && g_attn_path.load() == 0 && decode_attn_supported(geom)) {
-        if (workspace_bytes < decode_attn_workspace_bytes(geom)) return CF_ERR_WORKSPACE;
+        if (workspace_bytes < decode_attn_workspace_bytes(geom, batch->n_requests, span.n_layers)) return CF_ERR_WORKSPACE;
         return launch_decode_attn(geom, batch->n_requests, decode_cache_rows, span.n_layers, batch->doc_offsets, span, q, k_cache,
                                   v_cache, scale * kLog2e, out, lse, workspace, s);
     }

@@ -77,10 +77,12 @@ int configure_smem_once(PerDeviceOnce& once, K kernel, int bytes) {
     if (dev >= 0) once.done[dev] = true;
     return CF_OK;
 }
-// Launches a kernel that may be scheduled while its predecessor in the stream still runs (programmatic stream
-// serialisation): it must execute chain_wait() before it touches memory the predecessor wrote or reads, and
-// every kernel launched this way does so before it ends, so that a chain stays ordered.  Takes the launch latency
-// (1 to 1.5 us) out of chains of kernels that run for a few microseconds each.
+// Launches a kernel that may be scheduled while earlier kernels of the stream still run (programmatic stream
+// serialisation).  Kernels call chain_next() before their own chain_wait(), so a kernel may be resident while any number of
+// its predecessors are running or waiting themselves: until chain_wait() it touches no global memory at all, whoever wrote
+// it (its own parameters and shared memory are all it may use), and every kernel launched this way executes chain_wait()
+// before it ends, so that a chain stays ordered.  Takes the launch latency (1 to 1.5 us) out of chains of kernels that run
+// for a few microseconds each.
 template <typename... P, typename... A>
 int launch_chained_clusters(void (*kernel)(P...), dim3 grid, int threads, size_t smem, unsigned cluster, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg = {};
@@ -164,7 +166,7 @@ size_t attn_tc_part_rows();
 bool attn_tc_supported(const cf_geom* g, const cf_batch* b);
 // One query row per head over the final caches of a decoding step (doc_offsets: of the decode plan).
 bool decode_attn_supported(const cf_geom* g);
-size_t decode_attn_workspace_bytes(const cf_geom* g);
+size_t decode_attn_workspace_bytes(const cf_geom* g, int n_requests, int n_layers);
 int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_layers, const int* doc_offsets, const LayerSpan& span,
                        const void* q, const void* k, const void* v, float scale_log2, void* out, float* lse,
                        void* workspace, cudaStream_t stream);
@@ -201,7 +203,7 @@ int launch_docattn_tc(const cf_geom* g, const DocAttnArgs& a, const void* q, con
 int attn_path();
 
 // ---- device helpers -----------------------------------------------------------------------
-// The predecessor in the stream is complete and its writes are visible (returns at once for an ordinary launch).
+// Every earlier kernel of the stream is complete and its writes are visible (returns at once for an ordinary launch).
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The successor in the stream may be scheduled on what this grid leaves free.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

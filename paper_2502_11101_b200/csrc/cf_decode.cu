@@ -199,7 +199,7 @@ size_t cf_decode_workspace_bytes(const cf_geom* geom, int32_t n_requests, int32_
     decode_views(geom, n_requests, cache_rows, a, &g, &b);
     b.req_doc_begin = b.doc_offsets = b.doc_src_start = reinterpret_cast<const int32_t*>(geom);
     const size_t general = cf_attn_workspace_bytes_layers(&g, &b, n_layers);
-    return general == 0 || !decode_attn_supported(geom) ? general : general + decode_attn_workspace_bytes(geom);
+    return general == 0 || !decode_attn_supported(geom) ? general : general + decode_attn_workspace_bytes(geom, n_requests, n_layers);
 }
 
 int cf_decode_attn(const cf_geom* geom, int32_t n_requests, int32_t cache_rows, const void* decode_plan,

@@ -42,6 +42,7 @@ struct DecodeArgs {
     int n_requests, cache_rows, n_q_heads, n_kv_heads, row_tiles;
     float scale_log2;
     float *part_o, *part_m, *part_l;               // parts of units that lie in several shares of the line
+    int2* unit_parts;                              // [units] first share of a unit and the parts it was cut into (0: not cut)
 };
 
 __device__ __forceinline__ uint4 load_row(const __nv_bfloat16* p) {
@@ -91,16 +92,20 @@ __device__ __forceinline__ float2 peer_float2(uint32_t addr, uint32_t rank) {
 // A run of 16-key steps of one unit (layer, request, kv head, tile of query heads).
 struct Segment {
     int lb, head0, n_heads, kvh, used, s_begin, s_end, steps;
+    int unit;                                      // its number: (layer * B + request) * tiles + kv head and tile
 };
 
-// Where the steps of all units lie on one line (order: layer, request, kv head and tile, step), for the kernel that cuts
-// the line into equal shares and for the one that merges the shares of a unit.
+// Where the steps of all units lie on one line (order: layer, request, kv head and tile, step), which is cut into equal shares.
 struct Line {
     const int* pref;                               // [n_requests + 1] prefix sums of the requests' steps
     int n_requests, tiles;                         // tiles = kv heads * tiles of query heads
     int per_layer;
     int n_shares, each, rest;                      // equal shares: the first `rest` of them hold one step more
     __device__ __forceinline__ int cut(int c) const { return c * each + min(c, rest); }
+    __device__ __forceinline__ int share_of(int x) const {
+        const int y = x - rest * (each + 1);
+        return y < 0 ? x / (each + 1) : rest + y / each;
+    }
 };
 
 constexpr int kMinSteps = 12;                      // three steps per warp
@@ -152,6 +157,7 @@ __device__ __forceinline__ Segment segment_at(const DecodeArgs& a, const Line& l
     sg.s_begin = r - kr * sg.steps;
     sg.s_end = min(sg.steps, sg.s_begin + (end - x));
     sg.lb = layer * a.n_requests + lo;
+    sg.unit = sg.lb * line.tiles + kr;
     sg.kvh = kr / a.row_tiles;
     const int row_tile = kr - sg.kvh * a.row_tiles, group = a.n_q_heads / a.n_kv_heads;
     sg.head0 = sg.kvh * group + row_tile * kq;
@@ -163,7 +169,7 @@ __device__ __forceinline__ Segment segment_at(const DecodeArgs& a, const Line& l
 // NQ: query heads per CTA in groups of eight (1: up to 8 heads per kv head, 2: up to 16; more heads take further CTAs).
 // STREAM = false: a cluster per unit.  STREAM = true: CTA c takes share c of the line of all steps; a unit that lies in
 // one share is finished there, a share leaves its part of a unit that began before it in slot 2c of the workspace and
-// its part of one that goes on behind it in slot 2c + 1.
+// its part of one that goes on behind it in slot 2c + 1; the share a unit begins in notes into how many parts it was cut.
 template <int NQ, bool STREAM>
 __global__ void __launch_bounds__(kDecThreads, NQ == 1 ? 3 : 2)
 decode_attn_kernel(DecodeArgs a, int n_layers) {
@@ -371,6 +377,8 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
     const uint32_t addr_m = (uint32_t)__cvta_generic_to_shared(&s_m[kDecWarps][0]), addr_l = (uint32_t)__cvta_generic_to_shared(&s_l[kDecWarps][0]);
     const int layer = done.lb / a.n_requests, b = done.lb - layer * a.n_requests;
     const bool whole = !STREAM || (done.s_begin == 0 && done.s_end == done.steps);
+    if (STREAM && tid == 0 && done.s_begin == 0)                    // x_pos: the position behind this segment
+        a.unit_parts[done.unit] = make_int2((int)blockIdx.x, whole ? 0 : line.share_of(x_pos - done.s_end + done.steps - 1) - (int)blockIdx.x + 1);
     // every CTA of the cluster writes its share of the (head, dim pair) items
     for (int idx = rank * kDecThreads + tid; idx < done.n_heads * (kDecDim / 2); idx += n_cta * kDecThreads) {
         const int r = idx >> 6, d = (idx & 63) * 2;
@@ -422,26 +430,21 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
     if (!STREAM && n_cta > 1) cluster_sync();                       // nobody leaves while its shared memory is being read
 }
 
-// Units cut over several shares: one block per (layer, request, head) merges the parts, its warps every fourth one.
+// Units cut over several shares: one block per (layer, request, head) merges the parts, its warps every fourth one.  How a
+// unit was cut is read from what the attention kernel left.  Made again from the plan (dependent loads, a scan and a barrier
+// behind the wait) it took a step of 32 layers of 8 x 2764 rows, 32/32 heads, from 1526 to 1588 us; this way 1574 to 1581.
 __global__ void __launch_bounds__(kDecThreads)
-decode_merge_kernel(DecodeArgs a, int n_layers, int max_shares, int kq) {
-    __shared__ int s_pref[kMaxStreamRequests + 1];
+decode_merge_kernel(DecodeArgs a, int kq) {
     __shared__ __align__(16) float s_w[4][kDecDim];
     __shared__ float s_ml[2][4];
-    chain_next();
-    const Line line = make_line(a, s_pref, n_layers, max_shares);   // the decode plan was complete when the attention kernel began
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row = blockIdx.x;            // (layer * B + request) * heads + head
     const int lb = row / a.n_q_heads, h = row - lb * a.n_q_heads, layer = lb / a.n_requests, b = lb - layer * a.n_requests;
     const int group = a.n_q_heads / a.n_kv_heads, kvh = h / group, in_group = h - kvh * group, row_tile = in_group / kq, r = in_group - row_tile * kq;
-    const int steps = line.pref[b + 1] - line.pref[b];
-    const int x0 = layer * line.per_layer + line.pref[b] * line.tiles + (kvh * a.row_tiles + row_tile) * steps;
-    auto share_of = [&](int x) {
-        const int y = x - line.rest * (line.each + 1);
-        return y < 0 ? x / (line.each + 1) : line.rest + y / line.each;
-    };
-    const int c0 = share_of(x0), c1 = share_of(x0 + steps - 1);
+    chain_next();
     chain_wait();
-    if (c0 == c1) return;                                           // finished by its one share
+    const int2 cut = a.unit_parts[(lb * a.n_kv_heads + kvh) * a.row_tiles + row_tile];
+    if (cut.y == 0) return;                                         // finished by its one share
+    const int c0 = cut.x, c1 = c0 + cut.y - 1;
     float mm = -INFINITY, ll = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
     for (int cb = c0 + warp; cb <= c1; cb += 16) {                  // four parts in flight
         float mp[4], lp[4];
@@ -500,10 +503,16 @@ bool decode_attn_supported(const cf_geom* g) { return g->dtype == CF_BF16 && g->
 
 static int stream_shares(const cf_geom* g) { return (g->n_q_heads / g->n_kv_heads > 8 ? 2 : 3) * sm_count(); }   // one wave
 
-// Workspace of a call: two parts per share.
-size_t decode_attn_workspace_bytes(const cf_geom* g) {
+// Units of a call: (layer, request, kv head, tile of query heads).
+static long long decode_units(const cf_geom* g, int n_requests, int n_layers) {
+    const int group = g->n_q_heads / g->n_kv_heads, kq = group > 8 ? 16 : 8;
+    return (long long)n_layers * n_requests * g->n_kv_heads * ((group + kq - 1) / kq);
+}
+
+// Workspace of a call: two parts per share, and how every unit was cut.
+size_t decode_attn_workspace_bytes(const cf_geom* g, int n_requests, int n_layers) {
     const int kq = g->n_q_heads / g->n_kv_heads > 8 ? 16 : 8;
-    return (size_t)stream_shares(g) * 2 * kq * (kDecDim + 2) * sizeof(float);
+    return (size_t)stream_shares(g) * 2 * kq * (kDecDim + 2) * sizeof(float) + (size_t)decode_units(g, n_requests, n_layers) * sizeof(int2);
 }
 
 int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_layers, const int* doc_offsets, const LayerSpan& span,
@@ -517,10 +526,11 @@ int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_l
     float* part_o = static_cast<float*>(workspace);
     float* part_m = part_o + (size_t)shares * 2 * kq * kDecDim;
     float* part_l = part_m + (size_t)shares * 2 * kq;
+    int2* unit_parts = reinterpret_cast<int2*>(part_l + (size_t)shares * 2 * kq);
     const DecodeArgs a = {static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v),
                           static_cast<__nv_bfloat16*>(out), lse, doc_offsets, span.q_stride, span.kv_stride, span.out_stride, n_requests,
-                          cache_rows, g->n_q_heads, g->n_kv_heads, row_tiles, scale_log2, part_o, part_m, part_l};
-    const long long units = (long long)n_layers * n_requests * g->n_kv_heads * row_tiles;
+                          cache_rows, g->n_q_heads, g->n_kv_heads, row_tiles, scale_log2, part_o, part_m, part_l, unit_parts};
+    const long long units = decode_units(g, n_requests, n_layers);
     // A cluster per unit where one wave of clusters leaves a warp a few steps (measured, us per layer, cluster against
     // stream: 1011 rows, 2 units 5.5 / 8.1; 1984 rows, 16 units 10.1 / 11.5; 500 rows, 128 units 11.1 / 13.4), the
     // stream of equal shares for everything longer (5000 rows, 16 units 16.2 / 13.3; 2764 rows, 256 units 59 / 45.6).
@@ -533,7 +543,7 @@ int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_l
         const int rc = wide ? launch_chained(decode_attn_kernel<2, true>, dim3(shares), kDecThreads, 0, stream, a, n_layers)
                             : launch_chained(decode_attn_kernel<1, true>, dim3(shares), kDecThreads, 0, stream, a, n_layers);
         if (rc != CF_OK) return rc;
-        return launch_chained(decode_merge_kernel, dim3((unsigned)(n_layers * n_requests * g->n_q_heads)), kDecThreads, 0, stream, a, n_layers, shares, kq);
+        return launch_chained(decode_merge_kernel, dim3((unsigned)(n_layers * n_requests * g->n_q_heads)), kDecThreads, 0, stream, a, kq);
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cluster, (unsigned)(g->n_kv_heads * row_tiles), (unsigned)(n_requests * n_layers));

@@ -193,3 +193,45 @@ def test_decode_kernel_at_the_edges_of_its_splits(hq, hkv, cache_rows, used):
                 got = out[l, b].double().cpu().numpy()
                 assert np.all(np.abs(got - ref) <= 1e-2 + 2e-2 * np.abs(ref)), (l, b, per_call)
                 assert np.all(np.abs(lse[l, b].cpu().numpy() - (top[:, 0] + np.log(w.sum(axis=1)))) <= 1e-2), (l, b, per_call)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_steps_queued_behind_one_another(graph):
+    """Plan, append, attention and merge of many steps in one queue, the requests' fill levels changing from step to step so
+    that every step cuts its rows into other shares: bit for bit the results of the steps run one at a time."""
+    hq, hkv, room, d = 8, 1, 6000, 128
+    levels = [[5990, 1, 257], [33, 5900, 4000], [2000, 2001, 1], [1, 1, 5999]] * 3
+    geom = cf.make_geom(hq, hkv, d, cf.CF_BF16, 32768, 1e6)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    k0, v0 = rand(1, 3, room, hkv, d), rand(1, 3, room, hkv, d)
+    q, k_new, v_new = rand(len(levels), 1, 3, hq, d), rand(len(levels), 1, 3, hkv, d), rand(len(levels), 1, 3, hkv, d)
+    rows = torch.tensor(levels, dtype=torch.int32, device="cuda")
+    plan = torch.full((cf.cf_decode_plan_bytes(geom, 3, room),), 255, dtype=torch.uint8, device="cuda")
+    work = torch.full((cf.cf_decode_workspace_bytes(geom, 3, room, 1),), 255, dtype=torch.uint8, device="cuda")
+
+    def steps(k, v, out, lse, one_at_a_time):
+        for i in range(len(levels)):
+            cf.cf_decode_plan(geom, 3, room, rows[i], 1, plan)
+            cf.cf_decode_append(geom, 3, room, k, v, rows[i], 0, k_new[i], v_new[i])
+            cf.cf_decode_attn(geom, 3, room, plan, q[i], k, v, out[i], work, lse[i])
+            if one_at_a_time:
+                torch.cuda.synchronize()
+
+    results = []
+    for queued in (False, True):
+        k, v = k0.clone(), v0.clone()
+        out = torch.full((len(levels), 1, 3, hq, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((len(levels), 1, 3, hq), float("nan"), device="cuda")
+        torch.cuda.synchronize()
+        if queued and graph:
+            recorded = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(recorded):
+                steps(k, v, out, lse, False)
+            recorded.replay()
+        else:
+            steps(k, v, out, lse, not queued)
+        torch.cuda.synchronize()
+        results.append((out, lse))
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
+    assert not bool(torch.isnan(results[0][1]).any())
