@@ -18,10 +18,11 @@
 // Tensor memory: O (128 columns), the query tile (64: as the A operand of QK^T it costs no shared-memory reads, which this
 // kernel has none to spare of), three S buffers of 96 columns; P (bf16) overwrites the S columns already consumed.  S(n + 3) is issued behind PV(n), so a softmax warpgroup that has finished a
 // tile finds its next S waiting.
-// Softmax: both warpgroups accumulate into one O under one reference per row, fixed by the first 16 keys of the segment:
-// their maximum plus 40.  P and the sums keep their relative precision for logits up to 80 (log2 units) above that first
-// maximum and as far below as matters, so that no tile has to look at its maximum before its exponentials.  A row that
-// does leave this range is marked (NaN sum) and recomputed from scratch by the merge kernel.
+// Softmax: both warpgroups accumulate into one O under one reference per row, the maximum over the first 16 keys of the
+// segment.  P and the sums keep their relative precision for logits up to 80 (log2 units) above it and 126 below, so that no
+// tile has to look at its maximum before its exponentials.  (A reference 40 above that maximum, which centres the range, costs
+// three bits of the exponents and the log-sum-exps: 1.3e-6 off instead of 1.1e-7 for a row of one key.)  A row that does leave
+// the range is marked (NaN sum) and recomputed from scratch by the merge kernel.
 // What bounds it (per 96-key tile and 128 rows, in SM cycles): tensor cores 768 (8 x 48 + 6 x 64), exponentials 768 on
 // the shared MUFU, shared memory 1150 (copies 384, rotation 384, QK^T 192, PV 192), so these overlap only if nobody
 // waits for a chain.
@@ -51,8 +52,7 @@ constexpr int kPrefSlots = 48;
 constexpr int kLoadWarp = 9, kMmaWarp = 12;
 constexpr int kTrigBytes = kD / 2 * 8;
 constexpr uint32_t kColO = 0, kColQ = 128, kColS = 192;
-constexpr float kRefShift = 40.0f;                 // the reference of a row lies this far (log2 units) above its first maximum
-constexpr float kSumLimit = 1099511627776.0f;      // 2^40: a larger tile sum leaves the range the reference was chosen for
+constexpr float kSumLimit = 0x1p80f;               // a larger tile sum leaves the range: 2^47 are left for the values and the other tiles
 static_assert(kColS + kSBuffers * kTile <= 512, "tensor memory columns");
 static_assert(kTile % 16 == 0 && kTile <= 96, "three S buffers");
 static_assert(kKStages == 6 && kVStages == 3 && kSBuffers == 3, "rings of one period");
@@ -752,7 +752,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
                     float m = -INFINITY;
 #pragma unroll
                     for (int e = 0; e < 16; ++e) m = fmaxf(m, e < vis ? __uint_as_float(va[e]) : -INFINITY);
-                    sh.ref[par][r] = m > -INFINITY ? fmaf(m, src.scale_log2, kRefShift) : 0.f;   // a row that sees none of them sees none of the tile
+                    sh.ref[par][r] = m > -INFINITY ? m * src.scale_log2 : 0.f;   // a row that sees none of them sees none of the tile
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&bars.ref_full[par]));
                 }

@@ -16,9 +16,9 @@
 // one (tiles of 128 with one S buffer: the softmax waited 2200 cycles per tile for its S and worked for 2000), and the
 // epilogue is taken out of the chain.  Rows pass through 2 KB of staging per warp, so that a store instruction writes 64
 // bytes to each of 8 rows: one row per thread in 32-byte pieces kept the warps waiting for 2100 cycles per item.
-// Softmax: one fixed reference per row, the maximum over the item's first 16 keys (every row sees the first one) plus 40;
-// P and the sums keep their relative precision up to 80 (log2 units) above that maximum.  A row that leaves this range is
-// noted and computed again, alone, when the CTA's items are done.
+// Softmax: one fixed reference per row, the maximum over the item's first 16 keys (every row sees the first one); P and the
+// sums keep their relative precision up to 80 (log2 units) above that maximum.  A row that leaves this range is noted and
+// computed again, alone, when the CTA's items are done.
 // Bound by HBM for a few query heads per kv head: with 6 heads and a 64-token prefix 123 flops per byte.
 // Measured (400 documents of 128-192 tokens, 12/2 heads, 4 layers, prefix 64): 660 us before
 // (one issuing thread for copies and MMAs, two passes over S, rows staged through the value buffer), 449 us now; one layer
@@ -42,7 +42,7 @@ constexpr int kKeyHalf = kKeys * 128, kKeyTile = 2 * kKeyHalf;   // bytes: 64 di
 constexpr int kDocBoxes = 3;                                 // copy boxes of 16, 32 and 64 rows
 constexpr int kItemRing = 8, kSumRing = 4;                   // QK^T runs two tiles, perhaps two items, ahead of PV, and the epilogue one behind
 constexpr int kMarkedMost = 256;
-constexpr float kDocRefShift = 40.0f, kDocSumLimit = 1099511627776.0f;   // 2^40: see cf_attn_tc.cu
+constexpr float kDocSumLimit = 0x1p80f;                      // see cf_attn_tc.cu
 
 struct DocMaps {
     CUtensorMap k[kDocBoxes], v[kDocBoxes];        // the documents' keys and values, one map per box height
@@ -436,7 +436,7 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
                 tmem_ld16_wait(va);
                 if (c0 == 0) {
                     const float m = chunk16_max(va, min(lim, hole == 0 ? hole_valid : 16));
-                    ref = fmaf(m, p.a.scale_log2, kDocRefShift);
+                    ref = m * p.a.scale_log2;
                     neg_ref2 = pack_f2(-ref, -ref);
                 }
                 for (int c = 0; c < some; c += 2) {

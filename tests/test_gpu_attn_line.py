@@ -128,3 +128,27 @@ def test_scores_do_not_depend_on_the_layers_beside_them(heads, q_len, layers):
     for s in scores:
         total += s
     assert torch.equal(accum[[0, 1, 3, 4]], total[[0, 1, 3, 4]]) and float(scores[:, 2].abs().max()) == 0.0
+
+
+def test_log_sum_exp_of_a_single_key():
+    """A row that sees one key has its logit as log-sum-exp.  Queries of one non-zero element make the product exact, so what is
+    left are the roundings of the scale, the reference, the exponential (2^-22) and the logarithm: absolute 2^-22, relative
+    8 x 2^-24, as far as the row's own magnitude goes and no further."""
+    import paper_2502_11101_b200 as cf
+    from paper_2502_11101_b200.session import Session
+    q_len, heads = 128, 4
+    sess = Session(heads, heads, 128, torch.bfloat16, 32768, 1e6, q_len, np.ones(1, np.int32), np.asarray([0, 1], np.int32),
+                   np.zeros(1, np.int32), tail_reserve=q_len)
+    sess.init()
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    k = torch.randn(1, 1, heads, 128, generator=gen, device="cuda").bfloat16()
+    rotated, q = torch.empty_like(k), torch.zeros(1, 1, q_len, heads, 128, device="cuda", dtype=torch.bfloat16)
+    sess.reposition(k, rotated, 1, 0)
+    for j in range(q_len):
+        q[0, 0, j, :, j] = 8.0
+    lse = torch.empty(1, 1, heads, q_len, device="cuda")
+    sess.attend_layers(q, k, torch.ones_like(k), torch.empty_like(q), lse)
+    torch.cuda.synchronize()
+    want = rotated[0, 0].double() * 8.0 / np.sqrt(128.0)
+    error = (lse[0, 0].double() - want).abs()
+    assert bool((error <= 2.0 ** -22 + 8 * 2.0 ** -24 * want.abs()).all()), float(error.max())

@@ -172,3 +172,22 @@ def test_rows_far_outside_the_range_of_their_reference(lens, prefix_len, first):
     assert float(l1.max()) > 100.0
     torch.testing.assert_close(l0, l1, rtol=2e-3, atol=2e-3)
     torch.testing.assert_close(o0, o1, rtol=2e-2, atol=2e-2)
+
+
+def test_log_sum_exp_of_a_single_key():
+    """Documents of one token: the log-sum-exp is the logit.  Queries of one non-zero element make the product exact; left are
+    the roundings of the scale, the reference, the exponential (2^-22) and the logarithm."""
+    heads, n = 4, 128
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    k = torch.randn(1, n, heads, 128, generator=gen, device="cuda").bfloat16()
+    q = torch.zeros_like(k)
+    for j in range(n):
+        q[0, j, :, j] = 8.0
+    lse = torch.empty(1, heads, n, device="cuda")
+    geom = cf.make_geom(heads, heads, 128, torch.bfloat16, 4096, 1e4)
+    cf.cf_document_prefill_attn(geom, torch.arange(n + 1, dtype=torch.int32, device="cuda"), 1, q, k, torch.ones_like(k),
+                                torch.empty_like(q), None, None, lse)
+    torch.cuda.synchronize()
+    want = torch.diagonal(k[0].double(), dim1=0, dim2=2) * 8.0 / np.sqrt(128.0)
+    error = (lse[0].double() - want).abs()
+    assert bool((error <= 2.0 ** -22 + 8 * 2.0 ** -24 * want.abs()).all()), float(error.max())
