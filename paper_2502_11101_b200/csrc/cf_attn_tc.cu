@@ -31,6 +31,7 @@
 // for every phase in order.
 #include <algorithm>
 
+#include "cf_row_group.cuh"
 #include "cf_tc_util.cuh"
 
 namespace cf {
@@ -253,89 +254,186 @@ struct Params {
     __nv_bfloat16* const out_all = p.out;                                                                          \
     float* const lse = p.lse
 
-// One query row by one warp, keys one after the other under a running maximum: its output, its log-sum-exps and those of
-// its document tiles.  Only rows whose logits left the range of the shared reference come here.
+// Shared memory of a merge block that computes rows from scratch.
+struct RowScratch {
+    rows::Stage stage[8];          // of every warp
+    alignas(16) rows::Queries q;
+    alignas(16) float o[rows::kGroupRows][kD];
+    float m[8][rows::kGroupRows], l[8][rows::kGroupRows], docs[8][rows::kGroupRows];   // of every warp
+    Requests requests;
+};
+
+// Up to eight query rows (rg0 + every set bit of `set`, of one kv head) by a block of eight warps, each with every eighth key tile
+// under a running maximum of its own: outputs, log-sum-exps and those of the document tiles.  Only rows whose logits left the
+// range of the shared reference come here (keys that are not finite lead here too).  Bound by the instructions and mma.sync of a
+// step, 2 us for eight rows.  Measured with a warp per row and key after key, and this way: four layers of 50 documents of 160
+// tokens, 12/2 heads, 44 us without such rows, one row a layer 3.0 -> 0.19 ms, every row 10.1 -> 0.83 ms; one layer of 2 x 60
+// documents of 180, 32/32 heads, 93 us without, one row 6.1 -> 0.29, every row 27.1 -> 1.2 ms.
 template <int LAYOUT>
-__device__ __noinline__ void row_from_scratch(const Params& p, int lb, int rg, int n_doc) {
+__device__ __noinline__ void rows_from_scratch(const Params& p, RowScratch& sh, int lb, int rg0, unsigned set, int n_doc) {
     CF_PARAMS;
     const int n_prefix = (src.prefix_len + kTile - 1) / kTile, n_self = src.with_self ? (bv.q_len + kTile - 1) / kTile : 0;
-    const int lane = threadIdx.x & 31, lq = bv.q_len, group = n_q_heads / n_kv_heads;
-    const int layer = lb / bv.n_requests, b = lb - layer * bv.n_requests, h = rg / lq, j = rg - h * lq, kvh = h / group;
-    const int d0 = LAYOUT == CF_ROPE_HALF ? 2 * lane : 4 * lane, d1 = LAYOUT == CF_ROPE_HALF ? 64 + 2 * lane : 4 * lane + 2;
-    auto load = [&](const __nv_bfloat16* e, float (&x)[4]) {
-        const uint32_t u = *reinterpret_cast<const uint32_t*>(e + d0), t = *reinterpret_cast<const uint32_t*>(e + d1);
-        x[0] = __uint_as_float(u << 16);
-        x[1] = __uint_as_float(u & 0xffff0000u);
-        x[2] = __uint_as_float(t << 16);
-        x[3] = __uint_as_float(t & 0xffff0000u);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lq = bv.q_len, group = n_q_heads / n_kv_heads, rows_total = n_q_heads * lq;
+    const int layer = lb / bv.n_requests, b = lb - layer * bv.n_requests, n_rows = __popc(set);
+    const int rg = rg0 + rows::nth_bit(set, lane >> 2), h = rg / lq, j = rg - h * lq, kvh = h / group;
+    if (lane < 16) {                                                // a row of the group per warp
+        const int row = rg0 + rows::nth_bit(set, warp), hh = row / lq, jj = row - hh * lq;
+        sh.q.put(warp, lane, src.q + (size_t)layer * span.q_stride + (((size_t)b * lq + jj) * n_q_heads + hh) * kD);
+    }
+    __syncthreads();
+    // every eighth tile of the request: where its keys lie and which of them this lane's row sees
+    struct Tile {
+        const __nv_bfloat16 *k, *v;
+        size_t pitch;
+        const float2* trig;                                         // null: not a document's
+        int len, visible, index;
     };
-    float q[4], acc[4] = {0.f, 0.f, 0.f, 0.f}, m = -INFINITY, l = 0.f, docs_lse2 = -INFINITY;
-    load(src.q + (size_t)layer * span.q_stride + (((size_t)b * lq + j) * n_q_heads + h) * kD, q);
-    for (int t = 0; t < n_doc + n_prefix + n_self; ++t) {
-        const __nv_bfloat16 *kr, *vr;
-        size_t pitch = (size_t)n_kv_heads * kD;
-        int len, index = -1;
-        float2 cs0 = make_float2(1.f, 0.f), cs1 = cs0;
+    const int n_tiles = n_doc + n_prefix + n_self, tile0 = pv.tile_begin[b];
+    int next_row0 = 0, next_len = 0, next_doc = 0;                  // of the document tile behind the current one, asked for early
+    auto fetch = [&](int t) {
+        if (t >= n_doc) return;
+        next_row0 = pv.tile_row0[tile0 + t];
+        next_len = pv.tile_len[tile0 + t];
+        next_doc = pv.tile_doc[tile0 + t];
+    };
+    auto tile_at = [&](int t) {
+        Tile x;
+        x.pitch = (size_t)n_kv_heads * kD;
+        x.trig = nullptr;
+        x.index = -1;
         if (t < n_doc) {
-            index = pv.tile_begin[b] + t;
-            pitch = bv.token_stride;
-            const size_t at = (size_t)layer * span.kv_stride + (size_t)pv.tile_row0[index] * pitch + kvh * kD;
-            kr = src.k + at;
-            vr = src.v + at;
-            len = pv.tile_len[index];
-            const float2* trig = pv.trig + (size_t)pv.tile_doc[index] * (kD / 2) + 2 * lane;
-            cs0 = trig[0];
-            cs1 = trig[1];
+            x.index = tile0 + t;
+            x.pitch = bv.token_stride;
+            const size_t at = (size_t)layer * span.kv_stride + (size_t)next_row0 * x.pitch + kvh * kD;
+            x.k = src.k + at;
+            x.v = src.v + at;
+            x.len = x.visible = next_len;
+            x.trig = pv.trig + (size_t)next_doc * (kD / 2);
         } else if (t < n_doc + n_prefix) {
             const int row0 = (t - n_doc) * kTile;
-            const size_t at = (size_t)layer * src.prefix_stride + (size_t)row0 * pitch + kvh * kD;
-            kr = src.kp + at;
-            vr = src.vp + at;
-            len = min(kTile, src.prefix_len - row0);
+            const size_t at = (size_t)layer * src.prefix_stride + (size_t)row0 * x.pitch + kvh * kD;
+            x.k = src.kp + at;
+            x.v = src.vp + at;
+            x.len = x.visible = min(kTile, src.prefix_len - row0);
         } else {
             const int row0 = (t - n_doc - n_prefix) * kTile;
-            const size_t at = (size_t)layer * src.self_stride + ((size_t)b * lq + row0) * pitch + kvh * kD;
-            kr = src.ks + at;
-            vr = src.vs + at;
-            len = min(min(kTile, lq - row0), j + 1 - row0);
+            const size_t at = (size_t)layer * src.self_stride + ((size_t)b * lq + row0) * x.pitch + kvh * kD;
+            x.k = src.ks + at;
+            x.v = src.vs + at;
+            x.len = min(kTile, lq - row0);
+            x.visible = min(x.len, j + 1 - row0);                   // causal mask
         }
-        if (t == n_doc) docs_lse2 = l > 0.f ? m + log2f(l) : -INFINITY;
-        float tm = -INFINITY, tl = 0.f;
-        for (int i = 0; i < len; ++i) {
-            float k[4], v[4], y[4];
-            load(kr + i * pitch, k);
-            load(vr + i * pitch, v);
-            if (LAYOUT == CF_ROPE_HALF) {
-                rotate_pair(k[0], k[2], cs0.x, cs0.y, y[0], y[2]);
-                rotate_pair(k[1], k[3], cs1.x, cs1.y, y[1], y[3]);
-            } else {
-                rotate_pair(k[0], k[1], cs0.x, cs0.y, y[0], y[1]);
-                rotate_pair(k[2], k[3], cs1.x, cs1.y, y[2], y[3]);
-            }
-            float dot = 0.f;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) dot = fmaf(q[e], __bfloat162float(__float2bfloat16_rn(y[e])), dot);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-            const float s = dot * src.scale_log2;
-            const float m_new = fmaxf(m, s), alpha = exp2f(m - m_new), w = exp2f(s - m_new);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[e] = fmaf(acc[e], alpha, w * v[e]);
-            l = fmaf(l, alpha, w);
-            m = m_new;
-            const float tm_new = fmaxf(tm, s);
-            tl = fmaf(tl, exp2f(tm - tm_new), exp2f(s - tm_new));
-            tm = tm_new;
-        }
-        if (index >= 0 && lane == 0) ws.tile_lse2[((size_t)layer * ws.max_tiles + index) * n_q_heads * lq + rg] = tm + log2f(tl);
+        return x;
+    };
+    rows::Stage& stage = sh.stage[warp];
+    rows::Group acc;
+    acc.clear();
+    float docs = 0.f, in_tile = 0.f;                                // the parts of acc.l on documents and on the current tile
+    int t = warp, i = 0;
+    Tile now = {};
+    if (t < n_tiles) {
+        fetch(t);
+        now = tile_at(t);
+        fetch(t + 8);
+        rows::copy_step(stage.k, now.k, now.pitch, now.len);
+        rows::copies_end();
+        rows::copy_step(stage.v, now.v, now.pitch, now.len);
+        rows::copies_end();
     }
-    const float lse2 = l > 0.f ? m + log2f(l) : -INFINITY, inv = l > 0.f ? 1.f / l : 0.f;
-    __nv_bfloat16* dst = out_all + (size_t)layer * span.out_stride + (((size_t)b * lq + j) * n_q_heads + h) * kD;
-    *reinterpret_cast<uint32_t*>(dst + d0) = pack_bf16(acc[0] * inv, acc[1] * inv);
-    *reinterpret_cast<uint32_t*>(dst + d1) = pack_bf16(acc[2] * inv, acc[3] * inv);
-    if (lane == 0) {
-        ws.row_lse2[(size_t)lb * n_q_heads * lq + rg] = n_prefix + n_self > 0 ? docs_lse2 : lse2;
-        if (lse) lse[(size_t)lb * n_q_heads * lq + rg] = lse2 * kLn2;
+    while (t < n_tiles) {
+        rows::Keys keys;
+        rows::copies_wait();
+        keys.read(stage);
+        Tile next = now;                                            // the step behind this one
+        int next_i = i + rows::kStepKeys;
+        const bool last = next_i >= now.len;
+        if (last && t + 8 < n_tiles) {
+            next = tile_at(t + 8);
+            fetch(t + 16);
+            next_i = 0;
+        }
+        const bool more = next_i < next.len;
+        __syncwarp();                                               // every lane has its fragments
+        if (more) rows::copy_step(stage.k, next.k + next_i * next.pitch, next.pitch, next.len - next_i);
+        rows::copies_end();
+        if (now.trig) keys.rotate<LAYOUT>(now.trig);
+        float alpha;
+        const float sum = acc.scores(sh.q, keys, now.visible - i, src.scale_log2, alpha);
+        in_tile = fmaf(in_tile, alpha, sum);
+        docs = fmaf(docs, alpha, now.trig ? sum : 0.f);
+        rows::copies_wait();
+        acc.values(stage);
+        __syncwarp();
+        if (more) rows::copy_step(stage.v, next.v + next_i * next.pitch, next.pitch, next.len - next_i);
+        rows::copies_end();
+        if (last) {
+            in_tile = rows::over_keys(in_tile);
+            if (now.trig && (lane & 3) == 0 && (lane >> 2) < n_rows) ws.tile_lse2[((size_t)layer * ws.max_tiles + now.index) * rows_total + rg] = acc.m + log2f(in_tile);
+            in_tile = 0.f;
+            t += 8;
+        }
+        now = next;
+        i = next_i;
+    }
+    acc.l = rows::over_keys(acc.l);
+    docs = rows::over_keys(docs);
+    if ((lane & 3) == 0) {
+        sh.m[warp][lane >> 2] = acc.m;
+        sh.l[warp][lane >> 2] = acc.l;
+        sh.docs[warp][lane >> 2] = docs;
+    }
+    __syncthreads();
+    // join the warps, in order: a row's reference is the largest of theirs (-inf: nothing to attend)
+    float weight[2];                                                // of this warp's rows 2 t and 2 t + 1
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int r = 2 * (lane & 3) + x;
+        float top = sh.m[0][r];
+        for (int w = 1; w < 8; ++w) top = fmaxf(top, sh.m[w][r]);
+        weight[x] = sh.m[warp][r] > -INFINITY ? exp2f(sh.m[warp][r] - top) : sh.l[warp][r];   // nothing seen: 0 (or not a number)
+    }
+    for (int w = 0; w < 8; ++w) {
+        if (w == warp)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    float2& to = *reinterpret_cast<float2*>(&sh.o[2 * (lane & 3) + x][(i >> 2) * 64 + (lane >> 2) * 8 + 2 * (i & 3)]);
+                    const float2 was = w == 0 ? make_float2(0.f, 0.f) : to;
+                    to = make_float2(fmaf(acc.o[i][x], weight[x], was.x), fmaf(acc.o[i][x + 2], weight[x], was.y));
+                }
+        __syncthreads();
+    }
+    if (warp < n_rows) {                                            // a row per warp, four dims per lane
+        float top = sh.m[0][warp], l = 0.f, ld = 0.f;
+        for (int w = 1; w < 8; ++w) top = fmaxf(top, sh.m[w][warp]);
+        for (int w = 0; w < 8; ++w) {
+            const float f = sh.m[w][warp] > -INFINITY ? exp2f(sh.m[w][warp] - top) : 1.f;
+            l = fmaf(sh.l[w][warp], f, l);
+            ld = fmaf(sh.docs[w][warp], f, ld);
+        }
+        const int row = rg0 + rows::nth_bit(set, warp), hh = row / lq, jj = row - hh * lq;
+        const float inv = l == 0.f ? 0.f : 1.f / l;
+        const float4 o = *reinterpret_cast<const float4*>(&sh.o[warp][lane * 4]);
+        *reinterpret_cast<uint2*>(out_all + (size_t)layer * span.out_stride + (((size_t)b * lq + jj) * n_q_heads + hh) * kD + lane * 4) =
+            make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
+        if (lane == 0) {
+            ws.row_lse2[(size_t)lb * rows_total + row] = top + log2f(ld);
+            if (lse) lse[(size_t)lb * rows_total + row] = (top + log2f(l)) * kLn2;
+        }
+    }
+    __syncthreads();                                                // the shared memory may be used again
+}
+
+constexpr size_t kMergeSmem = sizeof(RowScratch);
+
+// All rows of a set, eight at a time.
+template <int LAYOUT>
+__device__ __forceinline__ void set_from_scratch(const Params& p, RowScratch& sh, int lb, int rg0, unsigned set, int n_doc) {
+    while (set) {
+        const unsigned now = rows::next_group(set);
+        rows_from_scratch<LAYOUT>(p, sh, lb, rg0, now, n_doc);
+        set ^= now;
     }
 }
 
@@ -839,6 +937,40 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
     }
 }
 
+// The rows of a merge block's slice that left the range of their reference: of the units finished in its shares (the sum of such
+// a row is not a number) and of those that were cut (cut_rows).
+template <int LAYOUT, int ROWS>
+__device__ __noinline__ void marked_from_scratch(const Params& p, const unsigned* cut_rows, int share0, int n_classes, int slice) {
+    extern __shared__ __align__(16) unsigned char merge_smem[];
+    RowScratch& sh = *reinterpret_cast<RowScratch*>(merge_smem);
+    const BatchView& bv = p.bv;
+    const PlanView& pv = p.pv;
+    const AttnWorkspace& ws = p.ws;
+    const int lane = threadIdx.x & 31, group = p.n_q_heads / p.n_kv_heads, rows_total = p.n_q_heads * bv.q_len;
+    for (int u = 0, share = share0; u < 32 / ROWS && share < p.max_shares; ++u, share += n_classes) {
+        const ShareHead head = reinterpret_cast<const ShareHead*>(ws.marks)[share];
+        if (head.marked) {
+            if (threadIdx.x < 32) scan_requests(bv, pv, p.n_prefix + p.n_self, sh.requests);
+            __syncthreads();
+            const Line line = make_line(bv, ws, sh.requests, p.n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, p.max_shares);
+            const int end = line.cut(share + 1);
+            for (int y = line.cut(share); y < end;) {
+                const Segment own = segment_at(bv, pv, ws, line, group, y, end);
+                y += own.t_end - own.t_begin;
+                if (own.t_end - own.t_begin != own.n_unit) continue;
+                const int rg0 = own.kvh * group * bv.q_len + own.row0 + slice * ROWS;
+                const bool mine = lane < ROWS && slice * ROWS + lane < own.rows_here;
+                const float v = mine ? ws.row_lse2[(size_t)own.lb * rows_total + rg0 + lane] : 0.f;
+                const unsigned todo = __ballot_sync(0xffffffffu, v != v);
+                __syncthreads();                                    // every warp has looked before the first row is written
+                set_from_scratch<LAYOUT>(p, sh, own.lb, rg0, todo, own.n_doc);
+            }
+        }
+        set_from_scratch<LAYOUT>(p, sh, head.lb, head.row_first + slice * ROWS, cut_rows[u], head.n_doc);
+        __syncthreads();
+    }
+}
+
 // Units that lie in several shares: the parts of a row are merged in the order of the line by eight lanes, in a block of the
 // share the unit begins in.  The blocks of a share also see to rows of its whole units that left the range of their reference,
 // those of the last share to the (empty) results of requests that have nothing to attend.  A chain of two memory latencies:
@@ -852,7 +984,10 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
     CF_PARAMS;
     constexpr int kRuns = 32 / ROWS, kSlices = kRowTile / ROWS, kRunThreads = 256 / kRuns;
     const int max_shares = p.max_shares;
-    __shared__ Requests s_rq;
+    __shared__ unsigned s_marked[4];                                // rows of the slice out of range, of the unit cut in every share
+    if (threadIdx.x < 4) s_marked[threadIdx.x] = 0;
+    __syncthreads();
+    bool marked = false;
     __shared__ float s_run[kRuns > 1 ? kRuns - 1 : 1][19][kRuns > 1 ? kRunThreads : 1];   // m, l, ld and 16 dims per thread
     const int lq = bv.q_len, rows_total = n_q_heads * lq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n_classes = (max_shares + kRuns - 1) / kRuns, share0 = blockIdx.x / kSlices, slice = blockIdx.x - share0 * kSlices;
@@ -881,23 +1016,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                             if (lse) lse[at + i] = -INFINITY;
                         }
                     }
-        if (head.marked) {
-            __syncthreads();
-            if (warp == 0) scan_requests(bv, pv, p.n_prefix + p.n_self, s_rq);
-            __syncthreads();
-            const Line line = make_line(bv, ws, s_rq, n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, max_shares);
-            const int group = n_q_heads / n_kv_heads, end = line.cut(share + 1);
-            for (int y = line.cut(share); y < end;) {
-                const Segment own = segment_at(bv, pv, ws, line, group, y, end);
-                if (own.t_end - own.t_begin == own.n_unit)
-                    for (int r = slice * ROWS + warp; r < min(own.rows_here, (slice + 1) * ROWS); r += 8) {
-                        const int rg = own.kvh * group * lq + own.row0 + r;
-                        const float v = ws.row_lse2[(size_t)own.lb * rows_total + rg];
-                        if (v != v) row_from_scratch<LAYOUT>(p, own.lb, rg, own.n_doc);
-                    }
-                y += own.t_end - own.t_begin;
-            }
-        }
+        marked |= head.marked != 0;
         const int n_parts = head.n_parts;
         if (n_parts == 0 || slice * ROWS >= head.rows_here) continue;                       // the whole block
         const int run = warp / (8 / kRuns), part_end = n_parts * (run + 1) / kRuns;
@@ -954,9 +1073,9 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 for (int e = 0; e < 16; ++e) mine[(3 + e) * kRunThreads] = acc[e];
             }
             __syncthreads();
-            if (run > 0) continue;
 #pragma unroll
             for (int k = 0; k < kRuns - 1; ++k) {
+                if (run > 0) break;
                 const float* other = &s_run[k][0][threadIdx.x];
                 const float mo = other[0];
                 if (mo == -INFINITY) continue;
@@ -981,10 +1100,12 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 if (lse) lse[(size_t)head.lb * rows_total + rg] = (l > 0.f ? m + log2f(l) : -INFINITY) * kLn2;
             }
         }
-        // marked: out of the range of its reference
-        for (unsigned todo = __ballot_sync(0xffffffffu, valid && l != l && (lane & 7) == 0); todo; todo &= todo - 1)
-            row_from_scratch<LAYOUT>(p, head.lb, __shfl_sync(0xffffffffu, rg, __ffs(todo) - 1), head.n_doc);
+        if (valid && l != l) {                                      // out of the range of its reference
+            marked = true;
+            if ((lane & 7) == 0) atomicOr(&s_marked[u], 1u << (r - slice * ROWS));
+        }
     }
+    if (__syncthreads_or(marked)) marked_from_scratch<LAYOUT, ROWS>(p, s_marked, share0, n_classes, slice);
 }
 
 // Exercises the bounded wait by itself: one CTA initialises an mbarrier that nothing ever arrives on,
@@ -1067,15 +1188,16 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
                             static_cast<In>(k_prefix), static_cast<In>(v_prefix), self_stride, prefix_stride, scale_log2, k_self ? 1 : 0, prefix_len};
     const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
                       k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, static_cast<__nv_bfloat16*>(out), lse};
-    static PerDeviceOnce configured[2];
+    static PerDeviceOnce configured[2], configured_merge[2][2];
     // Few units in many shares each.  Measured (attention and merge of a call, us, 32 rows against 8): 6 units of 25 parts 19.5
     // against 17.0; 24 units of 6 parts 33.0 against 36.2; 32 units of 5 parts 33.1 against 36.6.
     const bool many_parts = (long long)span.n_layers * b->n_requests * g->n_kv_heads * row_tiles * 8 <= shares;
     const int merge_rows = many_parts ? 8 : 32;
     auto run = [&](auto kernel, auto merge, int which) {
         if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return (int)CF_ERR_CUDA;
+        if (configure_smem_once(configured_merge[which][many_parts], merge, kMergeSmem) != CF_OK) return (int)CF_ERR_CUDA;
         const int rc = launch_chained(kernel, dim3((unsigned)shares), kThreads, kSmemBytes, stream, maps, p);
-        return rc != CF_OK ? rc : launch_chained(merge, dim3((unsigned)((shares + 32 / merge_rows - 1) / (32 / merge_rows) * (kRowTile / merge_rows))), 256, 0, stream, p);
+        return rc != CF_OK ? rc : launch_chained(merge, dim3((unsigned)((shares + 32 / merge_rows - 1) / (32 / merge_rows) * (kRowTile / merge_rows))), 256, kMergeSmem, stream, p);
     };
     constexpr int H = CF_ROPE_HALF, I = CF_ROPE_INTERLEAVED;
     if (g->rope_layout == H) return run(attn_tc_kernel<H>, many_parts ? attn_tc_merge_kernel<H, 8> : attn_tc_merge_kernel<H, 32>, 0);

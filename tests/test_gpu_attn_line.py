@@ -16,7 +16,8 @@ def _library():
     cf.load_library()
 
 
-def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_block=False, kept=None, peak=None):
+def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_block=False, kept=None, peak=None,
+                peak_every=1, rope_layout=0):
     """Outputs, log-sum-exps and scores of both kernel families on the same inputs."""
     import paper_2502_11101_b200 as cf
     from paper_2502_11101_b200.session import Session
@@ -27,7 +28,7 @@ def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_b
     rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
     q, k, v = rand(layers, b, q_len, hq, 128), rand(layers, total, hkv, 128), rand(layers, total, hkv, 128)
     if peak is not None:                                     # one key per kv head far above all others for every row
-        q.abs_()
+        q[:, :, ::peak_every].abs_()
         k[:, peak] = 40.0
     ks, vs = rand(layers, b, q_len, hkv, 128), rand(layers, b, q_len, hkv, 128)
     kp, vp = rand(layers, max(prefix, 1), hkv, 128), rand(layers, max(prefix, 1), hkv, 128)
@@ -36,7 +37,7 @@ def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_b
         for path in (1, 0):
             cf.cf_set_attn_path(path)
             sess = Session(hq, hkv, 128, torch.bfloat16, 32768, 1e6, q_len, np.asarray(lens, np.int32), begin,
-                           np.zeros(len(lens), np.int32), tail_reserve=q_len, prefix_len=prefix)
+                           np.zeros(len(lens), np.int32), tail_reserve=q_len, prefix_len=prefix, rope_layout=rope_layout)
             counts = None if kept is None else torch.tensor(kept, dtype=torch.int32, device="cuda")
             sess.init(kept_count=counts)
             out = torch.full_like(q, float("nan"))
@@ -152,3 +153,48 @@ def test_log_sum_exp_of_a_single_key():
     want = rotated[0, 0].double() * 8.0 / np.sqrt(128.0)
     error = (lse[0, 0].double() - want).abs()
     assert bool((error <= 2.0 ** -22 + 8 * 2.0 ** -24 * want.abs()).all()), float(error.max())
+
+
+@pytest.mark.parametrize("rope_layout", [0, 1])
+@pytest.mark.parametrize("heads,q_len,lens,docs,prefix,self_block,every", [
+    ((4, 2), 11, [97, 15, 1, 33, 130, 80], [6], 0, False, 1),        # odd tiles; the last group of rows is not whole
+    ((6, 2), 35, [64, 100, 47], [2, 1], 77, True, 3),                # some rows of a slice; prefix and query tokens as well
+    ((16, 16), 40, [50] * 24, [8, 8, 8], 0, True, 5),                # units finished by one share
+    ((1, 1), 3, [96] * 60, [60], 0, False, 1),                       # one unit in many shares, merged in runs
+])
+def test_rows_computed_from_scratch(heads, q_len, lens, docs, prefix, self_block, every, rope_layout):
+    """Rows that leave the range of their reference beside rows that do not, in every place they can lie."""
+    starts = np.concatenate([[0], np.cumsum(lens)])
+    peak = [int(starts[i + 1]) - 1 for i in range(len(lens)) if i % 2 == 1]
+    _both_paths(heads, q_len, lens, docs, 2, prefix, self_block, peak=peak, peak_every=every, rope_layout=rope_layout)
+
+
+def test_a_row_out_of_range_does_not_stop_the_call():
+    """One kv head whose rows leave the range of their reference: such rows are an exception, not a reason to take two hundred
+    times as long (they were computed by one warp each, a memory latency after the other).  The factor is about twenty."""
+    import paper_2502_11101_b200 as cf
+    from paper_2502_11101_b200.session import Session
+    hq, hkv, q_len, docs, length, layers = 12, 2, 48, 50, 160, 4
+    sess = Session(hq, hkv, 128, torch.bfloat16, 32768, 1e6, q_len, np.full(docs, length, np.int32), np.asarray([0, docs], np.int32),
+                   np.zeros(docs, np.int32), tail_reserve=q_len)
+    sess.init()
+    gen = torch.Generator(device="cuda").manual_seed(0)
+    q = torch.randn(layers, 1, q_len, hq, 128, generator=gen, device="cuda").bfloat16()
+    k = torch.randn(layers, docs * length, hkv, 128, generator=gen, device="cuda").bfloat16()
+    v = torch.randn(layers, docs * length, hkv, 128, generator=gen, device="cuda").bfloat16()
+    out, work = torch.empty_like(q), torch.empty(cf.cf_attn_workspace_bytes_layers(sess.geom, sess.batch, layers), dtype=torch.uint8, device="cuda")
+    times = []
+    for peaked in (False, True):
+        if peaked:
+            q[..., :hq // hkv, :].abs_()
+            k[:, 2 * length - 1, 0] = 40.0
+        best = float("inf")
+        for _ in range(6):
+            begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            begin.record()
+            cf.cf_query_prefill_attn_layers(sess.geom, sess.batch, sess.plan, q, k, v, out, work)
+            end.record()
+            torch.cuda.synchronize()
+            best = min(best, begin.elapsed_time(end))
+        times.append(best)
+    assert sess.status() == 0 and times[1] <= 40 * times[0], times
