@@ -17,8 +17,8 @@
 // epilogue is taken out of the chain.  Rows pass through 2 KB of staging per warp, so that a store instruction writes 64
 // bytes to each of 8 rows: one row per thread in 32-byte pieces kept the warps waiting for 2100 cycles per item.
 // Softmax: one fixed reference per row, the maximum over the item's first 16 keys (every row sees the first one); P and the
-// sums keep their relative precision up to 80 (log2 units) above that maximum.  A row that leaves this range is noted and
-// computed again, alone, when the CTA's items are done.
+// sums keep their relative precision up to 80 (log2 units) above that maximum.  A row that leaves this range ends as not a
+// number and is computed again when the CTA's items are done.
 // Bound by HBM for a few query heads per kv head: with 6 heads and a 64-token prefix 123 flops per byte.
 // Measured (400 documents of 128-192 tokens, 12/2 heads, 4 layers, prefix 64): 660 us before
 // (one issuing thread for copies and MMAs, two passes over S, rows staged through the value buffer), 449 us now; one layer
@@ -28,6 +28,7 @@
 
 #include <algorithm>
 
+#include "cf_row_group.cuh"
 #include "cf_tc_util.cuh"
 
 namespace cf {
@@ -41,7 +42,7 @@ constexpr int kKeys = 64, kKeyChunks = kKeys / 16;           // keys of a tile
 constexpr int kKeyHalf = kKeys * 128, kKeyTile = 2 * kKeyHalf;   // bytes: 64 dims of a tile, a tile
 constexpr int kDocBoxes = 3;                                 // copy boxes of 16, 32 and 64 rows
 constexpr int kItemRing = 8, kSumRing = 4;                   // QK^T runs two tiles, perhaps two items, ahead of PV, and the epilogue one behind
-constexpr int kMarkedMost = 256;
+constexpr int kScratchWarps = 8;                             // of the CTA, that compute rows from scratch
 constexpr float kDocSumLimit = 0x1p80f;                      // see cf_attn_tc.cu
 
 struct DocMaps {
@@ -170,11 +171,10 @@ struct DocShared {
     unsigned long long item_full[kItemRing], sums_full[kSumRing];
     unsigned int tmem_base;
     volatile int abort_flag;
-    int n_marked;
+    int marked;                                               // a row left the range of its reference
     float row_sum[kSumRing][kTile128], row_ref[kSumRing][kTile128];   // sum NaN: the row left the range of its reference
     DocItem item[kItemRing];
-    DocWalk walk;
-    int2 marked[kMarkedMost];                                 // item, row
+    DocWalk walk;                                             // the share's first item
 };
 constexpr int kDocTcSmem = 3 * kTileBytes + (int)sizeof(DocShared) + 1024;   // Q, K, V tiles
 static_assert(2 * (kDocTcSmem + 1024) <= 228 * 1024, "two CTAs per SM");
@@ -187,40 +187,101 @@ struct DocParams {
     float* lse;
     int* status;
 };
-// One row of an item by one warp, keys one after the other under a running maximum.
-__device__ __noinline__ void doc_row_from_scratch(const DocParams& p, int w, int r) {
-    const int lane = threadIdx.x & 31;
+// What a warp that computes rows from scratch holds in the shared memory of the tiles.
+struct DocScratch {
+    rows::Queries q;
+    rows::Stage stage;
+};
+static_assert(kScratchWarps * sizeof(DocScratch) <= 3 * kTileBytes, "fits the tiles' memory");
+
+// Up to eight rows (r0 + every set bit of `set`) of an item by one warp, under a running maximum.
+__device__ __noinline__ void doc_rows_from_scratch(const DocParams& p, DocScratch& sh, int w, int r0, unsigned set) {
+    const int lane = threadIdx.x & 31, group = p.dg.group, n_rows = __popc(set);
     const DocItem it = doc_item(p.a, p.dg, w);
-    const int row = it.r0 + r, token = row / p.dg.group, h = it.kvh * p.dg.group + row - token * p.dg.group;
-    auto load = [&](const __nv_bfloat16* e, float (&x)[4]) {
-        const uint2 u = *reinterpret_cast<const uint2*>(e + lane * 4);
-        x[0] = __uint_as_float(u.x << 16);
-        x[1] = __uint_as_float(u.x & 0xffff0000u);
-        x[2] = __uint_as_float(u.y << 16);
-        x[3] = __uint_as_float(u.y & 0xffff0000u);
+    // of a row of the group: its token, and where it lies among the document's rows of queries
+    auto token_of = [&](int n) { return (it.r0 + r0 + rows::nth_bit(set, n)) / group; };
+    auto place_of = [&](int n) {
+        const int row = it.r0 + r0 + rows::nth_bit(set, n), token = row / group;
+        return (size_t)(it.row_first + token) * p.a.n_q_heads + it.kvh * group + row - token * group;
     };
-    const size_t at = ((size_t)(it.row_first + token) * p.a.n_q_heads + h) * kD;
-    float q[4], acc[4] = {0.f, 0.f, 0.f, 0.f}, m = -INFINITY, l = 0.f;
-    load(p.q + (size_t)it.layer * p.a.q_layer_stride + at, q);
-    for (int i = 0; i < p.dg.prefix_len + token + 1; ++i) {
-        const size_t off = i < p.dg.prefix_len ? (size_t)it.layer * p.a.prefix_layer_stride + ((size_t)i * p.a.n_kv_heads + it.kvh) * kD
-                                               : (size_t)it.layer * p.a.kv_layer_stride + (size_t)(it.row_first + i - p.dg.prefix_len) * p.a.token_stride + it.kvh * kD;
-        float k[4], v[4];
-        load((i < p.dg.prefix_len ? p.kp : p.k) + off, k);
-        load((i < p.dg.prefix_len ? p.vp : p.v) + off, v);
-        float dot = fmaf(q[0], k[0], fmaf(q[1], k[1], fmaf(q[2], k[2], q[3] * k[3])));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-        const float s = dot * p.a.scale_log2, m_new = fmaxf(m, s), alpha = exp2f(m - m_new), e = exp2f(s - m_new);
-#pragma unroll
-        for (int x = 0; x < 4; ++x) acc[x] = fmaf(acc[x], alpha, e * v[x]);
-        l = fmaf(l, alpha, e);
-        m = m_new;
+    for (int i = 0; i < rows::kGroupRows; i += 2) {
+        const int r = i + (lane >> 4);
+        sh.q.put(r, lane & 15, p.q + (size_t)it.layer * p.a.q_layer_stride + place_of(r) * kD);
     }
-    const float inv = 1.f / l;
-    *reinterpret_cast<uint2*>(p.out + (size_t)it.layer * p.a.out_layer_stride + at + lane * 4) =
-        make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
-    if (lane == 0 && p.lse) p.lse[((size_t)it.layer * p.a.n_q_heads + h) * p.a.total_tokens + it.row_first + token] = (m + log2f(l)) * kLn2;
+    const int token = token_of(lane >> 2), n_tokens = token_of(n_rows - 1) + 1;    // rows are numbered token by token
+    const int prefix_steps = (p.dg.prefix_len + rows::kStepKeys - 1) / rows::kStepKeys;
+    const int steps = prefix_steps + (n_tokens + rows::kStepKeys - 1) / rows::kStepKeys;
+    auto copy = [&](auto& to, const __nv_bfloat16* prefix, const __nv_bfloat16* tokens, int s) {
+        if (s < prefix_steps) {
+            const int i = s * rows::kStepKeys;
+            const size_t pitch = (size_t)p.a.n_kv_heads * kD;
+            rows::copy_step(to, prefix + (size_t)it.layer * p.a.prefix_layer_stride + i * pitch + it.kvh * kD, pitch, p.dg.prefix_len - i);
+        } else if (s < steps) {
+            const int i = (s - prefix_steps) * rows::kStepKeys;
+            rows::copy_step(to, tokens + (size_t)it.layer * p.a.kv_layer_stride + (size_t)(it.row_first + i) * p.a.token_stride + it.kvh * kD,
+                            (size_t)p.a.token_stride, n_tokens - i);
+        }
+        rows::copies_end();
+    };
+    rows::Group acc;
+    acc.clear();
+    copy(sh.stage.k, p.kp, p.k, 0);
+    copy(sh.stage.v, p.vp, p.v, 0);
+    for (int s = 0; s < steps; ++s) {
+        const int i = (s < prefix_steps ? s : s - prefix_steps) * rows::kStepKeys;
+        rows::Keys keys;
+        rows::copies_wait();
+        keys.read(sh.stage);
+        __syncwarp();                                               // every lane has its fragments
+        copy(sh.stage.k, p.kp, p.k, s + 1);
+        float alpha;
+        acc.scores(sh.q, keys, (s < prefix_steps ? p.dg.prefix_len : token + 1) - i, p.a.scale_log2, alpha);
+        rows::copies_wait();
+        acc.values(sh.stage);
+        __syncwarp();
+        copy(sh.stage.v, p.vp, p.v, s + 1);
+    }
+    const float l = rows::over_keys(acc.l), inv = 1.f / l;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {                                   // rows 2 t and 2 t + 1
+        const int r = 2 * (lane & 3) + x;
+        const float f = __shfl_sync(0xffffffffu, inv, 4 * r);
+        __nv_bfloat16* out = p.out + (size_t)it.layer * p.a.out_layer_stride + place_of(r) * kD + 8 * (lane >> 2);
+        if (r < n_rows)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<uint32_t*>(out + (i >> 2) * 64 + 2 * (i & 3)) = pack_bf16(acc.o[i][x] * f, acc.o[i][x + 2] * f);
+    }
+    if ((lane & 3) == 0 && (lane >> 2) < n_rows && p.lse) {
+        const size_t place = place_of(lane >> 2);
+        const int h = (int)(place % p.a.n_q_heads);
+        p.lse[((size_t)it.layer * p.a.n_q_heads + h) * p.a.total_tokens + it.row_first + token] = (acc.m + log2f(l)) * kLn2;
+    }
+    __syncwarp();                                                   // the queries have been read
+}
+
+// Rows that left the range of their reference, by one of kScratchWarps warps: the share's items are walked once more, the rows that
+// are not numbers computed by groups of eight in the memory of the tiles (whose copies and readers are done).  Other rows keep
+// what they have, whatever their neighbours' keys are.  Measured (400 documents of 128-192 tokens, 12/2 heads, four layers, 446 us
+// without such rows): a key far above the others in one kv head of every tenth document 74 -> 1.3 ms, in every document and head
+// 74 -> 6.2 ms, against a warp per row, key after key, and with more than 256 such rows in a CTA all of its rows.
+__device__ __noinline__ void doc_marked_from_scratch(const DocParams& p, DocScratch& sh, DocWalk walk) {
+    const DocGrid& dg = p.dg;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int turn = 0; walk.pos < walk.end; walk_next(p.a, dg, walk)) {
+        const DocItem it = doc_item(p.a, dg, walk.layer, walk.doc, walk.kvh, walk.x);
+        for (int r0 = 0; r0 < it.rows_here; r0 += 32) {
+            if (turn++ % kScratchWarps != warp) continue;
+            const int row = it.r0 + min(r0 + lane, it.rows_here - 1), token = row / dg.group;
+            const size_t place = (size_t)(it.row_first + token) * p.a.n_q_heads + it.kvh * dg.group + row - token * dg.group;
+            const float first = __bfloat162float(p.out[(size_t)it.layer * p.a.out_layer_stride + place * kD]);
+            for (unsigned set = __ballot_sync(0xffffffffu, first != first && r0 + lane < it.rows_here); set;) {
+                const unsigned now = rows::next_group(set);
+                doc_rows_from_scratch(p, sh, it.w, r0, now);
+                set ^= now;
+            }
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kDocTcThreads, 2)
@@ -255,7 +316,7 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
             mbar_init(smem_u32(&sh->o_free), 4);
             for (int i = 0; i < kItemRing; ++i) mbar_init(smem_u32(&sh->item_full[i]), 1);
             sh->abort_flag = 0;
-            sh->n_marked = 0;
+            sh->marked = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();
@@ -489,10 +550,7 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
                 if (p.lse)
                     p.lse[((size_t)it.layer * p.a.n_q_heads + it.kvh * group + row - token * group) * p.a.total_tokens + it.row_first + token] =
                         (sh->row_ref[n % kSumRing][r] + log2f(sum)) * kLn2;
-                if (sum != sum) {
-                    const int m = atomicAdd(&sh->n_marked, 1);
-                    if (m < kMarkedMost) sh->marked[m] = make_int2(it.w, r);
-                }
+                if (sum != sum) sh->marked = 1;                         // its output row is not a number either
             }
             ok = warp_wait(smem_u32(&sh->o_full), n & 1, abort_flag);
             if (!ok) break;
@@ -544,15 +602,7 @@ docattn_tc_kernel(const __grid_constant__ DocMaps maps, const __grid_constant__ 
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
     }
-    const int n_marked = sh->n_marked;
-    if (n_marked <= kMarkedMost) {
-        for (int i = warp; i < n_marked; i += kDocTcThreads / 32) doc_row_from_scratch(p, sh->marked[i].x, sh->marked[i].y);
-    } else {                                                        // more than the list holds: every row of this CTA
-        for (DocWalk walk = sh->walk; walk.pos < walk.end; walk_next(p.a, dg, walk)) {
-            const DocItem it = doc_item(p.a, dg, walk.layer, walk.doc, walk.kvh, walk.x);
-            for (int r = warp; r < it.rows_here; r += kDocTcThreads / 32) doc_row_from_scratch(p, it.w, r);
-        }
-    }
+    if (sh->marked && !sh->abort_flag && warp < kScratchWarps) doc_marked_from_scratch(p, reinterpret_cast<DocScratch*>(smem)[warp], sh->walk);
 }
 
 }  // namespace

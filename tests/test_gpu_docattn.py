@@ -191,3 +191,31 @@ def test_log_sum_exp_of_a_single_key():
     want = torch.diagonal(k[0].double(), dim1=0, dim2=2) * 8.0 / np.sqrt(128.0)
     error = (lse[0].double() - want).abs()
     assert bool((error <= 2.0 ** -22 + 8 * 2.0 ** -24 * want.abs()).all()), float(error.max())
+
+
+@pytest.mark.parametrize("every", [2, 12])
+def test_rows_do_not_depend_on_the_range_of_others(every):
+    """Rows of some documents leave the range of their reference, a few or very many per CTA: the other documents' results are,
+    bit for bit, those of a call without such rows."""
+    lens, hq, hkv, prefix = [97, 128, 40, 150] * 60, 12, 2, 33
+    total, off = sum(lens), np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rand(1, total, hq, 128), rand(1, total, hkv, 128), rand(1, total, hkv, 128)
+    kp, vp = rand(1, prefix, hkv, 128), rand(1, prefix, hkv, 128)
+    geom = cf.make_geom(hq, hkv, 128, torch.bfloat16, 4096, 1e4)
+    others = torch.ones(total, dtype=torch.bool, device="cuda")
+    results = []
+    for with_peaks in (False, True):
+        if with_peaks:
+            for d in range(3, len(lens), every):
+                others[off[d]:off[d + 1]] = False
+                q[:, off[d]:off[d + 1]].abs_()
+                k[:, int(off[d]) + 20] = 40.0
+        out, lse = torch.full_like(q, float("nan")), torch.full((1, hq, total), float("nan"), device="cuda")
+        cf.cf_document_prefill_attn(geom, torch.from_numpy(off).cuda(), max(lens), q, k, v, out, kp, vp, lse)
+        torch.cuda.synchronize()
+        results.append((out, lse))
+    assert torch.equal(results[0][0][:, others], results[1][0][:, others])
+    assert torch.equal(results[0][1][:, :, others], results[1][1][:, :, others])
+    assert not bool(torch.isnan(results[1][0]).any()) and float(results[1][1].max()) > 100.0
