@@ -1,11 +1,14 @@
 """Thin binding of libcachefocus.so: same names as the C ABI, argument marshalling only.  The calls a serving loop issues
-per layer or per token are marshalled natively (csrc/binding.cpp), the others through ctypes.
+per layer or per token are marshalled natively (csrc/binding.cpp; where that has not been built, marshal_ctypes.py), the others
+through ctypes.
 
 Tensors are torch tensors used purely as device (or host) buffers; every step of the path runs
 in the library's kernels."""
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import List, Optional, Sequence, Tuple
 
@@ -165,13 +168,24 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+def _load_native(path: str):
+    """The native marshalling module at `path`, None where it has not been built for this torch and Python."""
+    if not os.path.exists(path):
+        return None
+    loader = importlib.machinery.ExtensionFileLoader(__package__ + "._native", path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
+    loader.exec_module(module)
+    return module
+
+
 def _native():
-    """The native marshalling module (built next to the library; there is no fallback)."""
+    """What marshals the hot calls: the native module built next to the library, or the same calls through ctypes.  Both end in
+    the library, which has to be there."""
     global _NATIVE
     if _NATIVE is None:
         load_library()
-        from . import _native as module
-        _NATIVE = module
+        from . import build, marshal_ctypes
+        _NATIVE = _load_native(build.NATIVE_PATH) or marshal_ctypes
     return _NATIVE
 
 

@@ -5,12 +5,16 @@ import glob
 import os
 import shutil
 import subprocess
+import sys
 import sysconfig
+import warnings
+from importlib import metadata
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
 LIB_PATH = os.path.join(PKG_DIR, "libcachefocus.so")
-NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
+# the native part of the binding uses torch's and Python's C++ interfaces: a module built for others is another file
+NATIVE_PATH = os.path.join(PKG_DIR, "_native-torch%s-%s.so" % (metadata.version("torch"), sys.implementation.cache_tag))
 NATIVE_SOURCE = os.path.join(PKG_DIR, "csrc", "binding.cpp")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "--threads", "0"]
@@ -44,7 +48,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose:
             print(log)
     if force or _stale(NATIVE_PATH, [NATIVE_SOURCE] + headers):
-        build_native()
+        try:
+            build_native()
+        except (RuntimeError, OSError) as e:             # no g++, no torch headers: the binding goes through ctypes
+            if os.path.exists(NATIVE_PATH):
+                os.remove(NATIVE_PATH)                   # built from other sources
+            warnings.warn("the native part of the binding was not built (%s); calls are marshalled by ctypes" % e)
     return LIB_PATH
 
 

@@ -244,3 +244,82 @@ def test_slot_call_with_further_key_blocks_checks_its_arguments_on_the_host(lib)
     assert call(k_prefix=None) == cf.CF_ERR_INVALID_ARG
     assert call(slot=4) == cf.CF_ERR_INVALID_ARG and call(prefix_len=-1) == cf.CF_ERR_INVALID_ARG
     assert call(nbytes=full - 1) == cf.CF_ERR_WORKSPACE
+
+
+# ---- the two ways of marshalling the hot calls
+
+HOT_CALLS = ["plan_init", "prune_topk", "reposition_keys", "query_prefill_attn", "query_prefill_attn_slot", "accumulate_scores",
+             "assemble_final_cache", "document_prefill_attn", "decode_plan", "decode_attn", "decode_append", "run_stack"]
+
+
+def _marshallers():
+    from paper_2502_11101_b200 import binding, marshal_ctypes
+    native = binding._load_native(cf_build.NATIVE_PATH)
+    assert native is not None
+    return native, marshal_ctypes
+
+
+def test_calls_go_through_ctypes_where_the_native_module_is_missing(lib, tmp_path, monkeypatch):
+    """Without g++ or torch's headers the library is still usable: the build says so and the binding marshals by ctypes."""
+    from paper_2502_11101_b200 import binding, marshal_ctypes
+    assert binding._load_native(str(tmp_path / "none.so")) is None
+    monkeypatch.setattr(cf_build, "NATIVE_PATH", str(tmp_path / "_native.so"))
+    monkeypatch.setattr(binding, "_NATIVE", None)
+    monkeypatch.setattr(cf_build, "build_native", lambda: (_ for _ in ()).throw(RuntimeError("g++ failed")))
+    with pytest.warns(UserWarning, match="ctypes"):
+        assert cf_build.build() == cf_build.LIB_PATH
+    assert binding._native() is marshal_ctypes
+
+
+def test_a_native_module_of_another_torch_is_not_the_one_loaded():
+    import sys
+    import torch
+    assert torch.__version__ in cf_build.NATIVE_PATH and sys.implementation.cache_tag in cf_build.NATIVE_PATH
+
+
+def test_both_marshallers_have_the_same_calls(lib):
+    native, through_ctypes = _marshallers()
+    for name in HOT_CALLS:
+        assert callable(getattr(native, name)) and callable(getattr(through_ctypes, name))
+
+
+def test_both_marshallers_refuse_the_same_calls(lib):
+    """Every case ends on the host: with the same error code, or the same kind of exception for arguments that contradict each
+    other."""
+    import torch
+    geom = cf.make_geom(4, 2, 128, cf.CF_BF16, 4096, 1e4)
+    fake = 256
+    batch = cf.cf_batch(1, 3, 8, 0, 8, 0, 0, 0, 300, 2 * 128, fake, fake, fake)
+    small, ints = torch.zeros(256, dtype=torch.uint8), torch.zeros(4, dtype=torch.int32)
+    x, y = torch.zeros(2, 1, 8, 4, 128, dtype=torch.bfloat16), torch.zeros(2, 300, 2, 128, dtype=torch.bfloat16)
+    one = torch.zeros(1, 300, 2, 128, dtype=torch.bfloat16)
+    f = torch.zeros(8)
+    cases = [
+        ("plan_init", (geom, batch, small[1:], None, None, -1, None, 0)),                     # misaligned plan
+        ("plan_init", (geom, batch, small, None, None, 1 << 20, f, 0)),                       # too small
+        ("prune_topk", (geom, batch, small, f, -1, None, 1, 0)),                              # no number of documents to keep
+        ("reposition_keys", (geom, batch, small, y, y, 0, 0, 0)),                             # no layers
+        ("query_prefill_attn", (geom, batch, small, x, y, y, x, small, None, None, None, -1.0, 0)),
+        ("query_prefill_attn_slot", (geom, batch, small, 9, 4, x, y, y, x, small, None, 0.0, 0)),
+        ("accumulate_scores", (geom, batch, small, 5, 4, small, None, f, 0)),
+        ("assemble_final_cache", (geom, batch, small, y, y, y, y, y[:, ::2], y[:, ::2], ints, 0)),
+        ("assemble_final_cache", (geom, batch, small, y, y, y, y, one[None], one[None], f, 0)),
+        ("document_prefill_attn", (geom, f, 10, x[:, 0], y, y, x[:, 0], None, None, None, 0.0, None, None, 0)),
+        ("document_prefill_attn", (geom, ints, -1, x[:, 0], y, y, x[:, 0], None, None, None, 0.0, None, None, 0)),
+        ("decode_plan", (geom, 1, 300, ints, 0, small, 0)),
+        ("decode_attn", (geom, 1, 300, small, x[:, 0, :1], one, one, x[:, 0, :1], small, None, 0.0, 0)),
+        ("decode_attn", (geom, 0, 300, small, x[:1, 0, :1], one, one, x[:1, 0, :1], small, None, 0.0, 0)),
+        ("decode_append", (geom, 1, 300, one[None], one[None], ints, -1, one[None], one[None], None, 0)),
+        ("run_stack", (geom, batch, small, small, x, one, one, x, f, [], 1, True, None, None, None, None, None, 0.0, None, None,
+                       None, None, 0)),
+        ("run_stack", (geom, batch, small, small, x, y, y, x, f, [(1, 2)], 1, True, None, None, None, None, None, 0.0, None, None,
+                       None, None, 0)),                                                       # the workspace it asks for
+    ]
+    for name, args in cases:
+        got = []
+        for m in _marshallers():
+            try:
+                got.append(getattr(m, name)(*args))
+            except AssertionError:
+                got.append(AssertionError)
+        assert got[0] == got[1] and got[0] not in (0, (0, 0)), (name, got)

@@ -235,3 +235,45 @@ def test_steps_queued_behind_one_another(graph):
         results.append((out, lse))
     assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
     assert not bool(torch.isnan(results[0][1]).any())
+
+
+def test_both_marshallers_give_the_same_results(monkeypatch):
+    """A stack, its final caches, a decoding step and cache construction with the calls marshalled natively and by ctypes."""
+    from paper_2502_11101_b200 import binding, build, marshal_ctypes
+    from paper_2502_11101_b200.session import Session
+    native = binding._load_native(build.NATIVE_PATH)
+    assert native is not None
+    L, B, q_len, hq, hkv = 3, 2, 5, 4, 2
+    lens, begin = np.asarray([40, 97, 20, 130, 64], np.int32), np.asarray([0, 3, 5], np.int32)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rand(L, B, q_len, hq, 128), rand(L, int(lens.sum()), hkv, 128), rand(L, int(lens.sum()), hkv, 128)
+    ks, vs, qd = rand(L, B, q_len, hkv, 128), rand(L, B, q_len, hkv, 128), rand(L, B, hq, 128)
+    kn, vn, qt = rand(L, B, hkv, 128), rand(L, B, hkv, 128), rand(L, int(lens.sum()), hq, 128)
+    results = []
+    for module in (native, marshal_ctypes):
+        monkeypatch.setattr(binding, "_NATIVE", module)
+        room = int(lens.sum()) + q_len + 1
+        sess = Session(hq, hkv, 128, torch.bfloat16, 32768, 1e6, q_len, lens, begin, np.zeros(5, np.int32), tail_reserve=q_len)
+        out, outs, lse = torch.zeros_like(q), torch.zeros_like(q), torch.zeros(L, B, hq, q_len, device="cuda")
+        scores = torch.zeros(L, 5, device="cuda")
+        sess.run_stack(q, k, v, [(1, 2)], 1, out, lse, layer_scores=scores)
+        sess.run_stack(q, k, v, [(1, 2)], 1, outs, driver="calls")
+        k_cache, v_cache = (torch.zeros(L, B, room, hkv, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        rows = torch.zeros(B, dtype=torch.int32, device="cuda")
+        sess.assemble(k, v, ks, vs, k_cache, v_cache, rows)
+        moved = torch.zeros_like(k)
+        sess.reposition(k, moved, L, k.stride(0))
+        plan = torch.zeros(cf.cf_decode_plan_bytes(sess.geom, B, room), dtype=torch.uint8, device="cuda")
+        work = torch.zeros(cf.cf_decode_workspace_bytes(sess.geom, B, room, L), dtype=torch.uint8, device="cuda")
+        token, token_lse = torch.zeros_like(qd), torch.zeros(L, B, hq, device="cuda")
+        cf.cf_decode_plan(sess.geom, B, room, rows, 1, plan)
+        cf.cf_decode_append(sess.geom, B, room, k_cache, v_cache, rows, 0, kn, vn)
+        cf.cf_decode_attn(sess.geom, B, room, plan, qd, k_cache, v_cache, token, work, token_lse)
+        built, off = torch.zeros_like(qt), torch.from_numpy(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)).cuda()
+        cf.cf_document_prefill_attn(sess.geom, off, int(lens.max()), qt, k, v, built)
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        results.append((out, outs, lse, scores, sess.score_accum.clone(), k_cache, v_cache, rows, moved, token, token_lse, built))
+    for a, b in zip(*results):
+        assert torch.equal(a, b) and float(a.float().abs().max()) > 0
