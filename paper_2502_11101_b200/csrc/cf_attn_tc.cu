@@ -113,8 +113,10 @@ struct Segment {
     int t_begin, t_end, n_unit, n_doc, tile0;      // tiles of the unit this segment covers; documents' tiles; first in the plan
 };
 
-// A share has at least two tiles: at one layer per call, 28 calls of a small request take 582 us a pass with 1 or 2, 611 / 635 /
-// 676 / 753 with 3 / 4 / 6 / 8 (a longer share costs more than the parts it saves); larger calls do not notice.
+// A share has at least two tiles.  Measured, attention and merge of a call (us, a least of 1 / 2 / 3 / 4; larger calls do not
+// notice): 25 documents of 160 tokens, 12/2 heads 16.9 / 16.9 / 19.4 / 21.2; 6 documents 14.0 / 14.0 / 14.5 / 14.8; 20 documents of
+// 90, 32/8 heads 15.3 / 14.8; 3 of 180, 32/32 heads 13.8 / 12.8; units of three and five tiles, which two do not divide: 3 and 5 of
+// 90, 32/8 heads 12.5 / 15.6 and 13.3 / 16.1.  Three and more cost parallelism, between one and two it is even.
 constexpr int kMinShare = 2;
 
 // What the line is made from: prefix sums of the requests' tiles (one entry per `stride` requests), and with one entry per
@@ -977,7 +979,6 @@ __device__ __noinline__ void marked_from_scratch(const Params& p, const unsigned
 // what a block has to know about the unit was left by the CTA that began it, and four parts of a row are loaded together.
 // ROWS = 32: a block has 32 rows of one share's unit.  ROWS = 8: it has 8 rows of the units of four shares (of which few have
 // one), and the parts of a row are cut into four runs, walked side by side and joined in order through shared memory.
-// Measured (one layer of 25 documents, 12/2 heads, with the attention): 19.5 us with 32 rows, 17.0 us with 8.
 template <int LAYOUT, int ROWS>
 __global__ void __launch_bounds__(256, 2)
 attn_tc_merge_kernel(const __grid_constant__ Params p) {
@@ -1189,9 +1190,10 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
     const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
                       k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, static_cast<__nv_bfloat16*>(out), lse};
     static PerDeviceOnce configured[2], configured_merge[2][2];
-    // Few units in many shares each.  Measured (attention and merge of a call, us, 32 rows against 8): 6 units of 25 parts 19.5
-    // against 17.0; 24 units of 6 parts 33.0 against 36.2; 32 units of 5 parts 33.1 against 36.6.
-    const bool many_parts = (long long)span.n_layers * b->n_requests * g->n_kv_heads * row_tiles * 8 <= shares;
+    // Few units in many shares each: from thirteen parts to a unit on.  Measured (attention and merge of a call over 50 documents of
+    // 160 tokens, us, 32 rows against 8): 2 units (50 parts) 25.7 / 17.5; 6 (25) 22.2 / 18.8; 8 (18) 26.4 / 24.9; 10 (15) 24.3 /
+    // 23.3; 12 (12) 25.3 / 26.4 and 26.4 / 27.7; 14 (11) 25.1 / 25.1; 16 (9) 26.7 / 28.2; 24 (6) 32.4 / 34.9; 48 (3) 38.9 / 42.2.
+    const bool many_parts = (long long)span.n_layers * b->n_requests * g->n_kv_heads * row_tiles * 13 <= shares;
     const int merge_rows = many_parts ? 8 : 32;
     auto run = [&](auto kernel, auto merge, int which) {
         if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return (int)CF_ERR_CUDA;

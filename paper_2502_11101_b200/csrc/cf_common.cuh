@@ -116,7 +116,7 @@ struct AttnWorkspace {
     float* part_l;     // [L*B][n_splits][Hq*Lq]    sum_t 2^(t - m)
     float* tile_lse2;  // [L][max_tiles][Hq*Lq]     log2 of sum over the tile's tokens of 2^t
     float* row_lse2;   // [L*B][Hq*Lq]              log2 of the full softmax denominator
-    int* marks;        // [shares]                  tensor-core path: a unit of the share has rows to be computed from scratch
+    int* marks;        // [shares][8]               tensor-core path: what a share leaves for the merge (ShareHead, cf_attn_tc.cu)
     int n_splits;
     int n_layers;
     int max_tiles;     // tile slots per layer in tile_lse2

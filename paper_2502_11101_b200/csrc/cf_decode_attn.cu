@@ -531,9 +531,13 @@ int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_l
                           static_cast<__nv_bfloat16*>(out), lse, doc_offsets, span.q_stride, span.kv_stride, span.out_stride, n_requests,
                           cache_rows, g->n_q_heads, g->n_kv_heads, row_tiles, scale_log2, part_o, part_m, part_l, unit_parts};
     const long long units = decode_units(g, n_requests, n_layers);
-    // A cluster per unit where one wave of clusters leaves a warp a few steps (measured, us per layer, cluster against
-    // stream: 1011 rows, 2 units 5.5 / 8.1; 1984 rows, 16 units 10.1 / 11.5; 500 rows, 128 units 11.1 / 13.4), the
-    // stream of equal shares for everything longer (5000 rows, 16 units 16.2 / 13.3; 2764 rows, 256 units 59 / 45.6).
+    // A cluster per unit where one wave of clusters leaves a warp a few steps, the stream of equal shares for everything longer;
+    // the line is eight steps.  Measured (us per layer with the append, cold, cluster against stream, the steps of a warp in
+    // brackets): 2 units, 1000 rows (2) 9.6 / 12.4, 2000 (4) 11.9 / 12.2, 3000 (6) 14.1 / 12.1; 8 units, 2000 (4) 12.4 / 13.2, 3000 (6)
+    // 14.7 / 13.7; 16 units, 3000 (6) 14.0 / 15.2, 4000 (8) 17.5 / 17.0; 32 units, 3000 (6) 18.8 / 19.1, 4000 (8) 21.6 / 21.6; 256
+    // units, 500 (8) 20.5 / 21.5, 750 (12) 24.0 / 23.6, 2000 (31) 48.5 / 44.7.  So the two meet at four steps for a few units and
+    // at ten for many.  What the rule sees is the slot, not the rows in use, which are known on the device only: 1011 rows of 2
+    // units take 8.1 us in a slot of 1075 rows and 10.1 in one of 20 000.
     int cluster = 1;
     while (cluster < kMaxCluster && units * cluster * 2 <= shares) cluster *= 2;
     bool stream_k = cache_rows > kStepKeys * kDecWarps * cluster * 8;

@@ -81,7 +81,10 @@ __device__ __forceinline__ DocItem doc_item(const DocAttnArgs& a, const DocGrid&
 // The items of all layers, documents and kv heads lie on a line, each as long as its estimated cost, kItemCost + its keys;
 // a CTA takes those that start in its equal share of the line.  Items dealt out in turn instead leave the slowest of 296 CTAs
 // with 1.75 times the mean (60 ragged documents with 32 heads), since neighbours on a CTA come from row tiles of like number.
-// kItemCost is what an item costs beside its keys, in keys: the first QK^T, the last PV and the epilogue.
+// kItemCost is what an item costs beside its keys, in keys: the first QK^T, the last PV and the epilogue.  Measured (us, for 0 /
+// 128 / 256 / 512 / 1024): 60 documents of 47-391 tokens, 32/32 heads 136 / 110 / 114 / 114 / 120; 40 of 24-400, 32/8, two layers
+// 120 / 89 / 92 / 93 / 97; 30 of 300-400, 12/2, eight layers 194 / 191 / 191 / 196 / 200; 400 of 128-192, 12/2, four layers 447 /
+// 443 / 443 / 445 / 446: what it stands for matters, its value between 128 and 512 does not.
 constexpr int kItemCost = 256;
 struct DocWalk {
     int layer, doc, kvh, x, tiles, len;                       // the current item; row tiles and tokens of its document
