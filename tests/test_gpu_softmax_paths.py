@@ -1,5 +1,5 @@
-"""Parity of paths the diffuse synthetic workloads leave cold: the single-pass softmax moving its
-reference maximum (peaked attention), a caller-chosen softmax scale, a store with padded rows, the
+"""Parity of paths the diffuse synthetic workloads leave cold: logits far above the ones the
+single-pass softmax takes its reference from (peaked attention), a caller-chosen softmax scale, a store with padded rows, the
 "sort" allocation with several parallel windows on the tensor-core path, both stack drivers, and the
 bounded device-side wait.  Everything is compared with the fp64 oracle through the C ABI."""
 import numpy as np
@@ -23,15 +23,15 @@ def _library():
 
 
 def _peaked_inputs(meta, seed, self_level=0.0):
-    """Inputs whose logits sit on a few well separated levels, so that a row's running reference of the
-    softmax has to move several times, in the middle of a key tile and from tile to tile, while the keys
-    met before the move still carry a visible part of the result.
+    """Inputs whose logits sit on a few well separated levels: a running reference of the softmax would have
+    to move several times, in the middle of a key tile and from tile to tile, a fixed one (the maximum over a
+    unit's first keys) is left behind by 10 to 30 log2 units, well inside its range, while the lower levels still
+    carry a visible part of the result.  (Rows that leave the range: tests/test_gpu_attn_line.py.)
 
     Per (layer, request, kv head) a unit direction u; query rows a*u + noise with a in [6, 10]; a key
     that should score `level` (log2 units for a = 8) is level/(8*scale*log2 e) * u + noise, counter-
     rotated by the document's delta so that the library's re-positioning brings it back onto u.
-    Most keys are on level 0, about one in 20 on the second level (8.5 higher: just above the
-    threshold of the kernel for a = 8, below it for small a), one per request and layer on the third.
+    Most keys are on level 0, about one in 20 on the second level (8.5 higher), one per request and layer on the third.
     Values carry a level-dependent constant, so every level is visible in the output.
     With `self_level` the query tokens' own keys get one spike on that level (the largest logit then
     sits in the causal query-self block)."""
