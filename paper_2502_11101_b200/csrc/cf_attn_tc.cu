@@ -30,6 +30,7 @@
 // roles leave their loops, and the CTA frees its tensor memory and exits.  Each barrier has one kind of waiter, which waits
 // for every phase in order.
 #include <algorithm>
+#include <cstddef>
 
 #include "cf_row_group.cuh"
 #include "cf_tc_util.cuh"
@@ -257,125 +258,131 @@ struct Params {
     float* const lse = p.lse
 
 // Shared memory of a merge block that computes rows from scratch.
+struct RowTile {                   // where a key tile lies; row j of the query sees its keys up to j - first
+    const __nv_bfloat16 *k, *v;
+    const float2* trig;            // null: not a document's
+    long long pitch;
+    int len, first, index;
+};
+struct RowJob {
+    int lb, layer, b, kvh, n_doc, rg0;
+    unsigned set;                  // of rows rg0 .. that are still to be computed
+    int u, x, end;                 // share of the block, and its positions that are still to be looked at
+};
 struct RowScratch {
+    volatile RowJob job;           // what all warps know and none has registers for
+    int row[rows::kGroupRows];     // the group
     rows::Stage stage[8];          // of every warp
-    alignas(16) rows::Queries q;
+    RowTile tile[8][2];            // the current tile and the next one (registers are what the keys and sums need)
+    rows::Queries q;
     alignas(16) float o[rows::kGroupRows][kD];
     float m[8][rows::kGroupRows], l[8][rows::kGroupRows], docs[8][rows::kGroupRows];   // of every warp
     Requests requests;
+    Line line;
 };
 
 // Up to eight query rows (rg0 + every set bit of `set`, of one kv head) by a block of eight warps, each with every eighth key tile
 // under a running maximum of its own: outputs, log-sum-exps and those of the document tiles.  Only rows whose logits left the
 // range of the shared reference come here (keys that are not finite lead here too).  Bound by the instructions and mma.sync of a
-// step, 2 us for eight rows.  Measured with a warp per row and key after key, and this way: four layers of 50 documents of 160
-// tokens, 12/2 heads, 44 us without such rows, one row a layer 3.0 -> 0.19 ms, every row 10.1 -> 0.83 ms; one layer of 2 x 60
-// documents of 180, 32/32 heads, 93 us without, one row 6.1 -> 0.29, every row 27.1 -> 1.2 ms.
+// step, just under 2 us for eight rows.  Measured with a warp per row and key after key, and this way: four layers of 50 documents
+// of 160 tokens, 12/2 heads, 44 us without such rows, one row a layer 3.0 -> 0.17 ms, every row 10.1 -> 0.71 ms; one layer of
+// 2 x 60 documents of 180, 32/32 heads, 93 us without, one row 6.1 -> 0.27, every row 27.1 -> 1.1 ms.
 template <int LAYOUT>
-__device__ __noinline__ void rows_from_scratch(const Params& p, RowScratch& sh, int lb, int rg0, unsigned set, int n_doc) {
+__device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& sh) {
     CF_PARAMS;
-    const int n_prefix = (src.prefix_len + kTile - 1) / kTile, n_self = src.with_self ? (bv.q_len + kTile - 1) / kTile : 0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lq = bv.q_len, group = n_q_heads / n_kv_heads, rows_total = n_q_heads * lq;
-    const int layer = lb / bv.n_requests, b = lb - layer * bv.n_requests, n_rows = __popc(set);
-    const int rg = rg0 + rows::nth_bit(set, lane >> 2), h = rg / lq, j = rg - h * lq, kvh = h / group;
-    if (lane < 16) {                                                // a row of the group per warp
-        const int row = rg0 + rows::nth_bit(set, warp), hh = row / lq, jj = row - hh * lq;
-        sh.q.put(warp, lane, src.q + (size_t)layer * span.q_stride + (((size_t)b * lq + jj) * n_q_heads + hh) * kD);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lq = bv.q_len;
+    {
+        const int n_rows = min(rows::kGroupRows, __popc(sh.job.set));
+        const int row = sh.job.rg0 + rows::nth_bit(sh.job.set, min(warp, n_rows - 1));      // a row of the group per warp
+        if (lane == 0) sh.row[warp] = row;
+        const int hh = row / lq, jj = row - hh * lq;
+        if (lane < 16) sh.q.put(warp, lane, src.q + (size_t)sh.job.layer * span.q_stride + (((size_t)sh.job.b * lq + jj) * n_q_heads + hh) * kD);
     }
     __syncthreads();
-    // every eighth tile of the request: where its keys lie and which of them this lane's row sees
-    struct Tile {
-        const __nv_bfloat16 *k, *v;
-        size_t pitch;
-        const float2* trig;                                         // null: not a document's
-        int len, visible, index;
-    };
-    const int n_tiles = n_doc + n_prefix + n_self, tile0 = pv.tile_begin[b];
-    int next_row0 = 0, next_len = 0, next_doc = 0;                  // of the document tile behind the current one, asked for early
-    auto fetch = [&](int t) {
-        if (t >= n_doc) return;
-        next_row0 = pv.tile_row0[tile0 + t];
-        next_len = pv.tile_len[tile0 + t];
-        next_doc = pv.tile_doc[tile0 + t];
-    };
-    auto tile_at = [&](int t) {
-        Tile x;
-        x.pitch = (size_t)n_kv_heads * kD;
-        x.trig = nullptr;
-        x.index = -1;
-        if (t < n_doc) {
-            x.index = tile0 + t;
-            x.pitch = bv.token_stride;
-            const size_t at = (size_t)layer * span.kv_stride + (size_t)next_row0 * x.pitch + kvh * kD;
-            x.k = src.k + at;
-            x.v = src.v + at;
-            x.len = x.visible = next_len;
-            x.trig = pv.trig + (size_t)next_doc * (kD / 2);
-        } else if (t < n_doc + n_prefix) {
-            const int row0 = (t - n_doc) * kTile;
-            const size_t at = (size_t)layer * src.prefix_stride + (size_t)row0 * x.pitch + kvh * kD;
-            x.k = src.kp + at;
-            x.v = src.vp + at;
-            x.len = x.visible = min(kTile, src.prefix_len - row0);
-        } else {
-            const int row0 = (t - n_doc - n_prefix) * kTile;
-            const size_t at = (size_t)layer * src.self_stride + ((size_t)b * lq + row0) * x.pitch + kvh * kD;
-            x.k = src.ks + at;
-            x.v = src.vs + at;
-            x.len = min(kTile, lq - row0);
-            x.visible = min(x.len, j + 1 - row0);                   // causal mask
-        }
-        return x;
-    };
+    const int j = sh.row[lane >> 2] % lq;
+    // every eighth tile of the request
+    auto in_range = [&](int t) { return t < sh.job.n_doc + p.n_prefix + p.n_self; };
     rows::Stage& stage = sh.stage[warp];
+    RowTile(&tile)[2] = sh.tile[warp];
+    auto describe = [&](int t, RowTile& x) {
+        if (lane == 0) {
+            const int n_doc = sh.job.n_doc, b = sh.job.b;
+            const long long layer = sh.job.layer;
+            long long pitch = (long long)n_kv_heads * kD, at;
+            const __nv_bfloat16 *k = src.k, *v = src.v;
+            const float2* trig = nullptr;
+            int first = -(1 << 30), index = -1, len;
+            if (t < n_doc) {
+                index = pv.tile_begin[b] + t;
+                pitch = bv.token_stride;
+                at = layer * span.kv_stride + pv.tile_row0[index] * pitch;
+                len = pv.tile_len[index];
+                trig = pv.trig + (size_t)pv.tile_doc[index] * (kD / 2);
+            } else if (t < n_doc + p.n_prefix) {
+                const int row0 = (t - n_doc) * kTile;
+                k = src.kp;
+                v = src.vp;
+                at = layer * src.prefix_stride + row0 * pitch;
+                len = min(kTile, src.prefix_len - row0);
+            } else {
+                first = (t - n_doc - p.n_prefix) * kTile;           // causal mask
+                k = src.ks;
+                v = src.vs;
+                at = layer * src.self_stride + ((long long)b * lq + first) * pitch;
+                len = min(kTile, lq - first);
+            }
+            at += sh.job.kvh * kD;
+            x = {k + at, v + at, trig, pitch, len, first, index};
+        }
+        __syncwarp();
+    };
+    auto copy_keys = [&](const RowTile& x, int i) { rows::copy_step(stage.k, x.k + i * x.pitch, x.pitch, x.len - i); };
+    auto copy_values = [&](const RowTile& x, int i) { rows::copy_step(stage.v, x.v + i * x.pitch, x.pitch, x.len - i); };
     rows::Group acc;
     acc.clear();
     float docs = 0.f, in_tile = 0.f;                                // the parts of acc.l on documents and on the current tile
-    int t = warp, i = 0;
-    Tile now = {};
-    if (t < n_tiles) {
-        fetch(t);
-        now = tile_at(t);
-        fetch(t + 8);
-        rows::copy_step(stage.k, now.k, now.pitch, now.len);
+    int t = warp, i = 0;                                            // the t-th tile lies in tile[t / 8 mod 2]
+    if (in_range(t)) {
+        describe(t, tile[0]);
+        copy_keys(tile[0], 0);
         rows::copies_end();
-        rows::copy_step(stage.v, now.v, now.pitch, now.len);
+        copy_values(tile[0], 0);
         rows::copies_end();
     }
-    while (t < n_tiles) {
+#pragma unroll 1
+    while (in_range(t)) {
+        const int now = t >> 3 & 1;
         rows::Keys keys;
         rows::copies_wait();
         keys.read(stage);
-        Tile next = now;                                            // the step behind this one
-        int next_i = i + rows::kStepKeys;
-        const bool last = next_i >= now.len;
-        if (last && t + 8 < n_tiles) {
-            next = tile_at(t + 8);
-            fetch(t + 16);
-            next_i = 0;
-        }
-        const bool more = next_i < next.len;
+        const int visible = min(tile[now].len, j + 1 - tile[now].first) - i;
+        const bool last = i + rows::kStepKeys >= tile[now].len, more = !last || in_range(t + 8);
+        const int next = last ? now ^ 1 : now;                      // the tile of the step behind this one
+        i = last ? 0 : i + rows::kStepKeys;                         // and its place there
+        if (last && more) describe(t + 8, tile[next]);
         __syncwarp();                                               // every lane has its fragments
-        if (more) rows::copy_step(stage.k, next.k + next_i * next.pitch, next.pitch, next.len - next_i);
+        if (more) copy_keys(tile[next], i);
         rows::copies_end();
-        if (now.trig) keys.rotate<LAYOUT>(now.trig);
+        const float2* trig = tile[now].trig;
+        if (trig) keys.rotate<LAYOUT>(trig);
         float alpha;
-        const float sum = acc.scores(sh.q, keys, now.visible - i, src.scale_log2, alpha);
+        const float sum = acc.scores(sh.q, keys, visible, src.scale_log2, alpha);
         in_tile = fmaf(in_tile, alpha, sum);
-        docs = fmaf(docs, alpha, now.trig ? sum : 0.f);
+        docs = fmaf(docs, alpha, tile[now].trig ? sum : 0.f);
         rows::copies_wait();
         acc.values(stage);
         __syncwarp();
-        if (more) rows::copy_step(stage.v, next.v + next_i * next.pitch, next.pitch, next.len - next_i);
+        if (more) copy_values(tile[next], i);
         rows::copies_end();
         if (last) {
             in_tile = rows::over_keys(in_tile);
-            if (now.trig && (lane & 3) == 0 && (lane >> 2) < n_rows) ws.tile_lse2[((size_t)layer * ws.max_tiles + now.index) * rows_total + rg] = acc.m + log2f(in_tile);
+            const int index = tile[now].index;
+            if (index >= 0 && (lane & 3) == 0)                      // (rows beyond the group's repeat its last one)
+                ws.tile_lse2[((size_t)sh.job.layer * ws.max_tiles + index) * n_q_heads * lq + sh.row[lane >> 2]] = acc.m + log2f(in_tile);
             in_tile = 0.f;
             t += 8;
+            __syncwarp();                                           // the tile has been read
         }
-        now = next;
-        i = next_i;
     }
     acc.l = rows::over_keys(acc.l);
     docs = rows::over_keys(docs);
@@ -406,7 +413,7 @@ __device__ __noinline__ void rows_from_scratch(const Params& p, RowScratch& sh, 
                 }
         __syncthreads();
     }
-    if (warp < n_rows) {                                            // a row per warp, four dims per lane
+    if (warp < __popc(sh.job.set)) {                                // a row per warp, four dims per lane
         float top = sh.m[0][warp], l = 0.f, ld = 0.f;
         for (int w = 1; w < 8; ++w) top = fmaxf(top, sh.m[w][warp]);
         for (int w = 0; w < 8; ++w) {
@@ -414,30 +421,22 @@ __device__ __noinline__ void rows_from_scratch(const Params& p, RowScratch& sh, 
             l = fmaf(sh.l[w][warp], f, l);
             ld = fmaf(sh.docs[w][warp], f, ld);
         }
-        const int row = rg0 + rows::nth_bit(set, warp), hh = row / lq, jj = row - hh * lq;
+        const int row = sh.row[warp], hh = row / lq, jj = row - hh * lq;
         const float inv = l == 0.f ? 0.f : 1.f / l;
         const float4 o = *reinterpret_cast<const float4*>(&sh.o[warp][lane * 4]);
-        *reinterpret_cast<uint2*>(out_all + (size_t)layer * span.out_stride + (((size_t)b * lq + jj) * n_q_heads + hh) * kD + lane * 4) =
+        *reinterpret_cast<uint2*>(out_all + (size_t)sh.job.layer * span.out_stride + (((size_t)sh.job.b * lq + jj) * n_q_heads + hh) * kD + lane * 4) =
             make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
         if (lane == 0) {
-            ws.row_lse2[(size_t)lb * rows_total + row] = top + log2f(ld);
-            if (lse) lse[(size_t)lb * rows_total + row] = (top + log2f(l)) * kLn2;
+            const size_t at = (size_t)sh.job.lb * n_q_heads * lq + row;
+            ws.row_lse2[at] = top + log2f(ld);
+            if (lse) lse[at] = (top + log2f(l)) * kLn2;
         }
     }
     __syncthreads();                                                // the shared memory may be used again
 }
 
 constexpr size_t kMergeSmem = sizeof(RowScratch);
-
-// All rows of a set, eight at a time.
-template <int LAYOUT>
-__device__ __forceinline__ void set_from_scratch(const Params& p, RowScratch& sh, int lb, int rg0, unsigned set, int n_doc) {
-    while (set) {
-        const unsigned now = rows::next_group(set);
-        rows_from_scratch<LAYOUT>(p, sh, lb, rg0, now, n_doc);
-        set ^= now;
-    }
-}
+static_assert(alignof(RowScratch) == 16 && offsetof(RowScratch, stage) % 16 == 0 && offsetof(RowScratch, q) % 16 == 0 && offsetof(RowScratch, o) % 16 == 0, "16-byte accesses");
 
 template <int LAYOUT>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -941,35 +940,84 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
 
 // The rows of a merge block's slice that left the range of their reference: of the units finished in its shares (the sum of such
 // a row is not a number) and of those that were cut (cut_rows).
+// Inlined, with one place that computes and everything that is known about the work in shared memory: as a function that is
+// called, the path cost a merge in blocks of 32 rows 0.3 to 0.5 us whether a row is marked or not (one layer of 20 documents,
+// 32/32 heads, 48.8 -> 48.3 us; three runs of layers of 50 documents, 12/2, 159.4 -> 158.3), and marked rows a tenth more.  A merge
+// in blocks of 8 rows does not notice (28 calls 571 -> 573 us).
 template <int LAYOUT, int ROWS>
-__device__ __noinline__ void marked_from_scratch(const Params& p, const unsigned* cut_rows, int share0, int n_classes, int slice) {
+__device__ __forceinline__ void marked_from_scratch(const Params& p, const unsigned* cut_rows, int share0, int n_classes, int slice) {
     extern __shared__ __align__(16) unsigned char merge_smem[];
     RowScratch& sh = *reinterpret_cast<RowScratch*>(merge_smem);
-    const BatchView& bv = p.bv;
-    const PlanView& pv = p.pv;
-    const AttnWorkspace& ws = p.ws;
-    const int lane = threadIdx.x & 31, group = p.n_q_heads / p.n_kv_heads, rows_total = p.n_q_heads * bv.q_len;
-    for (int u = 0, share = share0; u < 32 / ROWS && share < p.max_shares; ++u, share += n_classes) {
-        const ShareHead head = reinterpret_cast<const ShareHead*>(ws.marks)[share];
-        if (head.marked) {
-            if (threadIdx.x < 32) scan_requests(bv, pv, p.n_prefix + p.n_self, sh.requests);
-            __syncthreads();
-            const Line line = make_line(bv, ws, sh.requests, p.n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, p.max_shares);
-            const int end = line.cut(share + 1);
-            for (int y = line.cut(share); y < end;) {
-                const Segment own = segment_at(bv, pv, ws, line, group, y, end);
-                y += own.t_end - own.t_begin;
-                if (own.t_end - own.t_begin != own.n_unit) continue;
-                const int rg0 = own.kvh * group * bv.q_len + own.row0 + slice * ROWS;
-                const bool mine = lane < ROWS && slice * ROWS + lane < own.rows_here;
-                const float v = mine ? ws.row_lse2[(size_t)own.lb * rows_total + rg0 + lane] : 0.f;
-                const unsigned todo = __ballot_sync(0xffffffffu, v != v);
-                __syncthreads();                                    // every warp has looked before the first row is written
-                set_from_scratch<LAYOUT>(p, sh, own.lb, rg0, todo, own.n_doc);
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        sh.job.set = 0;
+        sh.job.u = -1;
+        sh.job.x = sh.job.end = 0;
+    }
+#pragma unroll 1
+    while (true) {
+        if (tid < 32) {                                            // the next group, sought by the first warp
+            __syncwarp();
+            const int group = p.n_q_heads / p.n_kv_heads;
+            unsigned set = sh.job.set;
+            if (set) set ^= rows::next_group(set);
+            __syncwarp();
+            if (tid == 0) sh.job.set = set;
+#pragma unroll 1
+            while (set == 0) {
+                int lb, layer, b, kvh, n_doc, rg0, x = sh.job.x;
+                const int end = sh.job.end;
+                __syncwarp();
+                if (x < end) {                                      // the next unit of the share, if it was finished there
+                    const Segment own = segment_at(p.bv, p.pv, p.ws, sh.line, group, x, end);
+                    lb = own.lb;
+                    layer = own.layer;
+                    b = own.b;
+                    kvh = own.kvh;
+                    n_doc = own.n_doc;
+                    rg0 = kvh * group * p.bv.q_len + own.row0 + slice * ROWS;
+                    const bool mine = tid < ROWS && slice * ROWS + tid < own.rows_here && own.t_end - own.t_begin == own.n_unit;
+                    const float v = mine ? p.ws.row_lse2[(size_t)lb * p.n_q_heads * p.bv.q_len + rg0 + tid] : 0.f;
+                    set = __ballot_sync(0xffffffffu, v != v);
+                    if (tid == 0) sh.job.x = x + own.t_end - own.t_begin;
+                } else {                                            // the next share, and the unit cut there
+                    const int u = sh.job.u + 1, share = share0 + u * n_classes;
+                    __syncwarp();
+                    if (u == 32 / ROWS || share >= p.max_shares) break;
+                    const ShareHead head = reinterpret_cast<const ShareHead*>(p.ws.marks)[share];
+                    lb = head.lb;
+                    layer = head.layer;
+                    b = head.b;
+                    n_doc = head.n_doc;
+                    rg0 = head.row_first + slice * ROWS;
+                    kvh = rg0 / (group * p.bv.q_len);
+                    set = cut_rows[u];
+                    if (head.marked) scan_requests(p.bv, p.pv, p.n_prefix + p.n_self, sh.requests);
+                    __syncwarp();
+                    if (tid == 0) {
+                        sh.job.u = u;
+                        if (head.marked) {
+                            sh.line = make_line(p.bv, p.ws, sh.requests, p.n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, p.max_shares);
+                            sh.job.x = sh.line.cut(share);
+                            sh.job.end = sh.line.cut(share + 1);
+                        }
+                    }
+                }
+                if (tid == 0) {
+                    sh.job.lb = lb;
+                    sh.job.layer = layer;
+                    sh.job.b = b;
+                    sh.job.kvh = kvh;
+                    sh.job.n_doc = n_doc;
+                    sh.job.rg0 = rg0;
+                    sh.job.set = set;
+                }
+                __syncwarp();
             }
         }
-        set_from_scratch<LAYOUT>(p, sh, head.lb, head.row_first + slice * ROWS, cut_rows[u], head.n_doc);
         __syncthreads();
+        if (sh.job.set == 0) break;
+        rows_from_scratch<LAYOUT>(p, sh);                           // ends with a barrier
     }
 }
 

@@ -32,7 +32,7 @@ __device__ __forceinline__ void read16(const void* p, uint32_t (&w)[4]) {
 }
 
 // The queries of a group.  Rows 320 bytes apart: the pieces that eight lanes read together fall on all banks.
-struct Queries {
+struct alignas(16) Queries {
     __nv_bfloat16 row[kGroupRows][kDim + 32];
     // Row r of the group, by sixteen lanes (piece = 0 .. 15).
     __device__ __forceinline__ void put(int r, int piece, const __nv_bfloat16* from) {
@@ -41,14 +41,15 @@ struct Queries {
 };
 
 // A warp's step on its way: sixteen keys and sixteen values.  The pitches keep the fragments of either free of bank conflicts.
-struct Stage {
+struct alignas(16) Stage {
     __nv_bfloat16 k[kStepKeys][kDim + 32], v[kStepKeys][kDim + 8];
 };
+static_assert(sizeof(Stage) % 16 == 0 && (kDim + 32) * 2 % 16 == 0 && (kDim + 8) * 2 % 16 == 0, "16-byte pieces");
 // Copies rows first .. first + 15 (rows `pitch` elements apart, of which n exist; the others repeat the last one) by a warp.
 template <int PITCH>
 __device__ __forceinline__ void copy_step(__nv_bfloat16 (&to)[kStepKeys][PITCH], const __nv_bfloat16* first, size_t pitch, int n) {
     const int lane = threadIdx.x & 31, piece = 8 * (lane & 15);
-#pragma unroll
+#pragma unroll 2
     for (int i = 0; i < kStepKeys / 2; ++i) {
         const int r = 2 * i + (lane >> 4);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(shared_at(&to[r][piece])), "l"(first + (size_t)min(r, n - 1) * pitch + piece) : "memory");
@@ -132,19 +133,19 @@ struct Group {
         const int lane = threadIdx.x & 31, t = lane & 3;
         // a short accumulation per chunk, joined in fp32, since mma.sync truncates what it adds: log-sum-exps near 200 were up to
         // 4.2e-5 off with one chain of eight, 3.0e-5 this way, 2.8e-5 with fused multiply-adds (one unit of the last place: 1.5e-5)
-        float s[2][2];
+        float s[2][2] = {};
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            float part[4][4] = {};
+        for (int c = 0; c < 4; ++c) {
+            uint32_t q[4];
+            read16(&queries.row[lane >> 2][8 * t + 32 * c], q);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                uint32_t q[4];
-                read16(&queries.row[lane >> 2][8 * t + 32 * c], q);
-                mma16816(part[c], q[0], 0u, q[1], 0u, keys.k[j][c][0], keys.k[j][c][1]);
-                mma16816(part[c], q[2], 0u, q[3], 0u, keys.k[j][c][2], keys.k[j][c][3]);
+            for (int j = 0; j < 2; ++j) {
+                float part[4] = {};
+                mma16816(part, q[0], 0u, q[1], 0u, keys.k[j][c][0], keys.k[j][c][1]);
+                mma16816(part, q[2], 0u, q[3], 0u, keys.k[j][c][2], keys.k[j][c][3]);
+                s[j][0] += part[0];
+                s[j][1] += part[1];
             }
-#pragma unroll
-            for (int x = 0; x < 2; ++x) s[j][x] = (part[0][x] + part[1][x]) + (part[2][x] + part[3][x]);
         }
         float e[4] = {s[0][0] * scale_log2, s[0][1] * scale_log2, s[1][0] * scale_log2, s[1][1] * scale_log2};
 #pragma unroll
