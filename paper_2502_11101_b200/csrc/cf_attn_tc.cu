@@ -22,7 +22,7 @@
 // segment.  P and the sums keep their relative precision for logits up to 80 (log2 units) above it and 126 below, so that no
 // tile has to look at its maximum before its exponentials.  (A reference 40 above that maximum, which centres the range, costs
 // three bits of the exponents and the log-sum-exps: 1.3e-6 off instead of 1.1e-7 for a row of one key.)  A row that does leave
-// the range is marked (NaN sum) and recomputed from scratch by the merge kernel.
+// the range is marked (NaN sum) and computed from scratch over the CTA's own share once the roles have left their loops.
 // What bounds it (per 96-key tile and 128 rows, in SM cycles): tensor cores 768 (8 x 48 + 6 x 64), exponentials 768 on
 // the shared MUFU, shared memory 1150 (copies 384, rotation 384, QK^T 192, PV 192), so these overlap only if nobody
 // waits for a chain.
@@ -73,7 +73,7 @@ struct Barriers {
     unsigned long long ref_full[2], sum_full[2];                        // [segment parity]
     unsigned int tmem_base;
     volatile int abort_flag;
-    volatile int marked;                           // a row of a unit finished here has to be computed from scratch
+    volatile int marked;                           // a row of the share has to be computed from scratch
 };
 
 // Tile descriptions: flags beside the length, and which keys they are.
@@ -207,10 +207,9 @@ __device__ __forceinline__ Segment segment_at(const BatchView& bv, const PlanVie
     return sg;
 }
 
-// What a CTA leaves for the merge kernel: the unit that begins in its share and goes on behind it (n_parts = 0: none), and
-// whether a unit finished in the share has rows to be computed from scratch.
+// What a CTA leaves for the merge kernel: the unit that begins in its share and goes on behind it (n_parts = 0: none).
 struct ShareHead {
-    int n_parts, marked, lb, layer, b, row_first, rows_here, n_doc;      // row_first: of the unit among the rows of a request
+    int n_parts, lb, layer, b, row_first, rows_here, unused[2];          // row_first: of the unit among the rows of a request
 };
 static_assert(sizeof(ShareHead) == 32, "two 16-byte loads");
 
@@ -257,63 +256,57 @@ struct Params {
     __nv_bfloat16* const out_all = p.out;                                                                          \
     float* const lse = p.lse
 
-// Shared memory of a merge block that computes rows from scratch.
+// Shared memory of a CTA that computes rows of its share from scratch, over the rings of keys and values.
+constexpr int kRowWarps = kThreads / 32;
 struct RowTile {                   // where a key tile lies; row j of the query sees its keys up to j - first
     const __nv_bfloat16 *k, *v;
     const float2* trig;            // null: not a document's
     long long pitch;
     int len, first, index;
 };
-struct RowJob {
-    int lb, layer, b, kvh, n_doc, rg0;
-    unsigned set;                  // of rows rg0 .. that are still to be computed
-    int u, x, end;                 // share of the block, and its positions that are still to be looked at
-};
 struct RowScratch {
-    volatile RowJob job;           // what all warps know and none has registers for
-    int row[rows::kGroupRows];     // the group
-    rows::Stage stage[8];          // of every warp
-    RowTile tile[8][2];            // the current tile and the next one (registers are what the keys and sums need)
+    rows::Stage stage[kRowWarps];  // of every warp
+    RowTile tile[kRowWarps][2];    // the current tile and the next one (registers are what the keys and sums need)
     rows::Queries q;
     alignas(16) float o[rows::kGroupRows][kD];
-    float m[8][rows::kGroupRows], l[8][rows::kGroupRows], docs[8][rows::kGroupRows];   // of every warp
-    Requests requests;
-    Line line;
+    float m[kRowWarps][rows::kGroupRows], l[kRowWarps][rows::kGroupRows], docs[kRowWarps][rows::kGroupRows];   // of every warp
+    Segment sg;
+    unsigned todo[kRowTile / 32];  // rows of the segment that are still to be computed
+    int row[rows::kGroupRows];     // the group, as rows of the segment
+    int n_rows;
+    int x;                         // position of the share behind the segment
 };
+static_assert(sizeof(RowScratch) <= (kKStages + kVStages) * kKvBytes, "over the rings");
+static_assert(alignof(RowScratch) == 16 && offsetof(RowScratch, q) % 16 == 0 && offsetof(RowScratch, o) % 16 == 0, "16-byte accesses");
 
-// Up to eight query rows (rg0 + every set bit of `set`, of one kv head) by a block of eight warps, each with every eighth key tile
-// under a running maximum of its own: outputs, log-sum-exps and those of the document tiles.  Only rows whose logits left the
-// range of the shared reference come here (keys that are not finite lead here too).  Bound by the instructions and mma.sync of a
-// step, just under 2 us for eight rows.  Measured with a warp per row and key after key, and this way: four layers of 50 documents
-// of 160 tokens, 12/2 heads, 44 us without such rows, one row a layer 3.0 -> 0.17 ms, every row 10.1 -> 0.71 ms; one layer of
-// 2 x 60 documents of 180, 32/32 heads, 93 us without, one row 6.1 -> 0.27, every row 27.1 -> 1.1 ms.
+// Up to eight query rows (every set bit of `set`, from row `row0` of the segment on) over the segment's key tiles, every warp
+// with every sixteenth tile under a running maximum of its own.  Leaves what the epilogue leaves of a row - a finished row or
+// the part of one - and the log-sum-exps of the document tiles.
 template <int LAYOUT>
-__device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& sh) {
+__device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& sh, int row0, unsigned set) {
     CF_PARAMS;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lq = bv.q_len;
-    {
-        const int n_rows = min(rows::kGroupRows, __popc(sh.job.set));
-        const int row = sh.job.rg0 + rows::nth_bit(sh.job.set, min(warp, n_rows - 1));      // a row of the group per warp
-        if (lane == 0) sh.row[warp] = row;
-        const int hh = row / lq, jj = row - hh * lq;
-        if (lane < 16) sh.q.put(warp, lane, src.q + (size_t)sh.job.layer * span.q_stride + (((size_t)sh.job.b * lq + jj) * n_q_heads + hh) * kD);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lq = bv.q_len, group = n_q_heads / n_kv_heads, rows_total = n_q_heads * lq;
+    if (warp < rows::kGroupRows) {                                  // a row of the group per warp; beyond them the last one again
+        const int n_rows = min(rows::kGroupRows, __popc(set)), r = row0 + rows::nth_bit(set, min(warp, n_rows - 1)), row = sh.sg.row0 + r, g = row / lq, j = row - g * lq;
+        if (lane == 0) sh.row[warp] = r;
+        if (threadIdx.x == 0) sh.n_rows = n_rows;
+        if (lane < 16)
+            sh.q.put(warp, lane, src.q + (size_t)sh.sg.layer * span.q_stride + (((size_t)sh.sg.b * lq + j) * n_q_heads + sh.sg.kvh * group + g) * kD);
     }
     __syncthreads();
-    const int j = sh.row[lane >> 2] % lq;
-    // every eighth tile of the request
-    auto in_range = [&](int t) { return t < sh.job.n_doc + p.n_prefix + p.n_self; };
+    const int j = (sh.sg.row0 + sh.row[lane >> 2]) % lq;
     rows::Stage& stage = sh.stage[warp];
     RowTile(&tile)[2] = sh.tile[warp];
     auto describe = [&](int t, RowTile& x) {
         if (lane == 0) {
-            const int n_doc = sh.job.n_doc, b = sh.job.b;
-            const long long layer = sh.job.layer;
+            const int n_doc = sh.sg.n_doc, b = sh.sg.b;
+            const long long layer = sh.sg.layer;
             long long pitch = (long long)n_kv_heads * kD, at;
             const __nv_bfloat16 *k = src.k, *v = src.v;
             const float2* trig = nullptr;
             int first = -(1 << 30), index = -1, len;
             if (t < n_doc) {
-                index = pv.tile_begin[b] + t;
+                index = sh.sg.tile0 + t;
                 pitch = bv.token_stride;
                 at = layer * span.kv_stride + pv.tile_row0[index] * pitch;
                 len = pv.tile_len[index];
@@ -331,7 +324,7 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
                 at = layer * src.self_stride + ((long long)b * lq + first) * pitch;
                 len = min(kTile, lq - first);
             }
-            at += sh.job.kvh * kD;
+            at += sh.sg.kvh * kD;
             x = {k + at, v + at, trig, pitch, len, first, index};
         }
         __syncwarp();
@@ -341,8 +334,8 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
     rows::Group acc;
     acc.clear();
     float docs = 0.f, in_tile = 0.f;                                // the parts of acc.l on documents and on the current tile
-    int t = warp, i = 0;                                            // the t-th tile lies in tile[t / 8 mod 2]
-    if (in_range(t)) {
+    int t = sh.sg.t_begin + warp, i = 0, now = 0;                   // the current tile lies in tile[now]
+    if (t < sh.sg.t_end) {
         describe(t, tile[0]);
         copy_keys(tile[0], 0);
         rows::copies_end();
@@ -350,16 +343,15 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
         rows::copies_end();
     }
 #pragma unroll 1
-    while (in_range(t)) {
-        const int now = t >> 3 & 1;
+    while (t < sh.sg.t_end) {
         rows::Keys keys;
         rows::copies_wait();
         keys.read(stage);
         const int visible = min(tile[now].len, j + 1 - tile[now].first) - i;
-        const bool last = i + rows::kStepKeys >= tile[now].len, more = !last || in_range(t + 8);
+        const bool last = i + rows::kStepKeys >= tile[now].len, more = !last || t + kRowWarps < sh.sg.t_end;
         const int next = last ? now ^ 1 : now;                      // the tile of the step behind this one
         i = last ? 0 : i + rows::kStepKeys;                         // and its place there
-        if (last && more) describe(t + 8, tile[next]);
+        if (last && more) describe(t + kRowWarps, tile[next]);
         __syncwarp();                                               // every lane has its fragments
         if (more) copy_keys(tile[next], i);
         rows::copies_end();
@@ -378,9 +370,11 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
             in_tile = rows::over_keys(in_tile);
             const int index = tile[now].index;
             if (index >= 0 && (lane & 3) == 0)                      // (rows beyond the group's repeat its last one)
-                ws.tile_lse2[((size_t)sh.job.layer * ws.max_tiles + index) * n_q_heads * lq + sh.row[lane >> 2]] = acc.m + log2f(in_tile);
+                ws.tile_lse2[((size_t)sh.sg.layer * ws.max_tiles + index) * rows_total + (size_t)sh.sg.kvh * group * lq + sh.sg.row0 + sh.row[lane >> 2]] =
+                    acc.m + log2f(in_tile);
             in_tile = 0.f;
-            t += 8;
+            t += kRowWarps;
+            now = next;
             __syncwarp();                                           // the tile has been read
         }
     }
@@ -398,10 +392,10 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
     for (int x = 0; x < 2; ++x) {
         const int r = 2 * (lane & 3) + x;
         float top = sh.m[0][r];
-        for (int w = 1; w < 8; ++w) top = fmaxf(top, sh.m[w][r]);
+        for (int w = 1; w < kRowWarps; ++w) top = fmaxf(top, sh.m[w][r]);
         weight[x] = sh.m[warp][r] > -INFINITY ? exp2f(sh.m[warp][r] - top) : sh.l[warp][r];   // nothing seen: 0 (or not a number)
     }
-    for (int w = 0; w < 8; ++w) {
+    for (int w = 0; w < kRowWarps; ++w) {
         if (w == warp)
 #pragma unroll
             for (int i = 0; i < 8; ++i)
@@ -413,30 +407,76 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
                 }
         __syncthreads();
     }
-    if (warp < __popc(sh.job.set)) {                                // a row per warp, four dims per lane
+    if (warp < sh.n_rows) {                                         // a row per warp, four dims per lane
         float top = sh.m[0][warp], l = 0.f, ld = 0.f;
-        for (int w = 1; w < 8; ++w) top = fmaxf(top, sh.m[w][warp]);
-        for (int w = 0; w < 8; ++w) {
+        for (int w = 1; w < kRowWarps; ++w) top = fmaxf(top, sh.m[w][warp]);
+        for (int w = 0; w < kRowWarps; ++w) {
             const float f = sh.m[w][warp] > -INFINITY ? exp2f(sh.m[w][warp] - top) : 1.f;
             l = fmaf(sh.l[w][warp], f, l);
             ld = fmaf(sh.docs[w][warp], f, ld);
         }
-        const int row = sh.row[warp], hh = row / lq, jj = row - hh * lq;
-        const float inv = l == 0.f ? 0.f : 1.f / l;
+        const bool whole = sh.sg.t_end - sh.sg.t_begin == sh.sg.n_unit;
+        const int row = sh.sg.row0 + sh.row[warp], g = row / lq, jj = row - g * lq;
+        const size_t slot = ((size_t)2 * blockIdx.x + (sh.sg.t_begin == 0 ? 1 : 0)) * kRowTile + sh.row[warp];
+        const float f = !whole ? 1.f : l == 0.f ? 0.f : 1.f / l;
         const float4 o = *reinterpret_cast<const float4*>(&sh.o[warp][lane * 4]);
-        *reinterpret_cast<uint2*>(out_all + (size_t)sh.job.layer * span.out_stride + (((size_t)sh.job.b * lq + jj) * n_q_heads + hh) * kD + lane * 4) =
-            make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
-        if (lane == 0) {
-            const size_t at = (size_t)sh.job.lb * n_q_heads * lq + row;
+        __nv_bfloat16* dst = whole ? out_all + (size_t)sh.sg.layer * span.out_stride + (((size_t)sh.sg.b * lq + jj) * n_q_heads + sh.sg.kvh * group + g) * kD
+                                   : reinterpret_cast<__nv_bfloat16*>(ws.part_o) + slot * kD;
+        *reinterpret_cast<uint2*>(dst + lane * 4) = make_uint2(pack_bf16(o.x * f, o.y * f), pack_bf16(o.z * f, o.w * f));
+        if (lane == 0 && whole) {
+            const size_t at = (size_t)sh.sg.lb * rows_total + (size_t)sh.sg.kvh * group * lq + row;
             ws.row_lse2[at] = top + log2f(ld);
             if (lse) lse[at] = (top + log2f(l)) * kLn2;
+        } else if (lane == 0) {
+            ws.part_m[slot] = l == 0.f ? -INFINITY : top > -INFINITY ? top : 0.f;   // (a sum that is not a number has to be seen)
+            ws.part_l[slot] = l;
+            if (ws.part_ld) ws.part_ld[slot] = ld;
         }
     }
     __syncthreads();                                                // the shared memory may be used again
 }
 
-constexpr size_t kMergeSmem = sizeof(RowScratch);
-static_assert(alignof(RowScratch) == 16 && offsetof(RowScratch, stage) % 16 == 0 && offsetof(RowScratch, q) % 16 == 0 && offsetof(RowScratch, o) % 16 == 0, "16-byte accesses");
+// The rows of a share that left the range of their reference (their sums are not numbers), segment by segment, in eights of
+// neighbours.  Only rows whose logits lie more than 2^80 above the first 16 of the segment come here, and keys that are not
+// finite.  A segment's reference is its own, so a row that left it in one share is computed over that share's keys and joins the
+// other parts like any other.  In the merge kernel, over all keys of the row (one block of eight warps had to walk them), the path
+// cost every merge 0.3 to 0.5 us although nobody took it: one layer of 20 documents, 32/32 heads 48.3 -> 46.6 us, 28 one-layer
+// calls over 50 documents, 12/2 heads 574 -> 559.  Calls with such rows: four layers of 50 documents of 160 tokens, 12/2 heads, 44 us
+// without, one row a layer 166 -> 79, every row 759 -> 398; one layer of 2 x 60 documents of 180, 32/32 heads, 93 us, 265 -> 166 and
+// 1109 -> 646; of 4 x 50 of 160, 28/4 heads, 75 us, 202 -> 130 and 687 -> 720 (few tiles per share leave warps idle).
+template <int LAYOUT>
+__device__ __forceinline__ void marked_from_scratch(const Params& p, RowScratch& sh, const Line& line) {
+    const int group = p.n_q_heads / p.n_kv_heads;
+    if (threadIdx.x == 0) sh.x = line.cut(blockIdx.x);
+#pragma unroll 1
+    while (true) {
+        __syncthreads();                                            // the segment before has been read
+        if (sh.x >= line.cut(blockIdx.x + 1)) break;
+        if (threadIdx.x == 0) sh.sg = segment_at(p.bv, p.pv, p.ws, line, group, sh.x, line.cut(blockIdx.x + 1));
+        __syncthreads();
+        if (threadIdx.x < kRowTile) {
+            const int rows = group * p.bv.q_len;
+            float l = 0.f;
+            if ((int)threadIdx.x < sh.sg.rows_here)
+                l = sh.sg.t_end - sh.sg.t_begin == sh.sg.n_unit
+                        ? p.ws.row_lse2[(size_t)sh.sg.lb * p.n_q_heads * p.bv.q_len + (size_t)sh.sg.kvh * rows + sh.sg.row0 + threadIdx.x]
+                        : p.ws.part_l[((size_t)2 * blockIdx.x + (sh.sg.t_begin == 0 ? 1 : 0)) * kRowTile + threadIdx.x];
+            const unsigned set = __ballot_sync(0xffffffffu, l != l);
+            if ((threadIdx.x & 31) == 0) sh.todo[threadIdx.x >> 5] = set;
+        }
+        if (threadIdx.x == 0) sh.x += sh.sg.t_end - sh.sg.t_begin;
+#pragma unroll 1
+        while (true) {
+            __syncthreads();
+            const int w = sh.todo[0] ? 0 : sh.todo[1] ? 1 : sh.todo[2] ? 2 : 3;
+            const unsigned set = sh.todo[w];
+            if (set == 0) break;
+            __syncthreads();
+            if (threadIdx.x == 0) sh.todo[w] = set ^ rows::next_group(set);
+            rows_from_scratch<LAYOUT>(p, sh, w * 32, set);
+        }
+    }
+}
 
 template <int LAYOUT>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -578,7 +618,6 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
                 head.b = sg.b;
                 head.row_first = sg.kvh * rows + sg.row0;
                 head.rows_here = sg.rows_here;
-                head.n_doc = sg.n_doc;
             }
             sh.head = head;
         }
@@ -815,8 +854,8 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
                         } else {
                             ws.row_lse2[at] = marked ? l_all : ref + log2f(d_all);
                             if (lse) lse[at] = (ref + log2f(l_all)) * kLn2;
-                            if (marked) bars.marked = 1;
                         }
+                        if (marked) bars.marked = 1;
                     }
                 }
                 tc_fence_before();
@@ -920,9 +959,10 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
     if (tid == 0) {
         ShareHead head = {};
         if (n_items > 0) head = sh.head;
-        head.marked = bars.marked;
         reinterpret_cast<ShareHead*>(ws.marks)[blockIdx.x] = head;
     }
+    // every copy has landed and every MMA has read its operands: the rings are free
+    if (bars.marked && !bars.abort_flag) marked_from_scratch<LAYOUT>(p, *reinterpret_cast<RowScratch*>(smem), line);
     if (bars.abort_flag) {
         // a wait expired: let the copies in flight land before the shared memory is given back
         if (tid == 0) {
@@ -938,105 +978,17 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
     }
 }
 
-// The rows of a merge block's slice that left the range of their reference: of the units finished in its shares (the sum of such
-// a row is not a number) and of those that were cut (cut_rows).
-// Inlined, with one place that computes and everything that is known about the work in shared memory: as a function that is
-// called, the path cost a merge in blocks of 32 rows 0.3 to 0.5 us whether a row is marked or not (one layer of 20 documents,
-// 32/32 heads, 48.8 -> 48.3 us; three runs of layers of 50 documents, 12/2, 159.4 -> 158.3), and marked rows a tenth more.  A merge
-// in blocks of 8 rows does not notice (28 calls 571 -> 573 us).
-template <int LAYOUT, int ROWS>
-__device__ __forceinline__ void marked_from_scratch(const Params& p, const unsigned* cut_rows, int share0, int n_classes, int slice) {
-    extern __shared__ __align__(16) unsigned char merge_smem[];
-    RowScratch& sh = *reinterpret_cast<RowScratch*>(merge_smem);
-    const int tid = threadIdx.x;
-    if (tid == 0) {
-        sh.job.set = 0;
-        sh.job.u = -1;
-        sh.job.x = sh.job.end = 0;
-    }
-#pragma unroll 1
-    while (true) {
-        if (tid < 32) {                                            // the next group, sought by the first warp
-            __syncwarp();
-            const int group = p.n_q_heads / p.n_kv_heads;
-            unsigned set = sh.job.set;
-            if (set) set ^= rows::next_group(set);
-            __syncwarp();
-            if (tid == 0) sh.job.set = set;
-#pragma unroll 1
-            while (set == 0) {
-                int lb, layer, b, kvh, n_doc, rg0, x = sh.job.x;
-                const int end = sh.job.end;
-                __syncwarp();
-                if (x < end) {                                      // the next unit of the share, if it was finished there
-                    const Segment own = segment_at(p.bv, p.pv, p.ws, sh.line, group, x, end);
-                    lb = own.lb;
-                    layer = own.layer;
-                    b = own.b;
-                    kvh = own.kvh;
-                    n_doc = own.n_doc;
-                    rg0 = kvh * group * p.bv.q_len + own.row0 + slice * ROWS;
-                    const bool mine = tid < ROWS && slice * ROWS + tid < own.rows_here && own.t_end - own.t_begin == own.n_unit;
-                    const float v = mine ? p.ws.row_lse2[(size_t)lb * p.n_q_heads * p.bv.q_len + rg0 + tid] : 0.f;
-                    set = __ballot_sync(0xffffffffu, v != v);
-                    if (tid == 0) sh.job.x = x + own.t_end - own.t_begin;
-                } else {                                            // the next share, and the unit cut there
-                    const int u = sh.job.u + 1, share = share0 + u * n_classes;
-                    __syncwarp();
-                    if (u == 32 / ROWS || share >= p.max_shares) break;
-                    const ShareHead head = reinterpret_cast<const ShareHead*>(p.ws.marks)[share];
-                    lb = head.lb;
-                    layer = head.layer;
-                    b = head.b;
-                    n_doc = head.n_doc;
-                    rg0 = head.row_first + slice * ROWS;
-                    kvh = rg0 / (group * p.bv.q_len);
-                    set = cut_rows[u];
-                    if (head.marked) scan_requests(p.bv, p.pv, p.n_prefix + p.n_self, sh.requests);
-                    __syncwarp();
-                    if (tid == 0) {
-                        sh.job.u = u;
-                        if (head.marked) {
-                            sh.line = make_line(p.bv, p.ws, sh.requests, p.n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, p.max_shares);
-                            sh.job.x = sh.line.cut(share);
-                            sh.job.end = sh.line.cut(share + 1);
-                        }
-                    }
-                }
-                if (tid == 0) {
-                    sh.job.lb = lb;
-                    sh.job.layer = layer;
-                    sh.job.b = b;
-                    sh.job.kvh = kvh;
-                    sh.job.n_doc = n_doc;
-                    sh.job.rg0 = rg0;
-                    sh.job.set = set;
-                }
-                __syncwarp();
-            }
-        }
-        __syncthreads();
-        if (sh.job.set == 0) break;
-        rows_from_scratch<LAYOUT>(p, sh);                           // ends with a barrier
-    }
-}
-
 // Units that lie in several shares: the parts of a row are merged in the order of the line by eight lanes, in a block of the
-// share the unit begins in.  The blocks of a share also see to rows of its whole units that left the range of their reference,
-// those of the last share to the (empty) results of requests that have nothing to attend.  A chain of two memory latencies:
+// share the unit begins in.  The blocks of the last share also see to the (empty) results of requests that have nothing to attend.  A chain of two memory latencies:
 // what a block has to know about the unit was left by the CTA that began it, and four parts of a row are loaded together.
 // ROWS = 32: a block has 32 rows of one share's unit.  ROWS = 8: it has 8 rows of the units of four shares (of which few have
 // one), and the parts of a row are cut into four runs, walked side by side and joined in order through shared memory.
-template <int LAYOUT, int ROWS>
+template <int ROWS>
 __global__ void __launch_bounds__(256, 2)
 attn_tc_merge_kernel(const __grid_constant__ Params p) {
     CF_PARAMS;
     constexpr int kRuns = 32 / ROWS, kSlices = kRowTile / ROWS, kRunThreads = 256 / kRuns;
     const int max_shares = p.max_shares;
-    __shared__ unsigned s_marked[4];                                // rows of the slice out of range, of the unit cut in every share
-    if (threadIdx.x < 4) s_marked[threadIdx.x] = 0;
-    __syncthreads();
-    bool marked = false;
     __shared__ float s_run[kRuns > 1 ? kRuns - 1 : 1][19][kRuns > 1 ? kRunThreads : 1];   // m, l, ld and 16 dims per thread
     const int lq = bv.q_len, rows_total = n_q_heads * lq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n_classes = (max_shares + kRuns - 1) / kRuns, share0 = blockIdx.x / kSlices, slice = blockIdx.x - share0 * kSlices;
@@ -1052,7 +1004,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
         const int share = share0 + u * n_classes;
         if (share >= max_shares) break;
         const ShareHead head = {word(words.x, 2 * u), word(words.y, 2 * u), word(words.z, 2 * u), word(words.w, 2 * u),
-                                word(words.x, 2 * u + 1), word(words.y, 2 * u + 1), word(words.z, 2 * u + 1), word(words.w, 2 * u + 1)};
+                                word(words.x, 2 * u + 1), word(words.y, 2 * u + 1)};
         if (share == max_shares - 1 && p.n_prefix + p.n_self == 0)
             for (int b = slice; b < bv.n_requests; b += kSlices)
                 if (pv.n_tiles[b] == 0)
@@ -1065,7 +1017,6 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                             if (lse) lse[at + i] = -INFINITY;
                         }
                     }
-        marked |= head.marked != 0;
         const int n_parts = head.n_parts;
         if (n_parts == 0 || slice * ROWS >= head.rows_here) continue;                       // the whole block
         const int run = warp / (8 / kRuns), part_end = n_parts * (run + 1) / kRuns;
@@ -1137,24 +1088,19 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
             }
         }
         const int rg = head.row_first + r, h = rg / lq, j = rg - h * lq;
-        if (valid && l == l) {
-            const float inv = l > 0.f ? 1.f / l : 0.f;
+        if (valid) {
+            const float inv = l == 0.f ? 0.f : 1.f / l;              // a sum that is not a number stays one
             uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)head.layer * span.out_stride + (((size_t)head.b * lq + j) * n_q_heads + h) * kD + e0);
 #pragma unroll
             for (int e = 0; e < 2; ++e)
                 dst[e] = make_uint4(pack_bf16(acc[8 * e] * inv, acc[8 * e + 1] * inv), pack_bf16(acc[8 * e + 2] * inv, acc[8 * e + 3] * inv),
                                     pack_bf16(acc[8 * e + 4] * inv, acc[8 * e + 5] * inv), pack_bf16(acc[8 * e + 6] * inv, acc[8 * e + 7] * inv));
             if ((lane & 7) == 0) {
-                ws.row_lse2[(size_t)head.lb * rows_total + rg] = ld > 0.f ? m + log2f(ld) : -INFINITY;
-                if (lse) lse[(size_t)head.lb * rows_total + rg] = (l > 0.f ? m + log2f(l) : -INFINITY) * kLn2;
+                ws.row_lse2[(size_t)head.lb * rows_total + rg] = ld == 0.f ? -INFINITY : m + log2f(ld);
+                if (lse) lse[(size_t)head.lb * rows_total + rg] = (l == 0.f ? -INFINITY : m + log2f(l)) * kLn2;
             }
         }
-        if (valid && l != l) {                                      // out of the range of its reference
-            marked = true;
-            if ((lane & 7) == 0) atomicOr(&s_marked[u], 1u << (r - slice * ROWS));
-        }
     }
-    if (__syncthreads_or(marked)) marked_from_scratch<LAYOUT, ROWS>(p, s_marked, share0, n_classes, slice);
 }
 
 // Exercises the bounded wait by itself: one CTA initialises an mbarrier that nothing ever arrives on,
@@ -1237,21 +1183,19 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
                             static_cast<In>(k_prefix), static_cast<In>(v_prefix), self_stride, prefix_stride, scale_log2, k_self ? 1 : 0, prefix_len};
     const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
                       k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, static_cast<__nv_bfloat16*>(out), lse};
-    static PerDeviceOnce configured[2], configured_merge[2][2];
+    static PerDeviceOnce configured[2];
     // Few units in many shares each: from thirteen parts to a unit on.  Measured (attention and merge of a call over 50 documents of
     // 160 tokens, us, 32 rows against 8): 2 units (50 parts) 25.7 / 17.5; 6 (25) 22.2 / 18.8; 8 (18) 26.4 / 24.9; 10 (15) 24.3 /
     // 23.3; 12 (12) 25.3 / 26.4 and 26.4 / 27.7; 14 (11) 25.1 / 25.1; 16 (9) 26.7 / 28.2; 24 (6) 32.4 / 34.9; 48 (3) 38.9 / 42.2.
     const bool many_parts = (long long)span.n_layers * b->n_requests * g->n_kv_heads * row_tiles * 13 <= shares;
     const int merge_rows = many_parts ? 8 : 32;
-    auto run = [&](auto kernel, auto merge, int which) {
+    auto run = [&](auto kernel, int which) {
         if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return (int)CF_ERR_CUDA;
-        if (configure_smem_once(configured_merge[which][many_parts], merge, kMergeSmem) != CF_OK) return (int)CF_ERR_CUDA;
         const int rc = launch_chained(kernel, dim3((unsigned)shares), kThreads, kSmemBytes, stream, maps, p);
-        return rc != CF_OK ? rc : launch_chained(merge, dim3((unsigned)((shares + 32 / merge_rows - 1) / (32 / merge_rows) * (kRowTile / merge_rows))), 256, kMergeSmem, stream, p);
+        return rc != CF_OK ? rc : launch_chained(many_parts ? attn_tc_merge_kernel<8> : attn_tc_merge_kernel<32>,
+                                                 dim3((unsigned)((shares + 32 / merge_rows - 1) / (32 / merge_rows) * (kRowTile / merge_rows))), 256, 0, stream, p);
     };
-    constexpr int H = CF_ROPE_HALF, I = CF_ROPE_INTERLEAVED;
-    if (g->rope_layout == H) return run(attn_tc_kernel<H>, many_parts ? attn_tc_merge_kernel<H, 8> : attn_tc_merge_kernel<H, 32>, 0);
-    return run(attn_tc_kernel<I>, many_parts ? attn_tc_merge_kernel<I, 8> : attn_tc_merge_kernel<I, 32>, 1);
+    return g->rope_layout == CF_ROPE_HALF ? run(attn_tc_kernel<CF_ROPE_HALF>, 0) : run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, 1);
 }
 
 }  // namespace cf
