@@ -283,12 +283,12 @@ __device__ __forceinline__ void store_to_first(float* at, float v) {
 // to a load.  Measured against one block of 1024 threads per document: 28 calls of one layer each, 50 documents, 12 heads,
 // 660 -> 598 us a pass.
 __global__ void __launch_bounds__(kScoreThreads)
-score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, int cluster, float* __restrict__ doc_scores,
+score_kernel(BatchView bv, PlanView pv, AttnWorkspace ws, int rows_total, const __grid_constant__ Divisor by_cluster, float* __restrict__ doc_scores,
              float* __restrict__ score_accum) {
     __shared__ float s_red[kScoreThreads / 32];
     __shared__ float s_layer[CF_MAX_LAYERS_PER_CALL];
     chain_next();
-    const int doc = blockIdx.x / cluster, rank = blockIdx.x - doc * cluster;
+    const int cluster = (int)by_cluster.d, doc = by_cluster.quotient(blockIdx.x), rank = (int)blockIdx.x - doc * cluster;
     if (cluster > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     chain_wait();
     const int n_layers = ws.n_layers;
@@ -456,7 +456,7 @@ int launch_scores(const cf_geom* g, const cf_batch* b, const PlanView& pv, const
     const int cluster = (ws.n_layers + rounds - 1) / rounds;
     const int rows_total = g->n_q_heads * b->q_len;
     return launch_chained_clusters(score_kernel, dim3((unsigned)(cluster * b->n_docs_total)), kScoreThreads, 0, (unsigned)cluster, stream, make_batch_view(b), pv,
-                          ws, rows_total, cluster, doc_scores, score_accum);
+                          ws, rows_total, Divisor(cluster), doc_scores, score_accum);
 }
 
 }  // namespace cf

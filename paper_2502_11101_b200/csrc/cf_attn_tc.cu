@@ -243,18 +243,28 @@ struct Params {
     LayerSpan span;
     RowSources src;
     int n_q_heads, n_kv_heads, row_tiles, n_prefix, n_self, max_shares;   // n_prefix, n_self: key tiles
+    Divisor q_len, tiles_of_rows, kv_heads, requests, merge_slices;       // of the batch; merge_slices: of a unit's rows in merge blocks
     __nv_bfloat16* out;
     float* lse;
 };
+
+// What row_lse2 holds of a row whose unit was cut, until its parts are merged: the share the unit begins in and the number of its
+// parts, as a negative quiet NaN (a denominator that is not a number is written as the positive one).
+constexpr uint32_t kPartsOf = 0xffc00000u;
+constexpr int kMaxCodedShares = 1 << 10;
+__device__ __forceinline__ uint32_t parts_code(int share, int n_parts) { return kPartsOf | ((uint32_t)n_parts << 10) | (uint32_t)share; }
+__device__ __forceinline__ bool is_parts_code(uint32_t w) { return (w & kPartsOf) == kPartsOf; }
+__device__ __forceinline__ int first_share(uint32_t w) { return (int)(w & (kMaxCodedShares - 1)); }
+__device__ __forceinline__ int part_count(uint32_t w) { return (int)((w ^ kPartsOf) >> 10); }
 #define CF_PARAMS                                                                                                  \
-    const BatchView& bv = p.bv;                                                                                    \
-    const PlanView& pv = p.pv;                                                                                     \
-    const AttnWorkspace& ws = p.ws;                                                                                \
-    const LayerSpan& span = p.span;                                                                                \
-    const RowSources& src = p.src;                                                                                 \
-    const int n_q_heads = p.n_q_heads, n_kv_heads = p.n_kv_heads;                                                  \
-    __nv_bfloat16* const out_all = p.out;                                                                          \
-    float* const lse = p.lse
+    [[maybe_unused]] const BatchView& bv = p.bv;                                                                   \
+    [[maybe_unused]] const PlanView& pv = p.pv;                                                                    \
+    [[maybe_unused]] const AttnWorkspace& ws = p.ws;                                                               \
+    [[maybe_unused]] const LayerSpan& span = p.span;                                                               \
+    [[maybe_unused]] const RowSources& src = p.src;                                                                \
+    [[maybe_unused]] const int n_q_heads = p.n_q_heads, n_kv_heads = p.n_kv_heads;                                 \
+    [[maybe_unused]] __nv_bfloat16* const out_all = p.out;                                                         \
+[[maybe_unused]] float* const lse = p.lse
 
 // Shared memory of a CTA that computes rows of its share from scratch, over the rings of keys and values.
 constexpr int kRowWarps = kThreads / 32;
@@ -425,7 +435,8 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
         *reinterpret_cast<uint2*>(dst + lane * 4) = make_uint2(pack_bf16(o.x * f, o.y * f), pack_bf16(o.z * f, o.w * f));
         if (lane == 0 && whole) {
             const size_t at = (size_t)sh.sg.lb * rows_total + (size_t)sh.sg.kvh * group * lq + row;
-            ws.row_lse2[at] = top + log2f(ld);
+            const float row_lse2 = top + log2f(ld);
+            ws.row_lse2[at] = row_lse2 == row_lse2 ? row_lse2 : __int_as_float(0x7fffffff);
             if (lse) lse[at] = (top + log2f(l)) * kLn2;
         } else if (lane == 0) {
             ws.part_m[slot] = l == 0.f ? -INFINITY : top > -INFINITY ? top : 0.f;   // (a sum that is not a number has to be seen)
@@ -851,8 +862,11 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
                             ws.part_m[slot] = l_all == 0.f ? -INFINITY : ref;   // a row may see none of the segment's keys
                             ws.part_l[slot] = l_all;
                             if (ws.part_ld) ws.part_ld[slot] = d_all;   // what the document scores are measured against
+                            if (done.t_begin == 0)            // (the share's last segment)
+                                reinterpret_cast<uint32_t*>(ws.row_lse2)[at] =
+                                    parts_code(blockIdx.x, line.share_of(x_end - done.t_end + done.n_unit - 1) - (int)blockIdx.x + 1);
                         } else {
-                            ws.row_lse2[at] = marked ? l_all : ref + log2f(d_all);
+                            ws.row_lse2[at] = marked ? __int_as_float(0x7fffffff) : ref + log2f(d_all);
                             if (lse) lse[at] = (ref + log2f(l_all)) * kLn2;
                         }
                         if (marked) bars.marked = 1;
@@ -978,47 +992,79 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
     }
 }
 
-// Units that lie in several shares: the parts of a row are merged in the order of the line by eight lanes, in a block of the
-// share the unit begins in.  The blocks of the last share also see to the (empty) results of requests that have nothing to attend.  A chain of two memory latencies:
-// what a block has to know about the unit was left by the CTA that began it, and four parts of a row are loaded together.
-// ROWS = 32: a block has 32 rows of one share's unit.  ROWS = 8: it has 8 rows of the units of four shares (of which few have
-// one), and the parts of a row are cut into four runs, walked side by side and joined in order through shared memory.
+constexpr int kMergeThreads = 256;
+
+// Units that lie in several shares: the parts of a row are merged in the order of the line by eight lanes.  A chain of two memory
+// latencies: where the parts are was left by the CTA the unit begins in, and four parts of a row are loaded together.
+// ROWS = 32: a block has a slice of the unit that begins in one share and goes on behind it.  ROWS = 8, for few units of many parts: a
+// block has a slice of one unit and reads from its first row's word how it was cut (blocks that looked at four shares each, of
+// which few begin a unit: 28 calls over 50 documents, 12/2 heads, 553 us, this way 530); the parts of a row are cut into four
+// runs, walked side by side and joined in order through shared memory.  Either also sees to the (empty) results of requests that
+// have nothing to attend.
 template <int ROWS>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(kMergeThreads, 2)
 attn_tc_merge_kernel(const __grid_constant__ Params p) {
     CF_PARAMS;
-    constexpr int kRuns = 32 / ROWS, kSlices = kRowTile / ROWS, kRunThreads = 256 / kRuns;
-    const int max_shares = p.max_shares;
+    constexpr bool kByUnit = ROWS < 32;
+    constexpr int kRuns = 32 / ROWS, kRunThreads = kMergeThreads / kRuns;
     __shared__ float s_run[kRuns > 1 ? kRuns - 1 : 1][19][kRuns > 1 ? kRunThreads : 1];   // m, l, ld and 16 dims per thread
-    const int lq = bv.q_len, rows_total = n_q_heads * lq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n_classes = (max_shares + kRuns - 1) / kRuns, share0 = blockIdx.x / kSlices, slice = blockIdx.x - share0 * kSlices;
+    const int lq = bv.q_len, rows_total = n_q_heads * lq, rows = n_q_heads / n_kv_heads * lq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int slices = (int)p.merge_slices.d;
+    const int at = p.merge_slices.quotient(blockIdx.x), slice = (int)blockIdx.x - at * slices;          // unit or share; slice of its rows
+    ShareHead head;
+    int share = at;
+    if (kByUnit) {
+        const int u = p.tiles_of_rows.quotient(at), row_tile = at - u * p.row_tiles, kvh = p.kv_heads.remainder(u);
+        head.lb = p.kv_heads.quotient(u);
+        head.layer = p.requests.quotient(head.lb);
+        head.b = head.lb - head.layer * bv.n_requests;
+        head.row_first = kvh * rows + row_tile * ws.rg_rows;
+        head.rows_here = min(ws.rg_rows, rows - row_tile * ws.rg_rows);
+    }
     chain_next();
     chain_wait();
-    // lanes 2 i, 2 i + 1: the head of share share0 + i * n_classes
-    int4 words = make_int4(0, 0, 0, 0);
-    if (lane < 2 * kRuns && share0 + (lane >> 1) * n_classes < max_shares)
-        words = reinterpret_cast<const int4*>(reinterpret_cast<const ShareHead*>(ws.marks) + share0 + (lane >> 1) * n_classes)[lane & 1];
-    auto word = [&](int v, int from) { return __shfl_sync(0xffffffffu, v, from); };
-#pragma unroll 1
-    for (int u = 0; u < kRuns; ++u) {
-        const int share = share0 + u * n_classes;
-        if (share >= max_shares) break;
-        const ShareHead head = {word(words.x, 2 * u), word(words.y, 2 * u), word(words.z, 2 * u), word(words.w, 2 * u),
-                                word(words.x, 2 * u + 1), word(words.y, 2 * u + 1)};
-        if (share == max_shares - 1 && p.n_prefix + p.n_self == 0)
-            for (int b = slice; b < bv.n_requests; b += kSlices)
+    if (kByUnit) {
+        if (slice * ROWS >= head.rows_here) return;
+        const size_t first = (size_t)head.lb * rows_total + head.row_first + slice * ROWS;
+        const uint32_t word = reinterpret_cast<const uint32_t*>(ws.row_lse2)[first];
+        if (p.n_prefix + p.n_self == 0 && pv.n_tiles[head.b] == 0) {
+            const int n = min(ROWS, head.rows_here - slice * ROWS);
+            for (int i = threadIdx.x; i < n * (kD / 8); i += kMergeThreads) {
+                const int rg = head.row_first + slice * ROWS + i / (kD / 8), h = rg / lq, j = rg - h * lq;
+                reinterpret_cast<uint4*>(out_all + (size_t)head.layer * span.out_stride + (((size_t)head.b * lq + j) * n_q_heads + h) * kD)[i % (kD / 8)] =
+                    make_uint4(0u, 0u, 0u, 0u);
+            }
+            __syncthreads();                                        // every thread has its word
+            if (threadIdx.x < n) {
+                ws.row_lse2[first + threadIdx.x] = -INFINITY;
+                if (lse) lse[first + threadIdx.x] = -INFINITY;
+            }
+            return;
+        }
+        if (!is_parts_code(word)) return;                           // finished by its one share
+        __syncthreads();                                            // every thread has its word: a row's is written below
+        head.n_parts = part_count(word);
+        share = first_share(word);
+    } else {
+        const int4* from = reinterpret_cast<const int4*>(reinterpret_cast<const ShareHead*>(ws.marks) + share);
+        const int4 lo = from[0], hi = from[1];
+        head = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y};
+        if (share == p.max_shares - 1 && p.n_prefix + p.n_self == 0)
+            for (int b = slice; b < bv.n_requests; b += slices)
                 if (pv.n_tiles[b] == 0)
                     for (int layer = 0; layer < ws.n_layers; ++layer) {
                         uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)layer * span.out_stride + (size_t)b * rows_total * kD);
-                        for (int i = threadIdx.x; i < rows_total * (kD / 8); i += 256) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-                        const size_t at = ((size_t)layer * bv.n_requests + b) * rows_total;
-                        for (int i = threadIdx.x; i < rows_total; i += 256) {
-                            ws.row_lse2[at + i] = -INFINITY;
-                            if (lse) lse[at + i] = -INFINITY;
+                        for (int i = threadIdx.x; i < rows_total * (kD / 8); i += kMergeThreads) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+                        const size_t to = ((size_t)layer * bv.n_requests + b) * rows_total;
+                        for (int i = threadIdx.x; i < rows_total; i += kMergeThreads) {
+                            ws.row_lse2[to + i] = -INFINITY;
+                            if (lse) lse[to + i] = -INFINITY;
                         }
                     }
+        if (head.n_parts == 0 || slice * ROWS >= head.rows_here) return;
+    }
+    {
         const int n_parts = head.n_parts;
-        if (n_parts == 0 || slice * ROWS >= head.rows_here) continue;                       // the whole block
         const int run = warp / (8 / kRuns), part_end = n_parts * (run + 1) / kRuns;
         const int r = slice * ROWS + (warp - run * (8 / kRuns)) * 4 + (lane >> 3), e0 = (lane & 7) * 16;   // row of the unit; this lane's dims
         const bool valid = run == 0 && r < head.rows_here;
@@ -1042,7 +1088,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 o[x][1] = *reinterpret_cast<const uint4*>(part_o + slot * kD + 8);
             }
             const float m_new = fmaxf(fmaxf(m, fmaxf(mp[0], mp[1])), fmaxf(mp[2], mp[3]));
-            const float keep = m > -INFINITY ? exp2f(m - m_new) : 0.f;
+            const float keep = m > -INFINITY ? fast_exp2(m - m_new) : 0.f;
             m = m_new;
             l *= keep;
             ld *= keep;
@@ -1051,7 +1097,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
 #pragma unroll
             for (int x = 0; x < 4; ++x)
                 if (mp[x] > -INFINITY) {
-                    const float w = exp2f(mp[x] - m_new);
+                    const float w = fast_exp2(mp[x] - m_new);
                     l = fmaf(lp[x], w, l);
                     ld = fmaf(dp[x], w, ld);
                     const uint32_t pairs[8] = {o[x][0].x, o[x][0].y, o[x][0].z, o[x][0].w, o[x][1].x, o[x][1].y, o[x][1].z, o[x][1].w};
@@ -1063,7 +1109,6 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 }
         }
         if (kRuns > 1) {
-            __syncthreads();                                        // the unit before has been joined
             if (run > 0) {
                 float* mine = &s_run[run - 1][0][threadIdx.x % kRunThreads];
                 mine[0] = m;
@@ -1079,7 +1124,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 const float* other = &s_run[k][0][threadIdx.x];
                 const float mo = other[0];
                 if (mo == -INFINITY) continue;
-                const float m_new = fmaxf(m, mo), keep = m > -INFINITY ? exp2f(m - m_new) : 0.f, w = exp2f(mo - m_new);
+                const float m_new = fmaxf(m, mo), keep = m > -INFINITY ? fast_exp2(m - m_new) : 0.f, w = fast_exp2(mo - m_new);
                 m = m_new;
                 l = fmaf(other[kRunThreads], w, l * keep);
                 ld = fmaf(other[2 * kRunThreads], w, ld * keep);
@@ -1087,7 +1132,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 for (int e = 0; e < 16; ++e) acc[e] = fmaf(other[(3 + e) * kRunThreads], w, acc[e] * keep);
             }
         }
-        const int rg = head.row_first + r, h = rg / lq, j = rg - h * lq;
+        const int rg = head.row_first + r, h = p.q_len.quotient(rg), j = rg - h * lq;
         if (valid) {
             const float inv = l == 0.f ? 0.f : 1.f / l;              // a sum that is not a number stays one
             uint4* dst = reinterpret_cast<uint4*>(out_all + (size_t)head.layer * span.out_stride + (((size_t)head.b * lq + j) * n_q_heads + h) * kD + e0);
@@ -1177,23 +1222,27 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
         if (rc != CF_OK) return rc;
     }
     const BatchView bv = make_batch_view(b);
-    const int shares = sm_count();
+    const int shares = std::min(sm_count(), kMaxCodedShares);
     typedef const __nv_bfloat16* In;
     const RowSources src = {static_cast<In>(q), static_cast<In>(k), static_cast<In>(v), static_cast<In>(k_self), static_cast<In>(v_self),
                             static_cast<In>(k_prefix), static_cast<In>(v_prefix), self_stride, prefix_stride, scale_log2, k_self ? 1 : 0, prefix_len};
-    const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
-                      k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, static_cast<__nv_bfloat16*>(out), lse};
-    static PerDeviceOnce configured[2];
+    const long long units = (long long)span.n_layers * b->n_requests * g->n_kv_heads * row_tiles;
     // Few units in many shares each: from thirteen parts to a unit on.  Measured (attention and merge of a call over 50 documents of
     // 160 tokens, us, 32 rows against 8): 2 units (50 parts) 25.7 / 17.5; 6 (25) 22.2 / 18.8; 8 (18) 26.4 / 24.9; 10 (15) 24.3 /
     // 23.3; 12 (12) 25.3 / 26.4 and 26.4 / 27.7; 14 (11) 25.1 / 25.1; 16 (9) 26.7 / 28.2; 24 (6) 32.4 / 34.9; 48 (3) 38.9 / 42.2.
-    const bool many_parts = (long long)span.n_layers * b->n_requests * g->n_kv_heads * row_tiles * 13 <= shares;
-    const int merge_rows = many_parts ? 8 : 32;
+    const bool many_parts = units * 13 <= shares;
+    const int merge_rows = many_parts ? 8 : 32, slices = (ws.rg_rows + merge_rows - 1) / merge_rows;
+    const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
+                      k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, Divisor(b->q_len), Divisor((int)row_tiles), Divisor(g->n_kv_heads),
+                      Divisor(b->n_requests), Divisor(slices), static_cast<__nv_bfloat16*>(out), lse};
+    static PerDeviceOnce configured[2];
     auto run = [&](auto kernel, int which) {
         if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return (int)CF_ERR_CUDA;
         const int rc = launch_chained(kernel, dim3((unsigned)shares), kThreads, kSmemBytes, stream, maps, p);
-        return rc != CF_OK ? rc : launch_chained(many_parts ? attn_tc_merge_kernel<8> : attn_tc_merge_kernel<32>,
-                                                 dim3((unsigned)((shares + 32 / merge_rows - 1) / (32 / merge_rows) * (kRowTile / merge_rows))), 256, 0, stream, p);
+        if (rc != CF_OK) return rc;
+        const unsigned blocks = (unsigned)((many_parts ? units : shares) * slices);
+        const auto merge = many_parts ? attn_tc_merge_kernel<8> : attn_tc_merge_kernel<32>;
+        return launch_chained(merge, dim3(blocks), kMergeThreads, 0, stream, p);
     };
     return g->rope_layout == CF_ROPE_HALF ? run(attn_tc_kernel<CF_ROPE_HALF>, 0) : run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, 1);
 }

@@ -54,6 +54,21 @@ __host__ __device__ inline int tile_base(int doc_begin, int row_begin) {
     return doc_begin + row_begin / kTile;
 }
 
+// Division of 0 <= n < 2^31 by a divisor the host knows: three dependent instructions instead of the thirty of a division whose
+// divisor comes out of a register (and over a hundred in 64 bits), on the way to the first load of kernels that run for 3 us.
+struct Divisor {
+    unsigned d, mul, shift;
+    Divisor() = default;
+    explicit Divisor(int by) : d((unsigned)by), mul(0), shift(0) {
+        while (shift < 31 && (1u << shift) < d) ++shift;
+        mul = (unsigned)((((1ull << shift) - d) << 32) / d) + 1u;
+    }
+#ifdef __CUDACC__
+    __device__ __forceinline__ int quotient(int n) const { return (int)((__umulhi((unsigned)n, mul) + (unsigned)n) >> shift); }
+    __device__ __forceinline__ int remainder(int n) const { return n - quotient(n) * (int)d; }
+#endif
+};
+
 GeomView make_geom_view(const cf_geom* g);
 BatchView make_batch_view(const cf_batch* b);
 PlanView make_plan_view(const cf_geom* g, const cf_batch* b, void* plan);
