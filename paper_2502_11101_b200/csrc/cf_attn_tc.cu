@@ -4,6 +4,8 @@
 // rotated there in place by their document's delta (fp32, one rounding: bit for bit what cf_reposition_keys writes) and
 // handed to the tensor cores.
 //
+// Kv heads with several tiles of query rows are worked on by pairs of CTAs where shares are long enough (cf_attn_pair.cu).
+//
 // Work: the key tiles (runs of at most kTile rows of one document, from the plan) of every (layer, request, kv head, tile of
 // at most 128 query rows) laid on one line and cut into equal shares, one per SM: a CTA walks its share, which may end in the
 // middle of a unit and hold several whole ones.  A unit inside one share is finished there; parts of others meet in the merge
@@ -30,39 +32,31 @@
 // roles leave their loops, and the CTA frees its tensor memory and exits.  Each barrier has one kind of waiter, which waits
 // for every phase in order.
 #include <algorithm>
-#include <cstddef>
 
-#include "cf_row_group.cuh"
-#include "cf_tc_util.cuh"
+#include "cf_attn_roles.cuh"
 
 namespace cf {
 
-namespace {
+using namespace line;
 
-using namespace tc;
+namespace {
 
 constexpr int kThreads = 512;
 constexpr int kRotateWarps = 6;
-constexpr int kRowTile = 128;
 constexpr int kKvHalf = kTile * 128;               // one 64-column half of a key or value tile
 constexpr int kKvBytes = 2 * kKvHalf;
-constexpr int kBoxes = kTile / 16;                 // copy boxes are 16, 32, .. kTile rows high
 constexpr int kKStages = 6, kVStages = 3;          // with the three S buffers of two warpgroups: everything repeats after six tiles
 constexpr int kSBuffers = 3;
-constexpr int kMetaRing = 16, kSegRing = 16;
-constexpr int kPrefSlots = 48;
 constexpr int kLoadWarp = 9, kMmaWarp = 12;
-constexpr int kTrigBytes = kD / 2 * 8;
 constexpr uint32_t kColO = 0, kColQ = 128, kColS = 192;
-constexpr float kSumLimit = 0x1p80f;               // a larger tile sum leaves the range: 2^47 are left for the values and the other tiles
 static_assert(kColS + kSBuffers * kTile <= 512, "tensor memory columns");
 static_assert(kTile % 16 == 0 && kTile <= 96, "three S buffers");
 static_assert(kKStages == 6 && kVStages == 3 && kSBuffers == 3, "rings of one period");
 
-struct StoreMaps {
-    CUtensorMap k[kBoxes], v[kBoxes];              // the stores, one map per box height
-    CUtensorMap ks, vs;                            // keys and values of the query tokens themselves (whole tiles)
-    CUtensorMap kp, vp;                            // keys and values of a shared prefix cache (whole tiles)
+struct R {
+    static constexpr bool kPair = false;
+    static constexpr int kSoftmaxGroups = 2, kKStages = 6, kSBuffers = 3;
+    static constexpr uint32_t kColO = 0, kColQ = 128, kColS = 192;
 };
 
 struct Barriers {
@@ -76,143 +70,6 @@ struct Barriers {
     volatile int marked;                           // a row of the share has to be computed from scratch
 };
 
-// Tile descriptions: flags beside the length, and which keys they are.
-constexpr int kFirstOfSegment = 1 << 8, kLastOfSegment = 1 << 9;
-constexpr int kKindPrefix = -1, kKindSelf = -2;    // tile index of a prefix tile; kKindSelf - n: n-th tile of the query tokens
-
-// a / b for a >= 0, b > 0 from the reciprocal, exact after its correction: the few divisions on the way to a CTA's first
-// copy are a serial chain, and the integer division of the language is three times as long.
-__device__ __forceinline__ int quick_div(int a, int b) {
-    int q = (int)__fdividef((float)a, (float)b);
-    int r = a - q * b;
-    while (r < 0) {
-        --q;
-        r += b;
-    }
-    while (r >= b) {
-        ++q;
-        r -= b;
-    }
-    return q;
-}
-
-// The line of all key tiles (order: layer, request, kv head and tile of query rows, key tile).  A request's tiles are its
-// documents' (plan), then those of the prefix cache, then those of the query tokens.
-struct Line {
-    const int *pref, *begin;
-    int stride, n_requests, row_tiles, tiles;      // tiles = kv heads * tiles of query rows
-    int n_prefix, n_self, per_layer, n_shares, each, rest;
-    __device__ __forceinline__ int cut(int c) const { return c * each + min(c, rest); }
-    __device__ __forceinline__ int share_of(int x) const {
-        const int y = x - rest * (each + 1);
-        return y < 0 ? quick_div(x, each + 1) : rest + quick_div(y, each);
-    }
-};
-
-struct Segment {
-    int lb, layer, b, kvh, row0, rows_here;        // unit: query rows row0 .. of the kv head
-    int t_begin, t_end, n_unit, n_doc, tile0;      // tiles of the unit this segment covers; documents' tiles; first in the plan
-};
-
-// A share has at least two tiles.  Measured, attention and merge of a call (us, a least of 1 / 2 / 3 / 4; larger calls do not
-// notice): 25 documents of 160 tokens, 12/2 heads 16.9 / 16.9 / 19.4 / 21.2; 6 documents 14.0 / 14.0 / 14.5 / 14.8; 20 documents of
-// 90, 32/8 heads 15.3 / 14.8; 3 of 180, 32/32 heads 13.8 / 12.8; units of three and five tiles, which two do not divide: 3 and 5 of
-// 90, 32/8 heads 12.5 / 15.6 and 13.3 / 16.1.  Three and more cost parallelism, between one and two it is even.
-constexpr int kMinShare = 2;
-
-// What the line is made from: prefix sums of the requests' tiles (one entry per `stride` requests), and with one entry per
-// request also the requests' first tiles in the plan.  Filled by the first warp.
-struct Requests {
-    int pref[kPrefSlots + 1], begin[kPrefSlots];
-};
-
-__device__ __forceinline__ void scan_requests(const BatchView& bv, const PlanView& pv, int extra, Requests& rq) {
-    const int lane = threadIdx.x & 31, stride = (bv.n_requests + kPrefSlots - 1) / kPrefSlots;
-    int carry = 0;
-    for (int b0 = 0; b0 < bv.n_requests; b0 += 32) {
-        const int b = b0 + lane;
-        int n = 0, begin = 0;
-        if (b < bv.n_requests) {
-            n = pv.n_tiles[b] + extra;
-            if (stride == 1) begin = pv.tile_begin[b];
-        }
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int up = __shfl_up_sync(0xffffffffu, n, o);
-            if (lane >= o) n += up;
-        }
-        if (b < bv.n_requests) {
-            if (stride == 1) rq.begin[b] = begin;
-            if ((b + 1) % stride == 0 || b == bv.n_requests - 1) rq.pref[(b + stride) / stride] = carry + n;
-        }
-        carry += __shfl_sync(0xffffffffu, n, 31);
-    }
-    if (lane == 0) rq.pref[0] = 0;
-}
-
-__device__ __forceinline__ Line make_line(const BatchView& bv, const AttnWorkspace& ws, const Requests& rq, int n_kv_heads, int row_tiles,
-                                          int n_prefix, int n_self, int max_shares) {
-    Line line;
-    line.pref = rq.pref;
-    line.begin = rq.begin;
-    line.n_requests = bv.n_requests;
-    line.stride = (bv.n_requests + kPrefSlots - 1) / kPrefSlots;
-    line.n_prefix = n_prefix;
-    line.n_self = n_self;
-    line.row_tiles = row_tiles;
-    line.tiles = n_kv_heads * line.row_tiles;
-    line.per_layer = rq.pref[(bv.n_requests + line.stride - 1) / line.stride] * line.tiles;
-    const int total = line.per_layer * ws.n_layers;
-    line.n_shares = max(1, min(max_shares, total / kMinShare));
-    line.each = quick_div(total, line.n_shares);
-    line.rest = total - line.each * line.n_shares;
-    return line;
-}
-
-__device__ __forceinline__ Segment segment_at(const BatchView& bv, const PlanView& pv, const AttnWorkspace& ws, const Line& line, int group,
-                                              int x, int end) {
-    Segment sg;
-    sg.layer = quick_div(x, line.per_layer);
-    int r = x - sg.layer * line.per_layer;
-    int lo = 0, hi = (line.n_requests + line.stride - 1) / line.stride;     // the last slot that starts at or before r
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (line.pref[mid] * line.tiles <= r) lo = mid; else hi = mid;
-    }
-    const int extra = line.n_prefix + line.n_self;
-    int b = lo, start = line.pref[lo], n;
-    if (line.stride == 1) {
-        n = line.pref[b + 1] - start;
-        sg.tile0 = line.begin[b];
-    } else {
-        b = lo * line.stride;
-        n = pv.n_tiles[b] + extra;
-        while ((start + n) * line.tiles <= r) {
-            start += n;
-            n = pv.n_tiles[++b] + extra;
-        }
-        sg.tile0 = pv.tile_begin[b];
-    }
-    r -= start * line.tiles;
-    const int unit = quick_div(r, n);
-    sg.n_unit = n;
-    sg.n_doc = n - extra;
-    sg.t_begin = r - unit * n;
-    sg.t_end = min(n, sg.t_begin + (end - x));
-    sg.b = b;
-    sg.lb = sg.layer * line.n_requests + b;
-    sg.kvh = quick_div(unit, line.row_tiles);
-    sg.row0 = (unit - sg.kvh * line.row_tiles) * ws.rg_rows;
-    sg.rows_here = min(ws.rg_rows, group * bv.q_len - sg.row0);
-    return sg;
-}
-
-// What a CTA leaves for the merge kernel: the unit that begins in its share and goes on behind it (n_parts = 0: none).
-struct ShareHead {
-    int n_parts, lb, layer, b, row_first, rows_here, unused[2];          // row_first: of the unit among the rows of a request
-};
-static_assert(sizeof(ShareHead) == 32, "two 16-byte loads");
-
 struct Shared {
     Barriers bars;
     int4 meta[kMetaRing];                          // tiles in flight: length and flags, tile index or kind, first row, kv head and layer
@@ -221,273 +78,11 @@ struct Shared {
     Line line;
     float ref[2][kRowTile];                        // [segment parity][row]
     alignas(16) float2 trig[kKStages][kD / 2];     // cosines and sines of the documents of the key stages
-    float sum[2][2][kRowTile], docs[2][2][kRowTile];   // [segment parity][warpgroup][row]
+    Sums<2> sums;
     Requests requests;
 };
 constexpr int kSmemBytes = (kKStages + kVStages) * kKvBytes + (int)sizeof(Shared) + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
-
-// Keys and values of a call outside the tensor maps, for rows that are computed from scratch.
-struct RowSources {
-    const __nv_bfloat16 *q, *k, *v, *ks, *vs, *kp, *vp;
-    long long self_stride, prefix_stride;
-    float scale_log2;
-    int with_self, prefix_len;
-};
-
-// Everything a kernel of this file is told: one constant, so that the rarely taken paths can be handed its address.
-struct Params {
-    BatchView bv;
-    PlanView pv;
-    AttnWorkspace ws;
-    LayerSpan span;
-    RowSources src;
-    int n_q_heads, n_kv_heads, row_tiles, n_prefix, n_self, max_shares;   // n_prefix, n_self: key tiles
-    Divisor q_len, tiles_of_rows, kv_heads, requests, merge_slices;       // of the batch; merge_slices: of a unit's rows in merge blocks
-    __nv_bfloat16* out;
-    float* lse;
-};
-
-// What row_lse2 holds of a row whose unit was cut, until its parts are merged: the share the unit begins in and the number of its
-// parts, as a negative quiet NaN (a denominator that is not a number is written as the positive one).
-constexpr uint32_t kPartsOf = 0xffc00000u;
-constexpr int kMaxCodedShares = 1 << 10;
-__device__ __forceinline__ uint32_t parts_code(int share, int n_parts) { return kPartsOf | ((uint32_t)n_parts << 10) | (uint32_t)share; }
-__device__ __forceinline__ bool is_parts_code(uint32_t w) { return (w & kPartsOf) == kPartsOf; }
-__device__ __forceinline__ int first_share(uint32_t w) { return (int)(w & (kMaxCodedShares - 1)); }
-__device__ __forceinline__ int part_count(uint32_t w) { return (int)((w ^ kPartsOf) >> 10); }
-#define CF_PARAMS                                                                                                  \
-    [[maybe_unused]] const BatchView& bv = p.bv;                                                                   \
-    [[maybe_unused]] const PlanView& pv = p.pv;                                                                    \
-    [[maybe_unused]] const AttnWorkspace& ws = p.ws;                                                               \
-    [[maybe_unused]] const LayerSpan& span = p.span;                                                               \
-    [[maybe_unused]] const RowSources& src = p.src;                                                                \
-    [[maybe_unused]] const int n_q_heads = p.n_q_heads, n_kv_heads = p.n_kv_heads;                                 \
-    [[maybe_unused]] __nv_bfloat16* const out_all = p.out;                                                         \
-[[maybe_unused]] float* const lse = p.lse
-
-// Shared memory of a CTA that computes rows of its share from scratch, over the rings of keys and values.
-constexpr int kRowWarps = kThreads / 32;
-struct RowTile {                   // where a key tile lies; row j of the query sees its keys up to j - first
-    const __nv_bfloat16 *k, *v;
-    const float2* trig;            // null: not a document's
-    long long pitch;
-    int len, first, index;
-};
-struct RowScratch {
-    rows::Stage stage[kRowWarps];  // of every warp
-    RowTile tile[kRowWarps][2];    // the current tile and the next one (registers are what the keys and sums need)
-    rows::Queries q;
-    alignas(16) float o[rows::kGroupRows][kD];
-    float m[kRowWarps][rows::kGroupRows], l[kRowWarps][rows::kGroupRows], docs[kRowWarps][rows::kGroupRows];   // of every warp
-    Segment sg;
-    unsigned todo[kRowTile / 32];  // rows of the segment that are still to be computed
-    int row[rows::kGroupRows];     // the group, as rows of the segment
-    int n_rows;
-    int x;                         // position of the share behind the segment
-};
-static_assert(sizeof(RowScratch) <= (kKStages + kVStages) * kKvBytes, "over the rings");
-static_assert(alignof(RowScratch) == 16 && offsetof(RowScratch, q) % 16 == 0 && offsetof(RowScratch, o) % 16 == 0, "16-byte accesses");
-
-// Up to eight query rows (every set bit of `set`, from row `row0` of the segment on) over the segment's key tiles, every warp
-// with every sixteenth tile under a running maximum of its own.  Leaves what the epilogue leaves of a row - a finished row or
-// the part of one - and the log-sum-exps of the document tiles.
-template <int LAYOUT>
-__device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& sh, int row0, unsigned set) {
-    CF_PARAMS;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lq = bv.q_len, group = n_q_heads / n_kv_heads, rows_total = n_q_heads * lq;
-    if (warp < rows::kGroupRows) {                                  // a row of the group per warp; beyond them the last one again
-        const int n_rows = min(rows::kGroupRows, __popc(set)), r = row0 + rows::nth_bit(set, min(warp, n_rows - 1)), row = sh.sg.row0 + r, g = row / lq, j = row - g * lq;
-        if (lane == 0) sh.row[warp] = r;
-        if (threadIdx.x == 0) sh.n_rows = n_rows;
-        if (lane < 16)
-            sh.q.put(warp, lane, src.q + (size_t)sh.sg.layer * span.q_stride + (((size_t)sh.sg.b * lq + j) * n_q_heads + sh.sg.kvh * group + g) * kD);
-    }
-    __syncthreads();
-    const int j = (sh.sg.row0 + sh.row[lane >> 2]) % lq;
-    rows::Stage& stage = sh.stage[warp];
-    RowTile(&tile)[2] = sh.tile[warp];
-    auto describe = [&](int t, RowTile& x) {
-        if (lane == 0) {
-            const int n_doc = sh.sg.n_doc, b = sh.sg.b;
-            const long long layer = sh.sg.layer;
-            long long pitch = (long long)n_kv_heads * kD, at;
-            const __nv_bfloat16 *k = src.k, *v = src.v;
-            const float2* trig = nullptr;
-            int first = -(1 << 30), index = -1, len;
-            if (t < n_doc) {
-                index = sh.sg.tile0 + t;
-                pitch = bv.token_stride;
-                at = layer * span.kv_stride + pv.tile_row0[index] * pitch;
-                len = pv.tile_len[index];
-                trig = pv.trig + (size_t)pv.tile_doc[index] * (kD / 2);
-            } else if (t < n_doc + p.n_prefix) {
-                const int row0 = (t - n_doc) * kTile;
-                k = src.kp;
-                v = src.vp;
-                at = layer * src.prefix_stride + row0 * pitch;
-                len = min(kTile, src.prefix_len - row0);
-            } else {
-                first = (t - n_doc - p.n_prefix) * kTile;           // causal mask
-                k = src.ks;
-                v = src.vs;
-                at = layer * src.self_stride + ((long long)b * lq + first) * pitch;
-                len = min(kTile, lq - first);
-            }
-            at += sh.sg.kvh * kD;
-            x = {k + at, v + at, trig, pitch, len, first, index};
-        }
-        __syncwarp();
-    };
-    auto copy_keys = [&](const RowTile& x, int i) { rows::copy_step(stage.k, x.k + i * x.pitch, x.pitch, x.len - i); };
-    auto copy_values = [&](const RowTile& x, int i) { rows::copy_step(stage.v, x.v + i * x.pitch, x.pitch, x.len - i); };
-    rows::Group acc;
-    acc.clear();
-    float docs = 0.f, in_tile = 0.f;                                // the parts of acc.l on documents and on the current tile
-    int t = sh.sg.t_begin + warp, i = 0, now = 0;                   // the current tile lies in tile[now]
-    if (t < sh.sg.t_end) {
-        describe(t, tile[0]);
-        copy_keys(tile[0], 0);
-        rows::copies_end();
-        copy_values(tile[0], 0);
-        rows::copies_end();
-    }
-#pragma unroll 1
-    while (t < sh.sg.t_end) {
-        rows::Keys keys;
-        rows::copies_wait();
-        keys.read(stage);
-        const int visible = min(tile[now].len, j + 1 - tile[now].first) - i;
-        const bool last = i + rows::kStepKeys >= tile[now].len, more = !last || t + kRowWarps < sh.sg.t_end;
-        const int next = last ? now ^ 1 : now;                      // the tile of the step behind this one
-        i = last ? 0 : i + rows::kStepKeys;                         // and its place there
-        if (last && more) describe(t + kRowWarps, tile[next]);
-        __syncwarp();                                               // every lane has its fragments
-        if (more) copy_keys(tile[next], i);
-        rows::copies_end();
-        const float2* trig = tile[now].trig;
-        if (trig) keys.rotate<LAYOUT>(trig);
-        float alpha;
-        const float sum = acc.scores(sh.q, keys, visible, src.scale_log2, alpha);
-        in_tile = fmaf(in_tile, alpha, sum);
-        docs = fmaf(docs, alpha, tile[now].trig ? sum : 0.f);
-        rows::copies_wait();
-        acc.values(stage);
-        __syncwarp();
-        if (more) copy_values(tile[next], i);
-        rows::copies_end();
-        if (last) {
-            in_tile = rows::over_keys(in_tile);
-            const int index = tile[now].index;
-            if (index >= 0 && (lane & 3) == 0)                      // (rows beyond the group's repeat its last one)
-                ws.tile_lse2[((size_t)sh.sg.layer * ws.max_tiles + index) * rows_total + (size_t)sh.sg.kvh * group * lq + sh.sg.row0 + sh.row[lane >> 2]] =
-                    acc.m + log2f(in_tile);
-            in_tile = 0.f;
-            t += kRowWarps;
-            now = next;
-            __syncwarp();                                           // the tile has been read
-        }
-    }
-    acc.l = rows::over_keys(acc.l);
-    docs = rows::over_keys(docs);
-    if ((lane & 3) == 0) {
-        sh.m[warp][lane >> 2] = acc.m;
-        sh.l[warp][lane >> 2] = acc.l;
-        sh.docs[warp][lane >> 2] = docs;
-    }
-    __syncthreads();
-    // join the warps, in order: a row's reference is the largest of theirs (-inf: nothing to attend)
-    float weight[2];                                                // of this warp's rows 2 t and 2 t + 1
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        const int r = 2 * (lane & 3) + x;
-        float top = sh.m[0][r];
-        for (int w = 1; w < kRowWarps; ++w) top = fmaxf(top, sh.m[w][r]);
-        weight[x] = sh.m[warp][r] > -INFINITY ? exp2f(sh.m[warp][r] - top) : sh.l[warp][r];   // nothing seen: 0 (or not a number)
-    }
-    for (int w = 0; w < kRowWarps; ++w) {
-        if (w == warp)
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    float2& to = *reinterpret_cast<float2*>(&sh.o[2 * (lane & 3) + x][(i >> 2) * 64 + (lane >> 2) * 8 + 2 * (i & 3)]);
-                    const float2 was = w == 0 ? make_float2(0.f, 0.f) : to;
-                    to = make_float2(fmaf(acc.o[i][x], weight[x], was.x), fmaf(acc.o[i][x + 2], weight[x], was.y));
-                }
-        __syncthreads();
-    }
-    if (warp < sh.n_rows) {                                         // a row per warp, four dims per lane
-        float top = sh.m[0][warp], l = 0.f, ld = 0.f;
-        for (int w = 1; w < kRowWarps; ++w) top = fmaxf(top, sh.m[w][warp]);
-        for (int w = 0; w < kRowWarps; ++w) {
-            const float f = sh.m[w][warp] > -INFINITY ? exp2f(sh.m[w][warp] - top) : 1.f;
-            l = fmaf(sh.l[w][warp], f, l);
-            ld = fmaf(sh.docs[w][warp], f, ld);
-        }
-        const bool whole = sh.sg.t_end - sh.sg.t_begin == sh.sg.n_unit;
-        const int row = sh.sg.row0 + sh.row[warp], g = row / lq, jj = row - g * lq;
-        const size_t slot = ((size_t)2 * blockIdx.x + (sh.sg.t_begin == 0 ? 1 : 0)) * kRowTile + sh.row[warp];
-        const float f = !whole ? 1.f : l == 0.f ? 0.f : 1.f / l;
-        const float4 o = *reinterpret_cast<const float4*>(&sh.o[warp][lane * 4]);
-        __nv_bfloat16* dst = whole ? out_all + (size_t)sh.sg.layer * span.out_stride + (((size_t)sh.sg.b * lq + jj) * n_q_heads + sh.sg.kvh * group + g) * kD
-                                   : reinterpret_cast<__nv_bfloat16*>(ws.part_o) + slot * kD;
-        *reinterpret_cast<uint2*>(dst + lane * 4) = make_uint2(pack_bf16(o.x * f, o.y * f), pack_bf16(o.z * f, o.w * f));
-        if (lane == 0 && whole) {
-            const size_t at = (size_t)sh.sg.lb * rows_total + (size_t)sh.sg.kvh * group * lq + row;
-            const float row_lse2 = top + log2f(ld);
-            ws.row_lse2[at] = row_lse2 == row_lse2 ? row_lse2 : __int_as_float(0x7fffffff);
-            if (lse) lse[at] = (top + log2f(l)) * kLn2;
-        } else if (lane == 0) {
-            ws.part_m[slot] = l == 0.f ? -INFINITY : top > -INFINITY ? top : 0.f;   // (a sum that is not a number has to be seen)
-            ws.part_l[slot] = l;
-            if (ws.part_ld) ws.part_ld[slot] = ld;
-        }
-    }
-    __syncthreads();                                                // the shared memory may be used again
-}
-
-// The rows of a share that left the range of their reference (their sums are not numbers), segment by segment, in eights of
-// neighbours.  Only rows whose logits lie more than 2^80 above the first 16 of the segment come here, and keys that are not
-// finite.  A segment's reference is its own, so a row that left it in one share is computed over that share's keys and joins the
-// other parts like any other.  In the merge kernel, over all keys of the row (one block of eight warps had to walk them), the path
-// cost every merge 0.3 to 0.5 us although nobody took it: one layer of 20 documents, 32/32 heads 48.3 -> 46.6 us, 28 one-layer
-// calls over 50 documents, 12/2 heads 574 -> 559.  Calls with such rows: four layers of 50 documents of 160 tokens, 12/2 heads, 44 us
-// without, one row a layer 166 -> 79, every row 759 -> 398; one layer of 2 x 60 documents of 180, 32/32 heads, 93 us, 265 -> 166 and
-// 1109 -> 646; of 4 x 50 of 160, 28/4 heads, 75 us, 202 -> 130 and 687 -> 720 (few tiles per share leave warps idle).
-template <int LAYOUT>
-__device__ __forceinline__ void marked_from_scratch(const Params& p, RowScratch& sh, const Line& line) {
-    const int group = p.n_q_heads / p.n_kv_heads;
-    if (threadIdx.x == 0) sh.x = line.cut(blockIdx.x);
-#pragma unroll 1
-    while (true) {
-        __syncthreads();                                            // the segment before has been read
-        if (sh.x >= line.cut(blockIdx.x + 1)) break;
-        if (threadIdx.x == 0) sh.sg = segment_at(p.bv, p.pv, p.ws, line, group, sh.x, line.cut(blockIdx.x + 1));
-        __syncthreads();
-        if (threadIdx.x < kRowTile) {
-            const int rows = group * p.bv.q_len;
-            float l = 0.f;
-            if ((int)threadIdx.x < sh.sg.rows_here)
-                l = sh.sg.t_end - sh.sg.t_begin == sh.sg.n_unit
-                        ? p.ws.row_lse2[(size_t)sh.sg.lb * p.n_q_heads * p.bv.q_len + (size_t)sh.sg.kvh * rows + sh.sg.row0 + threadIdx.x]
-                        : p.ws.part_l[((size_t)2 * blockIdx.x + (sh.sg.t_begin == 0 ? 1 : 0)) * kRowTile + threadIdx.x];
-            const unsigned set = __ballot_sync(0xffffffffu, l != l);
-            if ((threadIdx.x & 31) == 0) sh.todo[threadIdx.x >> 5] = set;
-        }
-        if (threadIdx.x == 0) sh.x += sh.sg.t_end - sh.sg.t_begin;
-#pragma unroll 1
-        while (true) {
-            __syncthreads();
-            const int w = sh.todo[0] ? 0 : sh.todo[1] ? 1 : sh.todo[2] ? 2 : 3;
-            const unsigned set = sh.todo[w];
-            if (set == 0) break;
-            __syncthreads();
-            if (threadIdx.x == 0) sh.todo[w] = set ^ rows::next_group(set);
-            rows_from_scratch<LAYOUT>(p, sh, w * 32, set);
-        }
-    }
-}
 
 template <int LAYOUT>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -539,7 +134,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
             const Line l = make_line(bv, ws, sh.requests, n_kv_heads, p.row_tiles, p.n_prefix, p.n_self, (int)gridDim.x);
             sh.line = l;
             const int begin = (int)blockIdx.x < l.n_shares ? l.cut(blockIdx.x) : 0, end = (int)blockIdx.x < l.n_shares ? l.cut(blockIdx.x + 1) : 0;
-            if (begin < end) sh.segments[0] = segment_at(bv, pv, ws, l, group, begin, end);
+            if (begin < end) sh.segments[0] = segment_at<false>(bv, pv, ws, l, group, begin, end);
         }
     }
     tc_fence_before();
@@ -584,7 +179,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
                     const float2* trig = pv.trig + (size_t)doc * (kD / 2);
                     ++x;
                     if (++t == sg.t_end && x < x_end) {
-                        sg = segment_at(bv, pv, ws, line, group, x, x_end);
+                        sg = segment_at<false>(bv, pv, ws, line, group, x, x_end);
                         t = sg.t_begin;
                         sh.segments[segments & (kSegRing - 1)] = sg;
                         mbar_arrive(smem_u32(&bars.segment[segments & (kSegRing - 1)]));
@@ -675,10 +270,10 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
                 const uint64_t b0 = bk_desc + (uint64_t)(s.j * (kKvBytes >> 4));
                 const uint32_t s_tmem = tmem + kColS + (s.j >= 3 ? s.j - 3 : s.j) * kTile, q_tmem = tmem + kColQ;
                 if (lead) {
-                    umma_ts_lit<false>(s_tmem, q_tmem, b0, idesc);
+                    umma_ts_lit<1, false>(s_tmem, q_tmem, b0, idesc);
 #pragma unroll
                     for (int kk = 1; kk < 8; ++kk)                  // 16 dims per instruction
-                        umma_ts_lit<true>(s_tmem, q_tmem + kk * 8, b0 + (uint64_t)(((kk >> 2) * kKvHalf + (kk & 3) * 32) >> 4), idesc);
+                        umma_ts_lit<1, true>(s_tmem, q_tmem + kk * 8, b0 + (uint64_t)(((kk >> 2) * kKvHalf + (kk & 3) * 32) >> 4), idesc);
                     umma_commit(bar_s_full + s.j * 8);
                     umma_commit(bar_k_empty + s.j * 8);
                     if (m & kLastOfSegment) umma_commit(smem_u32(&bars.q_free));
@@ -698,7 +293,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
             const uint32_t p_tmem = tmem + kColS + buffer * kTile, o_tmem = tmem + kColO;
             if (lead) {
                 umma_ts(o_tmem, p_tmem, b0, idesc_o, (m & kFirstOfSegment) ? 0u : 1u);
-                for (int kk = 1; kk < steps; ++kk) umma_ts_lit<true>(o_tmem, p_tmem + kk * 8, b0 + (uint64_t)(kk * 128), idesc_o);
+                for (int kk = 1; kk < steps; ++kk) umma_ts_lit<1, true>(o_tmem, p_tmem + kk * 8, b0 + (uint64_t)(kk * 128), idesc_o);
                 umma_commit(bar_v_empty + buffer * 8);
                 if (m & kLastOfSegment) umma_commit(smem_u32(&bars.o_done));
             }
@@ -716,51 +311,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
             const int2 meta = *reinterpret_cast<const int2*>(&sh.meta[it & (kMetaRing - 1)]);
             if (meta.y >= 0) {                                      // a document's tile: its table came with the keys
                 const int len = meta.x & 0xff;
-                uint64_t c2[4], s2[4], n2[4];                       // cosines, sines and their negatives as pairs for the packed arithmetic
-                const float4* trig = reinterpret_cast<const float4*>(sh.trig[stage]);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {                       // half layout: slices chunk*8 .. +7; interleaved: chunk*4 .. +3 of either half
-                    const float4 cs = trig[LAYOUT == CF_ROPE_HALF ? chunk * 4 + e : (e >> 1) * 16 + chunk * 2 + (e & 1)];
-                    c2[e] = pack_f2(cs.x, cs.z);
-                    s2[e] = pack_f2(cs.y, cs.w);
-                    n2[e] = pack_f2(-cs.y, -cs.w);
-                }
-                // rows 24 apart keep their swizzle phase: one pointer walks
-                unsigned char* at = smem + (size_t)stage * kKvBytes + swz(rsub, chunk);
-#pragma unroll 2
-                for (int r = rsub; r < len; r += kRotateWarps * 4, at += kRotateWarps * 4 * 128) {
-                    uint4* pa = reinterpret_cast<uint4*>(at);
-                    uint4* pb = reinterpret_cast<uint4*>(at + kKvHalf);
-                    const uint4 va = *pa, vb = *pb;
-                    uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
-                    if (LAYOUT == CF_ROPE_HALF) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const uint64_t fa = pack_f2(__uint_as_float(wa[e] << 16), __uint_as_float(wa[e] & 0xffff0000u));
-                            const uint64_t fb = pack_f2(__uint_as_float(wb[e] << 16), __uint_as_float(wb[e] & 0xffff0000u));
-                            float y0, y1;
-                            unpack_f2(fma_f2(fa, c2[e], mul_f2(fb, n2[e])), y0, y1);
-                            wa[e] = pack_bf16(y0, y1);
-                            unpack_f2(fma_f2(fa, s2[e], mul_f2(fb, c2[e])), y0, y1);
-                            wb[e] = pack_bf16(y0, y1);
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {               // the two elements of a word are a slice; words in pairs
-                            uint32_t& w0 = e < 2 ? wa[2 * e] : wb[2 * e - 4];
-                            uint32_t& w1 = e < 2 ? wa[2 * e + 1] : wb[2 * e - 3];
-                            const uint64_t fa = pack_f2(__uint_as_float(w0 << 16), __uint_as_float(w1 << 16));
-                            const uint64_t fb = pack_f2(__uint_as_float(w0 & 0xffff0000u), __uint_as_float(w1 & 0xffff0000u));
-                            float a0, a1, b0, b1;
-                            unpack_f2(fma_f2(fa, c2[e], mul_f2(fb, n2[e])), a0, a1);
-                            unpack_f2(fma_f2(fa, s2[e], mul_f2(fb, c2[e])), b0, b1);
-                            w0 = pack_bf16(a0, b0);
-                            w1 = pack_bf16(a1, b1);
-                        }
-                    }
-                    *pa = make_uint4(wa[0], wa[1], wa[2], wa[3]);
-                    *pb = make_uint4(wb[0], wb[1], wb[2], wb[3]);
-                }
+                rotate_rows<LAYOUT>(smem + (size_t)stage * kKvBytes, kKvHalf, reinterpret_cast<const float4*>(sh.trig[stage]), chunk, rsub, kRotateWarps * 4, len);
                 fence_proxy_async();
             }
             __syncwarp();
@@ -771,200 +322,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
             }
         }
     } else {
-        // ------------------------------------------------------------------ softmax, one row per thread
-        const int w = warp >> 2, r = tid & 127;                     // warpgroup; row of the tile = TMEM lane
-        const uint32_t lane_tmem = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint64_t scale2 = pack_f2(src.scale_log2, src.scale_log2);
-        const uint32_t bar_s_full = smem_u32(bars.s_full), bar_pv_ready = smem_u32(bars.pv_ready);
-        int k = w, phase = 0;                                       // this warpgroup's next tile, mod 6, and its parity
-        int it0 = 0;                                                // tiles before the current segment
-        float ref = 0.f, l_run = 0.f, l_docs = 0.f;
-        const bool wide_out = ((reinterpret_cast<uintptr_t>(out_all) | (uintptr_t)(span.out_stride * 2)) & 31) == 0;   // rows start at 32-byte addresses
-        bool ok = true;
-        for (int seg = 0; ok; ++seg) {
-            const bool more = it0 < n_items;
-            const int slot = seg & (kSegRing - 1);
-            if (more && seg > 0) {
-                ok = warp_wait(smem_u32(&bars.segment[slot]), (seg / kSegRing) & 1 ^ (slot == 0 ? 1 : 0), abort_flag);
-                if (!ok) break;
-            }
-            const Segment& sg = sh.segments[slot];
-            if (more) {
-                // the query tile of the segment goes into tensor memory, half of every row by each warpgroup (before the
-                // epilogue of the last segment)
-                const bool active = (warp & 3) * 32 < sg.rows_here;
-                const int row = sg.row0 + min(r, sg.rows_here - 1), g = row / lq, j = row - g * lq;
-                const uint4* q = reinterpret_cast<const uint4*>(src.q + (size_t)sg.layer * span.q_stride + (((size_t)sg.b * lq + j) * n_q_heads + sg.kvh * group + g) * kD) + w * 8;
-                uint32_t qw[32];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const uint4 v = __ldg(q + i);
-                    qw[4 * i] = v.x;
-                    qw[4 * i + 1] = v.y;
-                    qw[4 * i + 2] = v.z;
-                    qw[4 * i + 3] = v.w;
-                }
-                if (seg > 0) ok = warp_wait(smem_u32(&bars.q_free), (seg - 1) & 1, abort_flag);   // read by its last QK^T
-                if (!ok) break;
-                if (active) {
-                    tc_fence_after();
-                    tmem_st16_from<0>(lane_tmem + kColQ + w * 32, qw);
-                    tmem_st16_from<16>(lane_tmem + kColQ + w * 32 + 16, qw);
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    tc_fence_before();
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bars.q_ready));
-            }
-            if (seg > 0) {
-                // ---- end of a segment: the two sums meet, each warpgroup takes half of the columns of O
-                const int par = (seg - 1) & 1;
-                sh.sum[par][w][r] = l_run;
-                sh.docs[par][w][r] = l_docs;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bars.sum_full[par]));
-                ok = warp_wait(smem_u32(&bars.sum_full[par]), ((seg - 1) >> 1) & 1, abort_flag) && warp_wait(smem_u32(&bars.o_done), par, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                const Segment& done = sh.segments[(seg - 1) & (kSegRing - 1)];
-                const bool whole = done.t_end - done.t_begin == done.n_unit;
-                const int row = done.row0 + r;
-                const float l_all = sh.sum[par][0][r] + sh.sum[par][1][r], d_all = sh.docs[par][0][r] + sh.docs[par][1][r];
-                const bool row_valid = r < done.rows_here, marked = l_all != l_all;
-                const size_t at = (size_t)done.lb * rows_total + (size_t)done.kvh * rows + row;
-                if ((warp & 3) * 32 < done.rows_here) {
-                    const int g = row / lq, j = row - g * lq;
-                    const size_t slot = ((size_t)2 * blockIdx.x + (done.t_begin == 0 ? 1 : 0)) * kRowTile + r;
-                    const float f = whole ? (l_all > 0.f ? 1.f / l_all : 0.f) : 1.f;
-                    __nv_bfloat16* dst = (whole ? out_all + (size_t)done.layer * span.out_stride + (((size_t)done.b * lq + j) * n_q_heads + done.kvh * group + g) * kD
-                                                : reinterpret_cast<__nv_bfloat16*>(ws.part_o) + slot * kD) + w * 64;
-#pragma unroll 1
-                    for (int c = 0; c < 2; ++c) {
-                        uint32_t o[32];
-                        tmem_ld32(lane_tmem + kColO + w * 64 + c * 32, o);
-                        if (row_valid) {
-#pragma unroll
-                            for (int i = 0; i < 2; ++i) {           // whole 32-byte sectors: rows are 256 bytes apart
-                                uint32_t y[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) y[e] = pack_bf16(__uint_as_float(o[16 * i + 2 * e]) * f, __uint_as_float(o[16 * i + 2 * e + 1]) * f);
-                                if (wide_out) {
-                                    store32(dst + c * 32 + i * 16, y);
-                                } else {
-                                    *reinterpret_cast<uint4*>(dst + c * 32 + i * 16) = make_uint4(y[0], y[1], y[2], y[3]);
-                                    *reinterpret_cast<uint4*>(dst + c * 32 + i * 16 + 8) = make_uint4(y[4], y[5], y[6], y[7]);
-                                }
-                            }
-                        }
-                    }
-                    if (w == 0 && row_valid) {
-                        if (!whole) {
-                            ws.part_m[slot] = l_all == 0.f ? -INFINITY : ref;   // a row may see none of the segment's keys
-                            ws.part_l[slot] = l_all;
-                            if (ws.part_ld) ws.part_ld[slot] = d_all;   // what the document scores are measured against
-                            if (done.t_begin == 0)            // (the share's last segment)
-                                reinterpret_cast<uint32_t*>(ws.row_lse2)[at] =
-                                    parts_code(blockIdx.x, line.share_of(x_end - done.t_end + done.n_unit - 1) - (int)blockIdx.x + 1);
-                        } else {
-                            ws.row_lse2[at] = marked ? __int_as_float(0x7fffffff) : ref + log2f(d_all);
-                            if (lse) lse[at] = (ref + log2f(l_all)) * kLn2;
-                        }
-                        if (marked) bars.marked = 1;
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bars.o_free));
-            }
-            if (!more) break;
-            // ---- the tiles of the segment
-            const int n = sg.t_end - sg.t_begin, par = seg & 1;
-            const bool active = (warp & 3) * 32 < sg.rows_here, row_valid = r < sg.rows_here;
-            const int q_index = (sg.row0 + r) % lq;                 // position of this row's token in the query
-            float* tile_lse2 = ws.tile_lse2 + (size_t)sg.layer * ws.max_tiles * rows_total + (size_t)sg.kvh * rows + sg.row0 + r;
-            const bool leads = (it0 & 1) == w;                      // this warpgroup has the segment's first tile
-            bool have_ref = false, seen_extra = false;
-            l_run = l_docs = 0.f;
-            for (int i = leads ? 0 : 1; i < n; i += 2) {
-                ok = warp_wait(bar_s_full + k * 8, phase, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                const int4 meta = sh.meta[(it0 + i) & (kMetaRing - 1)];
-                const int len = meta.x & 0xff, n_chunks = (len + 15) >> 4;
-                // keys this row may see: a whole tile of a document or of the prefix, the query tokens up to its own (causal
-                // mask, footnote to Eq. 1)
-                const int vis = meta.y <= kKindSelf ? min(len, q_index + 1 - (kKindSelf - meta.y) * kTile) : len;
-                const uint32_t s_addr = lane_tmem + kColS + (k >= 3 ? k - 3 : k) * kTile;
-                uint32_t va[16], vb[16];
-                if (active) {
-                    tmem_ld16_async(s_addr, va);
-                    tmem_ld16_wait(va);
-                }
-                if (i == 0) {                                       // the reference of the segment, from its first 16 keys
-                    float m = -INFINITY;
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) m = fmaxf(m, e < vis ? __uint_as_float(va[e]) : -INFINITY);
-                    sh.ref[par][r] = m > -INFINITY ? m * src.scale_log2 : 0.f;   // a row that sees none of them sees none of the tile
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bars.ref_full[par]));
-                }
-                if (!have_ref) {
-                    ok = warp_wait(smem_u32(&bars.ref_full[par]), (seg >> 1) & 1, abort_flag);
-                    if (!ok) break;
-                    ref = sh.ref[par][r];
-                    have_ref = true;
-                }
-                if (meta.y < 0 && !seen_extra) {                    // from here on the keys are not the documents'
-                    l_docs = l_run;
-                    seen_extra = true;
-                }
-                if (active) {
-                    // single pass in chunks of 16 keys: P chunk c goes over the S columns 8c .. 8c + 7, which are in registers by then
-                    const uint64_t neg_ref2 = pack_f2(-ref, -ref);
-                    uint64_t sum2 = 0;
-                    auto finish = [&](uint32_t (&v)[16], int c) {
-                        if (vis - c * 16 < 16) {                    // the ragged end of a tile, the causal mask
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) v[e] = e < vis - c * 16 ? v[e] : 0xff800000u;
-                        }
-                        chunk16_exp(v, scale2, neg_ref2, sum2);
-                        tmem_st8_async(s_addr + c * 8, v);
-                    };
-#pragma unroll 1
-                    for (int c = 0;;) {
-                        if (c + 1 < n_chunks) tmem_ld16_async(s_addr + (c + 1) * 16, vb);
-                        finish(va, c);
-                        if (++c == n_chunks) break;
-                        tmem_ld16_wait(vb);
-                        if (c + 1 < n_chunks) tmem_ld16_async(s_addr + (c + 1) * 16, va);
-                        finish(vb, c);
-                        if (++c == n_chunks) break;
-                        tmem_ld16_wait(va);
-                    }
-                    float tile_sum, odd;
-                    unpack_f2(sum2, tile_sum, odd);
-                    tile_sum += odd;
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_pv_ready + k * 8);
-                    if (!(tile_sum < kSumLimit)) tile_sum = __int_as_float(0x7fffffff);     // out of range: the row is marked
-                    l_run += tile_sum;
-                    if (meta.y >= 0 && row_valid) tile_lse2[(size_t)meta.y * rows_total] = ref + __log2f(tile_sum);
-                } else if (lane == 0) {
-                    mbar_arrive(bar_pv_ready + k * 8);
-                }
-                k += 2;
-                if (k >= 6) {
-                    k -= 6;
-                    phase ^= 1;
-                }
-            }
-            if (ok && !have_ref) ok = warp_wait(smem_u32(&bars.ref_full[par]), (seg >> 1) & 1, abort_flag);   // every phase is waited for
-            if (!have_ref && ok) ref = sh.ref[par][r];
-            if (!seen_extra) l_docs = l_run;
-            it0 += n;
-        }
+        softmax_role<R>(p, sh, sh.sums, nullptr, tmem, blockIdx.x, x_end, n_items);
     }
 
     // ---------------------------------------------------------------------- teardown
@@ -976,7 +334,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
         reinterpret_cast<ShareHead*>(ws.marks)[blockIdx.x] = head;
     }
     // every copy has landed and every MMA has read its operands: the rings are free
-    if (bars.marked && !bars.abort_flag) marked_from_scratch<LAYOUT>(p, *reinterpret_cast<RowScratch*>(smem), line);
+    if (bars.marked && !bars.abort_flag) marked_from_scratch<LAYOUT, false>(p, *reinterpret_cast<RowScratch*>(smem), line);
     if (bars.abort_flag) {
         // a wait expired: let the copies in flight land before the shared memory is given back
         if (tid == 0) {
@@ -1014,7 +372,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
     ShareHead head;
     int share = at;
     if (kByUnit) {
-        const int u = p.tiles_of_rows.quotient(at), row_tile = at - u * p.row_tiles, kvh = p.kv_heads.remainder(u);
+        const int u = p.tiles_of_rows.quotient(at), row_tile = at - u * (int)p.tiles_of_rows.d, kvh = p.kv_heads.remainder(u);
         head.lb = p.kv_heads.quotient(u);
         head.layer = p.requests.quotient(head.lb);
         head.b = head.lb - head.layer * bv.n_requests;
@@ -1071,9 +429,9 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
         float acc[16], m = -INFINITY, l = 0.f, ld = 0.f;
 #pragma unroll
         for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-        // part i: the share's slot for what goes on behind it (i = 0), the others' for what began before them
-        const size_t slot0 = ((size_t)2 * share + 1) * kRowTile + min(r, head.rows_here - 1), slot1 = slot0 + kRowTile;
-        auto slot_of = [&](int i) { return i == 0 ? slot0 : slot1 + (size_t)(i - 1) * 2 * kRowTile; };
+        // part i: the CTA's slot for what goes on behind its share (i = 0), the others' for what began before theirs
+        const size_t slot0 = ((size_t)2 * share + 1) * kRowTile + min(r, head.rows_here - 1), slot1 = slot0 - kRowTile;
+        auto slot_of = [&](int i) { return i == 0 ? slot0 : slot1 + (size_t)i * p.ctas * 2 * kRowTile; };
         const __nv_bfloat16* part_o = reinterpret_cast<const __nv_bfloat16*>(ws.part_o) + e0;
         for (int i0 = n_parts * run / kRuns; i0 < part_end; i0 += 4) {
             float mp[4], lp[4], dp[4];
@@ -1186,12 +544,28 @@ int attn_tc_row_tile(const cf_geom* g, const cf_batch* b) {
 // Two parts per share of the line, one share per SM.
 size_t attn_tc_part_rows() { return (size_t)2 * sm_count() * kRowTile; }
 
+// Whether CTAs work in pairs on two tiles of query rows (cf_attn_pair.cu).  A pair copies and rotates every key tile once for both,
+// but starts later and leaves one of its CTAs without rows where their number is odd: what counts is how many key tiles a pair's share
+// has.  Measured, attention and merge of a call (us, alone / in pairs; tiles of a share in brackets, documents of 160 tokens).
+// Two tiles of rows, 32/8 heads: 25 documents (5) 31.7 / 31.7; 50 (11) 37.9 / 35.8; 4 x 50 (43) 74.7 / 60.4; four layers of 4 x 100 (346)
+// 419 / 292.  Four, 28/4: 25 (5) 31.7 / 31.7; 4 x 12 (10) 35.8 / 33.8; 4 x 50 (43) 72.7 / 58.4; 12/2, 50 (5) 29.7 / 31.7.  Three, 12/2:
+// 50 (5) 23.6 / 29.7; 4 x 100 (43) 58.4 / 58.4; four layers of that (173) 167 / 150; 28/4, 4 x 50 (43) 58.4 / 58.4; 4 x 100 (86) 95.2 /
+// 89.1.  Five, 28/4: 4 x 12 (16) 37.9 / 37.9; 4 x 50 (65) 85.0 / 74.7.  The tiles are those the host knows of, a bound.
+static bool work_in_pairs(const cf_geom* g, const cf_batch* b, int n_layers, long long row_tiles, int more_tiles) {
+    const long long documents = std::min((long long)b->n_requests * tiles_per_request_bound(b), (long long)b->n_docs_total + b->total_tokens / kTile + 1);
+    const long long tiles = (documents + (long long)b->n_requests * more_tiles) * g->n_kv_heads * n_layers * ((row_tiles + 1) / 2);
+    return row_tiles > 1 && tiles >= (row_tiles % 2 ? 44 : 8) * (long long)(sm_count() / 2);
+}
+
 int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span, const void* q,
                    const void* k, const void* v, const void* k_self, const void* v_self, long long self_stride,
                    const void* k_prefix, const void* v_prefix, long long prefix_stride, int prefix_len,
                    float scale_log2, const AttnWorkspace& ws, void* out, float* lse, cudaStream_t stream) {
     const int group = g->n_q_heads / g->n_kv_heads;
-    const long long row_tiles = ((long long)group * b->q_len + ws.rg_rows - 1) / ws.rg_rows;
+    long long row_tiles = ((long long)group * b->q_len + ws.rg_rows - 1) / ws.rg_rows;
+    const int n_prefix = (prefix_len + kTile - 1) / kTile, n_self = k_self ? (b->q_len + kTile - 1) / kTile : 0;
+    const int ctas = work_in_pairs(g, b, span.n_layers, row_tiles, n_prefix + n_self) ? 2 : 1;       // of a share
+    row_tiles = (row_tiles + ctas - 1) / ctas;                      // units of a kv head
     // the line's positions are 32-bit
     const long long most = ((long long)pv.max_tiles + (long long)b->n_requests * (prefix_len / kTile + b->q_len / kTile + 2)) *
                            g->n_kv_heads * row_tiles * span.n_layers;
@@ -1208,7 +582,7 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
     const unsigned long long dense = (unsigned long long)g->n_kv_heads * kD * 2;
     auto block_maps = [&](CUtensorMap* mk, CUtensorMap* mv, const void* pk, const void* pvv, unsigned long long n, long long stride) {
         const unsigned long long layer = span.n_layers > 1 ? (unsigned long long)stride * 2 : n * dense;
-        const int rc = make_rows_map(mk, pk, g->n_kv_heads, n, dense, span.n_layers, layer, kTile);
+        const int rc = make_rows_map(mk, pk, g->n_kv_heads, n, dense, span.n_layers, layer, kTile / ctas);
         return rc != CF_OK ? rc : make_rows_map(mv, pvv, g->n_kv_heads, n, dense, span.n_layers, layer, kTile);
     };
     maps.ks = maps.kp = maps.k[0];
@@ -1222,7 +596,7 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
         if (rc != CF_OK) return rc;
     }
     const BatchView bv = make_batch_view(b);
-    const int shares = std::min(sm_count(), kMaxCodedShares);
+    const int shares = std::min(sm_count(), kMaxCodedShares) / ctas;   // of the line
     typedef const __nv_bfloat16* In;
     const RowSources src = {static_cast<In>(q), static_cast<In>(k), static_cast<In>(v), static_cast<In>(k_self), static_cast<In>(v_self),
                             static_cast<In>(k_prefix), static_cast<In>(v_prefix), self_stride, prefix_stride, scale_log2, k_self ? 1 : 0, prefix_len};
@@ -1232,19 +606,19 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
     // 23.3; 12 (12) 25.3 / 26.4 and 26.4 / 27.7; 14 (11) 25.1 / 25.1; 16 (9) 26.7 / 28.2; 24 (6) 32.4 / 34.9; 48 (3) 38.9 / 42.2.
     const bool many_parts = units * 13 <= shares;
     const int merge_rows = many_parts ? 8 : 32, slices = (ws.rg_rows + merge_rows - 1) / merge_rows;
-    const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, (prefix_len + kTile - 1) / kTile,
-                      k_self ? (b->q_len + kTile - 1) / kTile : 0, shares, Divisor(b->q_len), Divisor((int)row_tiles), Divisor(g->n_kv_heads),
+    const Params p = {bv, pv, ws, span, src, g->n_q_heads, g->n_kv_heads, (int)row_tiles, n_prefix, n_self, shares * ctas, ctas, Divisor(b->q_len), Divisor((int)row_tiles * ctas), Divisor(g->n_kv_heads),
                       Divisor(b->n_requests), Divisor(slices), static_cast<__nv_bfloat16*>(out), lse};
     static PerDeviceOnce configured[2];
     auto run = [&](auto kernel, int which) {
         if (configure_smem_once(configured[which], kernel, kSmemBytes) != CF_OK) return (int)CF_ERR_CUDA;
-        const int rc = launch_chained(kernel, dim3((unsigned)shares), kThreads, kSmemBytes, stream, maps, p);
-        if (rc != CF_OK) return rc;
-        const unsigned blocks = (unsigned)((many_parts ? units : shares) * slices);
-        const auto merge = many_parts ? attn_tc_merge_kernel<8> : attn_tc_merge_kernel<32>;
-        return launch_chained(merge, dim3(blocks), kMergeThreads, 0, stream, p);
+        return launch_chained(kernel, dim3((unsigned)shares), kThreads, kSmemBytes, stream, maps, p);
     };
-    return g->rope_layout == CF_ROPE_HALF ? run(attn_tc_kernel<CF_ROPE_HALF>, 0) : run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, 1);
+    const int rc = ctas == 2 ? launch_attn_pair(maps, p, g->rope_layout, shares, stream)
+                             : g->rope_layout == CF_ROPE_HALF ? run(attn_tc_kernel<CF_ROPE_HALF>, 0) : run(attn_tc_kernel<CF_ROPE_INTERLEAVED>, 1);
+    if (rc != CF_OK) return rc;
+    const unsigned blocks = (unsigned)((many_parts ? units : shares) * ctas * slices);
+    const auto merge = many_parts ? attn_tc_merge_kernel<8> : attn_tc_merge_kernel<32>;
+    return launch_chained(merge, dim3(blocks), kMergeThreads, 0, stream, p);
 }
 
 }  // namespace cf

@@ -41,19 +41,44 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// Waits for arrivals from either CTA of a pair.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 // Bounded wait: false when the limit expired or another role already gave up.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           long long limit_cycles = kWaitLimitCycles) {
-    if (mbar_try_wait(bar, parity)) return true;
+    auto done = [&] { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (done()) return true;
     const long long t0 = clock64();
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (done()) return true;
         if (*abort_flag) return false;
         if (clock64() - t0 > limit_cycles) {
             *abort_flag = 1;
             return false;
         }
     }
+}
+// Arrives on the barrier at the same place in the first CTA of the cluster.
+__device__ __forceinline__ void mbar_arrive_first(uint32_t bar) {
+    asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, 0;\nmbarrier.arrive.shared::cluster.b64 _, [a];\n}" ::"r"(bar) : "memory");
+}
+// The same `times` times (as a form of the above with a count of 1 it cost 1 us per call of 12 us).
+__device__ __forceinline__ void mbar_arrive_first(uint32_t bar, int times) {
+    asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, 0;\nmbarrier.arrive.shared::cluster.b64 _, [a], %1;\n}" ::"r"(bar), "r"(times) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -77,10 +102,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
     return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) |
            ((uint64_t)(sbo_bytes >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
-// Instruction descriptor: bf16 x bf16 -> fp32, M = 128, A K-major; B K-major or MN-major.
-__device__ __forceinline__ uint32_t instr_desc(int n, bool b_mn_major) {
+// Instruction descriptor: bf16 x bf16 -> fp32, A K-major; B K-major or MN-major.
+__device__ __forceinline__ uint32_t instr_desc(int n, bool b_mn_major, int m = 128) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major ? (1u << 16) : 0u) | ((uint32_t)(n >> 3) << 17) |
-           ((uint32_t)(128 >> 4) << 24);
+           ((uint32_t)(m >> 4) << 24);
 }
 __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -89,16 +114,35 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a_desc, uint64_t 
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// Same with the A operand (bf16, two elements per 32-bit column) in tensor memory.
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// Same on both CTAs of a pair: each has its rows of A and half of the columns of B in its own shared memory, at the same places.
+__device__ __forceinline__ void umma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Same with the A operand (bf16, two elements per 32-bit column) in tensor memory; CTAS = 2: on the tensor cores of both CTAs of a
+// pair, each with its rows of A and D in its own tensor memory and half of the columns of B in its own shared memory.
+template <int CTAS = 1>
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    if (CTAS == 2)
+        asm volatile(
+            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}"
+            ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else asm volatile(
         "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+template <int CTAS = 1>                            // 2: on the barrier at the same place in both CTAs
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    if (CTAS == 2)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3) : "memory");
+    else asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane; returns after the data has arrived.
@@ -139,10 +183,21 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
 }
+// The same for the warp that issues MMAs.
+template <bool PAIR>
+__device__ __forceinline__ bool mma_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait<PAIR>(bar, parity, abort_flag));
+}
 // tcgen05.mma with the accumulate predicate a literal, in its two operand forms.
-template <bool ACCUMULATE>
+template <int CTAS, bool ACCUMULATE>
 __device__ __forceinline__ void umma_ts_lit(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc) {
-    asm volatile(
+    if (CTAS == 2)
+        asm volatile(
+            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}"
+            ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "n"(ACCUMULATE ? 1 : 0)
+            : "memory");
+    else asm volatile(
         "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "n"(ACCUMULATE ? 1 : 0)
@@ -217,7 +272,8 @@ __device__ __forceinline__ void tmem_ld16_wait(uint32_t (&v)[16]) {
                  : "memory");
 }
 // Eight columns (16 packed bf16) of the P operand.
-__device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t (&v)[16]) {
+template <int N>
+__device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t (&v)[N]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
                  : : "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(taddr)
                  : "memory");
@@ -227,6 +283,20 @@ __device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t (&
 __device__ __forceinline__ void chunk16_exp(uint32_t (&v)[16], uint64_t scale2, uint64_t neg_ref2, uint64_t& sum2) {
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
+        float p0, p1;
+        unpack_f2(fma_f2(pack_f2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), scale2, neg_ref2), p0, p1);
+        p0 = fast_exp2(p0);
+        p1 = fast_exp2(p1);
+        sum2 = add_f2(sum2, pack_f2(p0, p1));
+        v[i >> 1] = pack_bf16(p0, p1);
+    }
+}
+
+// The same for columns FIRST .. FIRST + 15 of 32, packed into v[FIRST / 2 ..].
+template <int FIRST>
+__device__ __forceinline__ void chunk_exp(uint32_t (&v)[32], uint64_t scale2, uint64_t neg_ref2, uint64_t& sum2) {
+#pragma unroll
+    for (int i = FIRST; i < FIRST + 16; i += 2) {
         float p0, p1;
         unpack_f2(fma_f2(pack_f2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), scale2, neg_ref2), p0, p1);
         p0 = fast_exp2(p0);
