@@ -126,15 +126,25 @@ __global__ void decode_append_kernel(int cache_rows, int row_elems, long long la
     chain_next();
     chain_wait();
     const int b = blockIdx.x, layer = blockIdx.y;
+    constexpr int E = 16 / sizeof(T);
+    const size_t src = (size_t)layer * new_layer_stride + (size_t)b * row_elems;
+    int i = threadIdx.x * E;
+    uint4 k0 = make_uint4(0u, 0u, 0u, 0u), v0 = k0;     // the first piece travels with the number of rows: one memory latency
+    if (i < row_elems) {
+        k0 = *reinterpret_cast<const uint4*>(k_new + src + i);
+        v0 = *reinterpret_cast<const uint4*>(v_new + src + i);
+    }
     const long long row = (long long)rows[b] + step;
     if (row < 0 || row >= cache_rows) {
         if (threadIdx.x == 0 && status) atomicCAS(status, 0, CF_ERR_RANGE);
         return;
     }
-    constexpr int E = 16 / sizeof(T);
     const size_t dst = (size_t)layer * layer_stride + ((size_t)b * cache_rows + (size_t)row) * row_elems;
-    const size_t src = (size_t)layer * new_layer_stride + (size_t)b * row_elems;
-    for (int i = threadIdx.x * E; i < row_elems; i += blockDim.x * E) {
+    if (i < row_elems) {
+        *reinterpret_cast<uint4*>(k_final + dst + i) = k0;
+        *reinterpret_cast<uint4*>(v_final + dst + i) = v0;
+    }
+    for (i += blockDim.x * E; i < row_elems; i += blockDim.x * E) {
         *reinterpret_cast<uint4*>(k_final + dst + i) = *reinterpret_cast<const uint4*>(k_new + src + i);
         *reinterpret_cast<uint4*>(v_final + dst + i) = *reinterpret_cast<const uint4*>(v_new + src + i);
     }

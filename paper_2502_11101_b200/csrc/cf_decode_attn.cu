@@ -39,7 +39,8 @@ struct DecodeArgs {
     float* lse;
     const int* doc_offsets;                        // of the decode plan: request b uses rows [2b] .. [2b + 1) of the store
     long long q_stride, kv_stride, out_stride;     // elements between layers
-    int n_requests, cache_rows, n_q_heads, n_kv_heads, row_tiles;
+    int n_requests, cache_rows, n_q_heads, n_kv_heads, row_tiles, group;   // group: query heads of a kv head
+    Divisor by_requests, by_row_tiles;
     float scale_log2;
     float *part_o, *part_m, *part_l;               // parts of units that lie in several shares of the line
     int2* unit_parts;                              // [units] first share of a unit and the parts it was cut into (0: not cut)
@@ -158,8 +159,8 @@ __device__ __forceinline__ Segment segment_at(const DecodeArgs& a, const Line& l
     sg.s_end = min(sg.steps, sg.s_begin + (end - x));
     sg.lb = layer * a.n_requests + lo;
     sg.unit = sg.lb * line.tiles + kr;
-    sg.kvh = kr / a.row_tiles;
-    const int row_tile = kr - sg.kvh * a.row_tiles, group = a.n_q_heads / a.n_kv_heads;
+    sg.kvh = a.by_row_tiles.quotient(kr);
+    const int row_tile = kr - sg.kvh * a.row_tiles, group = a.group;
     sg.head0 = sg.kvh * group + row_tile * kq;
     sg.n_heads = min(kq, group - row_tile * kq);
     sg.used = a.doc_offsets[2 * lo + 1] - a.doc_offsets[2 * lo];
@@ -183,7 +184,7 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
     chain_wait();
     Line line;
     Segment sg;
-    int x_pos = 0, x_end = 0;
+    int x_pos = 0, x_end = 0, used_from = 0, used_to = 0;
     if (STREAM) {
         line = make_line(a, s_pref, n_layers, (int)gridDim.x);
         if ((int)blockIdx.x >= line.n_shares) return;
@@ -191,18 +192,24 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
         x_end = line.cut(blockIdx.x + 1);
         sg = segment_at(a, line, x_pos, x_end, kQ);
     } else {
-        const int group = a.n_q_heads / a.n_kv_heads;
-        sg.kvh = blockIdx.y / a.row_tiles;
+        const int group = a.group;
+        sg.kvh = a.by_row_tiles.quotient(blockIdx.y);
         const int row_tile = blockIdx.y - sg.kvh * a.row_tiles;
         sg.lb = blockIdx.z;
         sg.head0 = sg.kvh * group + row_tile * kQ;
         sg.n_heads = min(kQ, group - row_tile * kQ);
-        const int b = sg.lb % a.n_requests;
-        sg.used = a.doc_offsets[2 * b + 1] - a.doc_offsets[2 * b];
-        sg.steps = (sg.used + kStepKeys - 1) / kStepKeys;          // every CTA of the cluster takes an equal share of them
-        sg.s_begin = (int)((long long)sg.steps * rank / n_cta);
-        sg.s_end = (int)((long long)sg.steps * (rank + 1) / n_cta);
+        const int b = a.by_requests.remainder(sg.lb);
+        used_from = a.doc_offsets[2 * b];
+        used_to = a.doc_offsets[2 * b + 1];
+        // The warps of the cluster take the steps in turn: a warp's first one is known before the rows in use are, and its loads
+        // travel with theirs.  Rows of the slot that are not in use are masked, their values replaced by zeros.  (Equal runs of steps,
+        // cut once the rows were known, by divisions out of registers: with the append a layer of 1011 rows, 12/2 heads, took 7.6 us,
+        // this way 6.6, of which 0.3 are the append's, which loads its first piece together with the number of rows.)
+        sg.s_begin = rank * kDecWarps;
+        sg.s_end = sg.s_begin + 1 + kDecWarps;                      // (the first step of every warp; the rest below)
+        sg.used = a.cache_rows;
     }
+    const int stride = n_cta * kDecWarps;
 
     uint4 qf[NQ][4], kf[2][4], vf[4][2];
     const __nv_bfloat16 *k, *v;
@@ -225,7 +232,7 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
     };
     // query fragments (chunk c = dims 32c + 8t .. + 7) and the first keys and values of a segment
     auto start = [&]() {
-        const int layer = sg.lb / a.n_requests, b = sg.lb - layer * a.n_requests;
+        const int layer = a.by_requests.quotient(sg.lb), b = sg.lb - layer * a.n_requests;
         const __nv_bfloat16* q = a.q + (size_t)layer * a.q_stride + ((size_t)b * a.n_q_heads + sg.head0) * kDecDim + t * 8;
         const size_t base = (size_t)layer * a.kv_stride + ((size_t)b * a.cache_rows * a.n_kv_heads + sg.kvh) * kDecDim;
         k = a.k + base + t * 8;
@@ -241,6 +248,15 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
         }
     };
     start();
+    if (!STREAM) {
+        sg.used = used_to - used_from;
+        sg.steps = sg.s_end = (sg.used + kStepKeys - 1) / kStepKeys;
+        const int valid = sg.used - (sg.s_begin + warp) * kStepKeys;
+        if (valid < kStepKeys)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (2 * t + (j & 1) + (j >> 1) * 8 >= valid) vf[j][0] = vf[j][1] = make_uint4(0u, 0u, 0u, 0u);
+    }
     while (true) {
     float o[NQ][8][4], m[NQ], l[NQ];
 #pragma unroll
@@ -252,8 +268,8 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) o[x][i][e] = 0.f;
     }
-    for (int s = sg.s_begin + warp; s < sg.s_end; s += kDecWarps) {
-        const bool more = s + kDecWarps < sg.s_end;
+    for (int s = sg.s_begin + warp; s < sg.s_end; s += stride) {
+        const bool more = s + stride < sg.s_end;
         float sc[2][4];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -264,7 +280,7 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
                 mma16816(sc[j], qf[0][c].z, NQ > 1 ? qf[NQ - 1][c].z : 0u, qf[0][c].w, NQ > 1 ? qf[NQ - 1][c].w : 0u, kf[j][c].z, kf[j][c].w);
             }
         }
-        if (more) load_k(s + kDecWarps);
+        if (more) load_k(s + stride);
         const int valid = sg.used - s * kStepKeys;                     // keys of this step that exist
         uint32_t p[NQ][2];
 #pragma unroll
@@ -311,7 +327,7 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
 #pragma unroll
                 for (int x = 0; x < NQ; ++x) mma16816(o[x][h * 4 + i], a0, a1, a2, a3, p[x][0], p[x][1]);
             }
-        if (more) load_v(s + kDecWarps);
+        if (more) load_v(s + stride);
     }
 
     // the next segment's first loads travel under the merge of this one
@@ -375,7 +391,7 @@ decode_attn_kernel(DecodeArgs a, int n_layers) {
     }
     const uint32_t addr_o = (uint32_t)__cvta_generic_to_shared(&s_o[0][0][0]);
     const uint32_t addr_m = (uint32_t)__cvta_generic_to_shared(&s_m[kDecWarps][0]), addr_l = (uint32_t)__cvta_generic_to_shared(&s_l[kDecWarps][0]);
-    const int layer = done.lb / a.n_requests, b = done.lb - layer * a.n_requests;
+    const int layer = a.by_requests.quotient(done.lb), b = done.lb - layer * a.n_requests;
     const bool whole = !STREAM || (done.s_begin == 0 && done.s_end == done.steps);
     if (STREAM && tid == 0 && done.s_begin == 0)                    // x_pos: the position behind this segment
         a.unit_parts[done.unit] = make_int2((int)blockIdx.x, whole ? 0 : line.share_of(x_pos - done.s_end + done.steps - 1) - (int)blockIdx.x + 1);
@@ -529,7 +545,7 @@ int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_l
     int2* unit_parts = reinterpret_cast<int2*>(part_l + (size_t)shares * 2 * kq);
     const DecodeArgs a = {static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v),
                           static_cast<__nv_bfloat16*>(out), lse, doc_offsets, span.q_stride, span.kv_stride, span.out_stride, n_requests,
-                          cache_rows, g->n_q_heads, g->n_kv_heads, row_tiles, scale_log2, part_o, part_m, part_l, unit_parts};
+                          cache_rows, g->n_q_heads, g->n_kv_heads, row_tiles, group, Divisor(n_requests), Divisor(row_tiles), scale_log2, part_o, part_m, part_l, unit_parts};
     const long long units = decode_units(g, n_requests, n_layers);
     // A cluster per unit where one wave of clusters leaves a warp a few steps, the stream of equal shares for everything longer;
     // the line is eight steps.  Measured (us per layer with the append, cold, cluster against stream, the steps of a warp in
@@ -537,7 +553,8 @@ int launch_decode_attn(const cf_geom* g, int n_requests, int cache_rows, int n_l
     // 14.7 / 13.7; 16 units, 3000 (6) 14.0 / 15.2, 4000 (8) 17.5 / 17.0; 32 units, 3000 (6) 18.8 / 19.1, 4000 (8) 21.6 / 21.6; 256
     // units, 500 (8) 20.5 / 21.5, 750 (12) 24.0 / 23.6, 2000 (31) 48.5 / 44.7.  So the two meet at four steps for a few units and
     // at ten for many.  What the rule sees is the slot, not the rows in use, which are known on the device only: 1011 rows of 2
-    // units take 8.1 us in a slot of 1075 rows and 10.1 in one of 20 000.
+    // units took 8.1 us in a slot of 1075 rows and 10.1 in one of 20 000.  (Figures of the kernel before a warp's first step was loaded
+    // early, which takes about 0.7 us off the cluster's side.)
     int cluster = 1;
     while (cluster < kMaxCluster && units * cluster * 2 <= shares) cluster *= 2;
     bool stream_k = cache_rows > kStepKeys * kDecWarps * cluster * 8;

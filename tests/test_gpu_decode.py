@@ -277,3 +277,32 @@ def test_both_marshallers_give_the_same_results(monkeypatch):
         results.append((out, outs, lse, scores, sess.score_accum.clone(), k_cache, v_cache, rows, moved, token, token_lse, built))
     for a, b in zip(*results):
         assert torch.equal(a, b) and float(a.float().abs().max()) > 0
+
+
+@pytest.mark.parametrize("heads,room", [((12, 2), 1075), ((20, 2), 513), ((4, 4), 40)])
+def test_rows_not_in_use_hold_anything(heads, room):
+    """Keys and values of a slot behind the rows in use may be read before their number is known, but count for nothing, whatever
+    they hold: around the steps of 16 keys, the 64 of a CTA's warps and the 512 of a cluster."""
+    import paper_2502_11101_b200 as cf
+    hq, hkv = heads
+    rows = [r for r in (1, 15, 16, 17, 63, 64, 65, 511, 512, 513, 1000) if r <= room]
+    b = len(rows)
+    gen = torch.Generator(device="cuda").manual_seed(room)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rand(1, b, hq, 128), rand(1, b, room, hkv, 128), rand(1, b, room, hkv, 128)
+    for i, r in enumerate(rows):
+        k[:, i, r:], v[:, i, r:] = float("nan"), float("inf")
+    geom = cf.make_geom(hq, hkv, 128, torch.bfloat16, 1 << 20, 1.0e4)
+    used = torch.tensor(rows, dtype=torch.int32, device="cuda")
+    plan = torch.zeros(cf.cf_decode_plan_bytes(geom, b, room), dtype=torch.uint8, device="cuda")
+    work = torch.empty(cf.cf_decode_workspace_bytes(geom, b, room, 1), dtype=torch.uint8, device="cuda")
+    out, lse = torch.empty_like(q), torch.empty(1, b, hq, device="cuda")
+    cf.cf_decode_plan(geom, b, room, used, 0, plan)
+    cf.cf_decode_attn(geom, b, room, plan, q, k, v, out, work, lse)
+    torch.cuda.synchronize()
+    for i, r in enumerate(rows):
+        kk, vv = (x[0, i, :r].double().repeat_interleave(hq // hkv, dim=1) for x in (k, v))
+        s = torch.einsum("hd,thd->ht", q[0, i].double(), kk) / np.sqrt(128.0)
+        # one bf16 rounding of the probabilities and of the output; fp32 sums for the log-sum-exp
+        assert torch.allclose(out[0, i].double(), torch.einsum("ht,thd->hd", s.softmax(-1), vv), rtol=1e-2, atol=1e-2), r
+        assert torch.allclose(lse[0, i].double(), s.logsumexp(-1), rtol=0, atol=1e-4), r
