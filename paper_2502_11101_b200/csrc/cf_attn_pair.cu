@@ -86,7 +86,7 @@ attn_pair_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__
     Barriers& bars = sh.bars;
     volatile int* abort_flag = &bars.abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int group = n_q_heads / n_kv_heads, lq = bv.q_len, rows = group * lq, rows_total = n_q_heads * lq;
+    const int group = n_q_heads / n_kv_heads, lq = bv.q_len, rows = group * lq;
     const int share = blockIdx.x >> 1, rank = blockIdx.x & 1;
     if (warp == kKeyWarp) {
         if (lane == 0) {
