@@ -397,7 +397,8 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
 // cost every merge 0.3 to 0.5 us although nobody took it: one layer of 20 documents, 32/32 heads 48.3 -> 46.6 us, 28 one-layer
 // calls over 50 documents, 12/2 heads 574 -> 559.  Calls with such rows: four layers of 50 documents of 160 tokens, 12/2 heads, 44 us
 // without, one row a layer 166 -> 79, every row 759 -> 398; one layer of 2 x 60 documents of 180, 32/32 heads, 93 us, 265 -> 166 and
-// 1109 -> 646; of 4 x 50 of 160, 28/4 heads, 75 us, 202 -> 130 and 687 -> 720 (few tiles per share leave warps idle).
+// 1109 -> 646; of 4 x 50 of 160, 28/4 heads, 75 us
+// (64 in pairs), 202 -> 128 and 687 -> 732 (few tiles per share leave warps idle, and a pair's kernel has registers for fewer).
 template <int LAYOUT, bool PAIR>
 __device__ __forceinline__ void marked_from_scratch(const Params& p, RowScratch& sh, const Line& line) {
     const int group = p.n_q_heads / p.n_kv_heads, share = blockIdx.x >> (PAIR ? 1 : 0);

@@ -142,61 +142,61 @@ __device__ __forceinline__ void softmax_role(const Params& p, SHARED& sh, Sums<R
             ok = warp_wait(smem_u32(&bars.sum_full[par]), ((seg - 1) >> 1) & 1, abort_flag) && (w >= 2 || warp_wait(smem_u32(&bars.o_done), par, abort_flag));
             if (!ok) break;
             if (kSoftmaxGroups == 2 || w < 2) {
-            tc_fence_after();
-            const Segment& done = sh.segments[(seg - 1) & (kSegRing - 1)];
-            const bool whole = done.t_end - done.t_begin == done.n_unit;
-            const int row = done.row0 + r;
-            float l_all = sums.all[par][0][r], d_all = sums.docs[par][0][r];
+                tc_fence_after();
+                const Segment& done = sh.segments[(seg - 1) & (kSegRing - 1)];
+                const bool whole = done.t_end - done.t_begin == done.n_unit;
+                const int row = done.row0 + r;
+                float l_all = sums.all[par][0][r], d_all = sums.docs[par][0][r];
 #pragma unroll
-            for (int x = 1; x < kSoftmaxGroups; ++x) {
-                l_all += sums.all[par][x][r];
-                d_all += sums.docs[par][x][r];
-            }
-            const bool row_valid = r < done.rows_here, marked = l_all != l_all;
-            const size_t at = (size_t)done.lb * rows_total + (size_t)done.kvh * rows + row;
-            if ((warp & 3) * 32 < done.rows_here) {
-                const int g = row / lq, j = row - g * lq;
-                const size_t slot = ((size_t)2 * blockIdx.x + (done.t_begin == 0 ? 1 : 0)) * kRowTile + r;
-                const float f = whole ? (l_all > 0.f ? 1.f / l_all : 0.f) : 1.f;
-                __nv_bfloat16* dst = (whole ? out_all + (size_t)done.layer * span.out_stride + (((size_t)done.b * lq + j) * n_q_heads + done.kvh * group + g) * kD
-                                            : reinterpret_cast<__nv_bfloat16*>(ws.part_o) + slot * kD) + w * 64;
+                for (int x = 1; x < kSoftmaxGroups; ++x) {
+                    l_all += sums.all[par][x][r];
+                    d_all += sums.docs[par][x][r];
+                }
+                const bool row_valid = r < done.rows_here, marked = l_all != l_all;
+                const size_t at = (size_t)done.lb * rows_total + (size_t)done.kvh * rows + row;
+                if ((warp & 3) * 32 < done.rows_here) {
+                    const int g = row / lq, j = row - g * lq;
+                    const size_t slot = ((size_t)2 * blockIdx.x + (done.t_begin == 0 ? 1 : 0)) * kRowTile + r;
+                    const float f = whole ? (l_all > 0.f ? 1.f / l_all : 0.f) : 1.f;
+                    __nv_bfloat16* dst = (whole ? out_all + (size_t)done.layer * span.out_stride + (((size_t)done.b * lq + j) * n_q_heads + done.kvh * group + g) * kD
+                                                : reinterpret_cast<__nv_bfloat16*>(ws.part_o) + slot * kD) + w * 64;
 #pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t o[32];
-                    tmem_ld32(lane_tmem + kColO + w * 64 + c * 32, o);
-                    if (row_valid) {
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t o[32];
+                        tmem_ld32(lane_tmem + kColO + w * 64 + c * 32, o);
+                        if (row_valid) {
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) {           // whole 32-byte sectors: rows are 256 bytes apart
-                            uint32_t y[8];
+                            for (int i = 0; i < 2; ++i) {           // whole 32-byte sectors: rows are 256 bytes apart
+                                uint32_t y[8];
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) y[e] = pack_bf16(__uint_as_float(o[16 * i + 2 * e]) * f, __uint_as_float(o[16 * i + 2 * e + 1]) * f);
-                            if (wide_out) {
-                                store32(dst + c * 32 + i * 16, y);
-                            } else {
-                                *reinterpret_cast<uint4*>(dst + c * 32 + i * 16) = make_uint4(y[0], y[1], y[2], y[3]);
-                                *reinterpret_cast<uint4*>(dst + c * 32 + i * 16 + 8) = make_uint4(y[4], y[5], y[6], y[7]);
+                                for (int e = 0; e < 8; ++e) y[e] = pack_bf16(__uint_as_float(o[16 * i + 2 * e]) * f, __uint_as_float(o[16 * i + 2 * e + 1]) * f);
+                                if (wide_out) {
+                                    store32(dst + c * 32 + i * 16, y);
+                                } else {
+                                    *reinterpret_cast<uint4*>(dst + c * 32 + i * 16) = make_uint4(y[0], y[1], y[2], y[3]);
+                                    *reinterpret_cast<uint4*>(dst + c * 32 + i * 16 + 8) = make_uint4(y[4], y[5], y[6], y[7]);
+                                }
                             }
                         }
                     }
-                }
-                if (w == 0 && row_valid) {
-                    if (!whole) {
-                        ws.part_m[slot] = l_all == 0.f ? -INFINITY : ref;   // a row may see none of the segment's keys
-                        ws.part_l[slot] = l_all;
-                        if (ws.part_ld) ws.part_ld[slot] = d_all;   // what the document scores are measured against
-                        if (done.t_begin == 0)            // (the share's last segment)
-                            reinterpret_cast<uint32_t*>(ws.row_lse2)[at] =
-                                parts_code(blockIdx.x, line.share_of(x_end - done.t_end + done.n_unit - 1) - share + 1);
-                    } else {
-                        ws.row_lse2[at] = marked ? __int_as_float(0x7fffffff) : ref + log2f(d_all);
-                        if (lse) lse[at] = (ref + log2f(l_all)) * kLn2;
+                    if (w == 0 && row_valid) {
+                        if (!whole) {
+                            ws.part_m[slot] = l_all == 0.f ? -INFINITY : ref;   // a row may see none of the segment's keys
+                            ws.part_l[slot] = l_all;
+                            if (ws.part_ld) ws.part_ld[slot] = d_all;   // what the document scores are measured against
+                            if (done.t_begin == 0)            // (the share's last segment)
+                                reinterpret_cast<uint32_t*>(ws.row_lse2)[at] =
+                                    parts_code(blockIdx.x, line.share_of(x_end - done.t_end + done.n_unit - 1) - share + 1);
+                        } else {
+                            ws.row_lse2[at] = marked ? __int_as_float(0x7fffffff) : ref + log2f(d_all);
+                            if (lse) lse[at] = (ref + log2f(l_all)) * kLn2;
+                        }
+                        if (marked) bars.marked = 1;
                     }
-                    if (marked) bars.marked = 1;
                 }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) arrive_mma(smem_u32(&bars.o_free));
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_mma(smem_u32(&bars.o_free));
             }
         }
         if (!more) {
