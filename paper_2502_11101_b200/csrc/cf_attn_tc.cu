@@ -358,7 +358,8 @@ constexpr int kMergeThreads = 256;
 // block has a slice of one unit and reads from its first row's word how it was cut (blocks that looked at four shares each, of
 // which few begin a unit: 28 calls over 50 documents, 12/2 heads, 553 us, this way 530); the parts of a row are cut into four
 // runs, walked side by side and joined in order through shared memory.  Either also sees to the (empty) results of requests that
-// have nothing to attend.
+// have nothing to attend.  Weights are exp2f's, which keeps numbers below 2^-126: the documents' share of a row whose prefix lies
+// that far above them is what their scores are measured against (with ex2.approx.ftz it was 0 and the scores infinite).
 template <int ROWS>
 __global__ void __launch_bounds__(kMergeThreads, 2)
 attn_tc_merge_kernel(const __grid_constant__ Params p) {
@@ -446,7 +447,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 o[x][1] = *reinterpret_cast<const uint4*>(part_o + slot * kD + 8);
             }
             const float m_new = fmaxf(fmaxf(m, fmaxf(mp[0], mp[1])), fmaxf(mp[2], mp[3]));
-            const float keep = m > -INFINITY ? fast_exp2(m - m_new) : 0.f;
+            const float keep = m > -INFINITY ? exp2f(m - m_new) : 0.f;
             m = m_new;
             l *= keep;
             ld *= keep;
@@ -455,7 +456,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
 #pragma unroll
             for (int x = 0; x < 4; ++x)
                 if (mp[x] > -INFINITY) {
-                    const float w = fast_exp2(mp[x] - m_new);
+                    const float w = exp2f(mp[x] - m_new);
                     l = fmaf(lp[x], w, l);
                     ld = fmaf(dp[x], w, ld);
                     const uint32_t pairs[8] = {o[x][0].x, o[x][0].y, o[x][0].z, o[x][0].w, o[x][1].x, o[x][1].y, o[x][1].z, o[x][1].w};
@@ -482,7 +483,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                 const float* other = &s_run[k][0][threadIdx.x];
                 const float mo = other[0];
                 if (mo == -INFINITY) continue;
-                const float m_new = fmaxf(m, mo), keep = m > -INFINITY ? fast_exp2(m - m_new) : 0.f, w = fast_exp2(mo - m_new);
+                const float m_new = fmaxf(m, mo), keep = m > -INFINITY ? exp2f(m - m_new) : 0.f, w = exp2f(mo - m_new);
                 m = m_new;
                 l = fmaf(other[kRunThreads], w, l * keep);
                 ld = fmaf(other[2 * kRunThreads], w, ld * keep);
