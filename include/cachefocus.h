@@ -341,11 +341,13 @@ int cf_query_prefill_attn_prefix(const cf_geom* geom, const cf_batch* batch, con
  * application that owns the allocator and hands out only input and output buffers, a serving
  * loop that has frozen its memory pool, a caller already inside a region where allocation would
  * synchronise the device.  Such a caller has nowhere to put the attention workspace, so here the
- * workspace is a fixed array of CF_STATIC_WORKSPACE_BYTES (32 MiB) that is part of the library
- * image: every GPU that loads the library holds those bytes until the process exits.
+ * workspace is a fixed array of CF_STATIC_WORKSPACE_BYTES (32 MiB), and 10 MiB for the low halves of
+ * partial results, that is part of the library image: every GPU that loads the library holds those
+ * bytes until the process exits.
  *   - Arguments are those of cf_query_prefill_attn without workspace / workspace_bytes.
- *   - Returns CF_ERR_WORKSPACE, launching nothing, when cf_attn_workspace_bytes(geom, batch) for
- *     this batch exceeds CF_STATIC_WORKSPACE_BYTES.  Use a smaller batch or the ordinary call.
+ *   - Returns CF_ERR_WORKSPACE, launching nothing, when this batch needs more than
+ *     CF_STATIC_WORKSPACE_BYTES without those low halves; it never does where
+ *     cf_attn_workspace_bytes(geom, batch) is within the limit.  Use a smaller batch or the ordinary call.
  *   - The first call on each device looks up the array's device address (one
  *     cudaGetSymbolAddress); make that first call outside any stream capture.  No call allocates
  *     or frees device memory.

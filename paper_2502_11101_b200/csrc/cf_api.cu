@@ -149,7 +149,7 @@ int choose_splits(const cf_geom* g, const cf_batch* b, int n_layers) {
 }
 
 size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, int n_layers, bool with_self,
-                             AttnWorkspace* ws, void* base_ptr, int part_layers) {
+                             AttnWorkspace* ws, void* base_ptr, int part_layers, bool low_halves) {
     const size_t rows = (size_t)g->n_q_heads * b->q_len;
     const size_t nlb = (size_t)b->n_requests * (size_t)(part_layers > 0 ? part_layers : n_layers);   // layers of partial results
     const size_t nlb_lse = (size_t)b->n_requests * (size_t)n_layers;
@@ -164,7 +164,7 @@ size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, 
     // room for the parts of either kernel family
     const size_t tc_rows = attn_tc_supported(g, b) ? attn_tc_part_rows() : 0;
     const size_t parts = std::max(nlb * n_splits * rows, tc_rows);
-    size_t o = take(std::max(nlb * n_splits * rows * g->head_dim, tc_rows * g->head_dim / 2));
+    size_t o = take(std::max(nlb * n_splits * rows * g->head_dim, tc_rows * g->head_dim / (low_halves ? 1 : 2)));
     size_t m = take(parts);
     size_t l = take(parts);
     size_t mk = take(tc_rows);
@@ -179,6 +179,7 @@ size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, 
     }
     if (ws) {
         ws->part_o = reinterpret_cast<float*>(base + o);
+        ws->part_low = reinterpret_cast<uint16_t*>(base + o) + tc_rows * g->head_dim;   // behind the bf16 parts
         ws->part_m = reinterpret_cast<float*>(base + m);
         ws->part_l = reinterpret_cast<float*>(base + l);
         ws->marks = reinterpret_cast<int*>(base + mk);

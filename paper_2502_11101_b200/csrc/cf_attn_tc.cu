@@ -428,6 +428,7 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
         const int r = slice * ROWS + (warp - run * (8 / kRuns)) * 4 + (lane >> 3), e0 = (lane & 7) * 16;   // row of the unit; this lane's dims
         const bool valid = run == 0 && r < head.rows_here;
         float acc[16], m = -INFINITY, l = 0.f, ld = 0.f;
+        uint32_t scratch = 0;
 #pragma unroll
         for (int e = 0; e < 16; ++e) acc[e] = 0.f;
         // part i: the CTA's slot for what goes on behind its share (i = 0), the others' for what began before theirs
@@ -451,14 +452,15 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
             m = m_new;
             l *= keep;
             ld *= keep;
+            scratch |= __float_as_uint(lp[0]) | __float_as_uint(lp[1]) | __float_as_uint(lp[2]) | __float_as_uint(lp[3]);
 #pragma unroll
             for (int e = 0; e < 16; ++e) acc[e] *= keep;
 #pragma unroll
             for (int x = 0; x < 4; ++x)
                 if (mp[x] > -INFINITY) {
                     const float w = exp2f(mp[x] - m_new);
-                    l = fmaf(lp[x], w, l);
-                    ld = fmaf(dp[x], w, ld);
+                    l = fmaf(fabsf(lp[x]), w, l);
+                    ld = fmaf(fabsf(dp[x]), w, ld);
                     const uint32_t pairs[8] = {o[x][0].x, o[x][0].y, o[x][0].z, o[x][0].w, o[x][1].x, o[x][1].y, o[x][1].z, o[x][1].w};
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
@@ -466,6 +468,21 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
                         acc[2 * e + 1] = fmaf(__uint_as_float(pairs[e] & 0xffff0000u), w, acc[2 * e + 1]);
                     }
                 }
+        }
+        if (scratch & kHasLowHalves) {                              // what the high halves leave of the parts computed from scratch
+#pragma unroll 1
+            for (int i = n_parts * run / kRuns; i < part_end; ++i) {
+                const size_t slot = slot_of(i);
+                const float mp = ws.part_m[slot];
+                if (mp == -INFINITY || !(__float_as_uint(ws.part_l[slot]) & kHasLowHalves)) continue;
+                const float w = exp2f(mp - m);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const uint32_t high = (uint32_t)reinterpret_cast<const uint16_t*>(part_o)[slot * kD + e] << 16;
+                    const float part = __uint_as_float(high), rest = __uint_as_float(high | ws.part_low[slot * kD + e0 + e]) - part;
+                    acc[e] = fmaf(fabsf(part) < INFINITY ? rest : 0.f, w, acc[e]);
+                }
+            }
         }
         if (kRuns > 1) {
             if (run > 0) {

@@ -129,9 +129,10 @@ struct AttnWorkspace {
     float* part_o;     // [L*B][n_splits][Hq*Lq][D] sum_t 2^(t - m) v_t, not normalised (unset if m = -inf)
     float* part_m;     // [L*B][n_splits][Hq*Lq]    reference maximum m (-inf if the part is empty)
     float* part_l;     // [L*B][n_splits][Hq*Lq]    sum_t 2^(t - m)
+    uint16_t* part_low; // [slots][D]               tensor-core path: low halves of part_o's numbers, of rows that have them
     float* tile_lse2;  // [L][max_tiles][Hq*Lq]     log2 of sum over the tile's tokens of 2^t
     float* row_lse2;   // [L*B][Hq*Lq]              log2 of the full softmax denominator
-    int* marks;        // [shares][8]               tensor-core path: what a share leaves for the merge (ShareHead, cf_attn_tc.cu)
+    int* marks;        // [shares][8]               tensor-core path: what a share leaves for the merge (ShareHead, cf_attn_line.cuh)
     int n_splits;
     int n_layers;
     int max_tiles;     // tile slots per layer in tile_lse2
@@ -146,10 +147,11 @@ struct AttnWorkspace {
     float* part_ld;    // like part_l, the documents' keys only (tensor-core path with further key blocks)
     int self_mode;
 };
+// low_halves = false: without part_low (the size that a limit stands on).
 // part_layers > 0: the partial results (and the further key blocks' buffers) are sized for that many layers only, the
 // per-tile and per-row log-sum-exps for n_layers (calls that fill one layer slot at a time and score the slots later).
 size_t attn_workspace_layout(const cf_geom* g, const cf_batch* b, int n_splits, int n_layers, bool with_self,
-                             AttnWorkspace* ws, void* base, int part_layers = 0);
+                             AttnWorkspace* ws, void* base, int part_layers = 0, bool low_halves = true);
 
 // Where the layers of a call sit (element strides between consecutive layers).
 struct LayerSpan {

@@ -7,11 +7,13 @@
 
 namespace cf {
 
-
 // The scratch itself.  Every GPU that loads this library holds these bytes until the process
 // exits.  In host code `g_static_scratch` is only a handle: the device address comes from
 // cudaGetSymbolAddress (static_scratch_address below).
-static __device__ __align__(256) unsigned char g_static_scratch[CF_STATIC_WORKSPACE_BYTES];
+// The limit stands on what a call needs without the low halves of partial results, which have room of their own behind it.
+constexpr size_t kLowHalvesBytes = 10u << 20;          // a call's: 2 x 128 rows of 256 bytes per SM
+constexpr size_t kStaticBytes = CF_STATIC_WORKSPACE_BYTES + kLowHalvesBytes;
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
 static std::mutex g_static_mutex;
 static void* g_static_address[kMaxDevices] = {};
@@ -30,6 +32,12 @@ static int static_scratch_address(void** out) {
     return CF_OK;
 }
 
+static bool static_scratch_fits(const cf_geom* geom, const cf_batch* batch) {
+    const int splits = choose_splits(geom, batch, 1);
+    return attn_workspace_layout(geom, batch, splits, 1, false, nullptr, nullptr, 0, false) <= (size_t)CF_STATIC_WORKSPACE_BYTES &&
+           attn_workspace_layout(geom, batch, splits, 1, false, nullptr, nullptr) <= kStaticBytes;
+}
+
 }  // namespace cf
 
 using namespace cf;
@@ -41,14 +49,12 @@ extern "C" int cf_query_prefill_attn_static(const cf_geom* geom, const cf_batch*
     if (!batch || !plan) return CF_ERR_INVALID_ARG;
     int rc = validate(geom, batch);
     if (rc != CF_OK) return rc;
-    if (attn_workspace_layout(geom, batch, choose_splits(geom, batch, 1), 1, false, nullptr, nullptr) >
-        (size_t)CF_STATIC_WORKSPACE_BYTES)
-        return CF_ERR_WORKSPACE;            // this batch needs more scratch than the library carries
+    if (!static_scratch_fits(geom, batch)) return CF_ERR_WORKSPACE;     // this batch needs more scratch than the library carries
     void* scratch = nullptr;
     rc = static_scratch_address(&scratch);
     if (rc != CF_OK) return rc;
     const LayerSpan span = {1, 0, 0, 0};
     return run_attn_layers(geom, batch, plan, span, q, k_cache, v_cache, nullptr, nullptr, 0, softmax_scale, out, lse,
-                           doc_scores, score_accum, scratch, (size_t)CF_STATIC_WORKSPACE_BYTES,
+                           doc_scores, score_accum, scratch, kStaticBytes,
                            static_cast<cudaStream_t>(stream));
 }
