@@ -36,6 +36,11 @@ int cf_profile_end(float* ms, int32_t capacity, int32_t* count);
 int cf_debug_wait_timeout(const cf_geom* geom, const cf_batch* batch, void* plan, int64_t limit_cycles,
                           void* stream);
 
+/* What the tensor-core path's merge makes of a row's word in the workspace, by a launch of `n_ctas` attention CTAs,
+ * `ctas_per_share` (1 or 2) of them on a share: the CTA that holds the row's first part (-1: the row was not cut) and the
+ * number of parts that are read from there on, one of every share (none where it is not positive).  Host arithmetic only. */
+int cf_debug_cut_row(uint32_t word, int32_t n_ctas, int32_t ctas_per_share, int32_t* first, int32_t* n_parts);
+
 #ifdef __cplusplus
 }
 #endif

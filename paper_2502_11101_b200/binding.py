@@ -34,7 +34,8 @@ EXPORTS = ["cf_error_string", "cf_allocate_positions", "cf_schedule_linear", "cf
            "cf_attn_workspace_bytes_full", "cf_query_prefill_attn_full", "cf_query_prefill_attn_prefix", "cf_assemble_final_cache", "cf_merge_attn",
            "cf_query_prefill_attn_static", "cf_prune_topk", "cf_prune_topk_host", "cf_run_stack_workspace_bytes",
            "cf_run_stack", "cf_document_prefill_attn", "cf_decode_plan_bytes", "cf_decode_plan", "cf_decode_status",
-           "cf_decode_workspace_bytes", "cf_decode_attn", "cf_decode_append", "cf_set_attn_path", "cf_profile_begin", "cf_profile_end", "cf_debug_wait_timeout"]
+           "cf_decode_workspace_bytes", "cf_decode_attn", "cf_decode_append", "cf_set_attn_path", "cf_profile_begin", "cf_profile_end", "cf_debug_wait_timeout",
+           "cf_debug_cut_row"]
 _SIZE_T_EXPORTS = ("cf_attn_workspace_bytes", "cf_attn_workspace_bytes_layers", "cf_attn_workspace_bytes_full",
                    "cf_attn_workspace_bytes_slots", "cf_attn_workspace_bytes_slots_full",
                    "cf_run_stack_workspace_bytes", "cf_decode_plan_bytes", "cf_decode_workspace_bytes")
@@ -147,6 +148,7 @@ def load_library() -> ctypes.CDLL:
     lib.cf_run_stack_workspace_bytes.argtypes = [gp, bp, sp]
     lib.cf_run_stack.argtypes = [gp, bp, sp, vp, ctypes.c_size_t, vp, ctypes.c_size_t, vp]
     lib.cf_debug_wait_timeout.argtypes = [gp, bp, vp, i64, vp]
+    lib.cf_debug_cut_row.argtypes = [ctypes.c_uint32, i32, i32, vp, vp]
     lib.cf_document_prefill_attn.argtypes = [gp, ctypes.POINTER(cf_doc_batch), i32, vp, i64, vp, vp, i64, vp, vp, i64,
                                              ctypes.c_float, vp, i64, vp, vp, vp]
     lib.cf_decode_plan_bytes.restype = ctypes.c_size_t
@@ -535,6 +537,13 @@ def cf_document_prefill_attn(geom: cf_geom, doc_offsets: torch.Tensor, max_doc_l
 def cf_debug_wait_timeout(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, limit_cycles: int, stream=None) -> None:
     _check(load_library().cf_debug_wait_timeout(ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(),
                                                 limit_cycles, _stream(stream)), "cf_debug_wait_timeout")
+
+
+def cf_debug_cut_row(word: int, n_ctas: int, ctas_per_share: int) -> Tuple[int, int]:
+    """(first CTA or -1, parts read) of a row's word in the workspace of the tensor-core path."""
+    first, n_parts = ctypes.c_int32(), ctypes.c_int32()
+    _check(load_library().cf_debug_cut_row(word, n_ctas, ctas_per_share, ctypes.byref(first), ctypes.byref(n_parts)), "cf_debug_cut_row")
+    return first.value, n_parts.value
 
 
 def cf_set_attn_path(path: int) -> None:

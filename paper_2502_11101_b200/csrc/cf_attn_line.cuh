@@ -195,9 +195,16 @@ struct Params {
 constexpr uint32_t kPartsOf = 0xffc00000u;
 constexpr int kMaxCodedShares = 1 << 10;
 __device__ __forceinline__ uint32_t parts_code(int share, int n_parts) { return kPartsOf | ((uint32_t)n_parts << 10) | (uint32_t)share; }
-__device__ __forceinline__ bool is_parts_code(uint32_t w) { return (w & kPartsOf) == kPartsOf; }
-__device__ __forceinline__ int first_share(uint32_t w) { return (int)(w & (kMaxCodedShares - 1)); }
-__device__ __forceinline__ int part_count(uint32_t w) { return (int)((w ^ kPartsOf) >> 10); }
+__host__ __device__ __forceinline__ bool is_parts_code(uint32_t w) { return (w & kPartsOf) == kPartsOf; }
+__host__ __device__ __forceinline__ int first_share(uint32_t w) { return (int)(w & (kMaxCodedShares - 1)); }
+__host__ __device__ __forceinline__ int part_count(uint32_t w) { return (int)((w ^ kPartsOf) >> 10); }
+// Parts that a merge may read from CTA `first` on, of `all` CTAs every one or every second (`ctas` to a share), where it was told of n.  A CTA whose wait ran out writes no
+// words for its rows, so that a merge by units finds what the workspace held before: its results are not used (CF_ERR_TIMEOUT), its
+// reads have to stay inside the workspace.  (A merge by shares needs no such bound, since that CTA leaves no ShareHead.)
+__host__ __device__ __forceinline__ int bounded_parts(int first, int n, int all, int ctas) {
+    const int most = (all - 1 - first >> (ctas == 2 ? 1 : 0)) + 1;      // (0 or less where there is no such CTA)
+    return n < most ? n : most;
+}
 
 // A part computed from scratch is left in fp32, as the halves of its numbers, and its sum (never negative) says so by its sign: such
 // rows are rounded to bf16 once, as results.  (Left in bf16 like other parts, whose probabilities are bf16 too, results of nine to

@@ -390,7 +390,7 @@ attn_pair_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__
     cluster_sync();
     if (tid == 0) {
         ShareHead head = {};
-        if (n_items > 0) head = sh.head;
+        if (n_items > 0 && !bars.abort_flag) head = sh.head;       // (as in cf_attn_tc.cu)
         reinterpret_cast<ShareHead*>(ws.marks)[blockIdx.x] = head;
     }
     // every copy has landed and every MMA has read its operands: the rings are free

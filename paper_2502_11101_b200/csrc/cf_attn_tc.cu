@@ -330,7 +330,7 @@ attn_tc_kernel(const __grid_constant__ StoreMaps maps, const __grid_constant__ P
     __syncthreads();
     if (tid == 0) {
         ShareHead head = {};
-        if (n_items > 0) head = sh.head;
+        if (n_items > 0 && !bars.abort_flag) head = sh.head;       // (roles that gave up may not have come to the share's last segment)
         reinterpret_cast<ShareHead*>(ws.marks)[blockIdx.x] = head;
     }
     // every copy has landed and every MMA has read its operands: the rings are free
@@ -402,8 +402,8 @@ attn_tc_merge_kernel(const __grid_constant__ Params p) {
         }
         if (!is_parts_code(word)) return;                           // finished by its one share
         __syncthreads();                                            // every thread has its word: a row's is written below
-        head.n_parts = part_count(word);
-        share = first_share(word);
+        share = first_share(word);                                  // (the CTA, for pairs that of this tile of rows)
+        head.n_parts = bounded_parts(share, part_count(word), p.max_shares, p.ctas);
     } else {
         const int4* from = reinterpret_cast<const int4*>(reinterpret_cast<const ShareHead*>(ws.marks) + share);
         const int4 lo = from[0], hi = from[1];
@@ -543,6 +543,13 @@ __global__ void __launch_bounds__(128) wait_probe_kernel(int* status, long long 
 }
 
 }  // namespace
+
+extern "C" int cf_debug_cut_row(uint32_t word, int32_t n_ctas, int32_t ctas_per_share, int32_t* first, int32_t* n_parts) {
+    if (n_ctas <= 0 || (ctas_per_share != 1 && ctas_per_share != 2) || !first || !n_parts) return CF_ERR_INVALID_ARG;
+    *first = is_parts_code(word) ? first_share(word) : -1;
+    *n_parts = is_parts_code(word) ? bounded_parts(*first, part_count(word), n_ctas, ctas_per_share) : 0;
+    return CF_OK;
+}
 
 int launch_wait_probe(const PlanView& pv, long long limit_cycles, cudaStream_t stream) {
     wait_probe_kernel<<<1, 128, 0, stream>>>(pv.status, limit_cycles);

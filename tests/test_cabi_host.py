@@ -323,3 +323,20 @@ def test_both_marshallers_refuse_the_same_calls(lib):
             except AssertionError:
                 got.append(AssertionError)
         assert got[0] == got[1] and got[0] not in (0, (0, 0)), (name, got)
+
+
+@pytest.mark.parametrize("n_ctas,per_share", [(148, 1), (148, 2), (1, 1), (2, 2), (132, 2), (1024, 1)])
+def test_a_merge_reads_parts_of_the_launch_only(lib, n_ctas, per_share):
+    """Whatever the workspace holds: after a wait that ran out, rows of a call have words of earlier ones or none at all."""
+    rng = np.random.default_rng(n_ctas)
+    code = lambda first, n: 0xFFC00000 | (n << 10) | first
+    words = [0xFFFFFFFF, 0xFFC00000, 0x7FFFFFFF, 0, code(n_ctas - 1, 2), code(n_ctas % 1024, 1), code(0, 4095)]
+    words += [int(w) for w in rng.integers(0, 1 << 32, 200, dtype=np.uint64)] + [0xFFC00000 | int(w) for w in rng.integers(0, 1 << 22, 500)]
+    for word in words:
+        first, n = cf.cf_debug_cut_row(word, n_ctas, per_share)
+        assert (first == -1 and n == 0) if word >> 22 != 0x3FF else first == word & 1023
+        assert n <= 0 or (first + (n - 1) * per_share < n_ctas), hex(word)
+    for first in range(0, n_ctas, 7):                        # what an attention kernel writes is read as it stands
+        n = (n_ctas - 1 - first) // per_share + 1
+        assert cf.cf_debug_cut_row(code(first, n), n_ctas, per_share) == (first, n)
+        assert cf.cf_debug_cut_row(code(first, 1), n_ctas, per_share) == (first, 1)
