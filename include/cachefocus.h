@@ -83,7 +83,8 @@ typedef struct cf_batch {
     int32_t tail_reserve;      /* positions kept free after query_start (query + new tokens)     */
     int32_t n_reuse;           /* number of parallel windows; 0 = Eq. 6                          */
     int32_t tiles_hint;        /* upper bound of live key tiles per request (0 = derive from
-                                  total_tokens); only steers grid sizes, never correctness       */
+                                  total_tokens); steers grid sizes and which attention kernel
+                                  runs, whose results agree within rounding, never correctness   */
     int32_t reserved;
     int64_t total_tokens;      /* rows in one layer of the store                                 */
     int64_t token_stride;      /* elements between consecutive rows, >= n_kv_heads*head_dim      */

@@ -36,6 +36,12 @@ int cf_profile_end(float* ms, int32_t capacity, int32_t* count);
 int cf_debug_wait_timeout(const cf_geom* geom, const cf_batch* batch, void* plan, int64_t limit_cycles,
                           void* stream);
 
+/* Which attention kernel a call over `n_layers` layers takes, with `prefix_len` rows of a prefix cache and, if with_self is
+ * not 0, the query tokens' own keys: 0 = CUDA cores, 1 = tensor cores, a CTA per tile of query rows, 2 = tensor cores, a pair
+ * of CTAs per two tiles.  (Without a GPU: for 148 multiprocessors.) */
+int cf_debug_attn_kernel(const cf_geom* geom, const cf_batch* batch, int32_t n_layers, int32_t prefix_len, int32_t with_self,
+                         int32_t* which);
+
 /* What the tensor-core path's merge makes of a row's word in the workspace, by a launch of `n_ctas` attention CTAs,
  * `ctas_per_share` (1 or 2) of them on a share: the CTA that holds the row's first part (-1: the row was not cut) and the
  * number of parts that are read from there on, one of every share (none where it is not positive).  Host arithmetic only. */

@@ -35,7 +35,7 @@ EXPORTS = ["cf_error_string", "cf_allocate_positions", "cf_schedule_linear", "cf
            "cf_query_prefill_attn_static", "cf_prune_topk", "cf_prune_topk_host", "cf_run_stack_workspace_bytes",
            "cf_run_stack", "cf_document_prefill_attn", "cf_decode_plan_bytes", "cf_decode_plan", "cf_decode_status",
            "cf_decode_workspace_bytes", "cf_decode_attn", "cf_decode_append", "cf_set_attn_path", "cf_profile_begin", "cf_profile_end", "cf_debug_wait_timeout",
-           "cf_debug_cut_row"]
+           "cf_debug_attn_kernel", "cf_debug_cut_row"]
 _SIZE_T_EXPORTS = ("cf_attn_workspace_bytes", "cf_attn_workspace_bytes_layers", "cf_attn_workspace_bytes_full",
                    "cf_attn_workspace_bytes_slots", "cf_attn_workspace_bytes_slots_full",
                    "cf_run_stack_workspace_bytes", "cf_decode_plan_bytes", "cf_decode_workspace_bytes")
@@ -148,6 +148,7 @@ def load_library() -> ctypes.CDLL:
     lib.cf_run_stack_workspace_bytes.argtypes = [gp, bp, sp]
     lib.cf_run_stack.argtypes = [gp, bp, sp, vp, ctypes.c_size_t, vp, ctypes.c_size_t, vp]
     lib.cf_debug_wait_timeout.argtypes = [gp, bp, vp, i64, vp]
+    lib.cf_debug_attn_kernel.argtypes = [gp, bp, i32, i32, i32, vp]
     lib.cf_debug_cut_row.argtypes = [ctypes.c_uint32, i32, i32, vp, vp]
     lib.cf_document_prefill_attn.argtypes = [gp, ctypes.POINTER(cf_doc_batch), i32, vp, i64, vp, vp, i64, vp, vp, i64,
                                              ctypes.c_float, vp, i64, vp, vp, vp]
@@ -537,6 +538,14 @@ def cf_document_prefill_attn(geom: cf_geom, doc_offsets: torch.Tensor, max_doc_l
 def cf_debug_wait_timeout(geom: cf_geom, batch: cf_batch, plan: torch.Tensor, limit_cycles: int, stream=None) -> None:
     _check(load_library().cf_debug_wait_timeout(ctypes.byref(geom), ctypes.byref(batch), plan.data_ptr(),
                                                 limit_cycles, _stream(stream)), "cf_debug_wait_timeout")
+
+
+def cf_debug_attn_kernel(geom: cf_geom, batch: cf_batch, n_layers: int, prefix_len: int = 0, with_self: bool = False) -> int:
+    """Which attention kernel a call takes: 0 CUDA cores, 1 tensor cores, 2 tensor cores by pairs of CTAs."""
+    which = ctypes.c_int32()
+    _check(load_library().cf_debug_attn_kernel(ctypes.byref(geom), ctypes.byref(batch), n_layers, prefix_len, int(with_self),
+                                               ctypes.byref(which)), "cf_debug_attn_kernel")
+    return which.value
 
 
 def cf_debug_cut_row(word: int, n_ctas: int, ctas_per_share: int) -> Tuple[int, int]:

@@ -575,11 +575,30 @@ size_t attn_tc_part_rows() { return (size_t)2 * sm_count() * kRowTile; }
 // Two tiles of rows, 32/8 heads: 25 documents (5) 31.7 / 31.7; 50 (11) 37.9 / 35.8; 4 x 50 (43) 74.7 / 60.4; four layers of 4 x 100 (346)
 // 419 / 292.  Four, 28/4: 25 (5) 31.7 / 31.7; 4 x 12 (10) 35.8 / 33.8; 4 x 50 (43) 72.7 / 58.4; 12/2, 50 (5) 29.7 / 31.7.  Three, 12/2:
 // 50 (5) 23.6 / 29.7; 4 x 100 (43) 58.4 / 58.4; four layers of that (173) 167 / 150; 28/4, 4 x 50 (43) 58.4 / 58.4; 4 x 100 (86) 95.2 /
-// 89.1.  Five, 28/4: 4 x 12 (16) 37.9 / 37.9; 4 x 50 (65) 85.0 / 74.7.  The tiles are those the host knows of, a bound.
+// 89.1.  Five, 28/4: 4 x 12 (16) 37.9 / 37.9; 4 x 50 (65) 85.0 / 74.7.  The tiles are those the host knows of, a bound.  Without a hint
+// that is all documents, however few are left (30 of 4 x 100 kept, 12/2, three tiles: 25.0 / 28.4; 3 kept: 12.5 / 15.0): an odd number,
+// which gains a tenth at most, then stays alone.  An even one gains up to a third and loses 1 to 2 us with three kept (32/8, 3 of
+// 4 x 100: 17.0 / 18.9).
 static bool work_in_pairs(const cf_geom* g, const cf_batch* b, int n_layers, long long row_tiles, int more_tiles) {
     const long long documents = std::min((long long)b->n_requests * tiles_per_request_bound(b), (long long)b->n_docs_total + b->total_tokens / kTile + 1);
     const long long tiles = (documents + (long long)b->n_requests * more_tiles) * g->n_kv_heads * n_layers * ((row_tiles + 1) / 2);
-    return row_tiles > 1 && tiles >= (row_tiles % 2 ? 44 : 8) * (long long)(sm_count() / 2);
+    if (row_tiles % 2) return row_tiles > 1 && b->tiles_hint > 0 && tiles >= 44LL * (sm_count() / 2);
+    return tiles >= 8LL * (sm_count() / 2);
+}
+
+static int more_tiles(const cf_batch* b, int prefix_len, bool with_self) {
+    return (prefix_len + kTile - 1) / kTile + (with_self ? (b->q_len + kTile - 1) / kTile : 0);
+}
+
+extern "C" int cf_debug_attn_kernel(const cf_geom* geom, const cf_batch* batch, int32_t n_layers, int32_t prefix_len, int32_t with_self, int32_t* which) {
+    if (!batch || !which || n_layers <= 0 || prefix_len < 0) return CF_ERR_INVALID_ARG;
+    const int rc = validate(geom, batch);
+    if (rc != CF_OK) return rc;
+    const int rg_rows = attn_tc_row_tile(geom, batch);
+    const long long rows = (long long)(geom->n_q_heads / geom->n_kv_heads) * batch->q_len;
+    *which = attn_path() != 0 || !attn_tc_supported(geom, batch) ? 0
+             : work_in_pairs(geom, batch, n_layers, (rows + rg_rows - 1) / rg_rows, more_tiles(batch, prefix_len, with_self != 0)) ? 2 : 1;
+    return CF_OK;
 }
 
 int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, const LayerSpan& span, const void* q,
@@ -589,7 +608,7 @@ int launch_attn_tc(const cf_geom* g, const cf_batch* b, const PlanView& pv, cons
     const int group = g->n_q_heads / g->n_kv_heads;
     long long row_tiles = ((long long)group * b->q_len + ws.rg_rows - 1) / ws.rg_rows;
     const int n_prefix = (prefix_len + kTile - 1) / kTile, n_self = k_self ? (b->q_len + kTile - 1) / kTile : 0;
-    const int ctas = work_in_pairs(g, b, span.n_layers, row_tiles, n_prefix + n_self) ? 2 : 1;       // of a share
+    const int ctas = work_in_pairs(g, b, span.n_layers, row_tiles, more_tiles(b, prefix_len, k_self != nullptr)) ? 2 : 1;      // of a share
     row_tiles = (row_tiles + ctas - 1) / ctas;                      // units of a kv head
     // the line's positions are 32-bit
     const long long most = ((long long)pv.max_tiles + (long long)b->n_requests * (prefix_len / kTile + b->q_len / kTile + 2)) *

@@ -55,7 +55,7 @@ std::vector<Call> calls_of(const cf_stack* st) {
 }
 
 // Upper bound of the key tiles a request can own while it keeps at most `keep` documents: the tile
-// counts of its `keep` longest documents (only steers grid sizes).  0 when the lengths are unknown.
+// counts of its `keep` longest documents (steers grid sizes and the choice of the attention kernel).  0 when the lengths are unknown.
 int live_tiles_hint(const cf_batch* b, const cf_stack* st, int keep) {
     if (!st->doc_len_host || !st->req_doc_begin_host) return b->tiles_hint;
     int worst = 1;

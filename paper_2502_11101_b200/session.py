@@ -53,7 +53,8 @@ class Session:
         self.score_accum = torch.zeros(self.n_docs_total, dtype=torch.float32, device=self.device)
 
     def set_live_docs(self, kept_per_request: int) -> None:
-        """Tell the library how many documents a request can still hold (sizes kernel grids only):
+        """Tell the library how many documents a request can still hold (sizes kernel grids and chooses
+        between attention kernels whose results agree within rounding):
         the hint is the tile count of the `kept_per_request` longest documents of any request."""
         k = max(0, min(kept_per_request, self.n_docs_total))
         self.batch.tiles_hint = max(1, int(self._live_tiles[k]))

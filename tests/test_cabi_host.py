@@ -340,3 +340,19 @@ def test_a_merge_reads_parts_of_the_launch_only(lib, n_ctas, per_share):
         n = (n_ctas - 1 - first) // per_share + 1
         assert cf.cf_debug_cut_row(code(first, n), n_ctas, per_share) == (first, n)
         assert cf.cf_debug_cut_row(code(first, 1), n_ctas, per_share) == (first, 1)
+
+
+@pytest.mark.parametrize("heads,q_len,docs,kept,layers,hinted,unhinted", [
+    ((12, 2), 48, 400, 120, 1, 1, 1),      # three tiles of query rows, few documents left: no pairs without a word about them
+    ((12, 2), 48, 400, 400, 4, 2, 1),      # all there: pairs where the caller says so
+    ((32, 8), 64, 400, 400, 1, 2, 2),      # two tiles
+    ((32, 8), 64, 400, 12, 1, 1, 2),       # an even number gains more than it can lose
+    ((12, 2), 20, 400, 400, 4, 1, 1),      # one tile
+])
+def test_pairs_of_ctas_where_they_pay(lib, heads, q_len, docs, kept, layers, hinted, unhinted):
+    geom = cf.make_geom(*heads, 128, cf.CF_BF16, 1 << 20, 1e4)
+    got = []
+    for hint in (2 * kept, 0):             # documents of 160 tokens are two tiles
+        batch = cf.cf_batch(1, docs, q_len, 0, q_len, 0, hint, 0, 160 * docs, heads[1] * 128, 256, 256, 256)
+        got.append(cf.cf_debug_attn_kernel(geom, batch, layers))
+    assert got == [hinted, unhinted]

@@ -17,8 +17,9 @@ def _library():
 
 
 def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_block=False, kept=None, peak=None,
-                peak_every=1, rope_layout=0):
-    """Outputs, log-sum-exps and scores of both kernel families on the same inputs."""
+                peak_every=1, rope_layout=0, kernel=None):
+    """Outputs, log-sum-exps and scores of both kernel families on the same inputs; `kernel`: the tensor-core one that has to run
+    (1: a CTA per tile of query rows, 2: pairs)."""
     import paper_2502_11101_b200 as cf
     from paper_2502_11101_b200.session import Session
     b = len(docs_per_request)
@@ -38,6 +39,7 @@ def _both_paths(heads, q_len, lens, docs_per_request, layers=1, prefix=0, self_b
             cf.cf_set_attn_path(path)
             sess = Session(hq, hkv, 128, torch.bfloat16, 32768, 1e6, q_len, np.asarray(lens, np.int32), begin,
                            np.zeros(len(lens), np.int32), tail_reserve=q_len, prefix_len=prefix, rope_layout=rope_layout)
+            assert path == 1 or kernel is None or cf.cf_debug_attn_kernel(sess.geom, sess.batch, layers, prefix, self_block) == kernel
             counts = None if kept is None else torch.tensor(kept, dtype=torch.int32, device="cuda")
             sess.init(kept_count=counts)
             out = torch.full_like(q, float("nan"))

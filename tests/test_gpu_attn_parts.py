@@ -43,6 +43,7 @@ def test_scores_of_documents_far_below_the_prefix(heads, q_len, docs, layers, ab
     hq, hkv = heads
     lens, prefix = [TILE] * sum(docs), 84 * TILE if len(docs) > 1 else 4 * TILE
     sess = _session(heads, q_len, lens, docs, prefix)
+    assert cf.cf_debug_attn_kernel(sess.geom, sess.batch, layers, prefix) == (2 if len(docs) > 1 else 1)
     gen = torch.Generator(device="cuda").manual_seed(7)
     rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
     b, total = len(docs), sum(lens)
@@ -78,6 +79,7 @@ def test_rows_from_scratch_are_rounded_once(heads, q_len, docs, every):
     hq, hkv = heads
     lens, total = [TILE] * sum(docs), TILE * sum(docs)
     sess = _session(heads, q_len, lens, docs)
+    assert cf.cf_debug_attn_kernel(sess.geom, sess.batch, 1) == (2 if docs[0] == 340 else 1)
     gen = torch.Generator(device="cuda").manual_seed(total)
     rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
     heavy = (torch.arange(total, device="cuda") % TILE >= 16) & (rand(total) > 0.7)
