@@ -26,10 +26,10 @@ struct StoreMaps {
     CUtensorMap kp, vp;                            // keys and values of a shared prefix cache (whole tiles)
 };
 
-// Tile descriptions: flags beside the length, and which keys they are.
 // Keys of a tile in either CTA of a pair: half of the MMA's columns, which come in 32s.
 __device__ __forceinline__ int pair_keys(int len) { return ((len + 31) >> 5) << 4; }
 
+// Tile descriptions: flags beside the length, and which keys they are.
 constexpr int kFirstOfSegment = 1 << 8, kLastOfSegment = 1 << 9;
 constexpr int kKindPrefix = -1, kKindSelf = -2;    // tile index of a prefix tile; kKindSelf - n: n-th tile of the query tokens
 
@@ -122,7 +122,7 @@ __device__ __forceinline__ Line make_line(const BatchView& bv, const AttnWorkspa
     return line;
 }
 
-// `rank`: of the CTA in a pair, which has two neighbouring tiles of query rows as its unit.
+// PAIR: a unit is two neighbouring tiles of query rows, of which either CTA of a pair (blockIdx.x & 1) has one.
 template <bool PAIR>
 __device__ __forceinline__ Segment segment_at(const BatchView& bv, const PlanView& pv, const AttnWorkspace& ws, const Line& line, int group,
                                               int x, int end) {
@@ -176,7 +176,7 @@ struct RowSources {
     int with_self, prefix_len;
 };
 
-// Everything a kernel of this file is told: one constant, so that the rarely taken paths can be handed its address.
+// Everything the attention and merge kernels are told: one constant, so that the rarely taken paths can be handed its address.
 struct Params {
     BatchView bv;
     PlanView pv;
@@ -417,7 +417,8 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
 // calls over 50 documents, 12/2 heads 574 -> 559.  Calls with such rows: four layers of 50 documents of 160 tokens, 12/2 heads, 44 us
 // without, one row a layer 166 -> 79, every row 759 -> 398; one layer of 2 x 60 documents of 180, 32/32 heads, 93 us, 265 -> 166 and
 // 1109 -> 646; of 4 x 50 of 160, 28/4 heads, 75 us
-// (64 in pairs), 202 -> 128 and 687 -> 732 (few tiles per share leave warps idle, and a pair's kernel has registers for fewer).
+// (64 in pairs), 202 -> 128 and 687 -> 732 (few tiles per share leave warps idle, and this path is where a pair's kernel spills: 96
+// registers, 76 to 80 bytes of stores and 120 to 128 of loads, none without it).
 template <int LAYOUT, bool PAIR>
 __device__ __forceinline__ void marked_from_scratch(const Params& p, RowScratch& sh, const Line& line) {
     const int group = p.n_q_heads / p.n_kv_heads, share = blockIdx.x >> (PAIR ? 1 : 0);

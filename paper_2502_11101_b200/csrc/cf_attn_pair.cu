@@ -17,10 +17,12 @@
 // wait for the values before them; 4 S buffers instead of 3 1620; loads and MMAs by warps of their own 1600, now bound by rotation,
 // eight warps on one tile; rotation a tile per warp 1520, bound by two softmax warpgroups (2500 per tile and 500 between tiles each);
 // three warpgroups 1250, where their exponentials take half of the MUFU's time.  32 keys to a softmax chunk instead of 16: no gain.
-// Barriers the MMA warps wait on are those of the first CTA.  An arrival from the second is an ordinary one (release at CTA scope):
-// what it orders are writes to its own shared and tensor memory, made visible by fence.proxy.async and the tcgen05 fences, which
-// its own SM's tensor core reads.  (With release at cluster scope an arrival waits for the thread's global stores: 2870 cycles per
-// tile.)  No CTA leaves, and none computes rows from scratch over its rings, before the other is done with the barriers.
+// Barriers the MMA warps wait on are those of the first CTA.  An arrival from the second is an ordinary one (release at CTA scope).
+// By the letter of the memory model that does not order the second CTA's writes for a thread of the first; that it is enough here is
+// an assumption about the hardware: what has to be ordered are writes to the second CTA's own shared and tensor memory, which fence.proxy.async
+// and the tcgen05 fences have completed for its own SM's tensor core before the arrival is issued, and nobody else reads them.  Release at
+// cluster scope costs more than pairs gain, since it waits for global stores: 2870 cycles per tile from the warps themselves, and from
+// one relaying warp per barrier that stores nothing itself 89 -> 134 us a call (4 x 100 documents, 32/8 heads).  No CTA leaves, and none computes rows from scratch over its rings, before the other is done with the barriers.
 #include "cf_attn_roles.cuh"
 
 namespace cf {

@@ -65,11 +65,16 @@ __device__ __forceinline__ void rotate_rows(unsigned char* base, int key_half, c
 
 // R: the rings of the kernel; SHARED: its shared memory (barriers, tile descriptions, segments, references).  `query`: where a pair's
 // query tile lies in shared memory.  Two warpgroups load the query tile and take finished rows out.
+// Where the groups do not divide the stages a warpgroup skips phases of s_full[k]: it meets tile t there and then tile t + stages *
+// groups.  Its wait for tile t can still not pass on the parity of tile t - stages, whose phase is over by then: the warpgroup has seen
+// S(t - groups), which was issued once PV(t - groups - buffers) had read its S buffer, and PVs are issued in order, each behind the
+// softmax of its tile, which has waited for that tile's S.
 template <class R, class SHARED>
 __device__ __forceinline__ void softmax_role(const Params& p, SHARED& sh, Sums<R::kSoftmaxGroups>& sums, unsigned char* query, uint32_t tmem, int share, int x_end,
                                              int n_items) {
     CF_PARAMS;
     constexpr bool PAIR = R::kPair;
+    static_assert(R::kKStages % R::kSoftmaxGroups == 0 || R::kKStages >= R::kSoftmaxGroups + R::kSBuffers, "the phase before a tile's is over");
     constexpr int kSoftmaxGroups = R::kSoftmaxGroups, kKStages = R::kKStages, kSBuffers = R::kSBuffers;
     constexpr uint32_t kColO = R::kColO, kColQ = R::kColQ, kColS = R::kColS;
     const Line& line = sh.line;

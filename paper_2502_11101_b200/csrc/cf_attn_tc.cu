@@ -30,7 +30,8 @@
 // waits for a chain.
 // Every wait on an mbarrier is bounded; when a wait expires the CTA raises CF_ERR_TIMEOUT in the plan's status word, all
 // roles leave their loops, and the CTA frees its tensor memory and exits.  Each barrier has one kind of waiter, which waits
-// for every phase in order.
+// for every phase in order, since a wait for a parity passes early where it skipped one (what a pair's softmax does instead stands at
+// softmax_role).
 #include <algorithm>
 
 #include "cf_attn_roles.cuh"
@@ -83,6 +84,7 @@ struct Shared {
 };
 constexpr int kSmemBytes = (kKStages + kVStages) * kKvBytes + (int)sizeof(Shared) + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
+static_assert(sizeof(RowScratch) <= (kKStages + kVStages) * kKvBytes, "over the rings");
 
 template <int LAYOUT>
 __global__ void __launch_bounds__(kThreads, 1)

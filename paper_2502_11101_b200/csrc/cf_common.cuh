@@ -56,6 +56,7 @@ __host__ __device__ inline int tile_base(int doc_begin, int row_begin) {
 
 // Division of 0 <= n < 2^31 by a divisor the host knows: three dependent instructions instead of the thirty of a division whose
 // divisor comes out of a register (and over a hundred in 64 bits), on the way to the first load of kernels that run for 3 us.
+// Multiplication by the reciprocal and a shift (Granlund and Montgomery, Division by Invariant Integers using Multiplication, 1994).
 struct Divisor {
     unsigned d, mul, shift;
     Divisor() = default;

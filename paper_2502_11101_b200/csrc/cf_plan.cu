@@ -3,9 +3,6 @@
 // Sec. 2.5), and what the hot kernels consume: per-document rotation tables (Eq. 2 angles of
 // the delta of Eq. 5) and the list of key tiles.  One thread block per request; everything
 // runs in stream order so a layer stack needs no host round trip between layers.
-#ifndef UNR
-#define UNR 4
-#endif
 #include <algorithm>
 #include <cmath>
 

@@ -272,8 +272,7 @@ __device__ __forceinline__ void tmem_ld16_wait(uint32_t (&v)[16]) {
                  : "memory");
 }
 // Eight columns (16 packed bf16) of the P operand.
-template <int N>
-__device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t (&v)[N]) {
+__device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t (&v)[16]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
                  : : "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(taddr)
                  : "memory");
@@ -283,20 +282,6 @@ __device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t (&
 __device__ __forceinline__ void chunk16_exp(uint32_t (&v)[16], uint64_t scale2, uint64_t neg_ref2, uint64_t& sum2) {
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        float p0, p1;
-        unpack_f2(fma_f2(pack_f2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), scale2, neg_ref2), p0, p1);
-        p0 = fast_exp2(p0);
-        p1 = fast_exp2(p1);
-        sum2 = add_f2(sum2, pack_f2(p0, p1));
-        v[i >> 1] = pack_bf16(p0, p1);
-    }
-}
-
-// The same for columns FIRST .. FIRST + 15 of 32, packed into v[FIRST / 2 ..].
-template <int FIRST>
-__device__ __forceinline__ void chunk_exp(uint32_t (&v)[32], uint64_t scale2, uint64_t neg_ref2, uint64_t& sum2) {
-#pragma unroll
-    for (int i = FIRST; i < FIRST + 16; i += 2) {
         float p0, p1;
         unpack_f2(fma_f2(pack_f2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), scale2, neg_ref2), p0, p1);
         p0 = fast_exp2(p0);
