@@ -270,8 +270,10 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
     }
     const int n_splits = choose_splits(geom, batch, span.n_layers);
     AttnWorkspace ws;
+    const int path = g_attn_path.load();
+    const bool low_halves = decode_cache_rows == 0;   // a decoding step never comes to the tensor-core kernel
     const size_t need = slotted ? attn_workspace_layout(geom, batch, n_splits, n_slots, with_self || with_prefix, &ws, workspace, 1)
-                                : attn_workspace_layout(geom, batch, n_splits, span.n_layers, with_self || with_prefix, &ws, workspace);
+                                : attn_workspace_layout(geom, batch, n_splits, span.n_layers, with_self || with_prefix, &ws, workspace, 0, low_halves);
     if (workspace_bytes < need) return CF_ERR_WORKSPACE;
     if (slotted) {                                    // this call sees its slot as the one layer it has
         const size_t rows_total = (size_t)geom->n_q_heads * batch->q_len;
@@ -281,12 +283,12 @@ int run_attn_layers(const cf_geom* geom, const cf_batch* batch, const void* plan
     }
     const float scale = softmax_scale == 0.0f ? 1.0f / std::sqrt((float)geom->head_dim) : softmax_scale;
     PlanView pv = make_plan_view(geom, batch, const_cast<void*>(plan));
-    if (decode_cache_rows > 0 && g_attn_path.load() == 0 && decode_attn_supported(geom)) {
+    if (decode_cache_rows > 0 && path == 0 && decode_attn_supported(geom)) {
         if (workspace_bytes < decode_attn_workspace_bytes(geom, batch->n_requests, span.n_layers)) return CF_ERR_WORKSPACE;
         return launch_decode_attn(geom, batch->n_requests, decode_cache_rows, span.n_layers, batch->doc_offsets, span, q, k_cache,
                                   v_cache, scale * kLog2e, out, lse, workspace, s);
     }
-    const bool tensor_core = g_attn_path.load() == 0 && attn_tc_supported(geom, batch);
+    const bool tensor_core = path == 0 && low_halves && attn_tc_supported(geom, batch);
     if (with_self && batch->q_len > 128) return CF_ERR_UNSUPPORTED;
     if (!tensor_core) ws.part_ld = nullptr;           // only the tensor-core kernel reports per-part document sums
     if ((with_self || with_prefix) && !tensor_core) { // the CUDA-core path computes these blocks as a part of their own

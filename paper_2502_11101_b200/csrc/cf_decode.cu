@@ -208,8 +208,9 @@ size_t cf_decode_workspace_bytes(const cf_geom* geom, int32_t n_requests, int32_
     cf_batch b;
     decode_views(geom, n_requests, cache_rows, a, &g, &b);
     b.req_doc_begin = b.doc_offsets = b.doc_src_start = reinterpret_cast<const int32_t*>(geom);
-    const size_t general = cf_attn_workspace_bytes_layers(&g, &b, n_layers);
-    return general == 0 || !decode_attn_supported(geom) ? general : general + decode_attn_workspace_bytes(geom, n_requests, n_layers);
+    if (cf_attn_workspace_bytes_layers(&g, &b, n_layers) == 0) return 0;
+    const size_t general = attn_workspace_layout(&g, &b, choose_splits(&g, &b, n_layers), n_layers, false, nullptr, nullptr, 0, false);
+    return decode_attn_supported(geom) ? general + decode_attn_workspace_bytes(geom, n_requests, n_layers) : general;
 }
 
 int cf_decode_attn(const cf_geom* geom, int32_t n_requests, int32_t cache_rows, const void* decode_plan,
