@@ -418,7 +418,11 @@ __device__ __forceinline__ void rows_from_scratch(const Params& p, RowScratch& s
 // without, one row a layer 166 -> 79, every row 759 -> 398; one layer of 2 x 60 documents of 180, 32/32 heads, 93 us, 265 -> 166 and
 // 1109 -> 646; of 4 x 50 of 160, 28/4 heads, 75 us
 // (64 in pairs), 202 -> 128 and 687 -> 732 (few tiles per share leave warps idle, and this path is where a pair's kernel spills: 96
-// registers, 76 to 80 bytes of stores and 120 to 128 of loads, none without it).
+// registers, 76 to 80 bytes of stores and 120 to 128 of loads, none without it).  With half of the rows out of range 4 x 50 documents,
+// 28/4 heads, took 242 us and take 273 to 277, 4 x 100 on 32/8 heads 456 and 486: shares of many such rows walk their keys once per eight.
+// Accuracy: a row that leaves its range in every share is off by 1.67e-3 of its size, one rounding, as when the merge computed it; one
+// that leaves it in some shares only has ordinary parts, of bf16 probabilities, in the others (two thirds of the shares: 1.67e-3 ->
+// 1.74e-3; rows that never leave it: 2.87e-3).
 template <int LAYOUT, bool PAIR>
 __device__ __forceinline__ void marked_from_scratch(const Params& p, RowScratch& sh, const Line& line) {
     const int group = p.n_q_heads / p.n_kv_heads, share = blockIdx.x >> (PAIR ? 1 : 0);
